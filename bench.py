@@ -38,8 +38,7 @@ L2_FLUSH_BYTES = 256 << 20
 # extra dM rho_ref part comes from the deviation form and is not counted as method work.
 KERNEL_FLOPS = {
     "gemm_M_f64": lambda N: 2 * N ** 3,
-    "gemm_Xre_f64": lambda N: 2 * N ** 3,
-    "gemm_Xim_f64": lambda N: 2 * N ** 3,
+    "gemm_X_f64": lambda N: 4 * N ** 3,
     "gemm_dM_f32": lambda N: 2 * N ** 3,
     "gemm_Xre_f32": lambda N: 2 * N ** 3,
     "gemm_Xim_f32": lambda N: 2 * N ** 3,

@@ -873,8 +873,7 @@ tdb_status md_forces(Ctx& c, int cur, bool first, int commit, int* n, StepTimer*
         if (n) *n += 7;
     } else {
         gemm_f64_ham(c.N, c.Sinv, c.H0, c.S, c.v_orb, c.M, c.stream);        // M = S^-1 H
-        gemm_f64(c.N, c.N, c.N, c.M, c.N, c.rho_re[cur], c.N, c.Xre, c.N, c.stream);
-        gemm_f64(c.N, c.N, c.N, c.M, c.N, c.rho_im[cur], c.N, c.Xim, c.N, c.stream);
+        gemm_f64_pair(c.N, c.M, c.rho_re[cur], c.rho_im[cur], c.Xre, c.Xim, c.stream);
     }
     MARK("md_forces");
     launch_wre(c.N, c.Xre, c.Wre, c.stream);
@@ -915,8 +914,7 @@ tdb_status enqueue_step_md(Ctx& c, int cur, bool euler, int* launches, StepTimer
         n += 3;
     } else {
         gemm_f64(c.N, c.N, c.N, c.Sinv, c.N, c.D, c.N, c.M, c.N, c.stream);   // Y = S^-1 D
-        gemm_f64(c.N, c.N, c.N, c.M, c.N, c.rho_re[cur], c.N, c.Zre, c.N, c.stream);
-        gemm_f64(c.N, c.N, c.N, c.M, c.N, c.rho_im[cur], c.N, c.Zim, c.N, c.stream);
+        gemm_f64_pair(c.N, c.M, c.rho_re[cur], c.rho_im[cur], c.Zre, c.Zim, c.stream);
     }
     const double factor = euler ? c.prm.dt : 2.0 * c.prm.dt;
     const double* bre = euler ? c.rho_re[cur] : c.rho_re[prv];
@@ -1139,11 +1137,9 @@ tdb_status enqueue_step(Ctx& c, int cur, bool euler, int* launches, StepTimer* t
     } else if (c.prm.precision == TDB_FP64) {
         MARK("gemm_M_f64");
         gemm_f64_ham(c.N, c.Sinv, c.H0, c.S, c.v_orb, c.M, c.stream);  // M = S^-1 H
-        MARK("gemm_Xre_f64");
-        gemm_f64(c.N, c.N, c.N, c.M, c.N, c.rho_re[cur], c.N, c.Xre, c.N, c.stream);
-        MARK("gemm_Xim_f64");
-        gemm_f64(c.N, c.N, c.N, c.M, c.N, c.rho_im[cur], c.N, c.Xim, c.N, c.stream);
-        n += 3;
+        MARK("gemm_X_f64");
+        gemm_f64_pair(c.N, c.M, c.rho_re[cur], c.rho_im[cur], c.Xre, c.Xim, c.stream);
+        n += 2;
         MARK("update");
         launch_update(c, c.Xre, c.Xim, bre, bim, c.rho_re[prv], c.rho_im[prv], factor, c.S,
                       c.partial, c.sc, c.stream);

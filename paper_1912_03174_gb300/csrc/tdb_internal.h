@@ -310,6 +310,9 @@ enum class BKind { Dense = 0, Hamiltonian = 1 };
 void gemm_f64(int M, int Ncol, int K, const double* A, int lda, const double* B, int ldb,
               double* C, int ldc, cudaStream_t st);
 // C = A * H with H_kj = H0_kj + 1/2 S_kj (v_k + v_j) formed while loading B (eq:hscc).
+// C0 = A B0 and C1 = A B1 (N x N) in one launch
+void gemm_f64_pair(int N, const double* A, const double* B0, const double* B1, double* C0,
+                   double* C1, cudaStream_t st);
 void gemm_f64_ham(int N, const double* A, const double* H0, const double* S, const double* v_orb,
                   double* C, cudaStream_t st);
 // FP32 SIMT: C = A * B (+ Cadd if non-null).
