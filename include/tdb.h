@@ -58,7 +58,8 @@ typedef enum {
 /* Arithmetic of the per-step matrix products (eq:eomrho).  The density matrix
  * master copy, charges, potentials, energies and forces are FP64 in every mode. */
 typedef enum {
-    TDB_FP64 = 0,     /* FP64 products (SIMT DFMA) */
+    TDB_FP64 = 0,     /* FP64 products: DFMA below N = 192, above it 55-bit integer slices on the
+                         tensor cores, summed exactly (N <= 4096; DFMA beyond) */
     TDB_FP32 = 1,     /* FP32 products (SIMT FFMA) on the deviation rho - rho_gs */
     TDB_BF16X3 = 2,   /* tcgen05 tensor cores, BF16 hi/lo pieces (~16 bits), 3 products,
                          FP32 accumulate, on the deviation rho - rho_gs */

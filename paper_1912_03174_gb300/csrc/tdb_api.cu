@@ -117,6 +117,16 @@ bool mixed(const Ctx& c) {
 bool md32(const Ctx& c) { return c.prm.move_nuclei && c.prm.precision == TDB_FP32; }
 // FP64-accurate integer-slice products (FP64 density and update), any nuclei.
 bool sliced(const Ctx& c) { return c.prm.precision == TDB_FP64_SLICED; }
+// FP64 form: from this size on its products run as integer slices (scheme kSeven), below it
+// as DFMA products.  A frozen SCC step with DFMA products / with slices, microseconds: 43 / 61
+// at N = 132, 53 / 63 at 160, 67.5 / 66.5 at 192, 98 / 69 at 224, 356 / 88 at 384; at
+// N = 1024 6324 / 265.  The slices pay two launches and their writes, the DFMA products
+// are bound by that pipe.
+constexpr int kSliceMinN = 192;
+bool use_slices(const Ctx& c) {
+    return sliced(c) || (c.prm.precision == TDB_FP64 && c.N >= kSliceMinN && c.N <= oz::kMaxK);
+}
+int slice_scheme(const Ctx& c) { return sliced(c) ? oz::kSix : oz::kSeven; }
 bool head3(const Ctx& c) { return c.prm.precision == TDB_FP16X6; }
 // The tensor-core X products (dM rho_ref, M Re(rho - rho_ref), M Im rho) are cut into
 // this many K slices with their own FP32 outputs, so that a slice of K <= 1024 keeps one
@@ -186,9 +196,9 @@ size_t carve(Ctx& c, char* base) {
         c.dv_f = k.take<float>(N);
         c.S_f = k.take<float>(NN);
     }
-    if (sliced(c)) {
+    if (use_slices(c)) {
         // slices of S^-1 (A), H or D (B), M or Y (A), Re rho and Im rho (B)
-        for (int q = 0; q < 5; ++q) c.oz_raw[q] = k.take<char>(oz::sliced_bytes(N, N));
+        for (int q = 0; q < 5; ++q) c.oz_raw[q] = k.take<char>(oz::sliced_bytes(N, N, slice_scheme(c)));
         c.oz_colmax = k.take<double>(N);
     }
     if (md32(c)) {
@@ -809,6 +819,31 @@ struct StepTimer {
 #define MARK(name) \
     if (tm) tm->mark(c.stream, name)
 
+// H of the current potential, sliced as a B operand (H is symmetric) without being stored
+oz::SliceJob ham_job(Ctx& c) {
+    oz::SliceJob j;
+    j.A = c.H0;
+    j.lda = c.N;
+    j.out = &c.oz[1];
+    j.S = c.S;
+    j.v = c.v_orb;
+    return j;
+}
+oz::SliceJob mat_job(const Ctx& c, const double* A, oz::Sliced& out, double sign = 1.0) {
+    oz::SliceJob j;
+    j.A = A;
+    j.lda = c.N;
+    j.sign = sign;
+    j.out = &out;
+    return j;
+}
+// M (A operand) and rho_n (B operands: Re rho symmetric, (Im rho)^T = -Im rho) in one launch
+void slice_m_rho(Ctx& c, int cur) {
+    const oz::SliceJob j[3] = {mat_job(c, c.M, c.oz[2]), mat_job(c, c.rho_re[cur], c.oz[3]),
+                               mat_job(c, c.rho_im[cur], c.oz[4], -1.0)};
+    oz::slice_rows(j, 3, c.stream);
+}
+
 // Sliced-form products: out = A B with A, B given through their slices (0: S^-1,
 // 1: H or D, 2: M or Y, 3: Re rho, 4: Im rho).
 tdb_status oz_product(Ctx& c, int a, int b, double* out) {
@@ -844,18 +879,14 @@ tdb_status md_forces(Ctx& c, int cur, bool first, int commit, int* n, StepTimer*
     launch_potential(c, c.gamma, c.dq, c.d_R, c.sc, c.v_orb, c.v_atom, c.gdq, c.hist, c.v_ref,
                      nullptr, c.stream);
     MARK("md_products_X");
-    if (sliced(c)) {
+    if (use_slices(c)) {
         // M = S^-1 H and X = M rho_n with integer-slice products (S^-1 sliced per step)
-        const int N = c.N;
-        launch_build_hamiltonian(N, c.H0, c.S, c.v_orb, c.Hs, c.stream);
-        oz::slice_rows(c.Sinv, N, 1.0, c.oz[0], c.stream);
-        oz::slice_rows(c.Hs, N, 1.0, c.oz[1], c.stream);          // H symmetric
+        const oz::SliceJob j[2] = {mat_job(c, c.Sinv, c.oz[0]), ham_job(c)};
+        oz::slice_rows(j, 2, c.stream);
         TRY(oz_product(c, 0, 1, c.M));
-        oz::slice_rows(c.M, N, 1.0, c.oz[2], c.stream);
-        oz::slice_rows(c.rho_re[cur], N, 1.0, c.oz[3], c.stream);  // Re rho symmetric
-        oz::slice_rows(c.rho_im[cur], N, -1.0, c.oz[4], c.stream); // (Im rho)^T = -Im rho
+        slice_m_rho(c, cur);
         TRY(oz_product_rho(c, 2, c.Xre, c.Xim));
-        if (n) *n += 5;
+        if (n) *n += 1;
     } else if (md32(c)) {
         // M = S^-1 H and X = M rho_n with FP32 operands and FFMA accumulation
         const int N = c.N;
@@ -894,7 +925,7 @@ tdb_status enqueue_step_md(Ctx& c, int cur, bool euler, int* launches, StepTimer
     int n = 0;
     TRY(md_forces(c, cur, euler, 1, &n, tm));
     MARK("md_products_Z");
-    if (sliced(c)) {
+    if (use_slices(c)) {
         // Y = S^-1 D (D is not symmetric: column slices) and Z = Y rho_n
         oz::slice_cols(c.D, c.N, c.oz[1], c.oz_colmax, c.stream);
         TRY(oz_product(c, 0, 1, c.M));
@@ -1116,20 +1147,17 @@ tdb_status enqueue_step(Ctx& c, int cur, bool euler, int* launches, StepTimer* t
                          nullptr, c.stream);
         ++n;
     }
-    if (sliced(c)) {
-        const int N = c.N;
+    if (use_slices(c)) {
         MARK("slice_H");
-        launch_build_hamiltonian(N, c.H0, c.S, c.v_orb, c.Hs, c.stream);
-        oz::slice_rows(c.Hs, N, 1.0, c.oz[1], c.stream);
+        const oz::SliceJob h = ham_job(c);
+        oz::slice_rows(&h, 1, c.stream);
         MARK("oz_gemm_M");
         TRY(oz_product(c, 0, 1, c.M));                          // M = S^-1 H
         MARK("slice_M_rho");
-        oz::slice_rows(c.M, N, 1.0, c.oz[2], c.stream);
-        oz::slice_rows(c.rho_re[cur], N, 1.0, c.oz[3], c.stream);
-        oz::slice_rows(c.rho_im[cur], N, -1.0, c.oz[4], c.stream);
+        slice_m_rho(c, cur);
         MARK("oz_gemm_X");
         TRY(oz_product_rho(c, 2, c.Xre, c.Xim));                // X = M rho
-        n += 7;
+        n += 4;
         MARK("update");
         launch_update(c, c.Xre, c.Xim, bre, bim, c.rho_re[prv], c.rho_im[prv], factor, c.S,
                       c.partial, c.sc, c.stream);
@@ -1451,11 +1479,12 @@ tdb_status tdb_create(const tdb_system* sys, const tdb_params* prm, void* worksp
         s = build_maps(*c);
         if (s != TDB_OK) return fail(s);
     }
-    if (sliced(*c)) {
+    if (use_slices(*c)) {
         const int N = c->N;
         bool ok = oz::prepare() == cudaSuccess;
         for (int q = 0; q < 5 && ok; ++q)
-            ok = oz::sliced_init(c->oz[q], c->oz_raw[q], N, N, q == 0 || q == 2 ? 128 : 64);
+            ok = oz::sliced_init(c->oz[q], c->oz_raw[q], N, N, q == 0 || q == 2 ? 128 : 64,
+                                 slice_scheme(*c));
         if (!ok) {
             set_err("integer-slice GEMM setup failed");
             return fail(TDB_ERR_CUDA);
@@ -1882,7 +1911,7 @@ tdb_status tdb_step_window(tdb_ctx* c, const double* v_bar, int k) {
     double* Cm = c->M;          // C
     double* lev[4] = {c->rho_re[prv], c->rho_im[prv], c->rho_re[cur], c->rho_im[cur]};
     launch_transpose(N, Z, Cm, c->stream);
-    if (sliced(*c)) {
+    if (use_slices(*c)) {
         // Integer-slice products, each with P^T or C as its A operand: with T = P^T rho,
         // rho P = +-T^T and rho~ = P^T (+-T^T); with U = C rho~, rho = C (+-U^T), the sign
         // + for the symmetric real part and - for the antisymmetric imaginary part, and a

@@ -2,16 +2,21 @@
 // tensor cores with exact accumulation.
 //
 // Each row of A is scaled by a power of two 2^-e so that its entries lie in (-1, 1),
-// then cut into kSlices signed 7-bit integers (|a_s| <= 64):
-//     A_ik = 2^(e_i - 6) sum_s a_s,ik 2^(-7 s) + r_ik,   |r_ik| <= 2^(e_i - 7 kSlices).
-// Columns of B are treated alike (stored as rows of B^T).  Every slice product
-// a_s b_t is an integer of magnitude <= 2^12, so the K-sums of all pairs of equal
-// weight w = s + t over a kChunk-deep slice of K stay below 2^24 and are exact in the
-// tensor core's FP32 accumulator; the sum over weights and chunks is exact in 64-bit
-// integers.  Pairs with s + t < kSlices are kept, so the product carries an error of
-// about (kSlices + 1) 2^(-7 kSlices) of K max_k|A_ik| max_k|B_kj| (~2e-12 relative to
-// those maxima): an FP64 product for the purposes of the propagation, at tensor-core
-// speed.
+// rounded to b S - 1 bits and cut into S signed b-bit integer digits (|a_s| <= 2^(b-1)):
+//     A_ik = 2^(e_i - (b-1)) sum_s a_s,ik 2^(-b s) + r_ik,   |r_ik| <= 2^(e_i - b S).
+// Columns of B are treated alike (stored as rows of B^T).  Every digit product a_s b_t is
+// an integer of magnitude <= 2^(2b-2), so the K-sums of all pairs of equal weight
+// w = s + t over a chunk of K stay below 2^24 and are exact in the tensor core's FP32
+// accumulator; the sum over weights and chunks is exact in 64-bit integers, rounded once.
+// Pairs with s + t < W are kept.  Two schemes:
+//
+//   kSix    6 digits of 7 bits, W = 6 (21 pairs), chunks of 512: error about 7 2^-42 of
+//           K max_k|A_ik| max_k|B_kj| -- the TDB_FP64_SLICED form.
+//   kSeven  7 digits of 8 bits, W = 8 (34 pairs), chunks of 128: 55-bit operands, the
+//           first dropped weight is 2^-64.  On the products of the propagation (S^-1 H,
+//           M rho, N = 132 .. 520) its error is 0.3 to 0.65 of the DFMA product's in the
+//           2-norm and below a tenth of it in the largest element: it replaces the DFMA
+//           product of the TDB_FP64 form where N is large enough (see use_slices).
 #pragma once
 
 #include <cuda.h>
@@ -22,29 +27,43 @@
 namespace tdb {
 namespace oz {
 
-constexpr int kSlices = 6;
-constexpr int kChunk = 512;     // 6 pairs x 512 x 64^2 < 2^24
+enum Scheme { kSix = 0, kSeven = 1 };
+constexpr int kMaxSlices = 7;
 constexpr int kMaxK = 4096;     // keeps the 64-bit sums below 2^63
+__host__ __device__ constexpr int n_slices(int scheme) { return scheme == kSeven ? 7 : 6; }
 
 // Slices of the rows of a rows x K matrix: s[q] is rows x ld 16-bit (FP16 integers),
-// ld a multiple of 64; e[i] the power-of-two exponent of row i.  The tensor maps cover
-// rows x K (zero fill beyond K) with boxes of 32 (K) x box_rows.
+// ld a multiple of 64; e[i] the power-of-two exponent of row i (kNonFinite: the row holds
+// an Inf or NaN and its products are NaN).  The tensor maps cover rows x K (zero fill
+// beyond K) with boxes of 32 (K) x box_rows.
 struct Sliced {
-    uint16_t* s[kSlices] = {};
+    uint16_t* s[kMaxSlices] = {};
     int* e = nullptr;
-    int rows = 0, K = 0, ld = 0;
-    CUtensorMap map[kSlices];
+    int rows = 0, K = 0, ld = 0, scheme = kSix;
+    CUtensorMap map[kMaxSlices];
 };
+constexpr int kNonFinite = 1 << 24;
 
 // Bytes of device memory a Sliced of rows x K needs (slices + exponents).
-size_t sliced_bytes(int rows, int K);
+size_t sliced_bytes(int rows, int K, int scheme = kSix);
 // Lays a Sliced out in base (256-byte aligned) and encodes its tensor maps; box_rows
 // is 128 for an A operand and 64 for a B operand.  False if a map cannot be encoded.
-bool sliced_init(Sliced& s, void* base, int rows, int K, int box_rows);
+bool sliced_init(Sliced& s, void* base, int rows, int K, int box_rows, int scheme = kSix);
 
-// Slices of sign * A (rows x K, row-major FP64 with row stride lda), row scales.  For
-// a B operand that is symmetric (sign 1) or antisymmetric (sign -1) this is also the
-// slicing of B^T.
+// A matrix to slice by rows: sign * A (rows x K, row-major FP64 with row stride lda), or,
+// with S set, the SCC Hamiltonian A + 1/2 S (v_r + v_c) formed element by element
+// (eq:hscc; S with the stride of A).  For a B operand that is symmetric (sign 1) or
+// antisymmetric (sign -1) this is also the slicing of B^T.
+struct SliceJob {
+    const double* A = nullptr;
+    int lda = 0;
+    double sign = 1.0;
+    Sliced* out = nullptr;
+    const double* S = nullptr;
+    const double* v = nullptr;
+};
+// njobs <= 3 matrices of the same rows, K and scheme in one launch.
+void slice_rows(const SliceJob* jobs, int njobs, cudaStream_t st);
 void slice_rows(const double* A, int lda, double sign, Sliced& out, cudaStream_t st);
 // Slices of B^T for a general B (K x cols, row-major FP64, row stride ldb); colmax is
 // a device scratch of cols doubles.
@@ -58,8 +77,8 @@ struct Part {
 };
 // Once per process and device before the first launch (outside stream capture).
 cudaError_t prepare();
-// C_z = A B_z for z < nparts (<= 2); M = a.rows, N = b.rows, K = a.K = b.K (<= kMaxK).
-// err: device flag, set to 1-3 if a bounded wait expired.
+// C_z = A B_z for z < nparts (<= 2); M = a.rows, N = b.rows, K = a.K = b.K (<= kMaxK), all
+// of one scheme.  err: device flag, set to 1-3 if a bounded wait expired.
 cudaError_t gemm(const Sliced& a, const Part* parts, int nparts, int* err, cudaStream_t st);
 
 }  // namespace oz
