@@ -40,8 +40,7 @@ KERNEL_FLOPS = {
     "gemm_M_f64": lambda N: 2 * N ** 3,
     "gemm_X_f64": lambda N: 4 * N ** 3,
     "gemm_dM_f32": lambda N: 2 * N ** 3,
-    "gemm_Xre_f32": lambda N: 2 * N ** 3,
-    "gemm_Xim_f32": lambda N: 2 * N ** 3,
+    "gemm_X_f32": lambda N: 4 * N ** 3,
     # tensor-core split GEMMs: algorithmic flops (the split products execute 3x or 6x this)
     "tc_gemm_dM": lambda N: 2 * N ** 3,
     "tc_gemm_X": lambda N: 4 * N ** 3,

@@ -26,15 +26,6 @@ struct Ham {
     }
 };
 
-// delta H_kj = 1/2 S_kj (dv_k + dv_j) in FP32
-struct DeltaHamF {
-    const float *S, *dv;
-    int N;
-    __device__ __forceinline__ float operator()(int k, int j) const {
-        return 0.5f * S[(size_t)k * N + j] * (dv[k] + dv[j]);
-    }
-};
-
 // FP64: an 8 x 8 tile of C per block of 64 threads, one output each; blockIdx.z picks one of
 // two products that share A.  DFMA issues at two lanes a clock per SM on this part, so the
 // product is bound by that pipe whatever the tile, and the tile only has to spread the work:
@@ -75,63 +66,119 @@ __global__ void __launch_bounds__(kT8* kT8)
     if (gm < M && gn < Ncol) (blockIdx.z ? C1 : C0)[(size_t)gm * ldc + gn] = acc;
 }
 
-// C[BM x BN] tile per block; each thread owns TM x TN outputs strided by the
-// thread-grid size, so shared-memory reads of a warp are conflict-free.
-template <typename T, int BM, int BN, int BK, int TM, int TN, class LA, class LB>
-__global__ void __launch_bounds__((BM / TM) * (BN / TN))
-    k_gemm(int M, int Ncol, int K, LA la, LB lb, T* C, int ldc,
-           const T* Cadd) {
-    constexpr int TX = BN / TN, TY = BM / TM, NT = TX * TY;
-    __shared__ T As[BK][BM + 1];
-    __shared__ T Bs[BK][BN];
-    const int tid = threadIdx.x;
-    const int tx = tid % TX, ty = tid / TX;
-    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-    T acc[TM][TN];
+// FP32: a 64 x 64 tile of C per block of 128 threads, 8 x 4 consecutive outputs each, for one
+// of up to three products of the same shape (blockIdx.z).  Bound by FFMA issue: a warp's step
+// of K reads 2 + 2 shared-memory wavefronts for its 32 FFMA, and the next 16-deep block is
+// loaded into registers while this one is multiplied.  64 x 64 rather than 128 x 128, so that
+// the three X products of a middle-sized system fill the chip (N = 532: 243 tiles; 128 x 128
+// tiles gave 25 blocks a product; the step there went from 425 to 100 us).  Each output sums its
+// K terms in order.
+constexpr int kF32Tile = 64, kF32K = 16, kF32Threads = 128;
+
+struct F32Parts {
+    F32Part p[3];
+};
+
+// B operand: dense, or delta H_kj = 1/2 S_kj (dv_k + dv_j) with S = b and dv set
+template <bool DHAM>
+__global__ void __launch_bounds__(kF32Threads, 4)
+    k_gemm_f32(int M, int Ncol, int K, const __grid_constant__ F32Parts parts,
+               const float* __restrict__ dv, const float* __restrict__ add, float* __restrict__ C2) {
+    __shared__ __align__(16) float As[2][kF32K][kF32Tile + 4];
+    __shared__ __align__(16) float Bs[2][kF32K][kF32Tile];
+    const F32Part& P = parts.p[blockIdx.z];
+    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
+    const int m0 = blockIdx.y * kF32Tile, n0 = blockIdx.x * kF32Tile;
+    // loads of a block: A rows ar, ar + 32 (4 consecutive k each), B rows bk, bk + 8 (4
+    // consecutive columns each)
+    const int ar = tid / 4, ak = 4 * (tid % 4), bk = tid / 16, bn = 4 * (tid % 16);
+    const bool va = (P.lda % 4 == 0) && (reinterpret_cast<uintptr_t>(P.A) & 15) == 0;
+    const bool vb = (P.ldb % 4 == 0) && (reinterpret_cast<uintptr_t>(P.B) & 15) == 0;
+    float ra[2][4], rb[2][4];
+    float dvn[4] = {0.f, 0.f, 0.f, 0.f};
+    pdl_launch_dependents();
+    pdl_wait();
+    if (DHAM)
 #pragma unroll
-    for (int i = 0; i < TM; ++i)
+        for (int j = 0; j < 4; ++j) dvn[j] = n0 + bn + j < Ncol ? __ldg(dv + n0 + bn + j) : 0.f;
+    auto load = [&](int k0) {
 #pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = T(0);
-    for (int k0 = 0; k0 < K; k0 += BK) {
+        for (int h = 0; h < 2; ++h) {
+            const int gm = m0 + ar + 32 * h, ga = k0 + ak;
+            const float* pa = P.A + (size_t)gm * P.lda + ga;
+            if (va && gm < M && ga + 4 <= K) {
+                const float4 v = *reinterpret_cast<const float4*>(pa);
+                ra[h][0] = v.x, ra[h][1] = v.y, ra[h][2] = v.z, ra[h][3] = v.w;
+            } else {
 #pragma unroll
-        for (int e = tid; e < BM * BK; e += NT) {
-            const int m = e / BK, k = e % BK;
-            const int gm = m0 + m, gk = k0 + k;
-            As[k][m] = (gm < M && gk < K) ? la(gm, gk) : T(0);
-        }
+                for (int j = 0; j < 4; ++j) ra[h][j] = gm < M && ga + j < K ? pa[j] : 0.f;
+            }
+            const int gk = k0 + bk + 8 * h, gn = n0 + bn;
+            const float* pb = P.B + (size_t)gk * P.ldb + gn;
+            if (vb && gk < K && gn + 4 <= Ncol) {
+                const float4 v = *reinterpret_cast<const float4*>(pb);
+                rb[h][0] = v.x, rb[h][1] = v.y, rb[h][2] = v.z, rb[h][3] = v.w;
+            } else {
 #pragma unroll
-        for (int e = tid; e < BK * BN; e += NT) {
-            const int k = e / BN, n = e % BN;
-            const int gk = k0 + k, gn = n0 + n;
-            Bs[k][n] = (gk < K && gn < Ncol) ? lb(gk, gn) : T(0);
-        }
-        __syncthreads();
+                for (int j = 0; j < 4; ++j) rb[h][j] = gk < K && gn + j < Ncol ? pb[j] : 0.f;
+            }
+            if (DHAM) {
+                const float dk = gk < K ? __ldg(dv + gk) : 0.f;
 #pragma unroll
-        for (int kk = 0; kk < BK; ++kk) {
-            T a[TM], b[TN];
-#pragma unroll
-            for (int i = 0; i < TM; ++i) a[i] = As[kk][ty + i * TY];
-#pragma unroll
-            for (int j = 0; j < TN; ++j) b[j] = Bs[kk][tx + j * TX];
-#pragma unroll
-            for (int i = 0; i < TM; ++i)
-#pragma unroll
-                for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int i = 0; i < TM; ++i) {
-        const int gm = m0 + ty + i * TY;
-        if (gm >= M) continue;
-#pragma unroll
-        for (int j = 0; j < TN; ++j) {
-            const int gn = n0 + tx + j * TX;
-            if (gn < Ncol) {
-                const size_t o = (size_t)gm * ldc + gn;
-                C[o] = Cadd ? acc[i][j] + Cadd[o] : acc[i][j];
+                for (int j = 0; j < 4; ++j) rb[h][j] = 0.5f * rb[h][j] * (dk + dvn[j]);
             }
         }
+    };
+    auto store = [&](int s) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) As[s][ak + j][ar + 32 * h] = ra[h][j];
+            *reinterpret_cast<float4*>(&Bs[s][bk + 8 * h][bn]) =
+                make_float4(rb[h][0], rb[h][1], rb[h][2], rb[h][3]);
+        }
+    };
+    float acc[8][4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+    load(0);
+    store(0);
+    __syncthreads();
+    int s = 0;
+    for (int k0 = 0; k0 < K; k0 += kF32K, s ^= 1) {
+        const bool more = k0 + kF32K < K;
+        if (more) load(k0 + kF32K);
+#pragma unroll
+        for (int kk = 0; kk < kF32K; ++kk) {
+            const float4 a0 = *reinterpret_cast<const float4*>(&As[s][kk][8 * ty]);
+            const float4 a1 = *reinterpret_cast<const float4*>(&As[s][kk][8 * ty + 4]);
+            const float4 b0 = *reinterpret_cast<const float4*>(&Bs[s][kk][4 * tx]);
+            const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+            const float b[4] = {b0.x, b0.y, b0.z, b0.w};
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+        }
+        if (more) {
+            store(s ^ 1);
+            __syncthreads();
+        }
+    }
+    const int gn = n0 + 4 * tx;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int gm = m0 + 8 * ty + i;
+        if (gm >= M) break;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (gn + j < Ncol) {
+                P.C[(size_t)gm * P.ldc + gn + j] = acc[i][j];
+                // M = M_gs + delta M beside delta M
+                if (DHAM && C2) C2[(size_t)gm * P.ldc + gn + j] = add[(size_t)gm * Ncol + gn + j] + acc[i][j];
+            }
     }
 }
 
@@ -140,15 +187,6 @@ void run_f64(int M, int Ncol, int K, LA la, LB lb0, LB lb1, double* C0, double* 
              cudaStream_t st) {
     const dim3 g((Ncol + kT8 - 1) / kT8, (M + kT8 - 1) / kT8, C1 ? 2 : 1);
     launch_pdl(k_gemm_f64<LA, LB>, g, dim3(kT8 * kT8), 0, st, M, Ncol, K, la, lb0, lb1, C0, C1, ldc);
-}
-
-template <class LA, class LB>
-void run_f32(int M, int Ncol, int K, LA la, LB lb, float* C, int ldc, const float* Cadd,
-             cudaStream_t st) {
-    constexpr int BM = 128, BN = 128, BK = 8, TM = 8, TN = 8;
-    dim3 g((Ncol + BN - 1) / BN, (M + BM - 1) / BM);
-    k_gemm<float, BM, BN, BK, TM, TN, LA, LB>
-        <<<g, (BM / TM) * (BN / TN), 0, st>>>(M, Ncol, K, la, lb, C, ldc, Cadd);
 }
 
 }  // namespace
@@ -170,21 +208,21 @@ void gemm_f64_ham(int N, const double* A, const double* H0, const double* S, con
     run_f64(N, N, N, Dense<double>{A, N}, h, h, C, static_cast<double*>(nullptr), N, st);
 }
 
-void gemm_f32(int M, int Ncol, int K, const float* A, int lda, const float* B, int ldb, float* C,
-              int ldc, cudaStream_t st) {
-    run_f32(M, Ncol, K, Dense<float>{A, lda}, Dense<float>{B, ldb}, C, ldc, nullptr, st);
+void gemm_f32(int M, int Ncol, int K, const F32Part* parts, int nparts, cudaStream_t st) {
+    F32Parts p{};
+    for (int z = 0; z < nparts; ++z) p.p[z] = parts[z];
+    const dim3 g((Ncol + kF32Tile - 1) / kF32Tile, (M + kF32Tile - 1) / kF32Tile, nparts);
+    launch_pdl(k_gemm_f32<false>, g, dim3(kF32Threads), 0, st, M, Ncol, K, p,
+               static_cast<const float*>(nullptr), static_cast<const float*>(nullptr),
+               static_cast<float*>(nullptr));
 }
 
-// C = A * dH + Cadd, dH_kj = 1/2 S_kj (dv_k + dv_j): delta M = S^-1 delta H, M = M_gs + delta M
-void gemm_f32_dham(int N, const float* A, const float* S, const float* dv, float* C, int ldc,
-                   const float* Cadd, cudaStream_t st) {
-    run_f32(N, N, N, Dense<float>{A, N}, DeltaHamF{S, dv, N}, C, ldc, Cadd, st);
-}
-
-// C = A * B + Cadd (FP32; Cadd may be C itself)
-void gemm_f32_add(int M, int Ncol, int K, const float* A, int lda, const float* B, int ldb,
-                  float* C, int ldc, const float* Cadd, cudaStream_t st) {
-    run_f32(M, Ncol, K, Dense<float>{A, lda}, Dense<float>{B, ldb}, C, ldc, Cadd, st);
+void gemm_f32_dham(int N, const float* A, const float* S, const float* dv, float* dM, float* Msum,
+                   int ldc, const float* Mgs, cudaStream_t st) {
+    F32Parts p{};
+    p.p[0] = {A, N, S, N, dM, ldc};
+    const dim3 g((N + kF32Tile - 1) / kF32Tile, (N + kF32Tile - 1) / kF32Tile);
+    launch_pdl(k_gemm_f32<true>, g, dim3(kF32Threads), 0, st, N, N, N, p, dv, Mgs, Msum);
 }
 
 }  // namespace tdb

@@ -656,15 +656,6 @@ __global__ void k_f32_to_f64(size_t n, const float* __restrict__ in, double* __r
         out[i] = (double)in[i];
 }
 
-// out[r][c] = a[r][c] + b[r][c] with row strides N (a), ldb (b), ldo (out)
-__global__ void k_add_f32(int N, const float* __restrict__ a, const float* __restrict__ b, int ldb,
-                          float* __restrict__ out, int ldo) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    const int r = blockIdx.y * blockDim.y + threadIdx.y;
-    if (r >= N || c >= N) return;
-    out[(size_t)r * ldo + c] = a[(size_t)r * N + c] + b[(size_t)r * ldb + c];
-}
-
 // out[0] = 1/2 sum_A dq_A (gamma dq)_A (eq:coul), out[1] = sum_{A<B} rep_A exp(-r/rep_b),
 // out[2] = nuclear kinetic energy (moving nuclei only)
 __global__ void k_small_energies(int nat, const double* __restrict__ dq,
@@ -738,12 +729,6 @@ void launch_f32_to_f64(size_t n, const float* in, double* out, cudaStream_t st) 
 
 void launch_f64_to_f32(size_t n, const double* in, float* out, cudaStream_t st) {
     k_f64_to_f32<<<1216, 256, 0, st>>>(n, in, out);
-}
-
-void launch_add_f32_strided(int N, const float* a, const float* b, int ldb, float* out, int ldo,
-                            cudaStream_t st) {
-    dim3 bl(32, 8);
-    k_add_f32<<<grid2(N, N, bl), bl, 0, st>>>(N, a, b, ldb, out, ldo);
 }
 
 void launch_small_energies(const Ctx& c, double* out, cudaStream_t st) {

@@ -12,10 +12,6 @@
 #include "tdb_internal.h"
 
 namespace tdb {
-void gemm_f32_dham(int N, const float* A, const float* S, const float* dv, float* C, int ldc,
-                   const float* Cadd, cudaStream_t st);
-void gemm_f32_add(int M, int Ncol, int K, const float* A, int lda, const float* B, int ldb,
-                  float* C, int ldc, const float* Cadd, cudaStream_t st);
 void launch_f64_to_f32(size_t n, const double* in, float* out, cudaStream_t st);
 void launch_f32_to_f64(size_t n, const float* in, double* out, cudaStream_t st);
 void launch_ns_update(int N, double* X, const double* Q, cudaStream_t st);
@@ -24,10 +20,6 @@ void launch_window(int N, const double* eps, double dt, int k, double* x0re, dou
                    double* x1re, double* x1im, cudaStream_t st);
 void launch_add_step(DevScalars* sc, int k, cudaStream_t st);
 }  // namespace learn
-void gemm_f32(int M, int Ncol, int K, const float* A, int lda, const float* B, int ldb, float* C,
-              int ldc, cudaStream_t st);
-void launch_add_f32_strided(int N, const float* a, const float* b, int ldb, float* out, int ldo,
-                            cudaStream_t st);
 void launch_small_energies(const Ctx& c, double* out, cudaStream_t st);
 void launch_absmax(size_t n, const double* x, double* out, cudaStream_t st,
                    const double* sub = nullptr);
@@ -211,6 +203,7 @@ size_t carve(Ctx& c, char* base) {
         c.md_xim = k.take<float>(NN);
     }
     if (c.prm.precision == TDB_FP32 && !c.prm.move_nuclei) {
+        c.Xa_f = k.take<float>(NN);
         c.Xre_f = k.take<float>(NN);
         c.Xim_f = k.take<float>(NN);
         c.Sinv_f = k.take<float>(NN);
@@ -867,6 +860,15 @@ tdb_status oz_product_rho(Ctx& c, int a, double* re, double* im) {
     return TDB_OK;
 }
 
+// md_m = S^-1 md_b and [md_xre | md_xim] = md_m rho_n in FP32
+void md32_products(Ctx& c) {
+    const int N = c.N;
+    const F32Part m = {c.md_sinv, N, c.md_b, N, c.md_m, N};
+    gemm_f32(N, N, N, &m, 1, c.stream);
+    const F32Part x[2] = {{c.md_m, N, c.md_rre, N, c.md_xre, N}, {c.md_m, N, c.md_rim, N, c.md_xim, N}};
+    gemm_f32(N, N, N, x, 2, c.stream);
+}
+
 // Everything of a moving-nuclei step up to the work rate, for rho_n in buffer cur
 // (Sec. 2.3 with the ordering: S_n, S^-1_n; q(rho_n), H_n; X_n; F_n; V_n; D_n; P_n).
 // commit = 1 inside a step (the work integral advances), 0 for observables.
@@ -896,9 +898,7 @@ tdb_status md_forces(Ctx& c, int cur, bool first, int commit, int* n, StepTimer*
         launch_f64_to_f32(NN, c.Hs, c.md_b, c.stream);
         launch_f64_to_f32(NN, c.rho_re[cur], c.md_rre, c.stream);
         launch_f64_to_f32(NN, c.rho_im[cur], c.md_rim, c.stream);
-        gemm_f32(N, N, N, c.md_sinv, N, c.md_b, N, c.md_m, N, c.stream);
-        gemm_f32(N, N, N, c.md_m, N, c.md_rre, N, c.md_xre, N, c.stream);
-        gemm_f32(N, N, N, c.md_m, N, c.md_rim, N, c.md_xim, N, c.stream);
+        md32_products(c);
         launch_f32_to_f64(NN, c.md_xre, c.Xre, c.stream);
         launch_f32_to_f64(NN, c.md_xim, c.Xim, c.stream);
         if (n) *n += 7;
@@ -937,9 +937,7 @@ tdb_status enqueue_step_md(Ctx& c, int cur, bool euler, int* launches, StepTimer
         const int N = c.N;
         const size_t NN = (size_t)N * N;
         launch_f64_to_f32(NN, c.D, c.md_b, c.stream);
-        gemm_f32(N, N, N, c.md_sinv, N, c.md_b, N, c.md_m, N, c.stream);
-        gemm_f32(N, N, N, c.md_m, N, c.md_rre, N, c.md_xre, N, c.stream);
-        gemm_f32(N, N, N, c.md_m, N, c.md_rim, N, c.md_xim, N, c.stream);
+        md32_products(c);
         launch_f32_to_f64(NN, c.md_xre, c.Zre, c.stream);
         launch_f32_to_f64(NN, c.md_xim, c.Zim, c.stream);
         n += 3;
@@ -1197,24 +1195,23 @@ tdb_status enqueue_step(Ctx& c, int cur, bool euler, int* launches, StepTimer* t
         const int N = c.N;
         // delta M = S^-1 delta H (left half of [dM | M]), M = M_gs + delta M (right half)
         MARK("gemm_dM_f32");
-        gemm_f32_dham(N, c.Sinv_f, c.S_f, c.dv_f, c.dM_f, 2 * N, nullptr, c.stream);
-        ++n;
-        MARK("add_M");
-        launch_add_f32_strided(N, c.Mgs_f, c.dM_f, 2 * N, c.M_f, 2 * N, c.stream);
-        ++n;
-        // X_re = dM rho_ref + M Re(rho - rho_ref);  X_im = M Im rho (master hi parts)
-        MARK("gemm_Xre_f32");
-        gemm_f32_add(N, N, N, c.dM_f, 2 * N, c.rref_f, N, c.Xre_f, N, nullptr, c.stream);
-        gemm_f32_add(N, N, N, c.M_f, 2 * N, c.ms[cur].re_hi, N, c.Xre_f, N, c.Xre_f, c.stream);
-        MARK("gemm_Xim_f32");
-        gemm_f32_add(N, N, N, c.M_f, 2 * N, c.ms[cur].im_hi, N, c.Xim_f, N, nullptr, c.stream);
-        n += 3;
+        gemm_f32_dham(N, c.Sinv_f, c.S_f, c.dv_f, c.dM_f, c.M_f, 2 * N, c.Mgs_f, c.stream);
+        // X_re = dM rho_ref + M Re(rho - rho_ref) (the update adds the two);
+        // X_im = M Im rho (master hi parts)
+        MARK("gemm_X_f32");
+        const F32Part x[3] = {{c.dM_f, 2 * N, c.rref_f, N, c.Xa_f, N},
+                              {c.M_f, 2 * N, c.ms[cur].re_hi, N, c.Xre_f, N},
+                              {c.M_f, 2 * N, c.ms[cur].im_hi, N, c.Xim_f, N}};
+        gemm_f32(N, N, N, x, 3, c.stream);
+        n += 2;
         MARK("update");
         UpdateOperands ops;
         ops.cur = cur;
-        ops.xre[0] = c.Xre_f;
+        ops.xre[0] = c.Xa_f;
+        ops.xre[1] = c.Xre_f;
         ops.xim[0] = c.Xim_f;
-        ops.nre = ops.nim = 1;
+        ops.nre = 2;
+        ops.nim = 1;
         ops.base_slot = euler ? cur : prv;
         launch_update_df(c, euler ? c.ms[cur] : c.ms[prv], c.ms[prv], factor, c.sc, ops,
                          level_args(c), c.stream);

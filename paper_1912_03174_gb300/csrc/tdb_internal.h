@@ -125,7 +125,7 @@ struct Ctx {
     float *dv_f = nullptr;                           // [N] v - v_ref per orbital
     float *S_f = nullptr, *Sinv_f = nullptr, *Mgs_f = nullptr, *rref_f = nullptr;
     float *dM_f = nullptr, *M_f = nullptr;           // delta M, M = M_gs + delta M
-    float *Xre_f = nullptr, *Xim_f = nullptr;
+    float *Xa_f = nullptr, *Xre_f = nullptr, *Xim_f = nullptr;
     // per-level evaluation of the reduced forms (LevelArgs)
     float2 *gam2 = nullptr, *R2 = nullptr, *lv_dq = nullptr, *lv_bsum = nullptr;
     float* c_res = nullptr;
@@ -310,6 +310,19 @@ enum class BKind { Dense = 0, Hamiltonian = 1 };
 void gemm_f64(int M, int Ncol, int K, const double* A, int lda, const double* B, int ldb,
               double* C, int ldc, cudaStream_t st);
 // C = A * H with H_kj = H0_kj + 1/2 S_kj (v_k + v_j) formed while loading B (eq:hscc).
+// FP32 products C = A B (row-major), up to three of the same shape in one launch
+struct F32Part {
+    const float* A;
+    int lda;
+    const float* B;
+    int ldb;
+    float* C;
+    int ldc;
+};
+void gemm_f32(int M, int Ncol, int K, const F32Part* parts, int nparts, cudaStream_t st);
+// dM = A dH with dH_kj = 1/2 S_kj (dv_k + dv_j), and Msum = Mgs + dM (row strides ldc; Mgs: N)
+void gemm_f32_dham(int N, const float* A, const float* S, const float* dv, float* dM, float* Msum,
+                   int ldc, const float* Mgs, cudaStream_t st);
 // C0 = A B0 and C1 = A B1 (N x N) in one launch
 void gemm_f64_pair(int N, const double* A, const double* B0, const double* B1, double* C0,
                    double* C1, cudaStream_t st);
