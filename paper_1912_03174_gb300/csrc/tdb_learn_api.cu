@@ -21,6 +21,10 @@ void launch_grad(int F, int H, const float* params, const float* X, const float*
                  float scale, float* grad, double* sse, cudaStream_t st);
 void launch_adam(int n, float* p, const float* g, float* m, float* v, float lr, float b1,
                  float b2, float c1, float c2, float eps, cudaStream_t st);
+int epoch_cluster();
+cudaError_t launch_epoch(int nc, int F, int H, float* params, float* m, float* v, const float* X,
+                         const float* Y, long n, long batch, float lr, float b1, float b2, float eps,
+                         long t0, double* sse, cudaStream_t st);
 }  // namespace learn
 }  // namespace tdb
 
@@ -31,10 +35,16 @@ struct tdb_shiftnet {
     float *X = nullptr, *Y = nullptr;
     long cap = 0;
     long t = 0;                  // Adam steps taken
+    int cluster = 8;             // CTAs of the epoch kernel
     cudaStream_t st = nullptr;
 };
 
 namespace {
+
+// Mini-batches up to this size train an epoch in one cluster launch; larger ones give every SM
+// 128-sample blocks of k_net_grad.  Microseconds a batch, cluster / grid, 16 x 64 network: 21 / 121
+// at 512 samples, 44 / 124 at 2048, 74 / 124 at 4096, 135 / 127 at 8192 (the cluster has 16 SMs).
+constexpr long kEpochBatch = 6144;
 
 tdb_status fail(const char* msg, tdb_status s) {
     tdb::set_last_error(msg);
@@ -89,6 +99,7 @@ tdb_status tdb_shiftnet_create(int n_features, int hidden, unsigned long long se
               cudaMalloc(&net->sse, sizeof(double)) == cudaSuccess &&
               tdb::learn::prepare(n_features, hidden) == cudaSuccess;
     if (ok) {
+        net->cluster = tdb::learn::epoch_cluster();
         // uniform weights in +-sqrt(3 / fan_in) (splitmix64 stream), zero biases
         std::vector<float> h(net->np, 0.f);
         uint64_t x = seed;
@@ -180,7 +191,16 @@ tdb_status tdb_shiftnet_train(tdb_shiftnet* net, const float* X, const float* Y,
     double last = 0.0;
     for (int ep = 0; ep < epochs; ++ep) {
         cudaMemsetAsync(net->sse, 0, sizeof(double), net->st);
-        for (long s = 0; s < n; s += batch) {
+        if (batch <= kEpochBatch) {
+            if (tdb::learn::launch_epoch(net->cluster, net->F, net->H, net->p, net->m, net->v, net->X,
+                                         net->Y, n, batch, lr, b1, b2, eps, net->t, net->sse,
+                                         net->st) != cudaSuccess) {
+                cudaGetLastError();
+                return fail("tdb_shiftnet_train: CUDA error", TDB_ERR_CUDA);
+            }
+            net->t += (n + batch - 1) / batch;
+        }
+        for (long s = 0; batch > kEpochBatch && s < n; s += batch) {
             const long nb = std::min(batch, n - s);
             cudaMemsetAsync(net->g, 0, sizeof(float) * net->np, net->st);
             tdb::learn::launch_grad(net->F, net->H, net->p, net->X + s * net->F, net->Y + s, nb,
