@@ -132,8 +132,8 @@ __device__ __forceinline__ double scaled_sum(long long hi, long long lo, int x) 
 
 // One CTA per 128 x 64 output tile; every CTA issues its own TMA loads of the A and B
 // slices it multiplies.  One product at N = 1024 (128 tiles), kSix: 41 us (79 us when the drain
-// used 64-bit conversions and the rounding FP64 arithmetic: 24 and 8 of those); kSeven 68 us;
-// at N = 2048 291 and 509 us.
+// used 64-bit conversions and the rounding FP64 arithmetic), kSeven: 68 us; at N = 2048 291 and
+// 509 us.
 template <int SCH>
 __global__ void __launch_bounds__(kThreads, 1)
     k_oz_gemm(const __grid_constant__ Maps maps, Params p) {

@@ -71,3 +71,73 @@ def test_slice_gemm_of_non_finite_rows_is_nan_there_and_only_there(B):
     assert np.all(np.isnan(C[bad]))
     assert np.array_equal(C[~bad], ref[~bad])
     assert np.all(B.tdb_slice_gemm(np.zeros((3, 5)), np.zeros((5, 2)))[0] == 0.0)
+
+
+# N = 4, 64 (one whole tile), 68 (one tile and a ragged one), 196
+@pytest.mark.parametrize("n_atoms", [1, 16, 17, 49])
+def test_fp32_form_matches_the_oracle_at_tile_edges(B, n_atoms):
+    # FP32 products on rho - rho_gs: the 1e-6 bounds of the reduced-form parity tests
+    sysm = I.small_flake(n_atoms, seed=8)
+    run = I.Run(dt=0.2, n_steps=0, scc=True, kick=1e-3, kT=I.SCC_KT)
+    n = 100
+    with B.Propagator(sysm, run, "fp32") as p:
+        p.setup()
+        p.step(n)
+        hist = B.tdb_dipole_history(p.ctx, n)
+        rho = B.tdb_get_rho(p.ctx)
+    ref, _, _, _ = O.setup(sysm, run)
+    tr = O.propagate(sysm, run, ref, n)
+    assert np.max(np.abs(hist - tr.dipole[:n])) < 1e-6
+    assert np.max(np.abs(rho - tr.rho)) < 1e-6
+
+
+@pytest.mark.parametrize("dt_over_damp", [0.0, 0.004, 0.5])
+@pytest.mark.parametrize("nsig,K,nw", [(1, 513, 24000), (3, 4608, 901), (10, 1023, 1300)])
+def test_damped_transform_of_large_problems_matches_the_oracle(B, nsig, K, nw, dt_over_damp):
+    # past the size from which samples go in blocks of 512 (one sample past a block, whole
+    # blocks, one short), undamped, damped, and damped too strongly within a block for that path;
+    # bound of the kernel's test at small sizes
+    from oracle import tdb_spectra as SP
+    rng = np.random.default_rng(nsig + K)
+    x = rng.normal(size=(nsig, K))
+    om = rng.uniform(0.0, 5.0, size=nw)
+    dt = 0.2
+    t_damp = dt / dt_over_damp if dt_over_damp else 0.0
+    got = B.tdb_damped_transform(x, dt, t_damp, om)
+    ref = SP.damped_transform(x, dt, t_damp or np.inf, om)
+    scale = dt * np.sum(np.abs(x), axis=1, keepdims=True)
+    assert np.max(np.abs(got - ref) / scale) < 1e-13
+
+
+# one sample; shares of a 16-CTA cluster that leave CTAs empty, one chunk of 32 per CTA, two
+# chunks with a ragged second; batch sizes that do not divide the samples; hidden and feature
+# counts that are not multiples of 4, and the largest network
+@pytest.mark.parametrize("F,H,n,batch", [(1, 1, 1, 1), (5, 7, 40, 9), (16, 64, 1100, 512),
+                                         (32, 64, 2000, 700), (3, 33, 600, 600)])
+def test_training_epochs_match_the_oracle_gradients_and_adam(B, F, H, n, batch):
+    # FP32 sums of at most 700 terms against FP64: the gradient agrees to ~1e-6 of its largest
+    # component, and an Adam step moves a parameter by lr g / |g| at first, so that parameters
+    # agree to lr times that error over the smallest gradients' scale.  Parameters are compared
+    # after two epochs with the bound lr / 20 per element and 1e-3 lr in the mean.
+    rng = np.random.default_rng(F * 100 + H)
+    p = (rng.normal(size=F * H + H + H * H + 2 * H + 1) * 0.3).astype(np.float32)
+    X = rng.normal(size=(n, F)).astype(np.float32)
+    Y = rng.normal(size=n).astype(np.float32)
+    lr = 1e-3
+    with B.ShiftNet(F, H) as net:
+        net.set_params(p)
+        loss = net.train(X, Y, epochs=2, batch=batch, lr=lr)
+        got = net.params()
+    q, m, v, t = p.astype(np.float64), 0.0, 0.0, 0
+    for ep in range(2):
+        sse = 0.0
+        for s in range(0, n, batch):
+            x, y = X[s:s + batch].astype(np.float64), Y[s:s + batch].astype(np.float64)
+            l, g = O.shiftnet_loss_grad(q, x, y, F, H)
+            sse += l * len(y)
+            t += 1
+            m, v = 0.9 * m + 0.1 * g, 0.999 * v + 0.001 * g * g
+            q = q - lr * (m / (1 - 0.9 ** t)) / (np.sqrt(v / (1 - 0.999 ** t)) + 1e-8)
+    assert abs(loss - sse / n) < 1e-4 * (sse / n)
+    assert np.max(np.abs(got - q)) < lr / 20
+    assert np.mean(np.abs(got - q)) < 1e-3 * lr + 1e-7
