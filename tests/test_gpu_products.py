@@ -115,10 +115,11 @@ def test_damped_transform_of_large_problems_matches_the_oracle(B, nsig, K, nw, d
 @pytest.mark.parametrize("F,H,n,batch", [(1, 1, 1, 1), (5, 7, 40, 9), (16, 64, 1100, 512),
                                          (32, 64, 2000, 700), (3, 33, 600, 600)])
 def test_training_epochs_match_the_oracle_gradients_and_adam(B, F, H, n, batch):
-    # FP32 sums of at most 700 terms against FP64: the gradient agrees to ~1e-6 of its largest
-    # component, and an Adam step moves a parameter by lr g / |g| at first, so that parameters
-    # agree to lr times that error over the smallest gradients' scale.  Parameters are compared
-    # after two epochs with the bound lr / 20 per element and 1e-3 lr in the mean.
+    # FP32 sums of at most 700 terms against FP64 agree to ~1e-6 of the largest gradient
+    # component; a master weight within that of a tie may round to the other bfloat16, which moves
+    # the gradient by up to ~3e-4 of its largest component.  Adam divides by sqrt(v): a parameter
+    # with a small gradient may differ by up to its whole step (2 lr), others by that error over
+    # sqrt(v) (factor 50: two moments over the steps), and the mean stays below 2% of a step.
     rng = np.random.default_rng(F * 100 + H)
     p = (rng.normal(size=F * H + H + H * H + 2 * H + 1) * 0.3).astype(np.float32)
     X = rng.normal(size=(n, F)).astype(np.float32)
@@ -129,6 +130,7 @@ def test_training_epochs_match_the_oracle_gradients_and_adam(B, F, H, n, batch):
         loss = net.train(X, Y, epochs=2, batch=batch, lr=lr)
         got = net.params()
     q, m, v, t = p.astype(np.float64), 0.0, 0.0, 0
+    allowed = 2.0 ** -22 * np.abs(q) + 1e-8
     for ep in range(2):
         sse = 0.0
         for s in range(0, n, batch):
@@ -137,7 +139,9 @@ def test_training_epochs_match_the_oracle_gradients_and_adam(B, F, H, n, batch):
             sse += l * len(y)
             t += 1
             m, v = 0.9 * m + 0.1 * g, 0.999 * v + 0.001 * g * g
-            q = q - lr * (m / (1 - 0.9 ** t)) / (np.sqrt(v / (1 - 0.999 ** t)) + 1e-8)
+            rms = np.sqrt(v / (1 - 0.999 ** t)) + 1e-8
+            q = q - lr * (m / (1 - 0.9 ** t)) / rms
+            allowed = allowed + lr * np.minimum(2.0, 50 * 3e-4 * np.max(np.abs(g)) / rms)
     assert abs(loss - sse / n) < 1e-4 * (sse / n)
-    assert np.max(np.abs(got - q)) < lr / 20
-    assert np.mean(np.abs(got - q)) < 1e-3 * lr + 1e-7
+    assert np.all(np.abs(got - q) <= allowed)
+    assert np.mean(np.abs(got - q)) < 0.02 * lr * t
