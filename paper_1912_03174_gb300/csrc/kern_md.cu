@@ -4,6 +4,7 @@
 // recomputed from the geometry where they are used and never stored.
 #include <cmath>
 
+#include "pdl.cuh"
 #include "tdb_internal.h"
 
 namespace tdb {
@@ -13,41 +14,6 @@ namespace {
 __device__ __forceinline__ double warp_sum_d(double v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
-}
-
-// Radial integrals and their r-derivatives (hopping if h, else overlap).
-__device__ __forceinline__ void radial(const ModelParams& mp, double r, bool h, double K[4],
-                                       double dK[4]) {
-    const double e = h ? exp(-r / mp.lam_H) : exp(-r / mp.lam_S);
-    const double lam = h ? mp.lam_H : mp.lam_S;
-    for (int k = 0; k < 4; ++k) {
-        K[k] = h ? mp.eta[k] * mp.t0 * e : -mp.eta[k] * mp.s0 * e;
-        dK[k] = -K[k] / lam;
-    }
-}
-
-// Gradient with respect to d = R_B - R_A of element (i, j) of the Slater-Koster
-// s/p block (ss = K0, s-a = c_a K1, a-s = -c_a K1, a-b = c_a c_b (K2 - K3) + d_ab K3),
-// using dr/dd_g = c_g and dc_a/dd_g = (d_ag - c_a c_g) / r.
-__device__ __forceinline__ void block_grad(int i, int j, const double c[3], double r,
-                                           const double K[4], const double dK[4], double g[3]) {
-    if (i == 0 && j == 0) {
-        for (int q = 0; q < 3; ++q) g[q] = dK[0] * c[q];
-    } else if (i == 0 || j == 0) {
-        const int a = (i == 0 ? j : i) - 1;
-        const double sg = i == 0 ? 1.0 : -1.0;
-        for (int q = 0; q < 3; ++q)
-            g[q] = sg * (((a == q ? 1.0 : 0.0) - c[a] * c[q]) / r * K[1] + c[a] * dK[1] * c[q]);
-    } else {
-        const int a = i - 1, b = j - 1;
-        const double dd = K[2] - K[3], ddk = dK[2] - dK[3];
-        for (int q = 0; q < 3; ++q) {
-            const double dca = ((a == q ? 1.0 : 0.0) - c[a] * c[q]) / r;
-            const double dcb = ((b == q ? 1.0 : 0.0) - c[b] * c[q]) / r;
-            g[q] = (dca * c[b] + c[a] * dcb) * dd + c[a] * c[b] * ddk * c[q] +
-                   (a == b ? dK[3] * c[q] : 0.0);
-        }
-    }
 }
 
 // d gamma_AB / dR for exponents ta, tb (tau = 16 U / 5): derivative of
@@ -83,8 +49,8 @@ __device__ double gamma_dR(double ta, double tb, double R) {
 //   + [p K1 + (M + M^T) c (K2 - K3)] / r.
 // nper = 1 (s only): w_00 K0' c.
 __device__ __forceinline__ void block_sum_grad(int nper, const double (&w)[16], const double c[3],
-                                               double r, const double K[4], const double dK[4],
-                                               double g[3]) {
+                                               double inv_r, const double K[4],
+                                               const double dK[4], double g[3]) {
     if (nper == 1) {
         for (int q = 0; q < 3; ++q) g[q] = w[0] * dK[0] * c[q];
         return;
@@ -99,151 +65,243 @@ __device__ __forceinline__ void block_sum_grad(int nper, const double (&w)[16], 
     const double cMc = c[0] * Mc[0] + c[1] * Mc[1] + c[2] * Mc[2];
     const double tr = w[5] + w[10] + w[15];
     const double d23 = K[2] - K[3];
-    const double inv_r = 1.0 / r;
     const double par = w[0] * dK[0] + pc * dK[1] + cMc * (dK[2] - dK[3]) + tr * dK[3] -
                        (pc * K[1] + 2.0 * cMc * d23) * inv_r;
     for (int q = 0; q < 3; ++q)
         g[q] = par * c[q] + (p[q] * K[1] + (Mc[q] + MTc[q]) * d23) * inv_r;
 }
 
-// One block per atom A, its threads over the partners B: F_A = sum over B != A of the pair
-// terms of eq:forces (energy-weighted form of the S-derivative terms, velocity terms
-// dropped):
+// Pair terms of the forces (eq:forces, energy-weighted form of the S-derivative terms, velocity
+// terms dropped), one thread per pair A < B (blockIdx.y = A): the force on A,
 //   sum over the (A, B) block of 2 Re rho_ij dH_ij/dR_B + (Re rho_ij (v_A + v_B) - 2 Re W_ij)
-//   dS_ij/dR_B, plus -dq_A dq_B dgamma/dR_A + rep_A/rep_b e^{-r/rep_b} u, and -dq_A E(t);
-// W = 1/2 (X + X^dagger), X = S^-1 H rho.  The block sums are differentiated in contracted
-// form (block_sum_grad); FP64.
-__global__ void __launch_bounds__(128)
-    k_forces(int nat, int nper, int scc, const double* __restrict__ R,
-             const double* __restrict__ rre, const double* __restrict__ wre,
-             const double* __restrict__ v_atom, const double* __restrict__ dq,
-             const double* __restrict__ U, ModelParams mp, const DevScalars* __restrict__ sc,
-             double* __restrict__ F) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int A = blockIdx.x;
-    const int N = nat * nper;
-    const double RA[3] = {R[3 * A], R[3 * A + 1], R[3 * A + 2]};
-    const double vA = v_atom[A], dqA = dq[A], tA = 3.2 * U[A];
-    double f[3] = {0.0, 0.0, 0.0};
-    for (int B = threadIdx.x; B < nat; B += blockDim.x) {
-        if (B == A) continue;
-        const double d[3] = {R[3 * B] - RA[0], R[3 * B + 1] - RA[1], R[3 * B + 2] - RA[2]};
-        const double r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-        const double inv_r = 1.0 / r;
-        const double c[3] = {d[0] * inv_r, d[1] * inv_r, d[2] * inv_r};
-        const double eh = exp(-r / mp.lam_H), es = exp(-r / mp.lam_S);
-        double KH[4], dKH[4], KS[4], dKS[4];
-        for (int k = 0; k < 4; ++k) {
-            KH[k] = mp.eta[k] * mp.t0 * eh;
-            dKH[k] = -KH[k] / mp.lam_H;
-            KS[k] = -mp.eta[k] * mp.s0 * es;
-            dKS[k] = -KS[k] / mp.lam_S;
-        }
-        const double vv = vA + v_atom[B];
-        double wh[16], ws[16];
-        for (int i = 0; i < nper; ++i) {
-            const size_t row = (size_t)(A * nper + i) * N + (size_t)B * nper;
-            for (int j = 0; j < nper; ++j) {
-                const double pr = rre[row + j], w = wre[row + j];
-                wh[4 * i + j] = 2.0 * pr;
-                ws[4 * i + j] = pr * vv - 2.0 * w;
-            }
-        }
-        double gh[3], gs[3];
-        block_sum_grad(nper, wh, c, r, KH, dKH, gh);
-        block_sum_grad(nper, ws, c, r, KS, dKS, gs);
-        for (int q = 0; q < 3; ++q) f[q] += gh[q] + gs[q];
-        // u = (R_A - R_B) / r = -c
-        if (scc) {
-            const double g = gamma_dR(tA, 3.2 * U[B], r);
-            const double s = dqA * dq[B] * g;
-            for (int q = 0; q < 3; ++q) f[q] += s * c[q];
-        }
-        if (mp.rep_A != 0.0) {
-            const double e = mp.rep_A / mp.rep_b * exp(-r / mp.rep_b);
-            for (int q = 0; q < 3; ++q) f[q] -= e * c[q];
-        }
-    }
-    for (int q = 0; q < 3; ++q) f[q] = warp_sum_d(f[q]);
-    __shared__ double red[3][4];
-    if (lane == 0)
-        for (int q = 0; q < 3; ++q) red[q][warp] = f[q];
-    __syncthreads();
-    if (threadIdx.x < 3) {
-        const int q = threadIdx.x;
-        F[3 * A + q] = ((red[q][0] + red[q][1]) + (red[q][2] + red[q][3])) - dqA * sc->E[q];
-    }
-}
+//   dS_ij/dR_B, plus -dq_A dq_B dgamma/dR_A + rep_A/rep_b e^{-r/rep_b} u;
+// W = 1/2 (X + X^dagger), X = S^-1 H rho, is formed from the blocks (A, B) and (B, A) of Re X.
+// The force on B is its negative: pf[A][B] = f, pf[B][A] = -f, so that an atom's row sums to its
+// force.  Bound by FP64 issue (two lanes a clock per SM): the block sums are differentiated in
+// contracted form (block_sum_grad) and each pair is evaluated once.
+constexpr int kPairThreads = 64;
 
-// Re W = 1/2 (Re X + Re X^T) through a shared-memory tile transpose.
-__global__ void k_wre(int N, const double* __restrict__ xre, double* __restrict__ wre) {
-    __shared__ double t[kTile][kTile + 1];
-    const int bx = blockIdx.x * kTile, by = blockIdx.y * kTile;
-    for (int y = threadIdx.y; y < kTile; y += blockDim.y) {
-        const int r = bx + y, c = by + threadIdx.x;   // transposed tile
-        t[y][threadIdx.x] = (r < N && c < N) ? xre[(size_t)r * N + c] : 0.0;
-    }
-    __syncthreads();
-    for (int y = threadIdx.y; y < kTile; y += blockDim.y) {
-        const int r = by + y, c = bx + threadIdx.x;
-        if (r < N && c < N) wre[(size_t)r * N + c] = 0.5 * (xre[(size_t)r * N + c] + t[threadIdx.x][y]);
-    }
-}
-
-// D_mu_nu = Rdot_B . grad_B S_mu_nu for mu in A, nu in B != A; on-site blocks 0.
-__global__ void k_build_nac(int nat, int nper, const double* __restrict__ R,
-                            const double* __restrict__ V, ModelParams mp, double* __restrict__ D) {
-    const int B = blockIdx.x * blockDim.x + threadIdx.x;
-    const int A = blockIdx.y * blockDim.y + threadIdx.y;
-    if (A >= nat || B >= nat) return;
-    const int N = nat * nper;
+__global__ void __launch_bounds__(kPairThreads)
+    k_pair_forces(int nat, int nper, int scc, const double* __restrict__ R,
+                  const double* __restrict__ rre, const double* __restrict__ xre,
+                  const double* __restrict__ v_atom, const double* __restrict__ dq,
+                  const double* __restrict__ U, ModelParams mp, double* __restrict__ pf) {
+    const int A = blockIdx.y, B = blockIdx.x * kPairThreads + threadIdx.x;
+    pdl_launch_dependents();
+    pdl_wait();
+    if (B < A || B >= nat) return;
+    const size_t ab = 3 * ((size_t)A * nat + B), ba = 3 * ((size_t)B * nat + A);
     if (A == B) {
-        for (int i = 0; i < nper; ++i)
-            for (int j = 0; j < nper; ++j) D[(size_t)(A * nper + i) * N + B * nper + j] = 0.0;
+        for (int q = 0; q < 3; ++q) pf[ab + q] = 0.0;
         return;
     }
+    const int N = nat * nper;
     const double d[3] = {R[3 * B] - R[3 * A], R[3 * B + 1] - R[3 * A + 1], R[3 * B + 2] - R[3 * A + 2]};
-    const double r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-    const double c[3] = {d[0] / r, d[1] / r, d[2] / r};
-    double KS[4], dKS[4];
-    radial(mp, r, false, KS, dKS);
-    for (int i = 0; i < nper; ++i)
-        for (int j = 0; j < nper; ++j) {
-            double g[3];
-            block_grad(i, j, c, r, KS, dKS, g);
-            D[(size_t)(A * nper + i) * N + B * nper + j] =
-                V[3 * B] * g[0] + V[3 * B + 1] * g[1] + V[3 * B + 2] * g[2];
+    const double vv = v_atom[A] + v_atom[B];
+    double wh[16], ws[16];
+    if (nper == 4) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const double2* pr = reinterpret_cast<const double2*>(rre + (size_t)(4 * A + i) * N + 4 * B);
+            const double2* px = reinterpret_cast<const double2*>(xre + (size_t)(4 * A + i) * N + 4 * B);
+            const double2 p0 = pr[0], p1 = pr[1], x0 = px[0], x1 = px[1];
+            wh[4 * i] = p0.x, wh[4 * i + 1] = p0.y, wh[4 * i + 2] = p1.x, wh[4 * i + 3] = p1.y;
+            ws[4 * i] = x0.x, ws[4 * i + 1] = x0.y, ws[4 * i + 2] = x1.x, ws[4 * i + 3] = x1.y;
         }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const double2* px = reinterpret_cast<const double2*>(xre + (size_t)(4 * B + j) * N + 4 * A);
+            const double2 x0 = px[0], x1 = px[1];
+            const double x[4] = {x0.x, x0.y, x1.x, x1.y};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) ws[4 * i + j] = fma(wh[4 * i + j], vv, -(ws[4 * i + j] + x[i]));
+        }
+    } else {
+        for (int k = 0; k < 16; ++k) wh[k] = ws[k] = 0.0;
+        wh[0] = rre[(size_t)A * N + B];
+        ws[0] = wh[0] * vv - (xre[(size_t)A * N + B] + xre[(size_t)B * N + A]);
+    }
+    const double r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
+    const double inv_r = 1.0 / r;
+    const double c[3] = {d[0] * inv_r, d[1] * inv_r, d[2] * inv_r};
+    // the hopping block carries 2 Re rho
+    const double eh = 2.0 * mp.t0 * exp(-r / mp.lam_H), es = -mp.s0 * exp(-r / mp.lam_S);
+    const double ih = -1.0 / mp.lam_H, is = -1.0 / mp.lam_S;
+    double K[4], dK[4], g[3], f[3];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        K[k] = mp.eta[k] * eh;
+        dK[k] = K[k] * ih;
+    }
+    block_sum_grad(nper, wh, c, inv_r, K, dK, f);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        K[k] = mp.eta[k] * es;
+        dK[k] = K[k] * is;
+    }
+    block_sum_grad(nper, ws, c, inv_r, K, dK, g);
+    double s = 0.0;
+    if (scc) s = dq[A] * dq[B] * gamma_dR(3.2 * U[A], 3.2 * U[B], r);
+    if (mp.rep_A != 0.0) s -= mp.rep_A / mp.rep_b * exp(-r / mp.rep_b);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const double t = f[q] + g[q] + s * c[q];   // u = (R_A - R_B) / r = -c
+        pf[ab + q] = t;
+        pf[ba + q] = -t;
+    }
 }
 
-// Per block: sum_ij Re X_ij (D_ji - D_ij)  (P = Re Tr[S^-1 H rho (D - D^T)]).
-__global__ void k_power(int N, const double* __restrict__ xre, const double* __restrict__ D,
-                        double* __restrict__ out) {
-    double s = 0.0;
-    const size_t NN = (size_t)N * N;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < NN;
-         i += (size_t)gridDim.x * blockDim.x) {
-        const size_t r = i / N, c = i % N;
-        s += xre[i] * (D[c * N + r] - D[i]);
+// F_A = sum_B pf[A][B] - dq_A E(t), one warp per atom; then V_n = V_{n-1/2} + F_n dt / 2m (V_0
+// itself at the first step).
+__global__ void __launch_bounds__(128)
+    k_force_sum(int nat, const double* __restrict__ pf, const double* __restrict__ dq,
+                const DevScalars* __restrict__ sc, const double* __restrict__ Vh,
+                const double* __restrict__ mass, double dt, int first, double* __restrict__ F,
+                double* __restrict__ Vn) {
+    const int lane = threadIdx.x & 31, A = blockIdx.x * 4 + (threadIdx.x >> 5);
+    pdl_launch_dependents();
+    pdl_wait();
+    if (A >= nat) return;
+    double f[3] = {0.0, 0.0, 0.0};
+    const double* p = pf + 3 * (size_t)A * nat;
+    for (int B = lane; B < nat; B += 32)
+        for (int q = 0; q < 3; ++q) f[q] += p[3 * B + q];
+    for (int q = 0; q < 3; ++q) f[q] = warp_sum_d(f[q]);
+    if (lane < 3) {
+        const int i = 3 * A + lane;
+        const double x = (lane == 0 ? f[0] : lane == 1 ? f[1] : f[2]) - dq[A] * sc->E[lane];
+        F[i] = x;
+        Vn[i] = first ? Vh[i] : Vh[i] + x * dt / (2.0 * (mass[A] * 1822.888486));
     }
-    __shared__ double red[32];
-    s = warp_sum_d(s);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+}
+
+// The non-adiabatic coupling D_mu_nu = Rdot_B . grad_B S_mu_nu (mu in A, nu in B != A, on-site
+// blocks 0; eq:nac, eq:onsite), or with `transposed` its transpose, and the pair sums of the work
+// rate P = Re Tr[S^-1 H rho (D - D^T)].  One thread per pair A < B (blockIdx.y = A): both blocks
+// of a pair are directional derivatives of one s/p block T(d), d = R_B - R_A,
+//   D_AB,ij = V_B . grad T_ij,  D_BA,ji = -V_A . grad T_ij,
+// with d(c_a) = (V_a - c_a (c.V)) / r and d(K) = K' (c.V) along V.
+__device__ __forceinline__ void block_along(int nper, const double c[3], double inv_r, const double K[4],
+                                            const double dK[4], const double V[3], double (&o)[16]) {
+    const double cv = c[0] * V[0] + c[1] * V[1] + c[2] * V[2];
+    o[0] = dK[0] * cv;
+    if (nper == 1) return;
+    double dc[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) dc[a] = (V[a] - c[a] * cv) * inv_r;
+    const double k1 = dK[1] * cv, d23 = K[2] - K[3], k23 = (dK[2] - dK[3]) * cv, k3 = dK[3] * cv;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const double sa = dc[a] * K[1] + c[a] * k1;
+        o[1 + a] = sa;
+        o[4 * (1 + a)] = -sa;
+#pragma unroll
+        for (int b = 0; b <= a; ++b) {
+            const double pp = (dc[a] * c[b] + c[a] * dc[b]) * d23 + c[a] * c[b] * k23 + (a == b ? k3 : 0.0);
+            o[4 * (1 + a) + 1 + b] = pp;
+            o[4 * (1 + b) + 1 + a] = pp;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kPairThreads)
+    k_nac_power(int nat, int nper, const double* __restrict__ R, const double* __restrict__ V,
+                ModelParams mp, const double* __restrict__ xre, int transposed, double* __restrict__ D,
+                double* __restrict__ part) {
+    const int A = blockIdx.y, B = blockIdx.x * kPairThreads + threadIdx.x;
+    const int N = nat * nper;
+    double p = 0.0;
+    pdl_launch_dependents();
+    pdl_wait();
+    if (B >= A && B < nat) {
+        double ab[16], ba[16];   // blocks (A, B) and, transposed, (B, A) of D
+        if (A == B) {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) ab[k] = ba[k] = 0.0;
+        } else {
+            const double d[3] = {R[3 * B] - R[3 * A], R[3 * B + 1] - R[3 * A + 1],
+                                 R[3 * B + 2] - R[3 * A + 2]};
+            const double r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
+            const double inv_r = 1.0 / r;
+            const double c[3] = {d[0] * inv_r, d[1] * inv_r, d[2] * inv_r};
+            const double es = -mp.s0 * exp(-r / mp.lam_S), is = -1.0 / mp.lam_S;
+            double K[4], dK[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                K[k] = mp.eta[k] * es;
+                dK[k] = K[k] * is;
+            }
+            const double vb[3] = {V[3 * B], V[3 * B + 1], V[3 * B + 2]};
+            const double va[3] = {-V[3 * A], -V[3 * A + 1], -V[3 * A + 2]};
+            block_along(nper, c, inv_r, K, dK, vb, ab);
+            block_along(nper, c, inv_r, K, dK, va, ba);
+            // P: X_AB,ij (D_BA,ji - D_AB,ij) + X_BA,ji (D_AB,ij - D_BA,ji)
+            if (nper == 4) {
+                double x[16];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const double2* px = reinterpret_cast<const double2*>(xre + (size_t)(4 * A + i) * N + 4 * B);
+                    const double2 x0 = px[0], x1 = px[1];
+                    x[4 * i] = x0.x, x[4 * i + 1] = x0.y, x[4 * i + 2] = x1.x, x[4 * i + 3] = x1.y;
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const double2* px = reinterpret_cast<const double2*>(xre + (size_t)(4 * B + j) * N + 4 * A);
+                    const double2 x0 = px[0], x1 = px[1];
+                    const double y[4] = {x0.x, x0.y, x1.x, x1.y};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        p = fma(x[4 * i + j] - y[i], ba[4 * i + j] - ab[4 * i + j], p);
+                }
+            } else {
+                p = (xre[(size_t)A * N + B] - xre[(size_t)B * N + A]) * (ba[0] - ab[0]);
+            }
+        }
+        // (A, B) holds ab and (B, A) the transpose of ba; in D^T the two change places
+        if (nper == 4) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                double2* o = reinterpret_cast<double2*>(D + (size_t)(4 * A + i) * N + 4 * B);
+                const double* s = transposed ? ba : ab;
+                o[0] = make_double2(s[4 * i], s[4 * i + 1]);
+                o[1] = make_double2(s[4 * i + 2], s[4 * i + 3]);
+            }
+            if (A != B)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    double2* o = reinterpret_cast<double2*>(D + (size_t)(4 * B + j) * N + 4 * A);
+                    const double* s = transposed ? ab : ba;
+                    o[0] = make_double2(s[j], s[4 + j]);
+                    o[1] = make_double2(s[8 + j], s[12 + j]);
+                }
+        } else {
+            D[(size_t)A * N + B] = transposed ? ba[0] : ab[0];
+            if (A != B) D[(size_t)B * N + A] = transposed ? ab[0] : ba[0];
+        }
+    }
+    p = warp_sum_d(p);
+    __shared__ double red[kPairThreads / 32];
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = p;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += red[k];
-        out[blockIdx.x] = t;
-    }
+    if (threadIdx.x == 0) part[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = red[0] + red[1];
 }
 
 // Sum the block partials into P_n; work_n = work_{n-1} + dt/2 (P_n + P_{n-1}) (none at
 // the first step).  commit = 0: only report (observables of the current state).
-__global__ void k_power_finish(int nb, const double* __restrict__ part, MdScalars* __restrict__ md,
-                               double dt, int first, int commit) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+__global__ void __launch_bounds__(1024)
+    k_power_finish(int nb, const double* __restrict__ part, MdScalars* __restrict__ md, double dt,
+                   int first, int commit) {
     double p = 0.0;
-    for (int k = 0; k < nb; ++k) p += part[k];
+    pdl_launch_dependents();
+    pdl_wait();
+    for (int k = threadIdx.x; k < nb; k += 1024) p += part[k];
+    p = warp_sum_d(p);
+    __shared__ double red[32];
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = p;
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    p = warp_sum_d(red[threadIdx.x]);
+    if (threadIdx.x != 0) return;
     const double w = first ? md->work : md->work + 0.5 * dt * (p + md->P_prev);
     md->P_now = p;
     md->work_now = w;
@@ -251,16 +309,6 @@ __global__ void k_power_finish(int nb, const double* __restrict__ part, MdScalar
         md->work = w;
         md->P_prev = p;
     }
-}
-
-// V_n = V_{n-1/2} + F_n dt / 2m (V_0 itself at the first step), into Vn.
-__global__ void k_vel_n(int nat, const double* __restrict__ Vh, const double* __restrict__ F,
-                        const double* __restrict__ mass, double dt, int first,
-                        double* __restrict__ Vn) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= 3 * nat) return;
-    const double m = mass[i / 3] * 1822.888486;
-    Vn[i] = first ? Vh[i] : Vh[i] + F[i] * dt / (2.0 * m);
 }
 
 // V_{n+1/2} = V_n + F_n dt / 2m;  R_{n+1} = R_n + dt V_{n+1/2}.
@@ -277,30 +325,24 @@ __global__ void k_vv(int nat, const double* __restrict__ Vn, const double* __res
 
 }  // namespace
 
-void launch_forces(const Ctx& c, const double* rre, const double* wre, double* F, cudaStream_t st) {
-    k_forces<<<c.nat, 128, 0, st>>>(c.nat, c.nper, c.prm.scc, c.d_R, rre, wre, c.v_atom, c.dq,
-                                    c.d_U, c.mp, c.sc, F);
+size_t pair_blocks(int nat) { return (size_t)nat * ((nat + kPairThreads - 1) / kPairThreads); }
+
+void launch_forces(const Ctx& c, const double* rre, const double* xre, double* F, int first,
+                   cudaStream_t st) {
+    const dim3 g((c.nat + kPairThreads - 1) / kPairThreads, c.nat);
+    launch_pdl(k_pair_forces, g, dim3(kPairThreads), 0, st, c.nat, c.nper, c.prm.scc, c.d_R, rre, xre,
+               c.v_atom, c.dq, c.d_U, c.mp, c.md_pf);
+    launch_pdl(k_force_sum, dim3((c.nat + 3) / 4), dim3(128), 0, st, c.nat, c.md_pf, c.dq, c.sc, c.d_V,
+               c.d_mass, c.prm.dt, first, F, c.d_Vn);
 }
 
-void launch_wre(int N, const double* xre, double* wre, cudaStream_t st) {
-    dim3 b(kTile, 8), g((N + kTile - 1) / kTile, (N + kTile - 1) / kTile);
-    k_wre<<<g, b, 0, st>>>(N, xre, wre);
-}
-
-void launch_build_nac(const Ctx& c, const double* V, double* D, cudaStream_t st) {
-    dim3 b(32, 8), g((c.nat + 31) / 32, (c.nat + 7) / 8);
-    k_build_nac<<<g, b, 0, st>>>(c.nat, c.nper, c.d_R, V, c.mp, D);
-}
-
-void launch_power(const Ctx& c, const double* xre, const double* D, double* part, int nb,
-                  int first, int commit, cudaStream_t st) {
-    k_power<<<nb, 256, 0, st>>>(c.N, xre, D, part);
-    k_power_finish<<<1, 32, 0, st>>>(nb, part, c.md, c.prm.dt, first, commit);
-}
-
-void launch_vel_n(const Ctx& c, const double* F, int first, cudaStream_t st) {
-    k_vel_n<<<(3 * c.nat + 255) / 256, 256, 0, st>>>(c.nat, c.d_V, F, c.d_mass, c.prm.dt, first,
-                                                      c.d_Vn);
+void launch_nac_power(const Ctx& c, const double* V, const double* xre, int transposed, double* D,
+                      int first, int commit, cudaStream_t st) {
+    const dim3 g((c.nat + kPairThreads - 1) / kPairThreads, c.nat);
+    launch_pdl(k_nac_power, g, dim3(kPairThreads), 0, st, c.nat, c.nper, c.d_R, V, c.mp, xre, transposed,
+               D, c.pw_part);
+    launch_pdl(k_power_finish, dim3(1), dim3(1024), 0, st, (int)pair_blocks(c.nat), c.pw_part, c.md,
+               c.prm.dt, first, commit);
 }
 
 void launch_vv(const Ctx& c, const double* F, cudaStream_t st) {

@@ -48,6 +48,10 @@ template <>
 struct Cfg<kSeven> {
     static constexpr int NS = 7, NW = 8, BITS = 8, CHUNK = 128, STAGES = 2;
 };
+template <>
+struct Cfg<kLow> {
+    static constexpr int NS = 3, NW = 3, BITS = 7, CHUNK = 512, STAGES = 4;
+};
 template <int SCH>
 constexpr int stage_bytes() {
     return Cfg<SCH>::NS * (A_TILE + B_TILE);
@@ -61,7 +65,9 @@ template <int SCH>
 constexpr int max_pairs() {
     return Cfg<SCH>::NW <= Cfg<SCH>::NS ? Cfg<SCH>::NW : Cfg<SCH>::NS;
 }
-static_assert(smem_bytes<kSix>() <= 227 * 1024 && smem_bytes<kSeven>() <= 227 * 1024, "shared memory");
+static_assert(smem_bytes<kSix>() <= 227 * 1024 && smem_bytes<kSeven>() <= 227 * 1024 &&
+                  smem_bytes<kLow>() <= 227 * 1024,
+              "shared memory");
 static_assert(Cfg<kSix>::NW * BN <= 512 && Cfg<kSeven>::NW * BN <= 512, "accumulators must fit in TMEM");
 static_assert(max_pairs<kSix>() * Cfg<kSix>::CHUNK * 64 * 64 < (1 << 24) &&
                   max_pairs<kSeven>() * Cfg<kSeven>::CHUNK * 128 * 128 < (1 << 24),
@@ -80,6 +86,7 @@ struct Params {
     int ldc[2];
     int* err;
     uint32_t idesc[5];   // [nb]: instruction descriptor of an N = 64 nb product
+    Gate gate;
 };
 
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
@@ -149,6 +156,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STAGES);
     const uint32_t cfull = smem_u32(bars + 2 * STAGES), cempty = smem_u32(bars + 2 * STAGES + 1);
 
+    if (p.gate.norm) {
+        pdl_wait();
+        if (__uint_as_float(__ldcg(p.gate.norm)) < p.gate.below) return;
+    }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int z = blockIdx.z;
     const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
@@ -256,8 +267,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int row = m0 + quarter * 32 + lane, col0 = n0 + cg * 16;
         const uint32_t lane_off = static_cast<uint32_t>(quarter * 32) << 16;
         // sum over the chunks of the weights below NW/2 (hi) and above (lo), each in units of
-        // its smallest weight: value = hi 2^(BITS NW/2) + lo
-        constexpr int NH = NW / 2, BITS = C::BITS;
+        // its smallest weight: value = hi 2^(BITS NL) + lo
+        constexpr int NH = NW / 2, NL = NW - NH, BITS = C::BITS;
         long long hi[16], lo[16];
 #pragma unroll
         for (int j = 0; j < 16; ++j) hi[j] = lo[j] = 0;
@@ -282,10 +293,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                     else
                         lo[j] += v;
                 }
-                if (w == kHalfW - 1 || w == NW - 1) {
+                constexpr int kFirst = (kHalfW < NW ? kHalfW : NW) - 1;
+                if (w == kFirst || w == NW - 1) {
                     fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(cempty + (w == NW - 1 ? 8 : 0));
+                    if (lane == 0 && w == kFirst) mbar_arrive(cempty);
+                    if (lane == 0 && w == NW - 1) mbar_arrive(cempty + 8);
                 }
             }
         }
@@ -303,7 +316,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int e = col0 + j0 + j < p.N ? __ldg(eb + j0 + j) : 0;
-                    v[j] = scaled_sum<BITS * NH>(hi[j0 + j], lo[j0 + j], ex + e);
+                    v[j] = scaled_sum<BITS * NL>(hi[j0 + j], lo[j0 + j], ex + e);
                     if (ea >= kNonFinite || e >= kNonFinite)
                         v[j] = __longlong_as_double(0x7ff8000000000000ll);
                 }
@@ -398,12 +411,14 @@ __device__ __forceinline__ double flip(double x, unsigned long long sgn) {
 
 struct RowJob {
     const double *A, *S, *v;
+    unsigned* resid;
     int lda;
     unsigned long long sgn;
     SlicePtrs out;
 };
 struct RowJobs {
     RowJob j[3];
+    Gate gate;
 };
 
 // One block per row (blockIdx.x) and matrix (blockIdx.y); every thread keeps its 4 PASS
@@ -418,10 +433,13 @@ __global__ void __launch_bounds__(256)
     const double* a = job.A + static_cast<size_t>(row) * job.lda;
     const double* s = job.S ? job.S + static_cast<size_t>(row) * job.lda : nullptr;
     __shared__ uint32_t red[8];
+    __shared__ float red_f[8];
     double x[PASS][4];
     uint32_t mh = 0;
+    float abs_sum = 0.f;
     pdl_launch_dependents();
     pdl_wait();
+    if (jobs.gate.norm && __uint_as_float(__ldcg(jobs.gate.norm)) < jobs.gate.below) return;
     const double vr = job.S ? __ldg(job.v + row) : 0.0;
     const bool vec = ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(s)) & 15) == 0;
 #pragma unroll
@@ -448,13 +466,31 @@ __global__ void __launch_bounds__(256)
                 if (s && k + j < K) x[i][j] += 0.5 * s[k + j] * (vr + __ldg(job.v + k + j));
             }
         }
+        if (job.resid) {
+            // row of 1 - A: only the diagonal needs arithmetic
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                x[i][j] = k + j == row ? 1.0 - x[i][j] : flip(x[i][j], 0x8000000000000000ull);
+                abs_sum += fabsf(static_cast<float>(x[i][j]));
+            }
+        }
 #pragma unroll
         for (int j = 0; j < 4; ++j)
             mh = max(mh, static_cast<uint32_t>(__double2hiint(x[i][j])) & 0x7fffffffu);
     }
     mh = __reduce_max_sync(0xffffffffu, mh);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mh;
+    if (job.resid) {
+        for (int o = 16; o > 0; o >>= 1) abs_sum += __shfl_xor_sync(0xffffffffu, abs_sum, o);
+        if ((threadIdx.x & 31) == 0) red_f[threadIdx.x >> 5] = abs_sum;
+    }
     __syncthreads();
+    if (job.resid && threadIdx.x == 0) {
+        float t = 0.f;
+        for (int w = 0; w < static_cast<int>(blockDim.x >> 5); ++w) t += red_f[w];
+        // a NaN counts as the largest norm
+        atomicMax(job.resid, t >= 0.f ? __float_as_uint(t) : 0x7f800000u);
+    }
     for (int w = 0; w < static_cast<int>(blockDim.x >> 5); ++w) mh = max(mh, red[w]);
     const int e = row_exponent(mh);
     if (threadIdx.x == 0) job.out.e[row] = e;
@@ -580,10 +616,11 @@ bool sliced_init(Sliced& s, void* base, int rows, int K, int box_rows, int schem
     return true;
 }
 
-void slice_rows(const SliceJob* jobs, int njobs, cudaStream_t st) {
+void slice_rows(const SliceJob* jobs, int njobs, cudaStream_t st, Gate gate) {
     RowJobs j{};
+    j.gate = gate;
     for (int i = 0; i < njobs; ++i)
-        j.j[i] = {jobs[i].A, jobs[i].S, jobs[i].v, jobs[i].lda,
+        j.j[i] = {jobs[i].A, jobs[i].S, jobs[i].v, jobs[i].resid, jobs[i].lda,
                   jobs[i].sign < 0 ? 0x8000000000000000ull : 0ull, ptrs(*jobs[i].out)};
     const Sliced& o = *jobs[0].out;
     if (o.scheme == kSeven)
@@ -619,12 +656,18 @@ cudaError_t prepare() {
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_oz_gemm<kSeven>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  smem_bytes<kSeven>());
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_oz_gemm<kLow>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 smem_bytes<kLow>());
     return e;
 }
 
-cudaError_t gemm(const Sliced& a, const Part* parts, int nparts, int* err, cudaStream_t st) {
-    if (nparts < 1 || nparts > 2 || a.K < 1 || a.K > kMaxK) return cudaErrorInvalidValue;
-    const int N = parts[0].b->rows, ns = n_slices(a.scheme);
+cudaError_t gemm(const Sliced& a, const Part* parts, int nparts, int* err, cudaStream_t st,
+                 Gate gate, bool low) {
+    if (nparts < 1 || nparts > 2 || a.K < 1 || a.K > kMaxK || (low && a.scheme != kSix))
+        return cudaErrorInvalidValue;
+    const int scheme = low ? static_cast<int>(kLow) : a.scheme;
+    const int N = parts[0].b->rows, ns = n_slices(scheme);
     Maps m{};
     Params p{};
     for (int q = 0; q < ns; ++q) m.a[q] = a.map[q];
@@ -641,9 +684,11 @@ cudaError_t gemm(const Sliced& a, const Part* parts, int nparts, int* err, cudaS
     p.K = a.K;
     p.ea = a.e;
     p.err = err;
+    p.gate = gate;
     for (int nb = 1; nb <= 4; ++nb) p.idesc[nb] = tc::idesc_f16(0, nb * BN);
     const dim3 grid((N + BN - 1) / BN, (a.rows + BM - 1) / BM, nparts);
-    return a.scheme == kSeven ? run_gemm<kSeven>(m, p, grid, st) : run_gemm<kSix>(m, p, grid, st);
+    if (scheme == kLow) return run_gemm<kLow>(m, p, grid, st);
+    return scheme == kSeven ? run_gemm<kSeven>(m, p, grid, st) : run_gemm<kSix>(m, p, grid, st);
 }
 
 }  // namespace oz

@@ -60,58 +60,6 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// One thread per (A, B) atom pair writes the nper x nper blocks of S and H0.
-// Off-site: Slater-Koster s/p table with direction cosines c of R_B - R_A:
-//   ss = K0, s-a = c_a K1, a-s = -c_a K1, a-b = c_a c_b (K2 - K3) + delta_ab K3,
-// with hopping K = eta t0 exp(-r/lam_H) and overlap K = -eta s0 exp(-r/lam_S).
-__global__ void k_build_model(int nat, int nper, const double* __restrict__ R,
-                              const double* __restrict__ onsite, ModelParams mp,
-                              double* __restrict__ S, double* __restrict__ H0) {
-    const int B = blockIdx.x * blockDim.x + threadIdx.x;
-    const int A = blockIdx.y * blockDim.y + threadIdx.y;
-    if (A >= nat || B >= nat) return;
-    const int N = nat * nper;
-    double hb[4][4], sb[4][4];
-    if (A == B) {
-        for (int i = 0; i < 4; ++i)
-            for (int j = 0; j < 4; ++j) {
-                sb[i][j] = (i == j) ? 1.0 : 0.0;
-                hb[i][j] = (i == j && i < nper) ? onsite[A * nper + i] : 0.0;
-            }
-    } else {
-        const double dx = R[3 * B] - R[3 * A], dy = R[3 * B + 1] - R[3 * A + 1],
-                     dz = R[3 * B + 2] - R[3 * A + 2];
-        const double r = sqrt(dx * dx + dy * dy + dz * dz);
-        const double c[3] = {dx / r, dy / r, dz / r};
-        const double eh = exp(-r / mp.lam_H), es = exp(-r / mp.lam_S);
-        double kh[4], ks[4];
-        for (int k = 0; k < 4; ++k) {
-            kh[k] = mp.eta[k] * mp.t0 * eh;
-            ks[k] = -mp.eta[k] * mp.s0 * es;
-        }
-        hb[0][0] = kh[0];
-        sb[0][0] = ks[0];
-        for (int a = 0; a < 3; ++a) {
-            hb[0][1 + a] = c[a] * kh[1];
-            sb[0][1 + a] = c[a] * ks[1];
-            hb[1 + a][0] = -c[a] * kh[1];
-            sb[1 + a][0] = -c[a] * ks[1];
-            for (int b = 0; b < 3; ++b) {
-                const double cc = c[a] * c[b];
-                hb[1 + a][1 + b] = cc * (kh[2] - kh[3]) + (a == b ? kh[3] : 0.0);
-                sb[1 + a][1 + b] = cc * (ks[2] - ks[3]) + (a == b ? ks[3] : 0.0);
-            }
-        }
-    }
-    for (int i = 0; i < nper; ++i) {
-        const size_t row = (size_t)(A * nper + i) * N + (size_t)B * nper;
-        for (int j = 0; j < nper; ++j) {
-            S[row + j] = sb[i][j];
-            H0[row + j] = hb[i][j];
-        }
-    }
-}
-
 // Short-range part zeta(R) of gamma for exponents ta, tb (tau = 16 U / 5):
 // Coulomb integral of two normalised exp(-tau r) densities is 1/R - zeta(R).
 __device__ double gamma_short(double ta, double tb, double R) {
@@ -131,21 +79,86 @@ __device__ double gamma_short(double ta, double tb, double R) {
     return z;
 }
 
-__global__ void k_build_gamma(int nat, const double* __restrict__ R, const double* __restrict__ U,
-                              double* __restrict__ G) {
-    const int B = blockIdx.x * blockDim.x + threadIdx.x;
-    const int A = blockIdx.y * blockDim.y + threadIdx.y;
-    if (A >= nat || B >= nat) return;
-    double g;
+// One thread per atom pair A <= B (blockIdx.y = A) writes the nper x nper blocks (A, B) and
+// (B, A) of S and H0 and gamma_AB = gamma_BA (eq:coul).  Off-site: Slater-Koster s/p table with
+// direction cosines c of R_B - R_A:
+//   ss = K0, s-a = c_a K1, a-s = -c_a K1, a-b = c_a c_b (K2 - K3) + delta_ab K3,
+// with hopping K = eta t0 exp(-r/lam_H) and overlap K = -eta s0 exp(-r/lam_S); the block (B, A)
+// is the transpose, element for element.  FP64 issue bounds it (two lanes a clock per SM): every
+// pair is evaluated once.
+constexpr int kPairThreads = 64;
+
+__global__ void __launch_bounds__(kPairThreads)
+    k_build_pair(int nat, int nper, const double* __restrict__ R, const double* __restrict__ onsite,
+                 const double* __restrict__ U, ModelParams mp, double* __restrict__ S,
+                 double* __restrict__ H0, double* __restrict__ G) {
+    const int A = blockIdx.y, B = blockIdx.x * kPairThreads + threadIdx.x;
+    pdl_launch_dependents();
+    pdl_wait();
+    if (B < A || B >= nat) return;
+    const int N = nat * nper;
+    double hb[4][4], sb[4][4];
     if (A == B) {
-        g = U[A];
+        for (int i = 0; i < 4; ++i)
+            for (int j = 0; j < 4; ++j) {
+                sb[i][j] = (i == j) ? 1.0 : 0.0;
+                hb[i][j] = (i == j && i < nper) ? onsite[A * nper + i] : 0.0;
+            }
+        G[(size_t)A * nat + A] = U[A];
     } else {
         const double dx = R[3 * B] - R[3 * A], dy = R[3 * B + 1] - R[3 * A + 1],
                      dz = R[3 * B + 2] - R[3 * A + 2];
         const double r = sqrt(dx * dx + dy * dy + dz * dz);
-        g = 1.0 / r - gamma_short(3.2 * U[A], 3.2 * U[B], r);
+        const double c[3] = {dx / r, dy / r, dz / r};
+        const double eh = exp(-r / mp.lam_H), es = exp(-r / mp.lam_S);
+        double kh[4], ks[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            kh[k] = mp.eta[k] * mp.t0 * eh;
+            ks[k] = -mp.eta[k] * mp.s0 * es;
+        }
+        hb[0][0] = kh[0];
+        sb[0][0] = ks[0];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            hb[0][1 + a] = c[a] * kh[1];
+            sb[0][1 + a] = c[a] * ks[1];
+            hb[1 + a][0] = -hb[0][1 + a];
+            sb[1 + a][0] = -sb[0][1 + a];
+#pragma unroll
+            for (int b = 0; b <= a; ++b) {
+                const double cc = c[a] * c[b];
+                hb[1 + a][1 + b] = cc * (kh[2] - kh[3]) + (a == b ? kh[3] : 0.0);
+                sb[1 + a][1 + b] = cc * (ks[2] - ks[3]) + (a == b ? ks[3] : 0.0);
+                hb[1 + b][1 + a] = hb[1 + a][1 + b];
+                sb[1 + b][1 + a] = sb[1 + a][1 + b];
+            }
+        }
+        const double g = 1.0 / r - gamma_short(3.2 * U[A], 3.2 * U[B], r);
+        G[(size_t)A * nat + B] = g;
+        G[(size_t)B * nat + A] = g;
     }
-    G[(size_t)A * nat + B] = g;
+    if (nper == 4) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const size_t ab = (size_t)(4 * A + i) * N + 4 * B, ba = (size_t)(4 * B + i) * N + 4 * A;
+            double2 *s0 = reinterpret_cast<double2*>(S + ab), *h0 = reinterpret_cast<double2*>(H0 + ab);
+            s0[0] = make_double2(sb[i][0], sb[i][1]);
+            s0[1] = make_double2(sb[i][2], sb[i][3]);
+            h0[0] = make_double2(hb[i][0], hb[i][1]);
+            h0[1] = make_double2(hb[i][2], hb[i][3]);
+            if (A != B) {
+                double2 *s1 = reinterpret_cast<double2*>(S + ba), *h1 = reinterpret_cast<double2*>(H0 + ba);
+                s1[0] = make_double2(sb[0][i], sb[1][i]);
+                s1[1] = make_double2(sb[2][i], sb[3][i]);
+                h1[0] = make_double2(hb[0][i], hb[1][i]);
+                h1[1] = make_double2(hb[2][i], hb[3][i]);
+            }
+        }
+    } else {
+        S[(size_t)A * N + B] = S[(size_t)B * N + A] = sb[0][0];
+        H0[(size_t)A * N + B] = H0[(size_t)B * N + A] = hb[0][0];
+    }
 }
 
 // Row-major upper triangle -> lower triangle (after a column-major lower potri).
@@ -540,14 +553,11 @@ inline dim3 grid2(int nx, int ny, dim3 b) {
 
 }  // namespace
 
-void launch_build_model(const Ctx& c, const double* R, double* S, double* H0, cudaStream_t st) {
-    dim3 b(32, 8);
-    k_build_model<<<grid2(c.nat, c.nat, b), b, 0, st>>>(c.nat, c.nper, R, c.d_onsite, c.mp, S, H0);
-}
-
-void launch_build_gamma(const Ctx& c, const double* R, double* gamma, cudaStream_t st) {
-    dim3 b(32, 8);
-    k_build_gamma<<<grid2(c.nat, c.nat, b), b, 0, st>>>(c.nat, R, c.d_U, gamma);
+void launch_build_pair(const Ctx& c, const double* R, double* S, double* H0, double* gamma,
+                       cudaStream_t st) {
+    const dim3 g((c.nat + kPairThreads - 1) / kPairThreads, c.nat);
+    launch_pdl(k_build_pair, g, dim3(kPairThreads), 0, st, c.nat, c.nper, R, c.d_onsite, c.d_U, c.mp, S,
+               H0, gamma);
 }
 
 void launch_symmetrize_upper_to_lower(int N, double* A, cudaStream_t st) {
@@ -640,14 +650,43 @@ __global__ void k_f64_to_f32(size_t n, const double* __restrict__ in, float* __r
         out[i] = (float)in[i];
 }
 
-// Newton-Schulz step for the inverse of S: X <- 2 X - 1/2 (Q + Q^T) with Q = X S X and X
-// symmetric (the symmetric part keeps the iterate exactly symmetric).
-__global__ void k_ns_update(int N, double* __restrict__ X, const double* __restrict__ Q) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    const int r = blockIdx.y * blockDim.y + threadIdx.y;
-    if (r >= N || c >= N) return;
-    const size_t i = (size_t)r * N + c, j = (size_t)c * N + r;
-    X[i] = 2.0 * X[i] - 0.5 * (Q[i] + Q[j]);
+// Start of the Newton-Schulz inverse at the next geometry: X <- 2 X - P (the line through the
+// last two inverses; P = null: X stays), P <- X, and a zeroed residual norm.
+__global__ void k_ns_start(size_t n, double* __restrict__ X, double* __restrict__ P, int line,
+                           unsigned* __restrict__ norm) {
+    pdl_launch_dependents();
+    pdl_wait();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *norm = 0u;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+         i += (size_t)gridDim.x * blockDim.x) {
+        const double x = X[i];
+        if (line) X[i] = 2.0 * x - P[i];
+        P[i] = x;
+    }
+}
+
+// X <- X + 1/2 (Q + Q^T) for a symmetric X: one block per tile pair, so X stays exactly
+// symmetric.  With a gate: nothing if *gate (float bits) is below `below`.
+__global__ void __launch_bounds__(256)
+    k_ns_update(int N, double* __restrict__ X, const double* __restrict__ Q,
+                const unsigned* __restrict__ gate, float below) {
+    __shared__ double a[kTile][kTile + 1], b[kTile][kTile + 1];
+    const int bi = blockIdx.y, bj = blockIdx.x;
+    pdl_launch_dependents();
+    pdl_wait();
+    if (bi > bj || (gate && __uint_as_float(__ldcg(gate)) < below)) return;
+    const int tx = threadIdx.x;
+    for (int y = threadIdx.y; y < kTile; y += 8) {
+        const int r = bi * kTile + y, c = bj * kTile + tx, r2 = bj * kTile + y, c2 = bi * kTile + tx;
+        a[y][tx] = r < N && c < N ? Q[(size_t)r * N + c] : 0.0;
+        b[y][tx] = r2 < N && c2 < N ? Q[(size_t)r2 * N + c2] : 0.0;
+    }
+    __syncthreads();
+    for (int y = threadIdx.y; y < kTile; y += 8) {
+        const int r = bi * kTile + y, c = bj * kTile + tx, r2 = bj * kTile + y, c2 = bi * kTile + tx;
+        if (r < N && c < N) X[(size_t)r * N + c] += 0.5 * (a[y][tx] + b[tx][y]);
+        if (bi != bj && r2 < N && c2 < N) X[(size_t)r2 * N + c2] += 0.5 * (b[y][tx] + a[tx][y]);
+    }
 }
 
 __global__ void k_f32_to_f64(size_t n, const float* __restrict__ in, double* __restrict__ out) {
@@ -718,9 +757,14 @@ void launch_absmax(size_t n, const double* x, double* out, cudaStream_t st, cons
     k_absmax<<<608, 256, 0, st>>>(n, x, sub, out);
 }
 
-void launch_ns_update(int N, double* X, const double* Q, cudaStream_t st) {
-    dim3 b(32, 8);
-    k_ns_update<<<grid2(N, N, b), b, 0, st>>>(N, X, Q);
+void launch_ns_start(int N, double* X, double* P, int line, unsigned* norm, cudaStream_t st) {
+    launch_pdl(k_ns_start, dim3(1216), dim3(256), 0, st, (size_t)N * N, X, P, line, norm);
+}
+
+void launch_ns_update(int N, double* X, const double* Q, const unsigned* gate, float below,
+                      cudaStream_t st) {
+    const int nt = (N + kTile - 1) / kTile;
+    launch_pdl(k_ns_update, dim3(nt, nt), dim3(kTile, 8), 0, st, N, X, Q, gate, below);
 }
 
 void launch_f32_to_f64(size_t n, const float* in, double* out, cudaStream_t st) {

@@ -14,7 +14,9 @@
 namespace tdb {
 void launch_f64_to_f32(size_t n, const double* in, float* out, cudaStream_t st);
 void launch_f32_to_f64(size_t n, const float* in, double* out, cudaStream_t st);
-void launch_ns_update(int N, double* X, const double* Q, cudaStream_t st);
+void launch_ns_start(int N, double* X, double* P, int line, unsigned* norm, cudaStream_t st);
+void launch_ns_update(int N, double* X, const double* Q, const unsigned* gate, float below,
+                      cudaStream_t st);
 namespace learn {
 void launch_window(int N, const double* eps, double dt, int k, double* x0re, double* x0im,
                    double* x1re, double* x1im, cudaStream_t st);
@@ -191,7 +193,6 @@ size_t carve(Ctx& c, char* base) {
     if (use_slices(c)) {
         // slices of S^-1 (A), H or D (B), M or Y (A), Re rho and Im rho (B)
         for (int q = 0; q < 5; ++q) c.oz_raw[q] = k.take<char>(oz::sliced_bytes(N, N, slice_scheme(c)));
-        c.oz_colmax = k.take<double>(N);
     }
     if (md32(c)) {
         c.md_sinv = k.take<float>(NN);
@@ -231,8 +232,10 @@ size_t carve(Ctx& c, char* base) {
         c.D = k.take<double>(NN);
         c.Zre = k.take<double>(NN);
         c.Zim = k.take<double>(NN);
-        c.Wre = k.take<double>(NN);
-        c.pw_part = k.take<double>(kObsBlocks);
+        c.md_pf = k.take<double>(3 * nat * nat);
+        c.pw_part = k.take<double>(pair_blocks(c.nat));
+        c.inv_norm = k.take<unsigned>(1);
+        if (sliced(c)) c.Sinv_p = k.take<double>(NN);
         c.md = k.take<MdScalars>(1);
     }
     c.d_err = k.take<int>(4);
@@ -746,11 +749,16 @@ tdb_status build_maps(Ctx& c) {
     return TDB_OK;
 }
 
-// S^-1 at the current geometry without synchronising (moving nuclei): Cholesky
-// and inverse in the preallocated workspace; a non-positive-definite S shows up as
-// NaN through tdb_check.
+// S^-1 at the current geometry without synchronising (moving nuclei); a non-positive-definite
+// S shows up as NaN through tdb_check.  Small systems use the library's own kernels, larger ones
+// a Cholesky factorisation and inverse in the preallocated workspace.
 tdb_status enqueue_inverse(Ctx& c) {
     const int N = c.N;
+    if (N <= kSmallInverseN) {
+        launch_small_inverse(N, c.S, c.Sinv, c.M, c.Hs, c.Xre, c.inv_norm, c.stream);
+        CKL();
+        return TDB_OK;
+    }
     CK(cudaMemcpyAsync(c.Sinv, c.S, sizeof(double) * N * N, cudaMemcpyDeviceToDevice, c.stream));
     CKS(cusolverDnDpotrf(c.solver, CUBLAS_FILL_MODE_LOWER, N, c.Sinv, N, c.inv_work, c.inv_lwork,
                          c.inv_info));
@@ -761,36 +769,66 @@ tdb_status enqueue_inverse(Ctx& c) {
     return TDB_OK;
 }
 
-tdb_status oz_product(Ctx& c, int a, int b, double* out);
+oz::SliceJob mat_job(const Ctx& c, const double* A, oz::Sliced& out, double sign = 1.0) {
+    oz::SliceJob j;
+    j.A = A;
+    j.lda = c.N;
+    j.sign = sign;
+    j.out = &out;
+    return j;
+}
 
-// S^-1 at a new geometry from the inverse at the previous one (FP64_SLICED form):
-// Newton-Schulz steps X <- 2 X - X S X with integer-slice products.  They converge
-// quadratically while ||1 - S X|| < 1; between two steps the nuclei move by ~1e-4 bohr,
-// so the start is within ~1e-5 and two steps reach the products' precision.
+// S^-1 at a new geometry from the inverses at the previous ones (FP64_SLICED form) by a
+// Newton-Schulz step X <- X + X E, E = 1 - S X, from the line through the last two inverses
+// (from the last one after a restart).  E is a full-precision product; X E only corrects, so the
+// leading slices do (6 pairs of 21).  The nuclei move by ~1e-4 bohr a step: the line leaves
+// ||E|| ~ 1e-9 .. 1e-7, the last inverse alone ~1e-5, and the step squares it.  Where ||E||
+// exceeds kNsDone a second step follows, its launches doing nothing otherwise.  (Two full steps
+// from the last inverse: four 21-pair products instead of one and a 6-pair one.)
+constexpr float kNsDone = 3e-7f;
+
 tdb_status ns_inverse(Ctx& c) {
     const int N = c.N;
-    oz::slice_rows(c.S, N, 1.0, c.oz[2], c.stream);                 // A = S
+    launch_ns_start(N, c.Sinv, c.Sinv_p, c.line_n == c.n - 2 ? 1 : 0, c.inv_norm, c.stream);
     for (int it = 0; it < 2; ++it) {
-        oz::slice_rows(c.Sinv, N, 1.0, c.oz[1], c.stream);          // B = X (symmetric)
-        TRY(oz_product(c, 2, 1, c.M));                              // P = S X
-        oz::slice_rows(c.Sinv, N, 1.0, c.oz[0], c.stream);          // A = X
-        oz::slice_cols(c.M, N, c.oz[1], c.oz_colmax, c.stream);     // B = P
-        TRY(oz_product(c, 0, 1, c.Hs));                             // Q = X P
-        launch_ns_update(N, c.Sinv, c.Hs, c.stream);
+        const oz::Gate gate = it ? oz::Gate{c.inv_norm, kNsDone} : oz::Gate{};
+        const oz::SliceJob xs[2] = {mat_job(c, c.Sinv, c.oz[0]), mat_job(c, c.S, c.oz[1])};
+        oz::slice_rows(xs, 2, c.stream, gate);
+        oz::Part part;
+        part.b = &c.oz[1];
+        part.C = c.M;
+        part.ldc = N;
+        CK(oz::gemm(c.oz[0], &part, 1, c.d_err, c.stream, gate));           // X S = (S X)^T
+        oz::SliceJob e = mat_job(c, c.M, c.oz[1]);                          // rows of E^T = 1 - X S
+        e.resid = c.inv_norm;
+        oz::slice_rows(&e, 1, c.stream, gate);
+        part.C = c.Hs;
+        CK(oz::gemm(c.oz[0], &part, 1, c.d_err, c.stream, gate, true));     // X E
+        launch_ns_update(N, c.Sinv, c.Hs, gate.norm, gate.below, c.stream);
     }
     CKL();
     return TDB_OK;
 }
 
-// S, H0, gamma and S^-1 at the current device geometry (moving nuclei).  Inside a step
-// of the FP64_SLICED form S^-1 follows from the previous one (ns_inverse); otherwise
-// (and after a ground state, kick or checkpoint load) it is factorised anew.
+// S, H0, gamma and S^-1 at the current device geometry (moving nuclei).  Inside a step they are
+// kept when they already belong to this step's geometry (observables were read before it, or a
+// kick or state load made them), and S^-1 of the FP64_SLICED form follows from the previous one
+// (ns_inverse); otherwise it is computed anew.
 tdb_status md_model(Ctx& c, bool in_step = false) {
-    launch_build_model(c, c.d_R, c.S, c.H0, c.stream);
-    launch_build_gamma(c, c.d_R, c.gamma, c.stream);
+    if (in_step && c.model_n == c.n) return TDB_OK;
+    launch_build_pair(c, c.d_R, c.S, c.H0, c.gamma, c.stream);
     CKL();
-    if (in_step && sliced(c)) return ns_inverse(c);
-    return enqueue_inverse(c);
+    const long long last = c.model_n;
+    c.model_n = -10;
+    if (in_step && sliced(c) && c.N > kSmallInverseN && last == c.n - 1) {
+        TRY(ns_inverse(c));
+        c.line_n = last;
+    } else {
+        TRY(enqueue_inverse(c));
+        c.line_n = -10;
+    }
+    c.model_n = c.n;
+    return TDB_OK;
 }
 
 // Optional per-kernel timing of an enqueued step: an event before each launch.
@@ -820,14 +858,6 @@ oz::SliceJob ham_job(Ctx& c) {
     j.out = &c.oz[1];
     j.S = c.S;
     j.v = c.v_orb;
-    return j;
-}
-oz::SliceJob mat_job(const Ctx& c, const double* A, oz::Sliced& out, double sign = 1.0) {
-    oz::SliceJob j;
-    j.A = A;
-    j.lda = c.N;
-    j.sign = sign;
-    j.out = &out;
     return j;
 }
 // M (A operand) and rho_n (B operands: Re rho symmetric, (Im rho)^T = -Im rho) in one launch
@@ -907,12 +937,10 @@ tdb_status md_forces(Ctx& c, int cur, bool first, int commit, int* n, StepTimer*
         gemm_f64_pair(c.N, c.M, c.rho_re[cur], c.rho_im[cur], c.Xre, c.Xim, c.stream);
     }
     MARK("md_forces");
-    launch_wre(c.N, c.Xre, c.Wre, c.stream);
-    launch_forces(c, c.rho_re[cur], c.Wre, c.d_F, c.stream);
-    launch_vel_n(c, c.d_F, first ? 1 : 0, c.stream);
+    launch_forces(c, c.rho_re[cur], c.Xre, c.d_F, first ? 1 : 0, c.stream);
     MARK("md_nac_power");
-    launch_build_nac(c, c.d_Vn, c.D, c.stream);
-    launch_power(c, c.Xre, c.D, c.pw_part, kObsBlocks, first ? 1 : 0, commit, c.stream);
+    // the slice products take D through the rows of D^T
+    launch_nac_power(c, c.d_Vn, c.Xre, use_slices(c) ? 1 : 0, c.D, first ? 1 : 0, commit, c.stream);
     CKL();
     if (n) *n += 16;
     return TDB_OK;
@@ -926,8 +954,8 @@ tdb_status enqueue_step_md(Ctx& c, int cur, bool euler, int* launches, StepTimer
     TRY(md_forces(c, cur, euler, 1, &n, tm));
     MARK("md_products_Z");
     if (use_slices(c)) {
-        // Y = S^-1 D (D is not symmetric: column slices) and Z = Y rho_n
-        oz::slice_cols(c.D, c.N, c.oz[1], c.oz_colmax, c.stream);
+        // Y = S^-1 D (c.D holds D^T) and Z = Y rho_n
+        oz::slice_rows(c.D, c.N, 1.0, c.oz[1], c.stream);
         TRY(oz_product(c, 0, 1, c.M));
         oz::slice_rows(c.M, c.N, 1.0, c.oz[2], c.stream);
         TRY(oz_product_rho(c, 2, c.Zre, c.Zim));
@@ -1435,8 +1463,7 @@ tdb_status tdb_create(const tdb_system* sys, const tdb_params* prm, void* worksp
             return fail(TDB_ERR_CUDA);
     if (upload_clock(*c, 0, 0, 0.0) != TDB_OK) return fail(TDB_ERR_CUDA);
     if (upload_field(*c) != TDB_OK) return fail(TDB_ERR_CUDA);
-    launch_build_model(*c, c->d_R, c->S, c->H0, c->stream);
-    launch_build_gamma(*c, c->d_R, c->gamma, c->stream);
+    launch_build_pair(*c, c->d_R, c->S, c->H0, c->gamma, c->stream);
     if (cudaGetLastError() != cudaSuccess) {
         set_err("model build launch failed");
         return fail(TDB_ERR_CUDA);
@@ -1632,6 +1659,7 @@ tdb_status tdb_ground_state(tdb_ctx* c, int* iters_out, double* residual_out) {
         if (tensor(*c)) TRY(setup_tensor(*c));
     }
     TRY(upload_clock(*c, 0, 0, 0.0));
+    c->model_n = 0;
     TRY(refresh_derived(*c));
     CK(cudaStreamSynchronize(c->stream));
     return TDB_OK;
@@ -1816,6 +1844,8 @@ tdb_status tdb_clone(tdb_ctx* src, void* cuda_stream, void* workspace, size_t wo
     c->work = src->work;
     c->field = src->field;
     c->field_on = src->field_on;
+    c->model_n = src->model_n;
+    c->line_n = src->line_n;
     return TDB_OK;
 }
 
@@ -2242,6 +2272,7 @@ tdb_status tdb_set_state(tdb_ctx* c, const void* buf, size_t bytes) {
         CK(cudaStreamSynchronize(c->stream));
     } else {
         TRY(upload_clock(*c, hd.n, hd.n_base, hd.t_base));
+        c->model_n = hd.n;   // moving nuclei: md_model ran at the loaded positions
         TRY(refresh_derived(*c));
         CK(cudaStreamSynchronize(c->stream));
     }

@@ -148,7 +148,7 @@ struct Ctx {
     // FP64_SLICED form: slices of S^-1, H or D, M or Y, Re rho, Im rho
     oz::Sliced oz[5];
     char* oz_raw[5] = {};
-    double* oz_colmax = nullptr;
+
     // moving nuclei, FP32 form: FP32 copies of S^-1, H or D, rho_n; M or Y; X or Z
     float *md_sinv = nullptr, *md_b = nullptr, *md_rre = nullptr, *md_rim = nullptr;
     float *md_m = nullptr, *md_xre = nullptr, *md_xim = nullptr;
@@ -175,9 +175,13 @@ struct Ctx {
     // moving nuclei (Ehrenfest): per-step buffers
     double *d_Vn = nullptr;                          // V_n (d_V holds V_{n-1/2}, or V_0)
     double *d_F = nullptr;                           // [nat][3] forces F_n
-    double *D = nullptr, *Zre = nullptr, *Zim = nullptr, *Wre = nullptr;   // N x N
+    double *D = nullptr, *Zre = nullptr, *Zim = nullptr, *md_pf = nullptr;   // N x N; pair forces
     double *pw_part = nullptr;                       // work-rate block partials
     MdScalars* md = nullptr;
+    double* Sinv_p = nullptr;    // FP64_SLICED: the inverse one step earlier
+    unsigned* inv_norm = nullptr;
+    // steps whose geometry S, H0, gamma and S^-1 (and Sinv_p) on the device belong to
+    long long model_n = -10, line_n = -10;
     double* inv_work = nullptr;                      // cuSOLVER workspace (potrf/potri)
     int inv_lwork = 0;
     int* inv_info = nullptr;
@@ -194,8 +198,13 @@ struct Ctx {
 };
 
 // ---- kernels (launchers) ----
-void launch_build_model(const Ctx& c, const double* R, double* S, double* H0, cudaStream_t st);
-void launch_build_gamma(const Ctx& c, const double* R, double* gamma, cudaStream_t st);
+// S, H0 and gamma at positions R
+void launch_build_pair(const Ctx& c, const double* R, double* S, double* H0, double* gamma,
+                       cudaStream_t st);
+// S^-1 for N <= kSmallInverseN; t0, t1, t2: N x N scratch, norm: one word (kern_inv.cu)
+constexpr int kSmallInverseN = 192;
+void launch_small_inverse(int N, const double* S, double* Sinv, double* t0, double* t1, double* t2,
+                          unsigned* norm, cudaStream_t st);
 void launch_symmetrize_upper_to_lower(int N, double* A, cudaStream_t st);
 void launch_transpose(int N, const double* in, double* out, cudaStream_t st);
 void launch_mulliken_partials(int N, const double* rho_re, const double* S, double* partial,
@@ -243,12 +252,13 @@ void launch_obs_reduce(int N, const double* rho_re, const double* rho_im, const 
 void launch_obs_finish(int n_blocks, const double* block_out, double* out4, cudaStream_t st);
 void launch_scale_rows_f(int N, const double* in, const double* f, double* out, cudaStream_t st);
 // moving nuclei (kern_md.cu)
-void launch_forces(const Ctx& c, const double* rre, const double* wre, double* F, cudaStream_t st);
-void launch_wre(int N, const double* xre, double* wre, cudaStream_t st);
-void launch_build_nac(const Ctx& c, const double* V, double* D, cudaStream_t st);
-void launch_power(const Ctx& c, const double* xre, const double* D, double* part, int nb, int first,
-                  int commit, cudaStream_t st);
-void launch_vel_n(const Ctx& c, const double* F, int first, cudaStream_t st);
+// F_n from Re rho and Re X, and V_n; pair_blocks: work-rate partials of launch_nac_power
+size_t pair_blocks(int nat);
+void launch_forces(const Ctx& c, const double* rre, const double* xre, double* F, int first,
+                   cudaStream_t st);
+// D(V) (or its transpose) and the work rate
+void launch_nac_power(const Ctx& c, const double* V, const double* xre, int transposed, double* D,
+                      int first, int commit, cudaStream_t st);
 void launch_vv(const Ctx& c, const double* F, cudaStream_t st);
 // reduced-precision master (kern_step.cu)
 // Arguments of one update of the reduced forms (one problem of a grouped launch).

@@ -27,10 +27,10 @@
 namespace tdb {
 namespace oz {
 
-enum Scheme { kSix = 0, kSeven = 1 };
+enum Scheme { kSix = 0, kSeven = 1, kLow = 2 };   // kLow: leading slices of kSix operands
 constexpr int kMaxSlices = 7;
 constexpr int kMaxK = 4096;     // keeps the 64-bit sums below 2^63
-__host__ __device__ constexpr int n_slices(int scheme) { return scheme == kSeven ? 7 : 6; }
+__host__ __device__ constexpr int n_slices(int scheme) { return scheme == kSeven ? 7 : scheme == kLow ? 3 : 6; }
 
 // Slices of the rows of a rows x K matrix: s[q] is rows x ld 16-bit (FP16 integers),
 // ld a multiple of 64; e[i] the power-of-two exponent of row i (kNonFinite: the row holds
@@ -61,9 +61,16 @@ struct SliceJob {
     Sliced* out = nullptr;
     const double* S = nullptr;
     const double* v = nullptr;
+    unsigned* resid = nullptr;   // slice 1 - A instead; atomicMax of its largest absolute row sum
+                                 // (FP32, as float bits)
+};
+// A launch that does nothing if *norm (float bits, device) is below `below`.
+struct Gate {
+    const unsigned* norm = nullptr;
+    float below = 0.f;
 };
 // njobs <= 3 matrices of the same rows, K and scheme in one launch.
-void slice_rows(const SliceJob* jobs, int njobs, cudaStream_t st);
+void slice_rows(const SliceJob* jobs, int njobs, cudaStream_t st, Gate gate = {});
 void slice_rows(const double* A, int lda, double sign, Sliced& out, cudaStream_t st);
 // Slices of B^T for a general B (K x cols, row-major FP64, row stride ldb); colmax is
 // a device scratch of cols doubles.
@@ -79,7 +86,10 @@ struct Part {
 cudaError_t prepare();
 // C_z = A B_z for z < nparts (<= 2); M = a.rows, N = b.rows, K = a.K = b.K (<= kMaxK), all
 // of one scheme.  err: device flag, set to 1-3 if a bounded wait expired.
-cudaError_t gemm(const Sliced& a, const Part* parts, int nparts, int* err, cudaStream_t st);
+// low: only the three leading slices of each operand and the six pairs s + t < 3 (kSix;
+// relative error about 2^-20 of K max|A_i.| max|B_.j|).
+cudaError_t gemm(const Sliced& a, const Part* parts, int nparts, int* err, cudaStream_t st,
+                 Gate gate = {}, bool low = false);
 
 }  // namespace oz
 }  // namespace tdb

@@ -145,3 +145,55 @@ def test_training_epochs_match_the_oracle_gradients_and_adam(B, F, H, n, batch):
     assert abs(loss - sse / n) < 1e-4 * (sse / n)
     assert np.all(np.abs(got - q) <= allowed)
     assert np.mean(np.abs(got - q)) < 0.02 * lr * t
+
+
+# N = 188, 192 (the largest size of the library's own inverse), 196 (cuSOLVER / Newton-Schulz)
+@pytest.mark.parametrize("form,tol", [("fp64", 1e-9), ("fp64s", 1e-8)])
+@pytest.mark.parametrize("n_atoms", [47, 48, 49])
+def test_ehrenfest_matches_the_oracle_on_both_sides_of_the_inverse_rule(B, n_atoms, form, tol):
+    # bounds of the Ehrenfest parity tests of the two forms
+    sysm = I.small_cluster(n_atoms, seed=7, T=3000.0, rep_A=60.0)
+    run = I.Run(dt=0.2, n_steps=0, scc=True, move_nuclei=True, kick=1e-2, kT=I.SCC_KT)
+    n = 40
+    with B.Propagator(sysm, run, form) as p:
+        p.setup()
+        p.step(n // 2)
+        p.observables()                 # the next step keeps what this evaluated
+        p.step(n // 2)
+        hist = B.tdb_dipole_history(p.ctx, n)
+        obs = p.observables(forces=True)
+        again = p.observables(forces=True)
+        rho = B.tdb_get_rho(p.ctx)
+    rho0, gs, S, Sinv = O.setup(sysm, run)
+    tr = O.propagate(sysm, run, rho0, n, keep_forces=True)
+    assert np.max(np.abs(hist - tr.dipole[:n])) < tol
+    assert np.max(np.abs(obs["forces"] - tr.forces[-1])) < tol
+    assert np.max(np.abs(rho - tr.rho)) < tol
+    assert abs(obs["work"] - tr.work[-1]) < 1e-9
+    assert np.array_equal(obs["forces"], again["forces"])
+
+
+@pytest.mark.parametrize("s0", [0.3, np.float64(7.1373463)])
+def test_ill_conditioned_overlaps_are_inverted_in_fp64(B, s0):
+    # the overlap amplitude of the other systems and one that brings the smallest eigenvalue of S
+    # to ~1e-6 of the largest: past what two Newton-Schulz steps from an FP32 inverse reach.  Forces of the ground
+    # state against the oracle: an inverse accurate to cond(S) 2^-52 of its largest element (1e6
+    # here) leaves about cond^2 2^-52 of S^-1 H rho's terms, which are O(1).
+    import dataclasses
+    sysm = dataclasses.replace(I.small_cluster(12, seed=5), s0=s0)
+    S, H0 = O.model_matrices(sysm, sysm.R)
+    ev = np.linalg.eigvalsh(S)
+    cond = ev[-1] / ev[0]
+    run = I.Run(dt=1e-6, n_steps=0, scc=False, move_nuclei=True, kT=I.SCC_KT)
+    with B.Propagator(sysm, run, "fp64") as p:
+        p.setup()
+        f = p.observables(forces=True)["forces"]
+    rho, gs, S, Sinv = O.setup(sysm, run)
+    G = O.gamma_matrix(sysm, sysm.R)
+    q = O.mulliken(sysm, rho, S) - O.reference_populations(sysm)
+    E = np.zeros(3)
+    v = O.atom_potential(G, q, sysm.R, E, False)
+    H = O.scc_hamiltonian(sysm, H0, S, v)
+    ref = O.forces(sysm, rho, S, Sinv, H, G, q, v, sysm.R, E, False)
+    assert np.all(np.isfinite(f))
+    assert np.max(np.abs(f - ref)) < 1e-10 + 100 * cond ** 2 * 2.0 ** -52 * np.max(np.abs(ref))
