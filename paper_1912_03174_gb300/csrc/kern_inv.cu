@@ -17,13 +17,16 @@ namespace tdb {
 
 namespace {
 
-// In-place Gauss-Jordan inversion, thread (tx, ty) of 32 x 32 holding the elements
-// (ty + 32 a, tx + 32 b), a, b < T (rows and columns past N: identity).  A pivot that is not
-// positive makes the result NaN.
+// In-place Gauss-Jordan inversion, thread (tx, ty) of 16 x 16 holding the elements
+// (ty + 16 a, tx + 16 b), a, b < T (rows and columns past N: identity).  A pivot that is not
+// positive makes the result NaN.  One barrier a pivot: the pivot row and column go through
+// double-buffered shared memory.  Bound by the issue of the T^2 updates plus that round trip; 256
+// threads with large register tiles rather than 1024 with small ones, which spent their time on
+// the shared-memory reads, the fix-ups and the barrier.
 template <int T>
-__global__ void __launch_bounds__(1024)
+__global__ void __launch_bounds__(256)
     k_inv_f32(int N, const double* __restrict__ S, double* __restrict__ X, unsigned* __restrict__ norm) {
-    __shared__ float row_s[2][32 * T], col_s[2][32 * T];
+    __shared__ float row_s[2][16 * T], col_s[2][16 * T];
     const int tx = threadIdx.x, ty = threadIdx.y;
     float r[T][T];
     pdl_launch_dependents();
@@ -33,47 +36,45 @@ __global__ void __launch_bounds__(1024)
     for (int a = 0; a < T; ++a)
 #pragma unroll
         for (int b = 0; b < T; ++b) {
-            const int i = ty + 32 * a, j = tx + 32 * b;
+            const int i = ty + 16 * a, j = tx + 16 * b;
             r[a][b] = i < N && j < N ? static_cast<float>(S[(size_t)i * N + j]) : (i == j ? 1.f : 0.f);
         }
     bool bad = false;
     int s = 0;
 #pragma unroll
     for (int kb = 0; kb < T; ++kb)
-        for (int kk = 0; kk < 32 && kb * 32 + kk < N; ++kk, s ^= 1) {
+        for (int kk = 0; kk < 16 && kb * 16 + kk < N; ++kk, s ^= 1) {
             if (ty == kk)
 #pragma unroll
-                for (int b = 0; b < T; ++b) row_s[s][tx + 32 * b] = r[kb][b];
+                for (int b = 0; b < T; ++b) row_s[s][tx + 16 * b] = r[kb][b];
             if (tx == kk)
 #pragma unroll
-                for (int a = 0; a < T; ++a) col_s[s][ty + 32 * a] = r[a][kb];
+                for (int a = 0; a < T; ++a) col_s[s][ty + 16 * a] = r[a][kb];
             __syncthreads();
-            const float piv = col_s[s][kb * 32 + kk];
+            const float piv = col_s[s][kb * 16 + kk];
             bad |= !(piv > 0.f);
-            const float inv = 1.f / piv;
-            float rj[T], ci[T];
+            const float inv = __fdividef(1.f, piv);   // refined in FP64 afterwards
+            float rj[T];
 #pragma unroll
-            for (int b = 0; b < T; ++b) rj[b] = row_s[s][tx + 32 * b] * inv;
+            for (int b = 0; b < T; ++b) rj[b] = row_s[s][tx + 16 * b] * inv;
 #pragma unroll
-            for (int a = 0; a < T; ++a) ci[a] = col_s[s][ty + 32 * a];
+            for (int a = 0; a < T; ++a) {
+                const float ci = col_s[s][ty + 16 * a];
 #pragma unroll
-            for (int a = 0; a < T; ++a)
-#pragma unroll
-                for (int b = 0; b < T; ++b) r[a][b] = fmaf(-ci[a], rj[b], r[a][b]);
-            if (ty == kk)
+                for (int b = 0; b < T; ++b) r[a][b] = fmaf(-ci, rj[b], r[a][b]);
+                if (tx == kk) r[a][kb] = -ci * inv;
+            }
+            if (ty == kk) {
 #pragma unroll
                 for (int b = 0; b < T; ++b) r[kb][b] = rj[b];
-            if (tx == kk) {
-#pragma unroll
-                for (int a = 0; a < T; ++a) r[a][kb] = -ci[a] * inv;
-                if (ty == kk) r[kb][kb] = inv;
+                if (tx == kk) r[kb][kb] = inv;
             }
         }
 #pragma unroll
     for (int a = 0; a < T; ++a)
 #pragma unroll
         for (int b = 0; b < T; ++b) {
-            const int i = ty + 32 * a, j = tx + 32 * b;
+            const int i = ty + 16 * a, j = tx + 16 * b;
             if (i < N && j < N)
                 X[(size_t)i * N + j] = bad ? __longlong_as_double(0x7ff8000000000000ll)
                                            : static_cast<double>(r[a][b]);
@@ -180,14 +181,20 @@ __global__ void __launch_bounds__(1024)
 
 void launch_small_inverse(int N, const double* S, double* Sinv, double* t0, double* t1, double* t2,
                           unsigned* norm, cudaStream_t st) {
-    const dim3 b(32, 32);
-    switch ((N + 31) / 32) {
+    const dim3 b(16, 16);
+    switch ((N + 15) / 16) {
         case 1: launch_pdl(k_inv_f32<1>, dim3(1), b, 0, st, N, S, t0, norm); break;
         case 2: launch_pdl(k_inv_f32<2>, dim3(1), b, 0, st, N, S, t0, norm); break;
         case 3: launch_pdl(k_inv_f32<3>, dim3(1), b, 0, st, N, S, t0, norm); break;
         case 4: launch_pdl(k_inv_f32<4>, dim3(1), b, 0, st, N, S, t0, norm); break;
         case 5: launch_pdl(k_inv_f32<5>, dim3(1), b, 0, st, N, S, t0, norm); break;
-        default: launch_pdl(k_inv_f32<6>, dim3(1), b, 0, st, N, S, t0, norm); break;
+        case 6: launch_pdl(k_inv_f32<6>, dim3(1), b, 0, st, N, S, t0, norm); break;
+        case 7: launch_pdl(k_inv_f32<7>, dim3(1), b, 0, st, N, S, t0, norm); break;
+        case 8: launch_pdl(k_inv_f32<8>, dim3(1), b, 0, st, N, S, t0, norm); break;
+        case 9: launch_pdl(k_inv_f32<9>, dim3(1), b, 0, st, N, S, t0, norm); break;
+        case 10: launch_pdl(k_inv_f32<10>, dim3(1), b, 0, st, N, S, t0, norm); break;
+        case 11: launch_pdl(k_inv_f32<11>, dim3(1), b, 0, st, N, S, t0, norm); break;
+        default: launch_pdl(k_inv_f32<12>, dim3(1), b, 0, st, N, S, t0, norm); break;
     }
     const dim3 g((N + kT - 1) / kT, (N + kT - 1) / kT), tb(kT * kT);
     unsigned* none = nullptr;

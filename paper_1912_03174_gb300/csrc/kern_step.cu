@@ -1,6 +1,7 @@
 // O(N^2) kernels of the propagation step and of the setup: model build
 // (S, H0, gamma), Mulliken charges, SCC potential, leapfrog update, kick
 // helpers and observable reductions.  All arithmetic is FP64.
+#include <algorithm>
 #include <cmath>
 
 #include <cuda_fp16.h>
@@ -182,27 +183,45 @@ __global__ void k_transpose(int N, const double* __restrict__ in, double* __rest
     }
 }
 
+// Row sums of a 32 x 32 tile of products, by a 32 x 8 block: threads ty < 4 add eight
+// consecutive columns of row tx in order, thread ty = 0 the four sums pairwise (as few FP64
+// additions as a sequential sum, an eighth of its chain).  Valid in the threads ty = 0.  The
+// barrier in between is the caller's last access to `row`.
+__device__ __forceinline__ double tile_row_sum_f64(double (*row)[kTile + 1], double (*quarter)[kTile]) {
+    const int tx = threadIdx.x, ty = threadIdx.y;
+    if (ty < 4) {
+        double s = row[tx][8 * ty];
+#pragma unroll
+        for (int k = 1; k < 8; ++k) s += row[tx][8 * ty + k];
+        quarter[ty][tx] = s;
+    }
+    __syncthreads();
+    if (ty != 0) return 0.0;
+    return (quarter[0][tx] + quarter[1][tx]) + (quarter[2][tx] + quarter[3][tx]);
+}
+
 // partial[row][ct] = sum over the 32 columns of tile ct of Re rho[row][col] * S[row][col]
-// (eq:qmulik: q_A = sum_{nu in A} Re (rho S)_{nu nu}; S is symmetric).  Summed in
-// column order, exactly as the update kernel sums them, so a state loaded from a
-// checkpoint continues bitwise.
-__global__ void k_mulliken_partials(int N, int nct, const double* __restrict__ rre,
-                                    const double* __restrict__ S, double* __restrict__ partial) {
-    __shared__ double pv_s[kTile][kTile + 1];
+// (eq:qmulik: q_A = sum_{nu in A} Re (rho S)_{nu nu}; S is symmetric).  Summed as the update
+// kernel sums them, so a state loaded from a checkpoint continues bitwise.
+__global__ void __launch_bounds__(256)
+    k_mulliken_partials(int N, int nct, const double* __restrict__ rre, const double* __restrict__ S,
+                        double* __restrict__ partial) {
+    __shared__ double pv_s[kTile][kTile + 1], quarter[4][kTile];
     const int ct = blockIdx.x;
     const int col = ct * kTile + threadIdx.x;
-    for (int y = threadIdx.y; y < kTile; y += blockDim.y) {
-        const int row = blockIdx.y * kTile + y;
+    pdl_launch_dependents();
+    pdl_wait();
+#pragma unroll
+    for (int k = 0; k < kTile / 8; ++k) {
+        const int y = threadIdx.y + 8 * k, row = blockIdx.y * kTile + y;
         double v = 0.0;
         if (row < N && col < N) v = rre[(size_t)row * N + col] * S[(size_t)row * N + col];
         pv_s[y][threadIdx.x] = v;
     }
     __syncthreads();
+    const double sum = tile_row_sum_f64(pv_s, quarter);
     if (threadIdx.y == 0) {
         const int row = blockIdx.y * kTile + threadIdx.x;
-        double sum = 0.0;
-#pragma unroll 8
-        for (int k = 0; k < kTile; ++k) sum += pv_s[threadIdx.x][k];
         if (row < N) partial[(size_t)row * nct + ct] = sum;
     }
 }
@@ -216,6 +235,10 @@ __global__ void k_charges(int nat, int nper, int nct, const double* __restrict__
                           const double* __restrict__ qbase) {
     const int lane = threadIdx.x & 31;
     const int A = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    // the potentials kernel may start once the previous step's update is complete: it then
+    // evaluates the field at this step's time while the charges are summed
+    pdl_wait();
+    pdl_launch_dependents();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         if (reset0) *reset0 = 0.0;
         if (reset1) *reset1 = 0.0;
@@ -241,88 +264,88 @@ __global__ void k_charges(int nat, int nper, int nct, const double* __restrict__
 }
 
 // Warp per atom A: gdq_A = sum_B gamma_AB dq_B;  v_A = [scc] gdq_A + R_A . E(t_n)
-// (eq:hscc, eq:hsccvext with V_ext,A = R_A . E).  Block 0 also records E(t_n),
-// the dipole mu = -sum_A dq_A R_A into the history ring, and sum_A dq_A V_ext,A.
-__global__ void k_potential(int nat, int nper, int scc, const double* __restrict__ gamma,
-                            const double* __restrict__ dq, const double* __restrict__ R,
-                            DevScalars* __restrict__ sc, double* __restrict__ v_orb,
-                            double* __restrict__ v_atom, double* __restrict__ gdq,
-                            double* __restrict__ hist, const double* __restrict__ v_ref,
-                            float* __restrict__ dv_f, double* __restrict__ max_dv, int record) {
+// (eq:hscc, eq:hsccvext with V_ext,A = R_A . E).  With `record`, one more block (the last) puts
+// E(t_n), the dipole mu = -sum_A dq_A R_A (also into the history ring) and sum_A dq_A V_ext,A
+// into sc.  `early` (launched behind k_charges, whose blocks release it after the step counter's
+// writer has finished): the field is evaluated before the wait for the charges.
+__global__ void __launch_bounds__(256)
+    k_potential(int nat, int nper, int scc, const double* __restrict__ gamma,
+                const double* dq, const double* __restrict__ R,
+                DevScalars* sc, double* __restrict__ v_orb,
+                double* __restrict__ v_atom, double* __restrict__ gdq,
+                double* __restrict__ hist, const double* __restrict__ v_ref,
+                float* __restrict__ dv_f, double* __restrict__ max_dv, int record, int early) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nwarp = blockDim.x >> 5;
+    const int nab = gridDim.x - (record ? 1 : 0);
+    __shared__ double E_sh[3];
+    if (!early) pdl_wait();
     const long long n = sc->step;
     // the field at t_n, evaluated once per block
-    __shared__ double E_sh[3];
     if (threadIdx.x == 0) {
         const double t = sc->t_base + (double)(n - sc->n_base) * sc->dt;
         field_at(sc->field, t, E_sh);
     }
+    if (early) pdl_wait();
+    pdl_launch_dependents();
     __syncthreads();
     const double E[3] = {E_sh[0], E_sh[1], E_sh[2]};
-    for (int A = blockIdx.x * nwarp + warp; A < nat; A += gridDim.x * nwarp) {
-        double s = 0.0;
-        if (scc) {
-            const double* g = gamma + (size_t)A * nat;
+    if ((int)blockIdx.x < nab) {
+        for (int A = blockIdx.x * nwarp + warp; A < nat; A += nab * nwarp) {
+            double s = 0.0;
+            if (scc) {
+                const double* g = gamma + (size_t)A * nat;
 #pragma unroll 8
-            for (int B = lane; B < nat; B += 32) s += g[B] * dq[B];
-        }
-        s = warp_sum(s);
-        const double vA = s + R[3 * A] * E[0] + R[3 * A + 1] * E[1] + R[3 * A + 2] * E[2];
-        if (lane < nper) {
-            const int o = A * nper + lane;
-            v_orb[o] = vA;
-            if (dv_f) dv_f[o] = (float)(vA - v_ref[o]);
-        }
-        if (lane == 0) {
-            v_atom[A] = vA;
-            gdq[A] = s;
-            if (max_dv)
-                atomicMax(reinterpret_cast<unsigned long long*>(max_dv),
-                          (unsigned long long)__double_as_longlong(fabs(vA - v_ref[A * nper])));
-        }
-    }
-    if (blockIdx.x == 0 && record) {
-        __shared__ double red[4][32];
-        double m0 = 0, m1 = 0, m2 = 0, ee = 0;
-        for (int A = threadIdx.x; A < nat; A += blockDim.x) {
-            const double d = dq[A];
-            m0 -= d * R[3 * A];
-            m1 -= d * R[3 * A + 1];
-            m2 -= d * R[3 * A + 2];
-            ee += d * (R[3 * A] * E[0] + R[3 * A + 1] * E[1] + R[3 * A + 2] * E[2]);
-        }
-        m0 = warp_sum(m0);
-        m1 = warp_sum(m1);
-        m2 = warp_sum(m2);
-        ee = warp_sum(ee);
-        if (lane == 0) {
-            red[0][warp] = m0;
-            red[1][warp] = m1;
-            red[2][warp] = m2;
-            red[3][warp] = ee;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double a = 0, b = 0, c = 0, e = 0;
-            for (int w = 0; w < nwarp; ++w) {
-                a += red[0][w];
-                b += red[1][w];
-                c += red[2][w];
-                e += red[3][w];
+                for (int B = lane; B < nat; B += 32) s += g[B] * dq[B];
             }
-            sc->mu[0] = a;
-            sc->mu[1] = b;
-            sc->mu[2] = c;
-            sc->e_ext = e;
-            sc->E[0] = E[0];
-            sc->E[1] = E[1];
-            sc->E[2] = E[2];
+            s = warp_sum(s);
+            const double vA = s + R[3 * A] * E[0] + R[3 * A + 1] * E[1] + R[3 * A + 2] * E[2];
+            if (lane < nper) {
+                const int o = A * nper + lane;
+                v_orb[o] = vA;
+                if (dv_f) dv_f[o] = (float)(vA - v_ref[o]);
+            }
+            if (lane == 0) {
+                v_atom[A] = vA;
+                gdq[A] = s;
+                if (max_dv)
+                    atomicMax(reinterpret_cast<unsigned long long*>(max_dv),
+                              (unsigned long long)__double_as_longlong(fabs(vA - v_ref[A * nper])));
+            }
+        }
+        return;
+    }
+    __shared__ double red[4][32];
+    double m0 = 0, m1 = 0, m2 = 0, ee = 0;
+    for (int A = threadIdx.x; A < nat; A += blockDim.x) {
+        const double d = dq[A];
+        m0 -= d * R[3 * A];
+        m1 -= d * R[3 * A + 1];
+        m2 -= d * R[3 * A + 2];
+        ee += d * (R[3 * A] * E[0] + R[3 * A + 1] * E[1] + R[3 * A + 2] * E[2]);
+    }
+    m0 = warp_sum(m0);
+    m1 = warp_sum(m1);
+    m2 = warp_sum(m2);
+    ee = warp_sum(ee);
+    if (lane == 0) {
+        red[0][warp] = m0;
+        red[1][warp] = m1;
+        red[2][warp] = m2;
+        red[3][warp] = ee;
+    }
+    __syncthreads();
+    if (threadIdx.x < 4) {
+        double a = 0;
+        for (int w = 0; w < nwarp; ++w) a += red[threadIdx.x][w];
+        if (threadIdx.x < 3) {
+            sc->mu[threadIdx.x] = a;
+            sc->E[threadIdx.x] = E[threadIdx.x];
             const long long slot = n % sc->hist_cap;
             const long long s2 = slot < 0 ? slot + sc->hist_cap : slot;
-            hist[3 * s2] = a;
-            hist[3 * s2 + 1] = b;
-            hist[3 * s2 + 2] = c;
+            hist[3 * s2 + threadIdx.x] = a;
+        } else {
+            sc->e_ext = a;
         }
     }
 }
@@ -341,9 +364,11 @@ __global__ void k_build_hamiltonian(int N, const double* __restrict__ H0,
 //   out = base + factor * rhodot,  rhodot = -i (X - X^dagger) - (Z + Z^dagger),
 //   X = S^-1 H rho, Z = S^-1 D rho (moving nuclei only).
 // Re rhodot_ij = Im X_ij + Im X_ji;  Im rhodot_ij = -(Re X_ij - Re X_ji).
-// A block (32 x 8 threads) owns the tile pair (bi, bj), bi <= bj, so both halves
-// come out of the same operands and rho stays exactly Hermitian.  The Mulliken
-// row partials of the new rho are fused in.
+// A block (32 x 8 threads) owns the tile pair (bi, bj), bi <= bj: rhodot is formed once and used
+// for both halves, so rho stays exactly Hermitian.  Z joins X when the tiles are loaded,
+//   rhodot_re,ij = b_ij + b_ji, rhodot_im,ij = a_ji - a_ij, a = Re X + Im Z, b = Im X - Re Z.
+// The Mulliken row partials of the new rho are fused in.  Bound by HBM and, about equally, by FP64
+// issue (two lanes a clock per SM).
 __global__ void __launch_bounds__(256)
     k_update(int N, int nct, const double* __restrict__ Xre, const double* __restrict__ Xim,
              const double* __restrict__ bre, const double* __restrict__ bim,
@@ -351,12 +376,19 @@ __global__ void __launch_bounds__(256)
              const double* __restrict__ S, double* __restrict__ partial,
              DevScalars* __restrict__ sc, const double* __restrict__ zre,
              const double* __restrict__ zim) {
-    const int bi = blockIdx.y, bj = blockIdx.x;
-    if (bi > bj) return;
+    // block b = bj (bj + 1) / 2 + bi
+    const int blk = blockIdx.x;
+    int bj = (int)((sqrtf(8.0f * (float)blk + 1.0f) - 1.0f) * 0.5f);
+    while (bj * (bj + 1) / 2 > blk) --bj;
+    while ((bj + 1) * (bj + 2) / 2 <= blk) ++bj;
+    const int bi = blk - bj * (bj + 1) / 2;
     constexpr int RPT = kTile / 8;   // rows per thread
-    __shared__ double xr_ij[kTile][kTile + 1], xi_ij[kTile][kTile + 1];
-    __shared__ double xr_ji[kTile][kTile + 1], xi_ji[kTile][kTile + 1];
+    __shared__ double t_re[kTile][kTile + 1], t_im[kTile][kTile + 1];   // (j, i) tile of X, then rhodot
+    __shared__ double pv_s[kTile][kTile + 1], quarter[4][kTile];
     const int tx = threadIdx.x, ty = threadIdx.y;
+    pdl_launch_dependents();
+    pdl_wait();
+    double a_ij[RPT], b_ij[RPT];
 #pragma unroll
     for (int k = 0; k < RPT; ++k) {
         const int y = ty + 8 * k;
@@ -366,9 +398,13 @@ __global__ void __launch_bounds__(256)
             const size_t i = (size_t)r * N + c;
             a = Xre[i];
             b = Xim[i];
+            if (zre) {
+                a += zim[i];
+                b -= zre[i];
+            }
         }
-        xr_ij[y][tx] = a;
-        xi_ij[y][tx] = b;
+        a_ij[k] = a;
+        b_ij[k] = b;
         r = bj * kTile + y;
         c = bi * kTile + tx;
         a = 0;
@@ -377,12 +413,31 @@ __global__ void __launch_bounds__(256)
             const size_t i = (size_t)r * N + c;
             a = Xre[i];
             b = Xim[i];
+            if (zre) {
+                a += zim[i];
+                b -= zre[i];
+            }
         }
-        xr_ji[y][tx] = a;
-        xi_ji[y][tx] = b;
+        t_re[y][tx] = a;
+        t_im[y][tx] = b;
     }
     __syncthreads();
-    __shared__ double pv_s[kTile][kTile + 1];
+    // rhodot of the (i, j) tile into registers; then, through shared memory, to the other half
+    double dre[RPT], dim[RPT];
+#pragma unroll
+    for (int k = 0; k < RPT; ++k) {
+        const int y = ty + 8 * k;
+        dre[k] = b_ij[k] + t_im[tx][y];
+        dim[k] = t_re[tx][y] - a_ij[k];
+    }
+    if (bi != bj) {
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < RPT; ++k) {
+            t_re[ty + 8 * k][tx] = dre[k];
+            t_im[ty + 8 * k][tx] = dim[k];
+        }
+    }
     for (int half = 0; half < (bi == bj ? 1 : 2); ++half) {
         const int ti = half ? bj : bi, tj = half ? bi : bj;
         double b_re[RPT], b_im[RPT], s_v[RPT];
@@ -403,47 +458,26 @@ __global__ void __launch_bounds__(256)
             const int r = ti * kTile + y, c = tj * kTile + tx;
             double pv = 0.0;
             if (r < N && c < N) {
-                double x_ij_re, x_ij_im, x_ji_re, x_ji_im;
-                if (!half) {
-                    x_ij_re = xr_ij[y][tx];
-                    x_ij_im = xi_ij[y][tx];
-                    x_ji_re = xr_ji[tx][y];
-                    x_ji_im = xi_ji[tx][y];
-                } else {
-                    x_ij_re = xr_ji[y][tx];
-                    x_ij_im = xi_ji[y][tx];
-                    x_ji_re = xr_ij[tx][y];
-                    x_ji_im = xi_ij[tx][y];
-                }
-                // the (j,i) element repeats these operations on the swapped operands
-                double dre = x_ij_im + x_ji_im;
-                double dim = -(x_ij_re - x_ji_re);
+                const double d0 = half ? t_re[tx][y] : dre[k];
+                const double d1 = half ? -t_im[tx][y] : dim[k];
                 const size_t i = (size_t)r * N + c;
-                if (zre) {
-                    const size_t j = (size_t)c * N + r;
-                    dre -= zre[i] + zre[j];
-                    dim -= zim[i] - zim[j];
-                }
-                const double nre = b_re[k] + factor * dre;
-                const double nim = b_im[k] + factor * dim;
+                const double nre = b_re[k] + factor * d0;
+                const double nim = b_im[k] + factor * d1;
                 ore[i] = nre;
                 oim[i] = nim;
                 pv = nre * s_v[k];
             }
             pv_s[y][tx] = pv;
         }
-        // Mulliken row partials: thread (tx, ty == 0) sums row tx of this tile
+        // (also orders the writes of rhodot above before the second half's reads)
         __syncthreads();
+        const double sum = tile_row_sum_f64(pv_s, quarter);
         if (ty == 0) {
             const int r = ti * kTile + tx;
-            double sum = 0.0;
-#pragma unroll 8
-            for (int k = 0; k < kTile; ++k) sum += pv_s[tx][k];
             if (r < N) partial[(size_t)r * nct + tj] = sum;
         }
-        __syncthreads();
     }
-    if (bi == 0 && bj == 0 && threadIdx.x == 0 && threadIdx.y == 0) sc->step += 1;
+    if (blk == 0 && threadIdx.x == 0 && threadIdx.y == 0) sc->step += 1;
 }
 
 // C = diag(p) P diag(conj p), p_mu = exp(-i E0 dir . R_A(mu)): the phase factors of
@@ -479,63 +513,81 @@ __global__ void k_hermitian_half(int N, const double* __restrict__ Tre,
     oim[i] = 0.5 * (Tim[i] - Tim[j]);
 }
 
-// Per block: sum Re rho * H0, sum Re rho * S, sum Im rho * S, max |rho_ij - conj rho_ji|.
-__global__ void k_obs_reduce(int N, const double* __restrict__ rre, const double* __restrict__ rim,
-                             const double* __restrict__ H0, const double* __restrict__ S,
-                             double* __restrict__ out) {
+// Per block (persistent over tile pairs bi <= bj): sum Re rho * H0, sum Re rho * S, sum Im rho *
+// S, max |rho_ij - conj rho_ji|; the transposed tiles go through shared memory.
+__global__ void __launch_bounds__(256)
+    k_obs_reduce(int N, int npair, const double* __restrict__ rre, const double* __restrict__ rim,
+                 const double* __restrict__ H0, const double* __restrict__ S, double* __restrict__ out) {
+    __shared__ double t_re[kTile][kTile + 1], t_im[kTile][kTile + 1];
+    const int tx = threadIdx.x, ty = threadIdx.y;
     double a = 0, b = 0, c = 0, m = 0;
-    const size_t NN = (size_t)N * N;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < NN;
-         i += (size_t)gridDim.x * blockDim.x) {
-        const size_t r = i / N, col = i % N, j = col * N + r;
-        const double re = rre[i], im = rim[i];
-        a += re * H0[i];
-        b += re * S[i];
-        c += im * S[i];
-        const double e1 = fabs(re - rre[j]), e2 = fabs(im + rim[j]);
-        m = fmax(m, fmax(e1, e2));
+    for (int blk = blockIdx.x; blk < npair; blk += gridDim.x) {
+        int bj = (int)((sqrtf(8.0f * (float)blk + 1.0f) - 1.0f) * 0.5f);
+        while (bj * (bj + 1) / 2 > blk) --bj;
+        while ((bj + 1) * (bj + 2) / 2 <= blk) ++bj;
+        const int bi = blk - bj * (bj + 1) / 2;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < kTile / 8; ++k) {
+            const int y = ty + 8 * k, r = bj * kTile + y, col = bi * kTile + tx;
+            double re = 0, im = 0;
+            if (r < N && col < N) {
+                const size_t i = (size_t)r * N + col;
+                re = rre[i];
+                im = rim[i];
+                if (bi != bj) {
+                    a = fma(re, H0[i], a);
+                    b = fma(re, S[i], b);
+                    c = fma(im, S[i], c);
+                }
+            }
+            t_re[y][tx] = re;
+            t_im[y][tx] = im;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < kTile / 8; ++k) {
+            const int y = ty + 8 * k, r = bi * kTile + y, col = bj * kTile + tx;
+            if (r < N && col < N) {
+                const size_t i = (size_t)r * N + col;
+                const double re = rre[i], im = rim[i];
+                a = fma(re, H0[i], a);
+                b = fma(re, S[i], b);
+                c = fma(im, S[i], c);
+                const double e1 = fabs(re - t_re[tx][y]), e2 = fabs(im + t_im[tx][y]);
+                m = fmax(m, fmax(e1, e2));
+            }
+        }
     }
-    __shared__ double red[4][32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    __shared__ double red[4][8];
     a = warp_sum(a);
     b = warp_sum(b);
     c = warp_sum(c);
     for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (lane == 0) {
-        red[0][w] = a;
-        red[1][w] = b;
-        red[2][w] = c;
-        red[3][w] = m;
+    if (tx == 0) {
+        red[0][ty] = a;
+        red[1][ty] = b;
+        red[2][ty] = c;
+        red[3][ty] = m;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double s0 = 0, s1 = 0, s2 = 0, mx = 0;
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) {
-            s0 += red[0][k];
-            s1 += red[1][k];
-            s2 += red[2][k];
-            mx = fmax(mx, red[3][k]);
-        }
-        out[4 * blockIdx.x] = s0;
-        out[4 * blockIdx.x + 1] = s1;
-        out[4 * blockIdx.x + 2] = s2;
-        out[4 * blockIdx.x + 3] = mx;
+    if (ty == 0 && tx < 4) {
+        double s = red[tx][0];
+        for (int k = 1; k < 8; ++k) s = tx == 3 ? fmax(s, red[3][k]) : s + red[tx][k];
+        out[4 * blockIdx.x + tx] = s;
     }
 }
 
+// One warp per quantity: the block sums (and the maximum, quantity 3).
 __global__ void k_obs_finish(int nb, const double* __restrict__ in, double* __restrict__ out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double s0 = 0, s1 = 0, s2 = 0, mx = 0;
-    for (int k = 0; k < nb; ++k) {
-        s0 += in[4 * k];
-        s1 += in[4 * k + 1];
-        s2 += in[4 * k + 2];
-        mx = fmax(mx, in[4 * k + 3]);
+    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+    double s = 0;
+    for (int k = lane; k < nb; k += 32) s = q == 3 ? fmax(s, in[4 * k + q]) : s + in[4 * k + q];
+    for (int o = 16; o > 0; o >>= 1) {
+        const double t = __shfl_xor_sync(0xffffffffu, s, o);
+        s = q == 3 ? fmax(s, t) : s + t;
     }
-    out[0] = s0;
-    out[1] = s1;
-    out[2] = s2;
-    out[3] = mx;
+    if (lane == 0) out[q] = s;
 }
 
 // out[m][k] = in[m][k] * f[k]
@@ -574,25 +626,24 @@ void launch_transpose(int N, const double* in, double* out, cudaStream_t st) {
 void launch_mulliken_partials(int N, const double* rho_re, const double* S, double* partial,
                               cudaStream_t st) {
     const int nct = (N + kTile - 1) / kTile;
-    dim3 b(kTile, 8);
-    k_mulliken_partials<<<dim3(nct, nct), b, 0, st>>>(N, nct, rho_re, S, partial);
+    launch_pdl(k_mulliken_partials, dim3(nct, nct), dim3(kTile, 8), 0, st, N, nct, rho_re, S, partial);
 }
 
 void launch_charges(const Ctx& c, const double* partial, double* q, double* dq, cudaStream_t st,
                     double* reset0, double* reset1, tc::DynScales* dyn, int cur,
                     const double* qbase) {
-    k_charges<<<(c.nat + 7) / 8, 256, 0, st>>>(c.nat, c.nper, c.nct, partial, c.d_q0, q, dq,
-                                               reset0, reset1, dyn, cur, qbase);
+    launch_pdl(k_charges, dim3((c.nat + 7) / 8), dim3(256), 0, st, c.nat, c.nper, c.nct, partial,
+               (const double*)c.d_q0, q, dq, reset0, reset1, dyn, cur, qbase);
 }
 
 void launch_potential(const Ctx& c, const double* gamma, const double* dq, const double* R,
                       DevScalars* sc, double* v_orb, double* v_atom, double* gdq, double* hist,
                       const double* v_ref, float* dv_orb, cudaStream_t st, double* max_dv,
-                      int record) {
+                      int record, int after_charges) {
     const int warps = 8;
-    const int blocks = (c.nat + warps - 1) / warps;
-    k_potential<<<blocks, warps * 32, 0, st>>>(c.nat, c.nper, c.prm.scc, gamma, dq, R, sc, v_orb,
-                                               v_atom, gdq, hist, v_ref, dv_orb, max_dv, record);
+    const int blocks = (c.nat + warps - 1) / warps + (record ? 1 : 0);
+    launch_pdl(k_potential, dim3(blocks), dim3(warps * 32), 0, st, c.nat, c.nper, c.prm.scc, gamma, dq, R,
+               sc, v_orb, v_atom, gdq, hist, v_ref, dv_orb, max_dv, record, after_charges);
 }
 
 void launch_build_hamiltonian(int N, const double* H0, const double* S, const double* v_orb,
@@ -605,9 +656,8 @@ void launch_update(const Ctx& c, const double* Xre, const double* Xim, const dou
                    const double* base_im, double* out_re, double* out_im, double factor,
                    const double* S, double* partial, DevScalars* sc, cudaStream_t st,
                    const double* zre, const double* zim) {
-    dim3 b(kTile, 8);
-    k_update<<<dim3(c.nct, c.nct), b, 0, st>>>(c.N, c.nct, Xre, Xim, base_re, base_im, out_re,
-                                               out_im, factor, S, partial, sc, zre, zim);
+    launch_pdl(k_update, dim3(c.nct * (c.nct + 1) / 2), dim3(kTile, 8), 0, st, c.N, c.nct, Xre, Xim,
+               base_re, base_im, out_re, out_im, factor, S, partial, sc, zre, zim);
 }
 
 void launch_kick_phase(int N, int n_per, const double* R, double strength, const double* dir,
@@ -626,11 +676,13 @@ void launch_hermitian_half(int N, const double* Tre, const double* Tim, double* 
 
 void launch_obs_reduce(int N, const double* rho_re, const double* rho_im, const double* H0,
                        const double* S, double* block_out, int n_blocks, cudaStream_t st) {
-    k_obs_reduce<<<n_blocks, 256, 0, st>>>(N, rho_re, rho_im, H0, S, block_out);
+    const int nt = (N + kTile - 1) / kTile;
+    k_obs_reduce<<<n_blocks, dim3(kTile, 8), 0, st>>>(N, nt * (nt + 1) / 2, rho_re, rho_im, H0, S,
+                                                      block_out);
 }
 
 void launch_obs_finish(int n_blocks, const double* block_out, double* out4, cudaStream_t st) {
-    k_obs_finish<<<1, 32, 0, st>>>(n_blocks, block_out, out4);
+    k_obs_finish<<<1, 128, 0, st>>>(n_blocks, block_out, out4);
 }
 
 void launch_scale_rows_f(int N, const double* in, const double* f, double* out, cudaStream_t st) {
@@ -695,25 +747,39 @@ __global__ void k_f32_to_f64(size_t n, const float* __restrict__ in, double* __r
         out[i] = (double)in[i];
 }
 
-// out[0] = 1/2 sum_A dq_A (gamma dq)_A (eq:coul), out[1] = sum_{A<B} rep_A exp(-r/rep_b),
-// out[2] = nuclear kinetic energy (moving nuclei only)
+// Block sums of the pair repulsion rep_A exp(-r/rep_b): blocks take atoms A in turn, their
+// threads the partners B > A.
+__global__ void __launch_bounds__(128)
+    k_repulsion(int nat, const double* __restrict__ R, double rep_A, double rep_b,
+                double* __restrict__ part) {
+    double er = 0;
+    for (int A = blockIdx.x; A < nat; A += gridDim.x)
+        for (int B = A + 1 + threadIdx.x; B < nat; B += 128) {
+            const double dx = R[3 * B] - R[3 * A], dy = R[3 * B + 1] - R[3 * A + 1],
+                         dz = R[3 * B + 2] - R[3 * A + 2];
+            er += rep_A * exp(-sqrt(dx * dx + dy * dy + dz * dz) / rep_b);
+        }
+    er = warp_sum(er);
+    __shared__ double red[4];
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = er;
+    __syncthreads();
+    if (threadIdx.x == 0) part[blockIdx.x] = (red[0] + red[1]) + (red[2] + red[3]);
+}
+
+// out[0] = 1/2 sum_A dq_A (gamma dq)_A (eq:coul), out[1] = sum_{A<B} rep_A exp(-r/rep_b) from its
+// nrep block sums, out[2] = nuclear kinetic energy (moving nuclei only)
 __global__ void k_small_energies(int nat, const double* __restrict__ dq,
-                                 const double* __restrict__ gdq, const double* __restrict__ R,
-                                 const double* __restrict__ V, const double* __restrict__ mass,
-                                 double rep_A, double rep_b, int kinetic,
+                                 const double* __restrict__ gdq, const double* __restrict__ V,
+                                 const double* __restrict__ mass, int nrep,
+                                 const double* __restrict__ rep, int kinetic,
                                  double* __restrict__ out) {
     double ec = 0, er = 0, ek = 0;
+    for (int k = threadIdx.x; k < nrep; k += blockDim.x) er += rep[k];
     for (int A = threadIdx.x; A < nat; A += blockDim.x) {
         ec += 0.5 * dq[A] * gdq[A];
         if (kinetic)
             ek += 0.5 * mass[A] * 1822.888486 *
                   (V[3 * A] * V[3 * A] + V[3 * A + 1] * V[3 * A + 1] + V[3 * A + 2] * V[3 * A + 2]);
-        if (rep_A != 0.0)
-            for (int B = A + 1; B < nat; ++B) {
-                const double dx = R[3 * B] - R[3 * A], dy = R[3 * B + 1] - R[3 * A + 1],
-                             dz = R[3 * B + 2] - R[3 * A + 2];
-                er += rep_A * exp(-sqrt(dx * dx + dy * dy + dz * dz) / rep_b);
-            }
     }
     __shared__ double red[3][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -726,16 +792,10 @@ __global__ void k_small_energies(int nat, const double* __restrict__ dq,
         red[2][w] = ek;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double a = 0, b = 0, c = 0;
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) {
-            a += red[0][k];
-            b += red[1][k];
-            c += red[2][k];
-        }
-        out[0] = a;
-        out[1] = b;
-        out[2] = c;
+    if (threadIdx.x < 3) {
+        double a = 0;
+        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) a += red[threadIdx.x][k];
+        out[threadIdx.x] = a;
     }
 }
 
@@ -775,9 +835,11 @@ void launch_f64_to_f32(size_t n, const double* in, float* out, cudaStream_t st) 
     k_f64_to_f32<<<1216, 256, 0, st>>>(n, in, out);
 }
 
-void launch_small_energies(const Ctx& c, double* out, cudaStream_t st) {
-    k_small_energies<<<1, 256, 0, st>>>(c.nat, c.dq, c.gdq, c.d_R, c.d_Vn, c.d_mass, c.mp.rep_A,
-                                        c.mp.rep_b, c.prm.move_nuclei, out);
+void launch_small_energies(const Ctx& c, double* out, double* scratch, int nscratch, cudaStream_t st) {
+    const int nrep = c.mp.rep_A != 0.0 ? std::min(c.nat, nscratch) : 0;
+    if (nrep) k_repulsion<<<nrep, 128, 0, st>>>(c.nat, c.d_R, c.mp.rep_A, c.mp.rep_b, scratch);
+    k_small_energies<<<1, 256, 0, st>>>(c.nat, c.dq, c.gdq, c.d_Vn, c.d_mass, nrep, scratch,
+                                        c.prm.move_nuclei, out);
 }
 
 }  // namespace tdb

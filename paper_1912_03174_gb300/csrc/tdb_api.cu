@@ -22,7 +22,7 @@ void launch_window(int N, const double* eps, double dt, int k, double* x0re, dou
                    double* x1re, double* x1im, cudaStream_t st);
 void launch_add_step(DevScalars* sc, int k, cudaStream_t st);
 }  // namespace learn
-void launch_small_energies(const Ctx& c, double* out, cudaStream_t st);
+void launch_small_energies(const Ctx& c, double* out, double* scratch, int nscratch, cudaStream_t st);
 void launch_absmax(size_t n, const double* x, double* out, cudaStream_t st,
                    const double* sub = nullptr);
 }  // namespace tdb
@@ -814,8 +814,9 @@ tdb_status ns_inverse(Ctx& c) {
 // kept when they already belong to this step's geometry (observables were read before it, or a
 // kick or state load made them), and S^-1 of the FP64_SLICED form follows from the previous one
 // (ns_inverse); otherwise it is computed anew.
-tdb_status md_model(Ctx& c, bool in_step = false) {
+tdb_status md_model(Ctx& c, bool in_step = false, int* launches = nullptr) {
     if (in_step && c.model_n == c.n) return TDB_OK;
+    if (launches) ++*launches;
     launch_build_pair(c, c.d_R, c.S, c.H0, c.gamma, c.stream);
     CKL();
     const long long last = c.model_n;
@@ -823,9 +824,11 @@ tdb_status md_model(Ctx& c, bool in_step = false) {
     if (in_step && sliced(c) && c.N > kSmallInverseN && last == c.n - 1) {
         TRY(ns_inverse(c));
         c.line_n = last;
+        if (launches) *launches += 11;
     } else {
         TRY(enqueue_inverse(c));
         c.line_n = -10;
+        if (launches) *launches += c.N <= kSmallInverseN ? 6 : 1;
     }
     c.model_n = c.n;
     return TDB_OK;
@@ -904,12 +907,12 @@ void md32_products(Ctx& c) {
 // commit = 1 inside a step (the work integral advances), 0 for observables.
 tdb_status md_forces(Ctx& c, int cur, bool first, int commit, int* n, StepTimer* tm = nullptr) {
     MARK("md_model_inverse");
-    TRY(md_model(c, true));
+    TRY(md_model(c, true, n));
     MARK("md_charges_potential");
     launch_mulliken_partials(c.N, c.rho_re[cur], c.S, c.partial, c.stream);
     launch_charges(c, c.partial, c.q, c.dq, c.stream);
     launch_potential(c, c.gamma, c.dq, c.d_R, c.sc, c.v_orb, c.v_atom, c.gdq, c.hist, c.v_ref,
-                     nullptr, c.stream);
+                     nullptr, c.stream, nullptr, 1, 1);
     MARK("md_products_X");
     if (use_slices(c)) {
         // M = S^-1 H and X = M rho_n with integer-slice products (S^-1 sliced per step)
@@ -918,7 +921,7 @@ tdb_status md_forces(Ctx& c, int cur, bool first, int commit, int* n, StepTimer*
         TRY(oz_product(c, 0, 1, c.M));
         slice_m_rho(c, cur);
         TRY(oz_product_rho(c, 2, c.Xre, c.Xim));
-        if (n) *n += 1;
+        if (n) *n += 4;
     } else if (md32(c)) {
         // M = S^-1 H and X = M rho_n with FP32 operands and FFMA accumulation
         const int N = c.N;
@@ -931,10 +934,11 @@ tdb_status md_forces(Ctx& c, int cur, bool first, int commit, int* n, StepTimer*
         md32_products(c);
         launch_f32_to_f64(NN, c.md_xre, c.Xre, c.stream);
         launch_f32_to_f64(NN, c.md_xim, c.Xim, c.stream);
-        if (n) *n += 7;
+        if (n) *n += 9;
     } else {
         gemm_f64_ham(c.N, c.Sinv, c.H0, c.S, c.v_orb, c.M, c.stream);        // M = S^-1 H
         gemm_f64_pair(c.N, c.M, c.rho_re[cur], c.rho_im[cur], c.Xre, c.Xim, c.stream);
+        if (n) *n += 2;
     }
     MARK("md_forces");
     launch_forces(c, c.rho_re[cur], c.Xre, c.d_F, first ? 1 : 0, c.stream);
@@ -942,7 +946,7 @@ tdb_status md_forces(Ctx& c, int cur, bool first, int commit, int* n, StepTimer*
     // the slice products take D through the rows of D^T
     launch_nac_power(c, c.d_Vn, c.Xre, use_slices(c) ? 1 : 0, c.D, first ? 1 : 0, commit, c.stream);
     CKL();
-    if (n) *n += 16;
+    if (n) *n += 7;   // charges 3, forces 2, coupling and power 2
     return TDB_OK;
 }
 
@@ -959,7 +963,7 @@ tdb_status enqueue_step_md(Ctx& c, int cur, bool euler, int* launches, StepTimer
         TRY(oz_product(c, 0, 1, c.M));
         oz::slice_rows(c.M, c.N, 1.0, c.oz[2], c.stream);
         TRY(oz_product_rho(c, 2, c.Zre, c.Zim));
-        n += 2;
+        n += 4;
     } else if (md32(c)) {
         // Y = S^-1 D and Z = Y rho_n in FP32 (the FP32 copies of S^-1 and rho_n are current)
         const int N = c.N;
@@ -968,10 +972,11 @@ tdb_status enqueue_step_md(Ctx& c, int cur, bool euler, int* launches, StepTimer
         md32_products(c);
         launch_f32_to_f64(NN, c.md_xre, c.Zre, c.stream);
         launch_f32_to_f64(NN, c.md_xim, c.Zim, c.stream);
-        n += 3;
+        n += 5;
     } else {
         gemm_f64(c.N, c.N, c.N, c.Sinv, c.N, c.D, c.N, c.M, c.N, c.stream);   // Y = S^-1 D
         gemm_f64_pair(c.N, c.M, c.rho_re[cur], c.rho_im[cur], c.Zre, c.Zim, c.stream);
+        n += 2;
     }
     const double factor = euler ? c.prm.dt : 2.0 * c.prm.dt;
     const double* bre = euler ? c.rho_re[cur] : c.rho_re[prv];
@@ -982,7 +987,7 @@ tdb_status enqueue_step_md(Ctx& c, int cur, bool euler, int* launches, StepTimer
     launch_vv(c, c.d_F, c.stream);
     MARK("end");
     CKL();
-    if (launches) *launches = n + 5;
+    if (launches) *launches = n + 2;
     return TDB_OK;
 }
 
@@ -1170,7 +1175,7 @@ tdb_status enqueue_step(Ctx& c, int cur, bool euler, int* launches, StepTimer* t
         ++n;
         MARK("potential");
         launch_potential(c, c.gamma, c.dq, c.d_R, c.sc, c.v_orb, c.v_atom, c.gdq, c.hist, c.v_ref,
-                         nullptr, c.stream);
+                         nullptr, c.stream, nullptr, 1, 1);
         ++n;
     }
     if (use_slices(c)) {
@@ -1262,7 +1267,8 @@ tdb_status ensure_graph(Ctx& c, int cur) {
     cudaGraph_t g = nullptr;
     CK(cudaStreamBeginCapture(c.stream, cudaStreamCaptureModeThreadLocal));
     int nl = 0;
-    tdb_status st = enqueue_step(c, cur, false, &nl);
+    tdb_status st = c.prm.move_nuclei ? enqueue_step_md(c, cur, false, &nl)
+                                      : enqueue_step(c, cur, false, &nl);
     cudaError_t e = cudaStreamEndCapture(c.stream, &g);
     if (st != TDB_OK) {
         if (g) cudaGraphDestroy(g);
@@ -1744,12 +1750,26 @@ tdb_status step_checks(tdb_ctx* c) {
     return TDB_OK;
 }
 
+// Whether the next step of moving nuclei is the one its graph holds: a new geometry whose S^-1
+// takes no library call (small systems; FP64_SLICED on the line through the last two inverses).
+bool md_steady(const Ctx& c) {
+    if (c.euler_next || c.model_n == c.n) return false;
+    return c.N <= kSmallInverseN || (sliced(c) && c.model_n == c.n - 1 && c.line_n == c.n - 2);
+}
+
 // Enqueue one step of c on its stream: the captured graph of its leapfrog parity, or
-// the kernels themselves for an Euler step and for moving nuclei.
+// the kernels themselves for an Euler step and for an irregular step of moving nuclei.
 tdb_status step_one(tdb_ctx* c, long* launches) {
     int nl = 0;
-    if (c->prm.move_nuclei) {
+    if (c->prm.move_nuclei && !md_steady(*c)) {
         TRY(enqueue_step_md(*c, c->cur, c->euler_next, &nl));
+    } else if (c->prm.move_nuclei) {
+        TRY(ensure_graph(*c, c->cur));
+        CK(cudaGraphLaunch(c->graph[c->cur], c->stream));
+        nl = c->graph_launches;
+        // what md_model keeps of a step
+        c->line_n = c->N > kSmallInverseN ? c->n - 1 : -10;
+        c->model_n = c->n;
     } else if (c->euler_next) {
         TRY(enqueue_step(*c, c->cur, true, &nl));
     } else {
@@ -2056,7 +2076,7 @@ tdb_status tdb_observables(tdb_ctx* c, tdb_obs* o, double* charges, double* forc
     launch_obs_reduce(c->N, c->rho_re[cur], c->rho_im[cur], c->H0, c->S, c->obs_blocks, kObsBlocks,
                       c->stream);
     launch_obs_finish(kObsBlocks, c->obs_blocks, c->obs_out, c->stream);
-    launch_small_energies(*c, c->obs_out + 4, c->stream);
+    launch_small_energies(*c, c->obs_out + 4, c->obs_blocks, 4 * kObsBlocks, c->stream);
     CKL();
     double* red = reinterpret_cast<double*>(c->h_pinned + 256);
     DevScalars* hs = reinterpret_cast<DevScalars*>(c->h_pinned + 512);

@@ -218,7 +218,7 @@ void launch_charges(const Ctx& c, const double* partial, double* q, double* dq, 
 void launch_potential(const Ctx& c, const double* gamma, const double* dq, const double* R,
                       DevScalars* sc, double* v_orb, double* v_atom, double* gdq, double* hist,
                       const double* v_ref, float* dv_orb, cudaStream_t st,
-                      double* max_dv = nullptr, int record = 1);
+                      double* max_dv = nullptr, int record = 1, int after_charges = 0);
 void launch_build_hamiltonian(int N, const double* H0, const double* S, const double* v_orb,
                               double* H, cudaStream_t st);
 // FP64 leapfrog / Euler update (zre, zim: NAC term of moving nuclei, or null)
