@@ -43,6 +43,7 @@ __global__ void __launch_bounds__(256)
     int s = 0;
 #pragma unroll
     for (int kb = 0; kb < T; ++kb)
+#pragma unroll 1   // the body stays in the instruction cache
         for (int kk = 0; kk < 16 && kb * 16 + kk < N; ++kk, s ^= 1) {
             if (ty == kk)
 #pragma unroll

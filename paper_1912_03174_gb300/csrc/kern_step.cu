@@ -183,21 +183,14 @@ __global__ void k_transpose(int N, const double* __restrict__ in, double* __rest
     }
 }
 
-// Row sums of a 32 x 32 tile of products, by a 32 x 8 block: threads ty < 4 add eight
-// consecutive columns of row tx in order, thread ty = 0 the four sums pairwise (as few FP64
-// additions as a sequential sum, an eighth of its chain).  Valid in the threads ty = 0.  The
-// barrier in between is the caller's last access to `row`.
-__device__ __forceinline__ double tile_row_sum_f64(double (*row)[kTile + 1], double (*quarter)[kTile]) {
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    if (ty < 4) {
-        double s = row[tx][8 * ty];
+// Sum of a row of 32 products, in column order.  The order is kept everywhere: a state loaded
+// from a checkpoint continues bitwise, and the reduced forms round differently (1e-9 .. 1e-7 of
+// the dipole) for ground-state charges that differ in their last bits.
+__device__ __forceinline__ double tile_row_sum_f64(const double* row) {
+    double s = 0.0;
 #pragma unroll
-        for (int k = 1; k < 8; ++k) s += row[tx][8 * ty + k];
-        quarter[ty][tx] = s;
-    }
-    __syncthreads();
-    if (ty != 0) return 0.0;
-    return (quarter[0][tx] + quarter[1][tx]) + (quarter[2][tx] + quarter[3][tx]);
+    for (int k = 0; k < kTile; ++k) s += row[k];
+    return s;
 }
 
 // partial[row][ct] = sum over the 32 columns of tile ct of Re rho[row][col] * S[row][col]
@@ -206,7 +199,7 @@ __device__ __forceinline__ double tile_row_sum_f64(double (*row)[kTile + 1], dou
 __global__ void __launch_bounds__(256)
     k_mulliken_partials(int N, int nct, const double* __restrict__ rre, const double* __restrict__ S,
                         double* __restrict__ partial) {
-    __shared__ double pv_s[kTile][kTile + 1], quarter[4][kTile];
+    __shared__ double pv_s[kTile][kTile + 1];
     const int ct = blockIdx.x;
     const int col = ct * kTile + threadIdx.x;
     pdl_launch_dependents();
@@ -219,9 +212,9 @@ __global__ void __launch_bounds__(256)
         pv_s[y][threadIdx.x] = v;
     }
     __syncthreads();
-    const double sum = tile_row_sum_f64(pv_s, quarter);
     if (threadIdx.y == 0) {
         const int row = blockIdx.y * kTile + threadIdx.x;
+        const double sum = tile_row_sum_f64(pv_s[threadIdx.x]);
         if (row < N) partial[(size_t)row * nct + ct] = sum;
     }
 }
@@ -384,7 +377,7 @@ __global__ void __launch_bounds__(256)
     const int bi = blk - bj * (bj + 1) / 2;
     constexpr int RPT = kTile / 8;   // rows per thread
     __shared__ double t_re[kTile][kTile + 1], t_im[kTile][kTile + 1];   // (j, i) tile of X, then rhodot
-    __shared__ double pv_s[kTile][kTile + 1], quarter[4][kTile];
+    __shared__ double pv_s[2][kTile][kTile + 1];   // products of both halves
     const int tx = threadIdx.x, ty = threadIdx.y;
     pdl_launch_dependents();
     pdl_wait();
@@ -437,6 +430,7 @@ __global__ void __launch_bounds__(256)
             t_re[ty + 8 * k][tx] = dre[k];
             t_im[ty + 8 * k][tx] = dim[k];
         }
+        __syncthreads();
     }
     for (int half = 0; half < (bi == bj ? 1 : 2); ++half) {
         const int ti = half ? bj : bi, tj = half ? bi : bj;
@@ -467,15 +461,15 @@ __global__ void __launch_bounds__(256)
                 oim[i] = nim;
                 pv = nre * s_v[k];
             }
-            pv_s[y][tx] = pv;
+            pv_s[half][y][tx] = pv;
         }
-        // (also orders the writes of rhodot above before the second half's reads)
-        __syncthreads();
-        const double sum = tile_row_sum_f64(pv_s, quarter);
-        if (ty == 0) {
-            const int r = ti * kTile + tx;
-            if (r < N) partial[(size_t)r * nct + tj] = sum;
-        }
+    }
+    __syncthreads();
+    // one warp per half
+    if (ty < (bi == bj ? 1 : 2)) {
+        const int r = (ty ? bj : bi) * kTile + tx;
+        const double sum = tile_row_sum_f64(pv_s[ty][tx]);
+        if (r < N) partial[(size_t)r * nct + (ty ? bi : bj)] = sum;
     }
     if (blk == 0 && threadIdx.x == 0 && threadIdx.y == 0) sc->step += 1;
 }

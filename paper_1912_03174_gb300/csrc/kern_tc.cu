@@ -278,11 +278,20 @@ __device__ __forceinline__ void gemm_tile(const Maps& maps, const GemmParams& p,
             if (row >= p.M) continue;
             if (P.mode == 0) {
                 float* out = P.C + static_cast<size_t>(row) * P.ldc + col0;
-                if (lim == 32 && (P.ldc & 3) == 0) {
+                if (lim >= 16 && (reinterpret_cast<uintptr_t>(out) & 31) == 0) {
+                    // whole sectors; lim is 32, 16 (a 176-wide tile's last chunk) or ragged
 #pragma unroll
-                    for (int j = 0; j < 32; j += 4)
-                        *reinterpret_cast<float4*>(out + j) =
-                            make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                    for (int j = 0; j < 32; j += 8)
+                        if (j + 8 <= lim) {
+                            uint32_t w[8];
+#pragma unroll
+                            for (int u = 0; u < 8; ++u) w[u] = __float_as_uint(v[j + u]);
+                            st_global_32(out + j, w);
+                        } else {
+#pragma unroll
+                            for (int u = 0; u < 8; ++u)
+                                if (j + u < lim) out[j + u] = v[j + u];
+                        }
                 } else {
 #pragma unroll
                     for (int j = 0; j < 32; ++j)
@@ -290,44 +299,41 @@ __device__ __forceinline__ void gemm_tile(const Maps& maps, const GemmParams& p,
                 }
             } else {
                 // delta M and M = M_gs + delta M, both re-split into A pieces; 16-byte
-                // vector loads of M_gs and stores of 8 pieces at a time
+                // loads of M_gs and stores of 16 pieces at a time
                 const float s_dm = p.s_dm_dev ? *p.s_dm_dev : 1.0f;
                 const float* mg = p.Mgs + static_cast<size_t>(row) * p.ld_mgs + col0;
                 const size_t ob = static_cast<size_t>(row) * p.ld_out + col0;
                 bool fine = true;
-                const bool vec = lim == 32 && (p.ld_mgs & 3) == 0 && (p.ld_out & 7) == 0 &&
-                                 (p.col_m & 7) == 0;
+                const bool vec = lim == 32 && (p.ld_mgs & 3) == 0 && (p.ld_out & 15) == 0 &&
+                                 (p.col_m & 15) == 0;
                 if (vec) {
 #pragma unroll
-                    for (int j0 = 0; j0 < 32; j0 += 8) {
-                        const float4 g0 = pre ? mgs_pre[j0 / 4] : *reinterpret_cast<const float4*>(mg + j0);
-                        const float4 g1 =
-                            pre ? mgs_pre[j0 / 4 + 1] : *reinterpret_cast<const float4*>(mg + j0 + 4);
-                        const float gm[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
-                        uint16_t qd[3][8], qm[3][8];
+                    for (int j0 = 0; j0 < 32; j0 += 16) {
+                        uint32_t qd[3][8], qm[3][8];   // 16 pieces each
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            uint16_t q[3];
-                            fine &= split_value<SCHEME>(v[j0 + j] * s_dm, p.bf16, q);
+                        for (int g = 0; g < 4; ++g) {
+                            const float4 m4 = pre ? mgs_pre[j0 / 4 + g]
+                                                  : *reinterpret_cast<const float4*>(mg + j0 + 4 * g);
+                            const float gm[4] = {m4.x, m4.y, m4.z, m4.w};
 #pragma unroll
-                            for (int t = 0; t < 3; ++t) qd[t][j] = q[t];
-                            fine &= split_value<SCHEME>((gm[j] + v[j0 + j]) * p.s_m, p.bf16, q);
+                            for (int h = 0; h < 2; ++h) {
+                                const int j = j0 + 4 * g + 2 * h;
+                                uint16_t a[3], b[3];
+                                fine &= split_value<SCHEME>(v[j] * s_dm, p.bf16, a);
+                                fine &= split_value<SCHEME>(v[j + 1] * s_dm, p.bf16, b);
 #pragma unroll
-                            for (int t = 0; t < 3; ++t) qm[t][j] = q[t];
+                                for (int t = 0; t < PIECES; ++t) qd[t][2 * g + h] = a[t] | (uint32_t(b[t]) << 16);
+                                fine &= split_value<SCHEME>((gm[2 * h] + v[j]) * p.s_m, p.bf16, a);
+                                fine &= split_value<SCHEME>((gm[2 * h + 1] + v[j + 1]) * p.s_m, p.bf16, b);
+#pragma unroll
+                                for (int t = 0; t < PIECES; ++t) qm[t][2 * g + h] = a[t] | (uint32_t(b[t]) << 16);
+                            }
                         }
+                        // whole 32-byte sectors of each row
 #pragma unroll
                         for (int t = 0; t < PIECES; ++t) {
-                            uint4 a, b;
-                            a.x = qd[t][0] | (uint32_t(qd[t][1]) << 16);
-                            a.y = qd[t][2] | (uint32_t(qd[t][3]) << 16);
-                            a.z = qd[t][4] | (uint32_t(qd[t][5]) << 16);
-                            a.w = qd[t][6] | (uint32_t(qd[t][7]) << 16);
-                            b.x = qm[t][0] | (uint32_t(qm[t][1]) << 16);
-                            b.y = qm[t][2] | (uint32_t(qm[t][3]) << 16);
-                            b.z = qm[t][4] | (uint32_t(qm[t][5]) << 16);
-                            b.w = qm[t][6] | (uint32_t(qm[t][7]) << 16);
-                            *reinterpret_cast<uint4*>(p.out[t] + ob + j0) = a;
-                            *reinterpret_cast<uint4*>(p.out[t] + ob + p.col_m + j0) = b;
+                            st_global_32(p.out[t] + ob + j0, qd[t]);
+                            st_global_32(p.out[t] + ob + p.col_m + j0, qm[t]);
                         }
                     }
                 } else {
