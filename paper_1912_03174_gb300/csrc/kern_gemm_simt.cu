@@ -9,20 +9,36 @@ namespace tdb {
 
 namespace {
 
-template <typename T>
+// B operands: raw(k, j) are the loads of an element (anything outside the matrix), value(raw, v_j)
+// the element formed from them, col(j) what a column needs once.  (Ham loads without a branch:
+// under one, the compiler forms the element at the load and waits for it there.)
 struct Dense {
-    const T* p;
+    const double* p;
     int ld;
-    __device__ __forceinline__ T operator()(int r, int c) const { return p[(size_t)r * ld + c]; }
+    struct Raw {
+        double x;
+    };
+    __device__ __forceinline__ Raw raw(int r, int c, bool in) const {
+        return {in ? p[(size_t)r * ld + c] : 0.0};
+    }
+    __device__ __forceinline__ double col(int, bool) const { return 0.0; }
+    __device__ __forceinline__ double value(const Raw& x, double) const { return x.x; }
 };
 
 // H_kj = H0_kj + 1/2 S_kj (v_k + v_j)
 struct Ham {
     const double *H0, *S, *v;
     int N;
-    __device__ __forceinline__ double operator()(int k, int j) const {
-        const size_t i = (size_t)k * N + j;
-        return H0[i] + 0.5 * S[i] * (v[k] + v[j]);
+    struct Raw {
+        double h, s, vk;
+    };
+    __device__ __forceinline__ Raw raw(int k, int j, bool in) const {
+        const size_t i = in ? (size_t)k * N + j : 0;
+        return {H0[i], S[i], v[in ? k : 0]};
+    }
+    __device__ __forceinline__ double col(int j, bool in) const { return in ? v[j] : 0.0; }
+    __device__ __forceinline__ double value(const Raw& x, double vj) const {
+        return x.h + 0.5 * x.s * (x.vk + vj);
     }
 };
 
@@ -34,34 +50,43 @@ struct Ham {
 // product launches, 26 us with these and two.
 constexpr int kT8 = 8, kK8 = 64;
 
-template <class LA, class LB>
+template <class LB>
 __global__ void __launch_bounds__(kT8* kT8)
-    k_gemm_f64(int M, int Ncol, int K, LA la, LB lb0, LB lb1, double* C0, double* C1, int ldc) {
+    k_gemm_f64(int M, int Ncol, int K, const double* A, int lda, LB lb0, LB lb1, double* C0, double* C1,
+               int ldc) {
     __shared__ double As[kT8][kK8 + 2];
     __shared__ double Bs[kK8][kT8 + 1];
     const int tid = threadIdx.x, tx = tid % kT8, ty = tid / kT8;
     const int m0 = blockIdx.y * kT8, n0 = blockIdx.x * kT8;
     const LB lb = blockIdx.z ? lb1 : lb0;
-    pdl_launch_dependents();
     pdl_wait();
-    double acc = 0.0;
-    for (int k0 = 0; k0 < K; k0 += kK8) {
+    double acc = 0.0, ra[kT8];
+    typename LB::Raw rb[kT8];
+    const double vj = lb.col(n0 + tx, n0 + tx < Ncol);
+    auto load = [&](int k0) {
 #pragma unroll
         for (int i = 0; i < kT8; ++i) {
-            const int gm = m0 + i, gk = k0 + tid;
-            As[i][tid] = (gm < M && gk < K) ? la(gm, gk) : 0.0;
+            const int gm = m0 + i, ga = k0 + tid, gk = k0 + ty + kT8 * i, gn = n0 + tx;
+            ra[i] = (gm < M && ga < K) ? A[(size_t)gm * lda + ga] : 0.0;
+            rb[i] = lb.raw(gk, gn, gk < K && gn < Ncol);
         }
+    };
+    load(0);
+    for (int k0 = 0; k0 < K; k0 += kK8) {
+        if (k0) __syncthreads();
 #pragma unroll
-        for (int i = 0; i < kK8 / kT8; ++i) {
-            const int gk = k0 + ty + kT8 * i, gn = n0 + tx;
-            Bs[ty + kT8 * i][tx] = (gk < K && gn < Ncol) ? lb(gk, gn) : 0.0;
+        for (int i = 0; i < kT8; ++i) {
+            As[i][tid] = ra[i];
+            const bool in = k0 + ty + kT8 * i < K && n0 + tx < Ncol;
+            Bs[ty + kT8 * i][tx] = in ? lb.value(rb[i], vj) : 0.0;
         }
         __syncthreads();
+        if (k0 + kK8 < K) load(k0 + kK8);   // while this block is multiplied
         const int len = K - k0 < kK8 ? K - k0 : kK8;
 #pragma unroll 8
         for (int kk = 0; kk < len; ++kk) acc = fma(As[ty][kk], Bs[kk][tx], acc);
-        __syncthreads();
     }
+    pdl_launch_dependents();   // at the end: see pdl.cuh
     const int gm = m0 + ty, gn = n0 + tx;
     if (gm < M && gn < Ncol) (blockIdx.z ? C1 : C0)[(size_t)gm * ldc + gn] = acc;
 }
@@ -83,7 +108,7 @@ struct F32Parts {
 template <bool DHAM>
 __global__ void __launch_bounds__(kF32Threads, 4)
     k_gemm_f32(int M, int Ncol, int K, const __grid_constant__ F32Parts parts,
-               const float* __restrict__ dv, const float* __restrict__ add, float* __restrict__ C2) {
+               const float* dv, const float* add, float* C2) {
     __shared__ __align__(16) float As[2][kF32K][kF32Tile + 4];
     __shared__ __align__(16) float Bs[2][kF32K][kF32Tile];
     const F32Part& P = parts.p[blockIdx.z];
@@ -96,11 +121,10 @@ __global__ void __launch_bounds__(kF32Threads, 4)
     const bool vb = (P.ldb % 4 == 0) && (reinterpret_cast<uintptr_t>(P.B) & 15) == 0;
     float ra[2][4], rb[2][4];
     float dvn[4] = {0.f, 0.f, 0.f, 0.f};
-    pdl_launch_dependents();
     pdl_wait();
     if (DHAM)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) dvn[j] = n0 + bn + j < Ncol ? __ldg(dv + n0 + bn + j) : 0.f;
+        for (int j = 0; j < 4; ++j) dvn[j] = n0 + bn + j < Ncol ? dv[n0 + bn + j] : 0.f;
     auto load = [&](int k0) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -123,7 +147,7 @@ __global__ void __launch_bounds__(kF32Threads, 4)
                 for (int j = 0; j < 4; ++j) rb[h][j] = gk < K && gn + j < Ncol ? pb[j] : 0.f;
             }
             if (DHAM) {
-                const float dk = gk < K ? __ldg(dv + gk) : 0.f;
+                const float dk = gk < K ? dv[gk] : 0.f;
 #pragma unroll
                 for (int j = 0; j < 4; ++j) rb[h][j] = 0.5f * rb[h][j] * (dk + dvn[j]);
             }
@@ -167,6 +191,7 @@ __global__ void __launch_bounds__(kF32Threads, 4)
             __syncthreads();
         }
     }
+    pdl_launch_dependents();
     const int gn = n0 + 4 * tx;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
@@ -182,30 +207,30 @@ __global__ void __launch_bounds__(kF32Threads, 4)
     }
 }
 
-template <class LA, class LB>
-void run_f64(int M, int Ncol, int K, LA la, LB lb0, LB lb1, double* C0, double* C1, int ldc,
-             cudaStream_t st) {
+template <class LB>
+void run_f64(int M, int Ncol, int K, const double* A, int lda, LB lb0, LB lb1, double* C0, double* C1,
+             int ldc, cudaStream_t st) {
     const dim3 g((Ncol + kT8 - 1) / kT8, (M + kT8 - 1) / kT8, C1 ? 2 : 1);
-    launch_pdl(k_gemm_f64<LA, LB>, g, dim3(kT8 * kT8), 0, st, M, Ncol, K, la, lb0, lb1, C0, C1, ldc);
+    launch_pdl(k_gemm_f64<LB>, g, dim3(kT8 * kT8), 0, st, M, Ncol, K, A, lda, lb0, lb1, C0, C1, ldc);
 }
 
 }  // namespace
 
 void gemm_f64(int M, int Ncol, int K, const double* A, int lda, const double* B, int ldb,
               double* C, int ldc, cudaStream_t st) {
-    run_f64(M, Ncol, K, Dense<double>{A, lda}, Dense<double>{B, ldb}, Dense<double>{B, ldb}, C,
-            static_cast<double*>(nullptr), ldc, st);
+    const Dense b{B, ldb};
+    run_f64(M, Ncol, K, A, lda, b, b, C, static_cast<double*>(nullptr), ldc, st);
 }
 
 void gemm_f64_pair(int N, const double* A, const double* B0, const double* B1, double* C0,
                    double* C1, cudaStream_t st) {
-    run_f64(N, N, N, Dense<double>{A, N}, Dense<double>{B0, N}, Dense<double>{B1, N}, C0, C1, N, st);
+    run_f64(N, N, N, A, N, Dense{B0, N}, Dense{B1, N}, C0, C1, N, st);
 }
 
 void gemm_f64_ham(int N, const double* A, const double* H0, const double* S, const double* v_orb,
                   double* C, cudaStream_t st) {
     const Ham h{H0, S, v_orb, N};
-    run_f64(N, N, N, Dense<double>{A, N}, h, h, C, static_cast<double*>(nullptr), N, st);
+    run_f64(N, N, N, A, N, h, h, C, static_cast<double*>(nullptr), N, st);
 }
 
 void gemm_f32(int M, int Ncol, int K, const F32Part* parts, int nparts, cudaStream_t st) {

@@ -82,12 +82,11 @@ __device__ __forceinline__ void block_sum_grad(int nper, const double (&w)[16], 
 constexpr int kPairThreads = 64;
 
 __global__ void __launch_bounds__(kPairThreads)
-    k_pair_forces(int nat, int nper, int scc, const double* __restrict__ R,
-                  const double* __restrict__ rre, const double* __restrict__ xre,
-                  const double* __restrict__ v_atom, const double* __restrict__ dq,
-                  const double* __restrict__ U, ModelParams mp, double* __restrict__ pf) {
+    k_pair_forces(int nat, int nper, int scc, const double* R,
+                  const double* rre, const double* xre,
+                  const double* v_atom, const double* dq,
+                  const double* U, ModelParams mp, double* pf) {
     const int A = blockIdx.y, B = blockIdx.x * kPairThreads + threadIdx.x;
-    pdl_launch_dependents();
     pdl_wait();
     if (B < A || B >= nat) return;
     const size_t ab = 3 * ((size_t)A * nat + B), ba = 3 * ((size_t)B * nat + A);
@@ -154,10 +153,10 @@ __global__ void __launch_bounds__(kPairThreads)
 // F_A = sum_B pf[A][B] - dq_A E(t), one warp per atom; then V_n = V_{n-1/2} + F_n dt / 2m (V_0
 // itself at the first step).
 __global__ void __launch_bounds__(128)
-    k_force_sum(int nat, const double* __restrict__ pf, const double* __restrict__ dq,
-                const DevScalars* __restrict__ sc, const double* __restrict__ Vh,
-                const double* __restrict__ mass, double dt, int first, double* __restrict__ F,
-                double* __restrict__ Vn) {
+    k_force_sum(int nat, const double* pf, const double* dq,
+                const DevScalars* sc, const double* Vh,
+                const double* mass, double dt, int first, double* F,
+                double* Vn) {
     const int lane = threadIdx.x & 31, A = blockIdx.x * 4 + (threadIdx.x >> 5);
     pdl_launch_dependents();
     pdl_wait();
@@ -205,13 +204,12 @@ __device__ __forceinline__ void block_along(int nper, const double c[3], double 
 }
 
 __global__ void __launch_bounds__(kPairThreads)
-    k_nac_power(int nat, int nper, const double* __restrict__ R, const double* __restrict__ V,
-                ModelParams mp, const double* __restrict__ xre, int transposed, double* __restrict__ D,
-                double* __restrict__ part) {
+    k_nac_power(int nat, int nper, const double* R, const double* V,
+                ModelParams mp, const double* xre, int transposed, double* D,
+                double* part) {
     const int A = blockIdx.y, B = blockIdx.x * kPairThreads + threadIdx.x;
     const int N = nat * nper;
     double p = 0.0;
-    pdl_launch_dependents();
     pdl_wait();
     if (B >= A && B < nat) {
         double ab[16], ba[16];   // blocks (A, B) and, transposed, (B, A) of D
@@ -289,7 +287,7 @@ __global__ void __launch_bounds__(kPairThreads)
 // Sum the block partials into P_n; work_n = work_{n-1} + dt/2 (P_n + P_{n-1}) (none at
 // the first step).  commit = 0: only report (observables of the current state).
 __global__ void __launch_bounds__(1024)
-    k_power_finish(int nb, const double* __restrict__ part, MdScalars* __restrict__ md, double dt,
+    k_power_finish(int nb, const double* part, MdScalars* md, double dt,
                    int first, int commit) {
     double p = 0.0;
     pdl_launch_dependents();

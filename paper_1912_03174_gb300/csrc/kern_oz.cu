@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         // the tiles are summed: the next kernel's blocks may be scheduled
         pdl_launch_dependents();
         if (ok && row < p.M) {
-            const int ea = __ldg(p.ea + row);
+            const int ea = p.ea[row];
             const int ex = ea - 2 * (BITS - 1) - BITS * (NW - 1);
             const int* eb = p.eb[z] + col0;
             double* out = p.C[z] + static_cast<size_t>(row) * p.ldc[z] + col0;
@@ -315,7 +315,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 double v[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const int e = col0 + j0 + j < p.N ? __ldg(eb + j0 + j) : 0;
+                    const int e = col0 + j0 + j < p.N ? eb[j0 + j] : 0;
                     v[j] = scaled_sum<BITS * NL>(hi[j0 + j], lo[j0 + j], ex + e);
                     if (ea >= kNonFinite || e >= kNonFinite)
                         v[j] = __longlong_as_double(0x7ff8000000000000ll);
@@ -440,7 +440,7 @@ __global__ void __launch_bounds__(256)
     pdl_launch_dependents();
     pdl_wait();
     if (jobs.gate.norm && __uint_as_float(__ldcg(jobs.gate.norm)) < jobs.gate.below) return;
-    const double vr = job.S ? __ldg(job.v + row) : 0.0;
+    const double vr = job.S ? job.v[row] : 0.0;
     const bool vec = ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(s)) & 15) == 0;
 #pragma unroll
     for (int i = 0; i < PASS; ++i) {
@@ -457,13 +457,13 @@ __global__ void __launch_bounds__(256)
                 const double2 t1 = *reinterpret_cast<const double2*>(s + k + 2);
                 const double t[4] = {t0.x, t0.y, t1.x, t1.y};
 #pragma unroll
-                for (int j = 0; j < 4; ++j) x[i][j] += 0.5 * t[j] * (vr + __ldg(job.v + k + j));
+                for (int j = 0; j < 4; ++j) x[i][j] += 0.5 * t[j] * (vr + job.v[k + j]);
             }
         } else {
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 x[i][j] = k + j < K ? a[k + j] : 0.0;
-                if (s && k + j < K) x[i][j] += 0.5 * s[k + j] * (vr + __ldg(job.v + k + j));
+                if (s && k + j < K) x[i][j] += 0.5 * s[k + j] * (vr + job.v[k + j]);
             }
         }
         if (job.resid) {

@@ -6,36 +6,13 @@
 
 #include <cuda_fp16.h>
 
+#include "field.cuh"
 #include "pdl.cuh"
 #include "tdb_internal.h"
 
 namespace tdb {
 
 namespace {
-
-// E(t) of eq:pumpf: E0 sin(omega t + phase) f(t) dir.
-__device__ void field_at(const FieldDev& f, double t, double E[3]) {
-    if (!f.on) {
-        E[0] = E[1] = E[2] = 0.0;
-        return;
-    }
-    double env = 1.0;
-    if (f.envelope == 1) {
-        const double x = t - f.t_center;
-        env = exp(-x * x * 4.0 * 0.69314718055994530942 / (f.fwhm * f.fwhm));
-    } else if (f.envelope == 2) {
-        if (t >= 0.0 && t <= f.fwhm) {
-            const double s = sin(3.14159265358979323846 * t / f.fwhm);
-            env = s * s;
-        } else {
-            env = 0.0;
-        }
-    }
-    const double a = f.E0 * sin(f.omega * t + f.phase) * env;
-    E[0] = a * f.dir[0];
-    E[1] = a * f.dir[1];
-    E[2] = a * f.dir[2];
-}
 
 __device__ __forceinline__ uint16_t to16(float x, int bf16) {
     if (bf16) return __bfloat16_as_ushort(__float2bfloat16_rn(x));
@@ -90,11 +67,10 @@ __device__ double gamma_short(double ta, double tb, double R) {
 constexpr int kPairThreads = 64;
 
 __global__ void __launch_bounds__(kPairThreads)
-    k_build_pair(int nat, int nper, const double* __restrict__ R, const double* __restrict__ onsite,
-                 const double* __restrict__ U, ModelParams mp, double* __restrict__ S,
-                 double* __restrict__ H0, double* __restrict__ G) {
+    k_build_pair(int nat, int nper, const double* R, const double* onsite,
+                 const double* U, ModelParams mp, double* S,
+                 double* H0, double* G) {
     const int A = blockIdx.y, B = blockIdx.x * kPairThreads + threadIdx.x;
-    pdl_launch_dependents();
     pdl_wait();
     if (B < A || B >= nat) return;
     const int N = nat * nper;
@@ -135,9 +111,11 @@ __global__ void __launch_bounds__(kPairThreads)
                 sb[1 + b][1 + a] = sb[1 + a][1 + b];
             }
         }
-        const double g = 1.0 / r - gamma_short(3.2 * U[A], 3.2 * U[B], r);
+        // the two exponents' terms are summed in the order of the row's atom, as ever
+        const double ta = 3.2 * U[A], tb = 3.2 * U[B];
+        const double g = 1.0 / r - gamma_short(ta, tb, r);
         G[(size_t)A * nat + B] = g;
-        G[(size_t)B * nat + A] = g;
+        G[(size_t)B * nat + A] = ta == tb ? g : 1.0 / r - gamma_short(tb, ta, r);
     }
     if (nper == 4) {
 #pragma unroll
@@ -197,8 +175,8 @@ __device__ __forceinline__ double tile_row_sum_f64(const double* row) {
 // (eq:qmulik: q_A = sum_{nu in A} Re (rho S)_{nu nu}; S is symmetric).  Summed as the update
 // kernel sums them, so a state loaded from a checkpoint continues bitwise.
 __global__ void __launch_bounds__(256)
-    k_mulliken_partials(int N, int nct, const double* __restrict__ rre, const double* __restrict__ S,
-                        double* __restrict__ partial) {
+    k_mulliken_partials(int N, int nct, const double* rre, const double* S,
+                        double* partial) {
     __shared__ double pv_s[kTile][kTile + 1];
     const int ct = blockIdx.x;
     const int col = ct * kTile + threadIdx.x;
@@ -221,11 +199,11 @@ __global__ void __launch_bounds__(256)
 
 // q_A = sum of the Mulliken row partials of A's orbitals (contiguous in the
 // [row][ct] layout): one warp per atom.
-__global__ void k_charges(int nat, int nper, int nct, const double* __restrict__ partial,
-                          const double* __restrict__ q0, double* __restrict__ q,
-                          double* __restrict__ dq, double* reset0, double* reset1,
-                          tc::DynScales* __restrict__ dyn, int cur,
-                          const double* __restrict__ qbase) {
+__global__ void k_charges(int nat, int nper, int nct, const double* partial,
+                          const double* q0, double* q,
+                          double* dq, double* reset0, double* reset1,
+                          tc::DynScales* dyn, int cur,
+                          const double* qbase) {
     const int lane = threadIdx.x & 31;
     const int A = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     // the potentials kernel may start once the previous step's update is complete: it then
@@ -262,12 +240,12 @@ __global__ void k_charges(int nat, int nper, int nct, const double* __restrict__
 // into sc.  `early` (launched behind k_charges, whose blocks release it after the step counter's
 // writer has finished): the field is evaluated before the wait for the charges.
 __global__ void __launch_bounds__(256)
-    k_potential(int nat, int nper, int scc, const double* __restrict__ gamma,
-                const double* dq, const double* __restrict__ R,
-                DevScalars* sc, double* __restrict__ v_orb,
-                double* __restrict__ v_atom, double* __restrict__ gdq,
-                double* __restrict__ hist, const double* __restrict__ v_ref,
-                float* __restrict__ dv_f, double* __restrict__ max_dv, int record, int early) {
+    k_potential(int nat, int nper, int scc, const double* gamma,
+                const double* dq, const double* R,
+                DevScalars* sc, double* v_orb,
+                double* v_atom, double* gdq,
+                double* hist, const double* v_ref,
+                float* dv_f, double* max_dv, int record, int early) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nwarp = blockDim.x >> 5;
     const int nab = gridDim.x - (record ? 1 : 0);
@@ -363,12 +341,12 @@ __global__ void k_build_hamiltonian(int N, const double* __restrict__ H0,
 // The Mulliken row partials of the new rho are fused in.  Bound by HBM and, about equally, by FP64
 // issue (two lanes a clock per SM).
 __global__ void __launch_bounds__(256)
-    k_update(int N, int nct, const double* __restrict__ Xre, const double* __restrict__ Xim,
-             const double* __restrict__ bre, const double* __restrict__ bim,
-             double* __restrict__ ore, double* __restrict__ oim, double factor,
-             const double* __restrict__ S, double* __restrict__ partial,
-             DevScalars* __restrict__ sc, const double* __restrict__ zre,
-             const double* __restrict__ zim) {
+    k_update(int N, int nct, const double* Xre, const double* Xim,
+             const double* bre, const double* bim,
+             double* ore, double* oim, double factor,
+             const double* S, double* partial,
+             DevScalars* sc, const double* zre,
+             const double* zim) {
     // block b = bj (bj + 1) / 2 + bi
     const int blk = blockIdx.x;
     int bj = (int)((sqrtf(8.0f * (float)blk + 1.0f) - 1.0f) * 0.5f);
@@ -698,8 +676,8 @@ __global__ void k_f64_to_f32(size_t n, const double* __restrict__ in, float* __r
 
 // Start of the Newton-Schulz inverse at the next geometry: X <- 2 X - P (the line through the
 // last two inverses; P = null: X stays), P <- X, and a zeroed residual norm.
-__global__ void k_ns_start(size_t n, double* __restrict__ X, double* __restrict__ P, int line,
-                           unsigned* __restrict__ norm) {
+__global__ void k_ns_start(size_t n, double* X, double* P, int line,
+                           unsigned* norm) {
     pdl_launch_dependents();
     pdl_wait();
     if (blockIdx.x == 0 && threadIdx.x == 0) *norm = 0u;
@@ -714,8 +692,8 @@ __global__ void k_ns_start(size_t n, double* __restrict__ X, double* __restrict_
 // X <- X + 1/2 (Q + Q^T) for a symmetric X: one block per tile pair, so X stays exactly
 // symmetric.  With a gate: nothing if *gate (float bits) is below `below`.
 __global__ void __launch_bounds__(256)
-    k_ns_update(int N, double* __restrict__ X, const double* __restrict__ Q,
-                const unsigned* __restrict__ gate, float below) {
+    k_ns_update(int N, double* X, const double* Q,
+                const unsigned* gate, float below) {
     __shared__ double a[kTile][kTile + 1], b[kTile][kTile + 1];
     const int bi = blockIdx.y, bj = blockIdx.x;
     pdl_launch_dependents();
@@ -1122,7 +1100,7 @@ __device__ void level_final_block(const LevelArgs& a, int slot, long long n_lvl,
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                     const int b = b0 + 64 * u;
-                    qv[u] = b < a.nat ? __ldg(a.dq + b) : z;
+                    qv[u] = b < a.nat ? ldcg2(a.dq + b) : z;
                 }
 #pragma unroll
                 for (int u = 0; u < 8; ++u) acc = df2_add(acc, df2_mul(gv[u], qv[u]));

@@ -1505,6 +1505,8 @@ tdb_status tdb_create(const tdb_system* sys, const tdb_params* prm, void* worksp
     if (mixed(*c)) launch_f64_to_f32((size_t)c->N * c->N, c->S, c->S_f, c->stream);
     if (c->prm.precision == TDB_FP32 && !c->prm.move_nuclei)
         launch_f64_to_f32((size_t)c->N * c->N, c->Sinv, c->Sinv_f, c->stream);
+    if (prm->precision == TDB_FP64 && !prm->move_nuclei && c->N <= kSmallStepN)
+        c->small_steps = small_steps_prepare();
     if (tensor(*c)) {
         s = build_maps(*c);
         if (s != TDB_OK) return fail(s);
@@ -1757,10 +1759,47 @@ bool md_steady(const Ctx& c) {
     return c.N <= kSmallInverseN || (sliced(c) && c.model_n == c.n - 1 && c.line_n == c.n - 2);
 }
 
+// n leapfrog steps of a small FP64 system in cluster launches of at most kSmallChunk steps (some
+// tens of milliseconds).
+constexpr long kSmallChunk = 2048;
+
+tdb_status small_steps(tdb_ctx* c, long n, long* launches) {
+    SmallStepArgs a{};
+    a.N = c->N;
+    a.nat = c->nat;
+    a.nper = c->nper;
+    a.scc = c->prm.scc;
+    a.factor = 2.0 * c->prm.dt;
+    for (int l = 0; l < 2; ++l) {
+        a.rho_re[l] = c->rho_re[l];
+        a.rho_im[l] = c->rho_im[l];
+    }
+    a.S = c->S;
+    a.Sinv = c->Sinv;
+    a.H0 = c->H0;
+    a.gamma = c->gamma;
+    a.R = c->d_R;
+    a.q0 = c->d_q0;
+    a.partial = c->partial;
+    a.hist = c->hist;
+    a.sc = c->sc;
+    while (n > 0) {
+        a.cur = c->cur;
+        a.steps = std::min(n, kSmallChunk);
+        CK(launch_small_steps(a, c->stream));
+        ++*launches;
+        c->cur ^= a.steps & 1;
+        c->n += a.steps;
+        n -= a.steps;
+    }
+    return TDB_OK;
+}
+
 // Enqueue one step of c on its stream: the captured graph of its leapfrog parity, or
 // the kernels themselves for an Euler step and for an irregular step of moving nuclei.
 tdb_status step_one(tdb_ctx* c, long* launches) {
     int nl = 0;
+    if (c->small_steps && !c->euler_next) return small_steps(c, 1, launches);
     if (c->prm.move_nuclei && !md_steady(*c)) {
         TRY(enqueue_step_md(*c, c->cur, c->euler_next, &nl));
     } else if (c->prm.move_nuclei) {
@@ -1796,7 +1835,13 @@ tdb_status tdb_step(tdb_ctx* c, long n) {
         return TDB_ERR_ARG;
     }
     long launches = 0;
-    for (long k = 0; k < n; ++k) TRY(step_one(c, &launches));
+    for (long k = 0; k < n; ++k) {
+        if (c->small_steps && !c->euler_next) {
+            TRY(small_steps(c, n - k, &launches));
+            break;
+        }
+        TRY(step_one(c, &launches));
+    }
     c->last_launches = launches;
     return TDB_OK;
 }

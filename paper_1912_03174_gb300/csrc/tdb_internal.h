@@ -160,6 +160,7 @@ struct Ctx {
 
     // host-side trajectory state
     int cur = 0;                 // index of rho_n in rho_re/rho_im
+    bool small_steps = false;    // steps run in launch_small_steps
     bool have_gs = false, euler_next = true, sticky = false;
     long long n = 0;             // host mirror of the step counter
     long last_launches = 0;
@@ -315,6 +316,19 @@ void launch_master_absmax(const Ctx& c, const MasterPtrs& m, double* out, cudaSt
 void launch_master_pieces(const Ctx& c, const MasterPtrs& m, const UpdateOperands& ops,
                           const double* mx_exact, const float* dev_scale, cudaStream_t st);
 // FP16X6: head pieces of rho - rho_ref (scale from c.dyn->max_drho[slot]) into the B operands
+// FP64 form, frozen nuclei, N <= kSmallStepN: leapfrog steps in one cluster launch (kern_small.cu)
+constexpr int kSmallStepN = 64;
+struct SmallStepArgs {
+    int N, nat, nper, scc, cur;
+    long steps;
+    double factor;
+    double *rho_re[2], *rho_im[2];
+    const double *S, *Sinv, *H0, *gamma, *R, *q0;
+    double *partial, *hist;
+    DevScalars* sc;
+};
+bool small_steps_prepare();   // whether the device can place the cluster
+cudaError_t launch_small_steps(const SmallStepArgs& a, cudaStream_t st);
 // GEMM: C[M x Ncol] = A[M x K] * B[K x Ncol], row-major, FP64 SIMT.
 enum class BKind { Dense = 0, Hamiltonian = 1 };
 void gemm_f64(int M, int Ncol, int K, const double* A, int lda, const double* B, int ldb,

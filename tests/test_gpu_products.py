@@ -197,3 +197,35 @@ def test_ill_conditioned_overlaps_are_inverted_in_fp64(B, s0):
     ref = O.forces(sysm, rho, S, Sinv, H, G, q, v, sysm.R, E, False)
     assert np.all(np.isfinite(f))
     assert np.max(np.abs(f - ref)) < 1e-10 + 100 * cond ** 2 * 2.0 ** -52 * np.max(np.abs(ref))
+
+
+# N = 4 (fewer rows than CTAs), 36 (rows that do not divide), 64 (the largest); a laser and one
+# orbital per atom
+@pytest.mark.parametrize("n_atoms,n_species,laser,per", [(1, 1, False, 4), (9, 2, True, 4),
+                                                         (16, 1, False, 4), (13, 1, True, 1)])
+def test_cluster_steps_give_the_bits_of_the_separate_kernels(B, n_atoms, n_species, laser, per):
+    # tdb_step runs small FP64 systems in one launch, tdb_step_profiled always step by step in the
+    # separate kernels; the same steps taken either way, in pieces or at once, agree bit for bit
+    import dataclasses
+    sysm = I.small_flake(n_atoms, seed=8, n_species=n_species)
+    if per == 1:
+        sysm = dataclasses.replace(sysm, orbs_per_atom=1, n_electrons=1.0 * n_atoms)
+    fld = I.Field(E0=0.02, omega=0.3, phase=0.3, t_center=4.0, fwhm=3.0, envelope=1,
+                  dir=np.array([0.6, 0.8, 0.0])) if laser else None
+    run = I.Run(dt=0.2, n_steps=0, scc=True, kick=1e-2, field=fld, kT=I.SCC_KT)
+    out = []
+    for how in ("at once", "pieces", "profiled"):
+        with B.Propagator(sysm, run, "fp64") as p:
+            p.setup()
+            if how == "at once":
+                p.step(38)
+            elif how == "pieces":
+                for n in (1, 2, 1, 3, 31):
+                    p.step(n)
+            else:
+                for _ in range(38):
+                    B.tdb_step_profiled(p.ctx)
+            out.append((B.tdb_get_state(p.ctx), B.tdb_dipole_history(p.ctx, 38),
+                        p.observables()["E_total"]))
+    for o in out[1:]:
+        assert o[0] == out[0][0] and np.array_equal(o[1], out[0][1]) and o[2] == out[0][2]
