@@ -93,12 +93,13 @@ __global__ void __launch_bounds__(kT8* kT8)
 
 // FP32: a 64 x 64 tile of C per block of 128 threads, 8 x 4 consecutive outputs each, for one
 // of up to three products of the same shape (blockIdx.z).  Bound by FFMA issue: a warp's step
-// of K reads 2 + 2 shared-memory wavefronts for its 32 FFMA, and the next 16-deep block is
-// loaded into registers while this one is multiplied.  64 x 64 rather than 128 x 128, so that
+// of K reads 2 + 2 shared-memory wavefronts for its 32 FFMA, and the next 32-deep block is
+// loaded into registers while this one is multiplied (32 rather than 16: a block's multiplications
+// then outlast a load).  64 x 64 rather than 128 x 128, so that
 // the three X products of a middle-sized system fill the chip (N = 532: 243 tiles; 128 x 128
 // tiles gave 25 blocks a product; the step there went from 425 to 100 us).  Each output sums its
 // K terms in order.
-constexpr int kF32Tile = 64, kF32K = 16, kF32Threads = 128;
+constexpr int kF32Tile = 64, kF32K = 32, kF32Threads = 128, kF32Loads = 4;
 
 struct F32Parts {
     F32Part p[3];
@@ -106,7 +107,7 @@ struct F32Parts {
 
 // B operand: dense, or delta H_kj = 1/2 S_kj (dv_k + dv_j) with S = b and dv set
 template <bool DHAM>
-__global__ void __launch_bounds__(kF32Threads, 4)
+__global__ void __launch_bounds__(kF32Threads, 3)
     k_gemm_f32(int M, int Ncol, int K, const __grid_constant__ F32Parts parts,
                const float* dv, const float* add, float* C2) {
     __shared__ __align__(16) float As[2][kF32K][kF32Tile + 4];
@@ -114,12 +115,12 @@ __global__ void __launch_bounds__(kF32Threads, 4)
     const F32Part& P = parts.p[blockIdx.z];
     const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
     const int m0 = blockIdx.y * kF32Tile, n0 = blockIdx.x * kF32Tile;
-    // loads of a block: A rows ar, ar + 32 (4 consecutive k each), B rows bk, bk + 8 (4
-    // consecutive columns each)
-    const int ar = tid / 4, ak = 4 * (tid % 4), bk = tid / 16, bn = 4 * (tid % 16);
+    // loads of a block: A rows ar + 16 h (4 consecutive k each), B rows bk + 8 h (4 consecutive
+    // columns each)
+    const int ar = tid / 8, ak = 4 * (tid % 8), bk = tid / 16, bn = 4 * (tid % 16);
     const bool va = (P.lda % 4 == 0) && (reinterpret_cast<uintptr_t>(P.A) & 15) == 0;
     const bool vb = (P.ldb % 4 == 0) && (reinterpret_cast<uintptr_t>(P.B) & 15) == 0;
-    float ra[2][4], rb[2][4];
+    float ra[kF32Loads][4], rb[kF32Loads][4];
     float dvn[4] = {0.f, 0.f, 0.f, 0.f};
     pdl_wait();
     if (DHAM)
@@ -127,8 +128,8 @@ __global__ void __launch_bounds__(kF32Threads, 4)
         for (int j = 0; j < 4; ++j) dvn[j] = n0 + bn + j < Ncol ? dv[n0 + bn + j] : 0.f;
     auto load = [&](int k0) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int gm = m0 + ar + 32 * h, ga = k0 + ak;
+        for (int h = 0; h < kF32Loads; ++h) {
+            const int gm = m0 + ar + 16 * h, ga = k0 + ak;
             const float* pa = P.A + (size_t)gm * P.lda + ga;
             if (va && gm < M && ga + 4 <= K) {
                 const float4 v = *reinterpret_cast<const float4*>(pa);
@@ -155,9 +156,9 @@ __global__ void __launch_bounds__(kF32Threads, 4)
     };
     auto store = [&](int s) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < kF32Loads; ++h) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) As[s][ak + j][ar + 32 * h] = ra[h][j];
+            for (int j = 0; j < 4; ++j) As[s][ak + j][ar + 16 * h] = ra[h][j];
             *reinterpret_cast<float4*>(&Bs[s][bk + 8 * h][bn]) =
                 make_float4(rb[h][0], rb[h][1], rb[h][2], rb[h][3]);
         }

@@ -294,6 +294,21 @@ __global__ void __launch_bounds__(kEThreads)
     }
     double sq = 0.0;
     long step = t0;
+    // this thread's values of a chunk, loaded one chunk ahead (rows past the share: x = 0)
+    constexpr int kPre = kES * kEF / kEThreads;
+    float xn[kPre], yn = 0.f;
+    auto fetch = [&](long b0, long c0) {
+        const long nb = batch < n - b0 ? batch : n - b0;
+        const long per = (nb + NC - 1) / NC, lo = rank * per, hi = lo + per < nb ? lo + per : nb;
+#pragma unroll
+        for (int u = 0; u < kPre; ++u) {
+            const int e = t + u * kEThreads, q = e / F;
+            const long r = lo + c0 + q;
+            xn[u] = q < kES && r < hi ? __ldg(X + (b0 + r) * F + (e - q * F)) : 0.f;
+        }
+        yn = t < kES && lo + c0 + t < hi ? __ldg(Y + b0 + lo + c0 + t) : 0.f;
+    };
+    fetch(0, 0);
     for (long b0 = 0; b0 < n; b0 += batch) {
         const long nb = batch < n - b0 ? batch : n - b0;
         const long per = (nb + NC - 1) / NC, lo = rank * per, hi = lo + per < nb ? lo + per : nb;
@@ -301,13 +316,17 @@ __global__ void __launch_bounds__(kEThreads)
         for (long c0 = 0; c0 < per; c0 += kES) {
             // samples lo + c0 .. of the batch (rows past the share carry x = 0 and dy = 0)
             __syncthreads();
-            for (int e = t; e < kES * F; e += kEThreads) {
-                const int q = e / F, f = e % F;
-                const long r = lo + c0 + q;
-                s.x[q][f] = r < hi ? __ldg(X + (b0 + r) * F + f) : 0.f;
+#pragma unroll
+            for (int u = 0; u < kPre; ++u) {
+                const int e = t + u * kEThreads, q = e / F;
+                if (q < kES) s.x[q][e - q * F] = xn[u];
             }
-            if (t < kES) s.y[t] = lo + c0 + t < hi ? __ldg(Y + b0 + lo + c0 + t) : 0.f;
+            if (t < kES) s.y[t] = yn;
             __syncthreads();
+            if (c0 + kES < per)
+                fetch(b0, c0 + kES);
+            else if (b0 + batch < n)
+                fetch(b0 + batch, 0);
             float v[2][4], dv[2][4];
             auto bias = [&](const float* b) {
 #pragma unroll
