@@ -89,17 +89,6 @@ struct Params {
     Gate gate;
 };
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-          "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-}
-
 // (hi 2^SHIFT + lo) 2^x as the nearest double (ties to even), in integer arithmetic.
 template <int SHIFT>
 __device__ __forceinline__ double scaled_sum(long long hi, long long lo, int x) {
@@ -280,7 +269,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int w = 0; w < NW; ++w) {
                 uint32_t r[16];
-                tmem_ld16(tmem + static_cast<uint32_t>(w * BN + cg * 16) + lane_off, r);
+                tmem_ld(tmem + static_cast<uint32_t>(w * BN + cg * 16) + lane_off, r);
                 tmem_wait_ld();
                 // integers below 2^24: exact in 32-bit integers
                 const int wgt = 1 << (BITS * ((w < NH ? NH : NW) - 1 - w));

@@ -8,6 +8,7 @@
 
 #include "field.cuh"
 #include "pdl.cuh"
+#include "tc_split.cuh"
 #include "tdb_internal.h"
 
 namespace tdb {
@@ -1183,58 +1184,105 @@ __device__ __forceinline__ void update_df_block(const UpdateDfArgs& A, int b) {
     while (bj * (bj + 1) / 2 > b) --bj;
     while ((bj + 1) * (bj + 2) / 2 <= b) ++bj;
     const int bi = b - bj * (bj + 1) / 2;
-    constexpr int RPT = kTile / 8;
-    {
-        // every operand line of both halves (rows of 32 floats = one 128-byte line) is
-        // requested from DRAM at once; the loads below then hit L2
-        const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+    // a thread takes four consecutive columns x .. x + 3 of row y of a tile: 16-byte accesses where
+    // the rows are aligned (N a multiple of 4), a quarter of the memory instructions
+    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+    const int y = tid >> 3, x = 4 * (tid & 7);
+    const bool vec = (N & 3) == 0;
+    auto load4 = [&](const float* p, int r, int c, float (&v)[4]) {
+        v[0] = v[1] = v[2] = v[3] = 0.f;
+        if (r >= N || c >= N) return;
+        const float* q = p + (size_t)r * N + c;
+        if (vec) {
+            const float4 f = *reinterpret_cast<const float4*>(q);
+            v[0] = f.x, v[1] = f.y, v[2] = f.z, v[3] = f.w;
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (c + j < N) v[j] = q[j];
+        }
+    };
+    auto store4 = [&](float* p, int r, int c, const float (&v)[4]) {
+        float* q = p + (size_t)r * N + c;
+        if (vec) {
+            *reinterpret_cast<float4*>(q) = make_float4(v[0], v[1], v[2], v[3]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (c + j < N) q[j] = v[j];
+        }
+    };
+    // base level and S of a half: constants of this step (their writer finished two kernels ago)
+    float rh[4], rl[4], ih[4], il[4], sv[4];
+    auto load_base = [&](int half) {
+        const int r = (half ? bj : bi) * kTile + y, c = (half ? bi : bj) * kTile + x;
+        load4(base.re_hi, r, c, rh);
+        load4(base.re_lo, r, c, rl);
+        load4(base.im_hi, r, c, ih);
+        load4(base.im_lo, r, c, il);
+        load4(Sf, r, c, sv);
+    };
+    // before the wait for X: the first half's operands into registers, the second's lines (rows of
+    // 32 floats = one 128-byte line) into L2
+    load_base(0);
+    if (bi != bj) {
         const int arr = tid >> 5, row = tid & 31;
         if (arr < 5) {
             const float* p = arr == 0 ? base.re_hi : arr == 1 ? base.re_lo : arr == 2 ? base.im_hi
                              : arr == 3 ? base.im_lo : Sf;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int ti = h ? bj : bi, tj = h ? bi : bj;
-                const int r = ti * kTile + row, c = tj * kTile;
-                if ((h == 0 || bi != bj) && r < N && c < N)
-                    asm volatile("prefetch.global.L2 [%0];" ::"l"(p + (size_t)r * N + c));
-            }
+            const int r = bj * kTile + row, c = bi * kTile;
+            if (r < N && c < N) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + (size_t)r * N + c));
         }
     }
     // X, the scalars and the outputs belong to the previous kernels from here on
     pdl_wait();
     __shared__ float xr_ij[kTile][kTile + 1], xi_ij[kTile][kTile + 1];
     __shared__ float xr_ji[kTile][kTile + 1], xi_ji[kTile][kTile + 1];
-    __shared__ float2 pv_s[kTile][kTile + 1];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    // X = sum of its partial products, in a fixed order (all loads issued first)
-    auto load_x = [&](size_t i, float& a, float& b) {
-        float t[6];
+    __shared__ float2 pv_s[2][kTile][kTile + 1];   // Mulliken products of both halves
+    // X = sum of its partial products, in a fixed order: Re X = ((t0 + t1) + t2) + t3, Im X = t0 + t1;
+    // the first round's loads of both tiles in flight together, a second round for two K slices
+    {
+        float t[2][3][4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) t[q] = q < ops.nre ? ops.xre[q][i] : 0.f;
+        for (int h = 0; h < 2; ++h) {
+            const int r = (h ? bj : bi) * kTile + y, c = (h ? bi : bj) * kTile + x;
+            load4(ops.xre[0], r, c, t[h][0]);
+            if (ops.nre > 1) load4(ops.xre[1], r, c, t[h][1]);
+            load4(ops.xim[0], r, c, t[h][2]);
+        }
 #pragma unroll
-        for (int q = 0; q < 2; ++q) t[4 + q] = q < ops.nim ? ops.xim[q][i] : 0.f;
-        a = ((t[0] + t[1]) + t[2]) + t[3];
-        b = t[4] + t[5];
-    };
+        for (int h = 0; h < 2; ++h)
 #pragma unroll
-    for (int k = 0; k < RPT; ++k) {
-        const int y = ty + 8 * k;
-        int r = bi * kTile + y, c = bj * kTile + tx;
-        float a = 0.f, b = 0.f;
-        if (r < N && c < N) load_x((size_t)r * N + c, a, b);
-        xr_ij[y][tx] = a;
-        xi_ij[y][tx] = b;
-        r = bj * kTile + y;
-        c = bi * kTile + tx;
-        a = b = 0.f;
-        if (r < N && c < N) load_x((size_t)r * N + c, a, b);
-        xr_ji[y][tx] = a;
-        xi_ji[y][tx] = b;
+            for (int j = 0; j < 4; ++j)
+                if (ops.nre > 1) t[h][0][j] += t[h][1][j];
+        if (ops.nre > 2) {
+            float u[2][3][4];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int r = (h ? bj : bi) * kTile + y, c = (h ? bi : bj) * kTile + x;
+                load4(ops.xre[2], r, c, u[h][0]);
+                load4(ops.xre[3], r, c, u[h][1]);
+                load4(ops.xim[1], r, c, u[h][2]);
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    t[h][0][j] = (t[h][0][j] + u[h][0][j]) + u[h][1][j];
+                    t[h][2][j] += u[h][2][j];
+                }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                (h ? xr_ji : xr_ij)[y][x + j] = t[h][0][j];
+                (h ? xi_ji : xi_ij)[y][x + j] = t[h][2][j];
+            }
     }
     __shared__ float s_bound;
     __shared__ float eps_sh;
-    if (threadIdx.x == 0 && threadIdx.y == 0) {
+    if (tid == 0) {
         // both leapfrog chains are renormalised once every kRenormEvery steps
         const long long n = sc->step;
         eps_sh = (n % kRenormEvery) < 2 ? sc->eps_lvl[ops.base_slot] : 0.f;
@@ -1255,96 +1303,66 @@ __device__ __forceinline__ void update_df_block(const UpdateDfArgs& A, int b) {
     float dmax = 0.f;
     for (int half = 0; half < (bi == bj ? 1 : 2); ++half) {
         const int ti = half ? bj : bi, tj = half ? bi : bj;
-        float brh[RPT], brl[RPT], bih[RPT], bil[RPT], sv[RPT], gv[RPT];
+        const int r = ti * kTile + y, c0 = tj * kTile + x;
+        if (half) load_base(1);
+        float gv[4] = {0.f, 0.f, 0.f, 0.f};
+        if (eps != 0.f) load4(rgs, r, c0, gv);
+        const bool in = r < N && c0 < N;
 #pragma unroll
-        for (int k = 0; k < RPT; ++k) {
-            const int r = ti * kTile + ty + 8 * k, c = tj * kTile + tx;
-            brh[k] = brl[k] = bih[k] = bil[k] = sv[k] = gv[k] = 0.f;
-            if (r < N && c < N) {
-                const size_t i = (size_t)r * N + c;
-                brh[k] = base.re_hi[i];
-                brl[k] = base.re_lo[i];
-                bih[k] = base.im_hi[i];
-                bil[k] = base.im_lo[i];
-                sv[k] = Sf[i];
-                if (eps != 0.f) gv[k] = rgs[i];
+        for (int j = 0; j < 4; ++j) {
+            const float x_ij_re = (half ? xr_ji : xr_ij)[y][x + j], x_ij_im = (half ? xi_ji : xi_ij)[y][x + j];
+            const float x_ji_re = (half ? xr_ij : xr_ji)[x + j][y], x_ji_im = (half ? xi_ij : xi_ji)[x + j][y];
+            // rhodot = -i (X - X^dagger); the (j,i) element repeats these operations on
+            // the swapped operands, so the master stays exactly Hermitian
+            const float dre = x_ij_im + x_ji_im;
+            const float dim = -(x_ij_re - x_ji_re);
+            const float ire = fmaf(fh, dre, fl * dre);
+            const float iim = fmaf(fh, dim, fl * dim);
+            if (eps != 0.f) {
+                // renormalised base: f (rho_ref + dev) - rho_ref = dev + eps (rho_ref + dev)
+                df_add(rh[j], rl[j], eps * (gv[j] + rh[j]));
+                df_add(ih[j], il[j], eps * ih[j]);
             }
+            df_add(rh[j], rl[j], ire);
+            df_add(ih[j], il[j], iim);
+            const bool here = in && c0 + j < N;
+            pv_s[half][y][x + j] = here ? mulliken_elem(rh[j], rl[j], sv[j]) : make_float2(0.f, 0.f);
+            if (ops.dyn && here) dmax = fmaxf(dmax, fmaxf(fabsf(rh[j]), fabsf(ih[j])));
         }
-#pragma unroll
-        for (int k = 0; k < RPT; ++k) {
-            const int y = ty + 8 * k;
-            const int r = ti * kTile + y, c = tj * kTile + tx;
-            float2 pv = make_float2(0.f, 0.f);
-            if (r < N && c < N) {
-                float x_ij_re, x_ij_im, x_ji_re, x_ji_im;
-                if (!half) {
-                    x_ij_re = xr_ij[y][tx];
-                    x_ij_im = xi_ij[y][tx];
-                    x_ji_re = xr_ji[tx][y];
-                    x_ji_im = xi_ji[tx][y];
+        if (!in) continue;
+        store4(out.re_hi, r, c0, rh);
+        store4(out.re_lo, r, c0, rl);
+        store4(out.im_hi, r, c0, ih);
+        store4(out.im_lo, r, c0, il);
+        if (ops.re[0]) {
+            // operands of the tensor-core products are K-major: Re rho is symmetric, the transpose
+            // of Im rho is -Im rho; four pieces per 8-byte store (rows are padded to 64 columns;
+            // a ragged row writes zeros past N)
+            const size_t jr = (size_t)r * ops.ld_re + c0, ji = (size_t)r * ops.ld_im + c0;
+            uint32_t a[3], b[3];
+            auto put = [&](uint16_t* const* dst, size_t o, const float (&v)[4], float f) {
+                if (ops.re[2]) {
+                    tc::split_pair<tc::kHead3>(v[0] * f, v[1] * f, 0, a);
+                    tc::split_pair<tc::kHead3>(v[2] * f, v[3] * f, 0, b);
                 } else {
-                    x_ij_re = xr_ji[y][tx];
-                    x_ij_im = xi_ji[y][tx];
-                    x_ji_re = xr_ij[tx][y];
-                    x_ji_im = xi_ij[tx][y];
+                    tc::split_pair<tc::kHiLo>(v[0] * f, v[1] * f, ops.bf16, a);
+                    tc::split_pair<tc::kHiLo>(v[2] * f, v[3] * f, ops.bf16, b);
                 }
-                // rhodot = -i (X - X^dagger); the (j,i) element repeats these operations on
-                // the swapped operands, so the master stays exactly Hermitian
-                const float dre = x_ij_im + x_ji_im;
-                const float dim = -(x_ij_re - x_ji_re);
-                const float ire = fmaf(fh, dre, fl * dre);
-                const float iim = fmaf(fh, dim, fl * dim);
-                float rh = brh[k], rl = brl[k], ih = bih[k], il = bil[k];
-                if (eps != 0.f) {
-                    // renormalised base: f (rho_ref + dev) - rho_ref = dev + eps (rho_ref + dev)
-                    df_add(rh, rl, eps * (gv[k] + rh));
-                    df_add(ih, il, eps * ih);
-                }
-                df_add(rh, rl, ire);
-                df_add(ih, il, iim);
-                const size_t i = (size_t)r * N + c;
-                out.re_hi[i] = rh;
-                out.re_lo[i] = rl;
-                out.im_hi[i] = ih;
-                out.im_lo[i] = il;
-                pv = mulliken_elem(rh, rl, sv[k]);
-                if (ops.dyn) dmax = fmaxf(dmax, fmaxf(fabsf(rh), fabsf(ih)));
-                if (ops.re[0]) {
-                    // operands of the tensor-core products are K-major: Re rho is symmetric,
-                    // the transpose of Im rho is -Im rho
-                    const size_t jr = (size_t)r * ops.ld_re + c;
-                    const size_t ji = (size_t)r * ops.ld_im + c;
-                    if (ops.re[2]) {
-                        uint16_t q[3];
-                        split_head3(rh * op_scale, q);
-                        ops.re[0][jr] = q[0];
-                        ops.re[1][jr] = q[1];
-                        ops.re[2][jr] = q[2];
-                        split_head3(-ih * op_scale, q);
-                        ops.im[0][ji] = q[0];
-                        ops.im[1][ji] = q[1];
-                        ops.im[2][ji] = q[2];
-                    } else {
-                        const float xa = rh * op_scale;
-                        const uint16_t h1 = to16(xa, ops.bf16);
-                        ops.re[0][jr] = h1;
-                        ops.re[1][jr] = to16(xa - from16(h1, ops.bf16), ops.bf16);
-                        const float yb = -ih * op_scale;
-                        const uint16_t h2 = to16(yb, ops.bf16);
-                        ops.im[0][ji] = h2;
-                        ops.im[1][ji] = to16(yb - from16(h2, ops.bf16), ops.bf16);
-                    }
-                }
-            }
-            pv_s[y][tx] = pv;
+#pragma unroll
+                for (int t = 0; t < 3; ++t)
+                    if (t < 2 || ops.re[2]) *reinterpret_cast<uint2*>(dst[t] + o) = make_uint2(a[t], b[t]);
+            };
+            put(ops.re, jr, rh, op_scale);
+            put(ops.im, ji, ih, -op_scale);
         }
-        __syncthreads();
-        if (ty == 0) {
-            const int r = ti * kTile + tx;
-            const float2 sum = tile_row_sum(pv_s[tx]);
-            if (r < N) const_cast<float2*>(lv.partial)[(size_t)r * nct + tj] = sum;
-        }
-        __syncthreads();
+    }
+    __syncthreads();
+    // row sums, one warp per half
+    const int tx = tid & 31, ty = tid >> 5;
+    if (ty < (bi == bj ? 1 : 2)) {
+        const int r = (ty ? bj : bi) * kTile + tx;
+        const float2 sum = tile_row_sum(pv_s[ty][tx]);
+        if (r < N) const_cast<float2*>(lv.partial)[(size_t)r * nct + (ty ? bi : bj)] = sum;
     }
     if (ops.dyn) {
         // one atomic per block (the warps' maxima through shared memory)
@@ -1352,7 +1370,7 @@ __device__ __forceinline__ void update_df_block(const UpdateDfArgs& A, int b) {
         for (int o = 16; o > 0; o >>= 1) dmax = fmaxf(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
         if (tx == 0) wmax[ty] = dmax;
         __syncthreads();
-        if (tx == 0 && ty == 0) {
+        if (tid == 0) {
             for (int w = 1; w < 8; ++w) dmax = fmaxf(dmax, wmax[w]);
             atomicMax(reinterpret_cast<unsigned long long*>(&ops.dyn->max_drho[2]),
                       (unsigned long long)__double_as_longlong((double)dmax));

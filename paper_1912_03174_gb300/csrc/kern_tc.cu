@@ -134,16 +134,17 @@ __device__ __forceinline__ void gemm_tile(const Maps& maps, const GemmParams& p,
 
     // delta-M epilogue of 64-wide tiles (one 32-column chunk per warp): every thread loads
     // its row's 32 values of M_gs now, so that the loads overlap the products
-    float4 mgs_pre[8];
+    constexpr int CW = 32;   // columns of an epilogue chunk
+    float4 mgs_pre[CW / 4];
     bool pre = false;
     if (BN == 64 && P.mode == 1) {
-        const int row = m0 + (warp & 3) * 32 + lane, col0 = n0 + (warp >> 2) * 32;
-        pre = row < p.M && col0 + 32 <= p.N && (p.ld_mgs & 3) == 0;
+        const int row = m0 + (warp & 3) * 32 + lane, col0 = n0 + (warp >> 2) * CW;
+        pre = row < p.M && col0 + CW <= p.N && (p.ld_mgs & 3) == 0;
         if (pre) {
             const float4* mg4 =
                 reinterpret_cast<const float4*>(p.Mgs + static_cast<size_t>(row) * p.ld_mgs + col0);
 #pragma unroll
-            for (int u = 0; u < 8; ++u) mgs_pre[u] = __ldg(mg4 + u);
+            for (int u = 0; u < CW / 4; ++u) mgs_pre[u] = __ldg(mg4 + u);
         }
     }
     // everything above touches only constants and this CTA's own memory: the operands the
@@ -216,7 +217,8 @@ __device__ __forceinline__ void gemm_tile(const Maps& maps, const GemmParams& p,
     __syncwarp();
 
     // epilogue: warp w reads TMEM lanes (rows) 32 (w % 4) .. + 31 (the lane quarter a warp
-    // may access) and every second 32-column chunk starting at chunk w / 4
+    // may access) and every second 32-column chunk starting at chunk w / 4 (sixteen warps with
+    // half the chunks each: no faster, and 256-wide tiles spill)
     const bool ok = __all_sync(0xffffffffu, mbar_wait(done, 0, p.err, 3) ? 1 : 0) != 0;
     fence_after();
     // the products are done: the next kernel may be scheduled while the epilogue runs
@@ -227,48 +229,48 @@ __device__ __forceinline__ void gemm_tile(const Maps& maps, const GemmParams& p,
         const int quarter = warp & 3;
         const int row = m0 + quarter * 32 + lane;
         const uint32_t lane_off = static_cast<uint32_t>(quarter * 32) << 16;
-        for (int c = warp >> 2; c < (BN + 31) / 32; c += kThreads / 128) {
+        for (int c = warp >> 2; c < (BN + CW - 1) / CW; c += kThreads / 128) {
             // columns of this chunk inside the tile (a 176-wide tile ends in a 16-column
             // chunk; the TMEM columns read past it belong to the next accumulator or to
             // the unused end of the allocation) and inside the matrix
-            const int lim = min(min(32, BN - c * 32), p.N - (n0 + c * 32));
-            uint32_t r[32];
-            tmem_ld32(tmem + lane_off + c * 32, r);
-            float v[32];
+            const int lim = min(min(CW, BN - c * CW), p.N - (n0 + c * CW));
+            uint32_t r[CW];
+            tmem_ld(tmem + lane_off + c * CW, r);
+            float v[CW];
             if (SCHEME == kHead3) {
                 // heads summed first (exact while below 2^24), then the tail
-                uint32_t r1[32];
-                tmem_ld32(tmem + static_cast<uint32_t>(nheads * BN) + lane_off + c * 32, r1);
+                uint32_t r1[CW];
+                tmem_ld(tmem + static_cast<uint32_t>(nheads * BN) + lane_off + c * CW, r1);
                 tmem_wait_ld();
 #pragma unroll
-                for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+                for (int j = 0; j < CW; ++j) v[j] = __uint_as_float(r[j]);
                 for (int h = 1; h < nheads; ++h) {
-                    tmem_ld32(tmem + static_cast<uint32_t>(h * BN) + lane_off + c * 32, r);
+                    tmem_ld(tmem + static_cast<uint32_t>(h * BN) + lane_off + c * CW, r);
                     tmem_wait_ld();
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) v[j] += __uint_as_float(r[j]);
+                    for (int j = 0; j < CW; ++j) v[j] += __uint_as_float(r[j]);
                 }
                 // separate tail accumulators summed in a fixed order
                 for (int t = 1; t < n_tails(SCHEME, BN); ++t) {
-                    tmem_ld32(tmem + static_cast<uint32_t>((nheads + t) * BN) + lane_off + c * 32, r);
+                    tmem_ld(tmem + static_cast<uint32_t>((nheads + t) * BN) + lane_off + c * CW, r);
                     tmem_wait_ld();
 #pragma unroll
-                    for (int j = 0; j < 32; ++j)
+                    for (int j = 0; j < CW; ++j)
                         r1[j] = __float_as_uint(__uint_as_float(r1[j]) + __uint_as_float(r[j]));
                 }
 #pragma unroll
-                for (int j = 0; j < 32; ++j) v[j] = (v[j] + __uint_as_float(r1[j])) * inv;
+                for (int j = 0; j < CW; ++j) v[j] = (v[j] + __uint_as_float(r1[j])) * inv;
             } else {
                 tmem_wait_ld();
 #pragma unroll
-                for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]) * inv;
+                for (int j = 0; j < CW; ++j) v[j] = __uint_as_float(r[j]) * inv;
             }
-            const int col0 = n0 + c * 32;
+            const int col0 = n0 + c * CW;
             if (P.mode == 0 && p.max_out) {
                 float m = 0.f;
                 if (row < p.M)
 #pragma unroll
-                    for (int j = 0; j < 32; ++j)
+                    for (int j = 0; j < CW; ++j)
                         if (j < lim) m = fmaxf(m, fabsf(v[j]));
                 for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
                 if (lane == 0)
@@ -276,12 +278,12 @@ __device__ __forceinline__ void gemm_tile(const Maps& maps, const GemmParams& p,
                               static_cast<unsigned long long>(__double_as_longlong(static_cast<double>(m))));
             }
             if (row >= p.M) continue;
-            if (P.mode == 0) {
+            if (BN != 64 || P.mode == 0) {   // (the delta-M epilogue exists for 64-wide tiles)
                 float* out = P.C + static_cast<size_t>(row) * P.ldc + col0;
                 if (lim >= 16 && (reinterpret_cast<uintptr_t>(out) & 31) == 0) {
                     // whole sectors; lim is 32, 16 (a 176-wide tile's last chunk) or ragged
 #pragma unroll
-                    for (int j = 0; j < 32; j += 8)
+                    for (int j = 0; j < CW; j += 8)
                         if (j + 8 <= lim) {
                             uint32_t w[8];
 #pragma unroll
@@ -294,7 +296,7 @@ __device__ __forceinline__ void gemm_tile(const Maps& maps, const GemmParams& p,
                         }
                 } else {
 #pragma unroll
-                    for (int j = 0; j < 32; ++j)
+                    for (int j = 0; j < CW; ++j)
                         if (j < lim) out[j] = v[j];
                 }
             } else {
@@ -304,11 +306,11 @@ __device__ __forceinline__ void gemm_tile(const Maps& maps, const GemmParams& p,
                 const float* mg = p.Mgs + static_cast<size_t>(row) * p.ld_mgs + col0;
                 const size_t ob = static_cast<size_t>(row) * p.ld_out + col0;
                 bool fine = true;
-                const bool vec = lim == 32 && (p.ld_mgs & 3) == 0 && (p.ld_out & 15) == 0 &&
+                const bool vec = lim == CW && (p.ld_mgs & 3) == 0 && (p.ld_out & 15) == 0 &&
                                  (p.col_m & 15) == 0;
                 if (vec) {
 #pragma unroll
-                    for (int j0 = 0; j0 < 32; j0 += 16) {
+                    for (int j0 = 0; j0 < CW; j0 += 16) {
                         uint32_t qd[3][8], qm[3][8];   // 16 pieces each
 #pragma unroll
                         for (int g = 0; g < 4; ++g) {
@@ -318,15 +320,14 @@ __device__ __forceinline__ void gemm_tile(const Maps& maps, const GemmParams& p,
 #pragma unroll
                             for (int h = 0; h < 2; ++h) {
                                 const int j = j0 + 4 * g + 2 * h;
-                                uint16_t a[3], b[3];
-                                fine &= split_value<SCHEME>(v[j] * s_dm, p.bf16, a);
-                                fine &= split_value<SCHEME>(v[j + 1] * s_dm, p.bf16, b);
+                                uint32_t q[3];
+                                fine &= split_pair<SCHEME>(v[j] * s_dm, v[j + 1] * s_dm, p.bf16, q);
 #pragma unroll
-                                for (int t = 0; t < PIECES; ++t) qd[t][2 * g + h] = a[t] | (uint32_t(b[t]) << 16);
-                                fine &= split_value<SCHEME>((gm[2 * h] + v[j]) * p.s_m, p.bf16, a);
-                                fine &= split_value<SCHEME>((gm[2 * h + 1] + v[j + 1]) * p.s_m, p.bf16, b);
+                                for (int t = 0; t < PIECES; ++t) qd[t][2 * g + h] = q[t];
+                                fine &= split_pair<SCHEME>((gm[2 * h] + v[j]) * p.s_m,
+                                                           (gm[2 * h + 1] + v[j + 1]) * p.s_m, p.bf16, q);
 #pragma unroll
-                                for (int t = 0; t < PIECES; ++t) qm[t][2 * g + h] = a[t] | (uint32_t(b[t]) << 16);
+                                for (int t = 0; t < PIECES; ++t) qm[t][2 * g + h] = q[t];
                             }
                         }
                         // whole 32-byte sectors of each row
@@ -338,7 +339,7 @@ __device__ __forceinline__ void gemm_tile(const Maps& maps, const GemmParams& p,
                     }
                 } else {
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) {
+                    for (int j = 0; j < CW; ++j) {
                         if (j >= lim) continue;
                         uint16_t q[3];
                         fine &= split_value<SCHEME>(v[j] * s_dm, p.bf16, q);
@@ -566,7 +567,9 @@ bool launchable(int scheme, const GemmParams& p, int nparts, int bn) {
     if (nparts < 1 || nparts > kMaxParts || (bn != 64 && bn != 128 && bn != 176 && bn != 256))
         return false;
     for (int z = 0; z < nparts; ++z)
-        if (p.part[z].K < 1 || tmem_cols(scheme, p.part[z].K, bn) > 512) return false;
+        if (p.part[z].K < 1 || tmem_cols(scheme, p.part[z].K, bn) > 512 ||
+            (p.part[z].mode == 1 && bn != 64))
+            return false;
     return true;
 }
 

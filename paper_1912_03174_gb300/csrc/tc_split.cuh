@@ -6,6 +6,7 @@
 #include <cuda_fp16.h>
 
 #include <cstdint>
+#include <cstring>
 
 #include "tdb_tc.h"
 
@@ -40,6 +41,41 @@ __device__ __forceinline__ bool split_value(float x, int bf16, uint16_t (&q)[3])
         q[1] = __half_as_ushort(rh);
         q[2] = __half_as_ushort(__float2half_rn(r - __half2float(rh)));
         return fabsf(r) < 65000.f;
+    }
+}
+
+// The pieces of two values, packed (x0 in the low half): split_value with the paired conversions,
+// half as many instructions.
+template <int SCHEME>
+__device__ __forceinline__ bool split_pair(float x0, float x1, int bf16, uint32_t (&q)[3]) {
+    auto bits = [](auto v) {
+        uint32_t u;
+        memcpy(&u, &v, 4);
+        return u;
+    };
+    if (SCHEME == kHiLo) {
+        if (bf16) {
+            const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
+            const float2 f = __bfloat1622float2(h);
+            q[0] = bits(h);
+            q[1] = bits(__floats2bfloat162_rn(x0 - f.x, x1 - f.y));
+        } else {
+            const __half2 h = __floats2half2_rn(x0, x1);
+            const float2 f = __half22float2(h);
+            q[0] = bits(h);
+            q[1] = bits(__floats2half2_rn(x0 - f.x, x1 - f.y));
+        }
+        q[2] = 0;
+        return fabsf(x0) < 65000.f && fabsf(x1) < 65000.f;   // (false for a NaN)
+    } else {
+        const float h0 = fminf(fmaxf(rintf(x0), -127.f), 127.f), h1 = fminf(fmaxf(rintf(x1), -127.f), 127.f);
+        const float r0 = x0 - h0, r1 = x1 - h1;
+        const __half2 rh = __floats2half2_rn(r0, r1);
+        const float2 f = __half22float2(rh);
+        q[0] = bits(__floats2half2_rn(h0, h1));
+        q[1] = bits(rh);
+        q[2] = bits(__floats2half2_rn(r0 - f.x, r1 - f.y));
+        return fabsf(r0) < 65000.f && fabsf(r1) < 65000.f;
     }
 }
 
