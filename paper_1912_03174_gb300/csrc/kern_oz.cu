@@ -126,6 +126,28 @@ __device__ __forceinline__ double scaled_sum(long long hi, long long lo, int x) 
     return sign ? -v : v;
 }
 
+// The same for hi 2^SHIFT + lo below 2^63 in magnitude (kSix: 2^24 chunk sums, weights to 2^35, 8
+// chunks): a third of the instructions, which the epilogue is bound by.
+template <int SHIFT>
+__device__ __forceinline__ double scaled_sum64(long long hi, long long lo, int x) {
+    const long long t = static_cast<long long>(static_cast<unsigned long long>(hi) << SHIFT) + lo;
+    if (t == 0) return 0.0;
+    const unsigned long long sign = static_cast<unsigned long long>(t) & 0x8000000000000000ull;
+    unsigned long long m = static_cast<unsigned long long>(t < 0 ? -t : t);
+    const int lz = __clzll(m);
+    m <<= lz;
+    const unsigned r = static_cast<unsigned>(m) & 0x7ffu;
+    m >>= 11;
+    if (r > 0x400u || (r == 0x400u && (m & 1))) ++m;
+    // value = m 2^(63 - lz - 52 + x) with m in [2^52, 2^53]
+    const int be = 1023 + 63 - lz + x;
+    if (be >= 1 && be < 2046)
+        return __longlong_as_double(static_cast<long long>(
+            sign | ((static_cast<unsigned long long>(be - 1) << 52) + m)));
+    const double v = ldexp(static_cast<double>(m), be - 1023 - 52);
+    return sign ? -v : v;
+}
+
 // One CTA per 128 x 64 output tile; every CTA issues its own TMA loads of the A and B
 // slices it multiplies.  One product at N = 1024 (128 tiles), kSix: 41 us (79 us when the drain
 // used 64-bit conversions and the rounding FP64 arithmetic), kSeven: 68 us; at N = 2048 291 and
@@ -155,6 +177,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int nkb = (p.K + BK - 1) / BK;
     const int nchunk = (nkb + kChunkKB - 1) / kChunkKB;
 
+    if (warp == 3 && lane < 2 * NS) prefetch_map(lane < NS ? &maps.a[lane] : &maps.b[z][lane - NS]);
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(full0 + 8 * s, 1);
@@ -305,7 +328,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int e = col0 + j0 + j < p.N ? eb[j0 + j] : 0;
-                    v[j] = scaled_sum<BITS * NL>(hi[j0 + j], lo[j0 + j], ex + e);
+                    v[j] = SCH == kSeven ? scaled_sum<BITS * NL>(hi[j0 + j], lo[j0 + j], ex + e)
+                                         : scaled_sum64<BITS * NL>(hi[j0 + j], lo[j0 + j], ex + e);
                     if (ea >= kNonFinite || e >= kNonFinite)
                         v[j] = __longlong_as_double(0x7ff8000000000000ll);
                 }

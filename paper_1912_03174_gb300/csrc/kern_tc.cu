@@ -147,23 +147,42 @@ __device__ __forceinline__ void gemm_tile(const Maps& maps, const GemmParams& p,
             for (int u = 0; u < CW / 4; ++u) mgs_pre[u] = __ldg(mg4 + u);
         }
     }
-    // everything above touches only constants and this CTA's own memory: the operands the
-    // previous kernel wrote are read from here on
+    // K block kb into its stage: the A pieces, the B pieces
+    auto load_a = [&](int kb) {
+        const uint32_t st = base + (kb % STAGES) * SB, fb = full0 + 8 * (kb % STAGES);
+#pragma unroll
+        for (int q = 0; q < PIECES; ++q)
+            tma_load_2d(st + q * TILE_BYTES, &maps.a[q], P.k0_a + kb * BK, m0, fb);
+    };
+    auto load_b = [&](int kb) {
+        const uint32_t st = base + (kb % STAGES) * SB, fb = full0 + 8 * (kb % STAGES);
+#pragma unroll
+        for (int q = 0; q < PIECES; ++q)
+            tma_load_2d(st + PIECES * TILE_BYTES + q * BTILE, &maps.b[P.b_set][q], P.k0_b + kb * BK, n0, fb);
+    };
+    const int nfirst = nkb < STAGES ? nkb : STAGES;
+    if (warp == 0 && lane == 0)
+        // the first stages of a B operand that is older than the previous kernel
+        for (int kb = 0; kb < nfirst; ++kb) {
+            mbar_expect_tx(full0 + 8 * kb, SB);
+            if (p.early_b) load_b(kb);
+        }
+    // everything above touches only constants, older operands and this CTA's own memory: what
+    // the previous kernel wrote is read from here on
     pdl_wait();
     if (warp == 0 && lane == 0) {
-        // TMA producer: A pieces then B pieces of one 64-wide K block per stage
+        // TMA producer
         for (int kb = 0; kb < nkb; ++kb) {
             const int s = kb % STAGES, round = kb / STAGES;
-            if (kb >= STAGES && !mbar_wait(empty0 + 8 * s, (round - 1) & 1, p.err, 1)) break;
-            const uint32_t st = base + s * SB;
-            const uint32_t fb = full0 + 8 * s;
-            mbar_expect_tx(fb, SB);
-#pragma unroll
-            for (int q = 0; q < PIECES; ++q) {
-                tma_load_2d(st + q * TILE_BYTES, &maps.a[q], P.k0_a + kb * BK, m0, fb);
-                tma_load_2d(st + PIECES * TILE_BYTES + q * BTILE, &maps.b[P.b_set][q],
-                            P.k0_b + kb * BK, n0, fb);
+            if (kb < STAGES) {
+                load_a(kb);
+                if (!p.early_b) load_b(kb);
+                continue;
             }
+            if (!mbar_wait(empty0 + 8 * s, (round - 1) & 1, p.err, 1)) break;
+            mbar_expect_tx(full0 + 8 * s, SB);
+            load_a(kb);
+            load_b(kb);
         }
     } else if (warp == 1 && lane == 0) {
         const uint32_t tail = tmem + static_cast<uint32_t>(nheads * BN);
@@ -367,6 +386,11 @@ __device__ __forceinline__ void gemm_tile(const Maps& maps, const GemmParams& p,
 template <int SCHEME, int BN>
 __global__ void __launch_bounds__(kThreads, 1)
     k_split_gemm(const __grid_constant__ Maps maps, GemmParams p) {
+    // (threads past the first warp: its first lane sets up the barriers meanwhile)
+    if (threadIdx.x >= 96 && threadIdx.x < 96 + 2 * Cfg<SCHEME>::PIECES) {
+        const int q = threadIdx.x - 96, h = q / 2;
+        prefetch_map(q & 1 ? &maps.b[p.part[blockIdx.z].b_set][h] : &maps.a[h]);
+    }
     gemm_tile<SCHEME, BN>(maps, p, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
@@ -407,69 +431,85 @@ __global__ void k_split(int rows, int cols, const double* __restrict__ in,
     if (!ok && err) atomicCAS(err, 0, 4);
 }
 
-// delta H_kj = 1/2 S_kj (dv_k + dv_j) from FP32 copies of S and dv = v - v_ref; block
-// (bx, by) of a grid with gy block rows
+// delta H_kj = 1/2 S_kj (dv_k + dv_j) from FP32 copies of S and dv = v - v_ref, one block of 256
+// threads per 32 rows x 128 columns (block bx, by); a thread takes four consecutive columns of
+// four rows, whose values of S (a constant) are loaded before the wait for the potentials.
+constexpr int kDhRows = 32, kDhCols = 128;
+
 template <int SCHEME>
-__device__ __forceinline__ void split_dham_block(int N, const float* __restrict__ S,
-                                                 const float* __restrict__ dv, float scale_const,
-                                                 int bf16, const Pieces& out, int ld_out,
-                                                 const DynScales* __restrict__ dyn, int* err,
-                                                 int bx, int by, int gy) {
+__device__ __forceinline__ void split_dham_block(int N, const float* S, const float* dv,
+                                                 float scale_const, int bf16, const Pieces& out,
+                                                 int ld_out, const DynScales* dyn, int* err, int bx,
+                                                 int by) {
+    const int tid = threadIdx.x, c = bx * kDhCols + 4 * (tid & 31), r0 = by * kDhRows + (tid >> 5);
+    const bool vec = (N & 3) == 0;   // rows of S aligned to 16 bytes, no ragged columns
+    float sv[4][4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int row = r0 + 8 * u;
+        const float* p = S + static_cast<size_t>(row) * N + c;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) sv[u][j] = 0.f;
+        if (row >= N || c >= N) continue;
+        if (vec) {
+            const float4 f = *reinterpret_cast<const float4*>(p);
+            sv[u][0] = f.x, sv[u][1] = f.y, sv[u][2] = f.z, sv[u][3] = f.w;
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (c + j < N) sv[u][j] = p[j];
+        }
+    }
+    pdl_wait();
     // FP16X6: the delta-M product may be scheduled now (its CTAs set up their barriers and
     // tensor memory and load M_gs while this kernel runs, then wait for it).  Its CTAs cannot
     // share an SM with this kernel's, so they start as SMs drain; the smaller two-piece CTAs
     // can, and slowed the split (measured: FP16X6 +1.6%, BF16X3 -7% steps/s)
     if (SCHEME == kHead3) pdl_launch_dependents();
-    const int c = bx * blockDim.x + threadIdx.x;
-    const int r = by * blockDim.y + threadIdx.y;
+    if (c >= N) return;
     // FP16X6: the scale of this step, pscale(max |dv|), written with dv by the evaluation
     // of the level (|delta H| <= max |dv| since |S_kj| <= 1)
     const float s = dyn ? dyn->s_dh : scale_const;
-    if (c >= N) return;
-    // rows r, r + gridDim.y blockDim.y, ...: the scale prologue is paid once per block
-    const float dvc = __ldg(dv + c);
+    float dc[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) dc[j] = c + j < N ? dv[c + j] : 0.f;
     bool ok = true;
-    const int stride = gy * blockDim.y;
-    // eight rows per pass with their loads in flight together
-    for (int row0 = r; row0 < N; row0 += 8 * stride) {
-        float sv[8], dr[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int row = row0 + u * stride;
-            sv[u] = row < N ? __ldg(S + static_cast<size_t>(row) * N + c) : 0.f;
-            dr[u] = row < N ? __ldg(dv + row) : 0.f;
-        }
+    for (int u = 0; u < 4; ++u) {
+        const int row = r0 + 8 * u;
+        if (row >= N) break;
+        const float dr = dv[row];
+        uint32_t a[3], b[3];
+        float x[4];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int row = row0 + u * stride;
-            if (row >= N) break;
-            uint16_t q[3];
-            ok &= split_value<SCHEME>(0.5f * sv[u] * (dr[u] + dvc) * s, bf16, q);
-            const size_t o = static_cast<size_t>(row) * ld_out + c;
+        for (int j = 0; j < 4; ++j) x[j] = 0.5f * sv[u][j] * (dr + dc[j]) * s;
+        ok &= split_pair<SCHEME>(x[0], x[1], bf16, a);
+        ok &= split_pair<SCHEME>(x[2], x[3], bf16, b);
+        // (rows are padded to 64 columns: a ragged row writes zeros past N)
+        const size_t o = static_cast<size_t>(row) * ld_out + c;
 #pragma unroll
-            for (int t = 0; t < Cfg<SCHEME>::PIECES; ++t) out.p[t][o] = q[t];
-        }
+        for (int t = 0; t < Cfg<SCHEME>::PIECES; ++t)
+            *reinterpret_cast<uint2*>(out.p[t] + o) = make_uint2(a[t], b[t]);
     }
     if (!ok && err) atomicCAS(err, 0, 4);
 }
 
 template <int SCHEME>
-__global__ void k_split_dham(int N, const float* __restrict__ S, const float* __restrict__ dv,
-                             float scale_const, int bf16, Pieces out, int ld_out,
-                             DynScales* __restrict__ dyn, int* err) {
-    split_dham_block<SCHEME>(N, S, dv, scale_const, bf16, out, ld_out, dyn, err, blockIdx.x,
-                             blockIdx.y, gridDim.y);
+__global__ void __launch_bounds__(256)
+    k_split_dham(int N, const float* S, const float* dv, float scale_const, int bf16, Pieces out,
+                 int ld_out, DynScales* dyn, int* err) {
+    split_dham_block<SCHEME>(N, S, dv, scale_const, bf16, out, ld_out, dyn, err, blockIdx.x, blockIdx.y);
 }
 
 template <int SCHEME>
-__global__ void k_split_dham_grouped(const SplitDhArgs* __restrict__ args,
-                                     const int2* __restrict__ work) {
+__global__ void __launch_bounds__(256)
+    k_split_dham_grouped(const SplitDhArgs* __restrict__ args, const int2* __restrict__ work) {
     const int2 w = work[blockIdx.x];
     const SplitDhArgs& a = args[w.x];
-    const int gx = (a.N + 31) / 32, gy = (a.N + 63) / 64;
+    const int gx = (a.N + kDhCols - 1) / kDhCols;
     const Pieces out{{a.out[0], a.out[1], a.out[2]}};
     split_dham_block<SCHEME>(a.N, a.S, a.dv, a.scale, a.bf16, out, a.ld_out, a.dyn, a.err,
-                             w.y % gx, w.y / gx, gy);
+                             w.y % gx, w.y / gx);
 }
 
 // Failure-detection probe: one thread waits on an mbarrier that nothing arrives on, polling
@@ -652,27 +692,28 @@ SplitDhArgs split_dham_args(int scheme, int N, const float* S, const float* dv, 
     return a;
 }
 
-int split_dham_blocks(int N) { return ((N + 31) / 32) * ((N + 63) / 64); }
+int split_dham_blocks(int N) {
+    return ((N + kDhCols - 1) / kDhCols) * ((N + kDhRows - 1) / kDhRows);
+}
 
 void launch_split_dham_grouped(int scheme, const SplitDhArgs* args, const int2* work, int nwork,
                                cudaStream_t st) {
     if (scheme == kHiLo)
-        k_split_dham_grouped<kHiLo><<<nwork, dim3(32, 8), 0, st>>>(args, work);
+        launch_pdl(k_split_dham_grouped<kHiLo>, dim3(nwork), dim3(256), 0, st, args, work);
     else
-        k_split_dham_grouped<kHead3><<<nwork, dim3(32, 8), 0, st>>>(args, work);
+        launch_pdl(k_split_dham_grouped<kHead3>, dim3(nwork), dim3(256), 0, st, args, work);
 }
 
 void launch_split_dham(int scheme, int N, const float* S, const float* dv, float scale, int bf16,
                        uint16_t* const* pieces, int ld_out, DynScales* dyn, cudaStream_t st,
                        int* err) {
-    dim3 b(32, 8);
-    // about 8 rows per thread
-    dim3 g((N + 31) / 32, (N + 63) / 64);
+    const dim3 b(256), g((N + kDhCols - 1) / kDhCols, (N + kDhRows - 1) / kDhRows);
     Pieces o{{pieces[0], pieces[1], scheme == kHead3 ? pieces[2] : nullptr}};
     if (scheme == kHiLo)
-        k_split_dham<kHiLo><<<g, b, 0, st>>>(N, S, dv, scale, bf16, o, ld_out, nullptr, err);
+        launch_pdl(k_split_dham<kHiLo>, g, b, 0, st, N, S, dv, scale, bf16, o, ld_out,
+                   static_cast<DynScales*>(nullptr), err);
     else
-        k_split_dham<kHead3><<<g, b, 0, st>>>(N, S, dv, scale, bf16, o, ld_out, dyn, err);
+        launch_pdl(k_split_dham<kHead3>, g, b, 0, st, N, S, dv, scale, bf16, o, ld_out, dyn, err);
 }
 
 }  // namespace tc

@@ -60,6 +60,11 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
         : "memory");
 }
 
+// Fetches a tensor map in kernel parameters ahead of its first use.
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
+}
+
 // Shared-memory matrix descriptor: K-major operand, 64-byte swizzle (rows of BK = 32
 // 16-bit values), 8-row groups 512 bytes apart.
 __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {

@@ -84,7 +84,8 @@ void set_err(const char* fmt, ...) {
         if (s_ != TDB_OK) return s_;   \
     } while (0)
 
-constexpr int kObsBlocks = 304;  // 2 x 152 SMs
+constexpr int kSmCount = 152;
+constexpr int kObsBlocks = 2 * kSmCount;
 
 // Carves named sub-buffers out of one workspace, 256-byte aligned.
 struct Carver {
@@ -1035,7 +1036,7 @@ int x_params(Ctx& c, int bn, tc::GemmParams& x) {
 }
 
 // Autotuner of the X product's tile width (tensor-core forms), run once per context
-// before the first step is captured: each candidate width times three launches on the
+// before the first step is captured: each candidate width times a few launches on the
 // context's current operands (CUDA events on its stream) and the fastest is kept.  Every
 // output element keeps its K order whatever the width, so the choice changes the time,
 // not the result.  The launches write only the X partials and the X maxima, which the
@@ -1053,17 +1054,26 @@ tdb_status tune_x(Ctx& c) {
         tc::GemmParams x{};
         if (!make_x_maps(c, bn, m)) continue;   // width not encodable for this size
         const int np = x_params(c, bn, x);
-        cudaError_t e = tc::launch(c.scheme, m, x, np, c.stream, bn);   // warm-up
+        // a launch to warm up, one to see how long it takes, then as many as fill kTuneMs (events
+        // resolve about 2 us, a difference of 10% between widths at 20 us a launch)
+        float ms = 0.f;
+        auto timed = [&](int reps) {
+            cudaError_t e = cudaEventRecord(e0, c.stream);
+            for (int r = 0; r < reps && e == cudaSuccess; ++r) e = tc::launch(c.scheme, m, x, np, c.stream, bn);
+            if (e == cudaSuccess) e = cudaEventRecord(e1, c.stream);
+            if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+            if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+            ms /= (float)reps;
+            return e;
+        };
+        cudaError_t e = tc::launch(c.scheme, m, x, np, c.stream, bn);
         if (e == cudaErrorInvalidValue) {                               // width not valid here
             cudaGetLastError();
             continue;
         }
-        if (e == cudaSuccess) e = cudaEventRecord(e0, c.stream);
-        for (int r = 0; r < 3 && e == cudaSuccess; ++r) e = tc::launch(c.scheme, m, x, np, c.stream, bn);
-        if (e == cudaSuccess) e = cudaEventRecord(e1, c.stream);
-        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-        float ms = 0.f;
-        if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+        constexpr float kTuneMs = 0.3f;
+        if (e == cudaSuccess) e = timed(1);
+        if (e == cudaSuccess) e = timed(std::min(16, std::max(3, (int)(kTuneMs / std::max(ms, 0.001f)))));
         if (e != cudaSuccess) {
             set_err("X tile tuning: %s", cudaGetErrorString(e));
             st = TDB_ERR_CUDA;
@@ -1122,6 +1132,10 @@ TensorStep tensor_step_args(Ctx& c, int cur, bool euler, int bn) {
     g.err = c.d_err;
     ts.x_bn = bn;
     ts.x_parts = x_params(c, bn, ts.x);
+    // rho_ref, and rho_n from the previous step's update.  Only where the tiles are one wave: CTAs
+    // of a later wave wait for no kernel, and B before A delays their first products (N = 1024
+    // 68.0 -> 67.5 us a step with it, N = 2048 391 -> 401)
+    ts.x.early_b = ((N + bn - 1) / bn) * ((N + 127) / 128) * ts.x_parts <= kSmCount;
     // the update writes the pieces of rho_{n+1} - rho_ref itself (FP16X6: scaled from a
     // bound on their size) and tracks their maximum
     const int ns = x_split(c);

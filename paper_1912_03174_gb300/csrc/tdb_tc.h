@@ -36,6 +36,8 @@ struct GemmPart {
 
 struct GemmParams {
     int M, N;
+    int early_b;       // the B operand is older than the kernel before this one in the stream (and
+                       // than anything running when that one started): its first loads do not wait
     GemmPart part[kMaxParts];
     double* max_out;   // mode 0: atomicMax of |C| per part into max_out[part] (may be null)
     uint32_t idesc;
