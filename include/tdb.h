@@ -148,7 +148,11 @@ size_t tdb_workspace_bytes(const tdb_system* sys, const tdb_params* prm);
 /* Create a context: copy the system to the device and build S, H0, gamma
  * (Sec. 2.1).  workspace: caller-owned device memory of at least
  * tdb_workspace_bytes() bytes, 256-byte aligned, or NULL (the library
- * allocates).  Returns TDB_ERR_NOT_SPD if S is not positive definite. */
+ * allocates).  Returns TDB_ERR_NOT_SPD if S is not positive definite.
+ * Beside the workspace, and also when that is the caller's, a TDB_FP64 context of
+ * 192 <= N <= 4096 orbitals allocates the integer slices of its products (70 N^2
+ * bytes, rows padded to 64; freed by tdb_destroy).  If they cannot be had, its products
+ * run in FP64 arithmetic instead: slower, within the same accuracy. */
 tdb_status tdb_create(const tdb_system* sys, const tdb_params* prm, void* workspace,
                       size_t workspace_bytes, tdb_ctx** out);
 

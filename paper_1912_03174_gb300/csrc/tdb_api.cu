@@ -118,9 +118,12 @@ bool sliced(const Ctx& c) { return c.prm.precision == TDB_FP64_SLICED; }
 // N = 1024 6324 / 265.  The slices pay two launches and their writes, the DFMA products
 // are bound by that pipe.
 constexpr int kSliceMinN = 192;
-bool use_slices(const Ctx& c) {
-    return sliced(c) || (c.prm.precision == TDB_FP64 && c.N >= kSliceMinN && c.N <= oz::kMaxK);
+bool wants_slices(const Ctx& c) {
+    return c.prm.precision == TDB_FP64 && c.N >= kSliceMinN && c.N <= oz::kMaxK;
 }
+// The FP64 form's slices (14 bytes an element, 70 N^2 in all) live beside the workspace, whose
+// size stays that of the DFMA form; where they cannot be allocated the products stay DFMA's.
+bool use_slices(const Ctx& c) { return sliced(c) || c.oz_mem; }
 int slice_scheme(const Ctx& c) { return sliced(c) ? oz::kSix : oz::kSeven; }
 bool head3(const Ctx& c) { return c.prm.precision == TDB_FP16X6; }
 // The tensor-core X products (dM rho_ref, M Re(rho - rho_ref), M Im rho) are cut into
@@ -135,6 +138,24 @@ int piece_bf16(const Ctx& c) { return c.prm.precision == TDB_BF16X3 ? 1 : 0; }
 float pow2_scale(double m, double target) {
     if (!(m > 0)) return 1.0f;
     return (float)std::ldexp(1.0, (int)std::floor(std::log2(target / m)));
+}
+
+// slices of S^-1 (A), H or D (B), M or Y (A), Re rho and Im rho (B)
+void take_slices(Ctx& c, Carver& k) {
+    for (int q = 0; q < 5; ++q) c.oz_raw[q] = k.take<char>(oz::sliced_bytes(c.N, c.N, slice_scheme(c)));
+}
+
+// Lays the FP64 form's slices out in memory of the context's own, if it can be had.
+void alloc_slices(Ctx& c) {
+    Carver size{nullptr};
+    take_slices(c, size);
+    if (cudaMalloc(&c.oz_mem, size.off) != cudaSuccess) {
+        cudaGetLastError();
+        c.oz_mem = nullptr;
+        return;
+    }
+    Carver k{static_cast<char*>(c.oz_mem)};
+    take_slices(c, k);
 }
 
 size_t carve(Ctx& c, char* base) {
@@ -191,10 +212,7 @@ size_t carve(Ctx& c, char* base) {
         c.dv_f = k.take<float>(N);
         c.S_f = k.take<float>(NN);
     }
-    if (use_slices(c)) {
-        // slices of S^-1 (A), H or D (B), M or Y (A), Re rho and Im rho (B)
-        for (int q = 0; q < 5; ++q) c.oz_raw[q] = k.take<char>(oz::sliced_bytes(N, N, slice_scheme(c)));
-    }
+    if (sliced(c)) take_slices(c, k);
     if (md32(c)) {
         c.md_sinv = k.take<float>(NN);
         c.md_b = k.take<float>(NN);
@@ -1525,6 +1543,7 @@ tdb_status tdb_create(const tdb_system* sys, const tdb_params* prm, void* worksp
         s = build_maps(*c);
         if (s != TDB_OK) return fail(s);
     }
+    if (wants_slices(*c)) alloc_slices(*c);
     if (use_slices(*c)) {
         const int N = c->N;
         bool ok = oz::prepare() == cudaSuccess;
@@ -1892,6 +1911,16 @@ tdb_status tdb_clone(tdb_ctx* src, void* cuda_stream, void* workspace, size_t wo
     prm.cuda_stream = cuda_stream;
     TRY(tdb_create(&sys, &prm, workspace, workspace_bytes, out));
     tdb_ctx* c = *out;
+    // the source's kind of products, so that both step alike
+    if (!src->oz_mem && c->oz_mem) {
+        cudaFree(c->oz_mem);
+        c->oz_mem = nullptr;
+    } else if (src->oz_mem && !c->oz_mem) {
+        tdb_destroy(c);
+        *out = nullptr;
+        set_err("tdb_clone: cudaMalloc of the product slices failed");
+        return TDB_ERR_NOMEM;
+    }
     // the device state is the workspace (same layout: no device pointers inside it)
     tdb_status rc = TDB_OK;
     if (c->ws_need != src->ws_need || cudaStreamSynchronize(src->stream) != cudaSuccess ||
@@ -2460,6 +2489,7 @@ void tdb_destroy(tdb_ctx* c) {
         if (g) cudaGraphExecDestroy(g);
     if (c->solver) cusolverDnDestroy(c->solver);
     if (c->own_ws && c->ws) cudaFree(c->ws);
+    if (c->oz_mem) cudaFree(c->oz_mem);
     if (c->inv_work) cudaFree(c->inv_work);
     if (c->win_work) cudaFree(c->win_work);
     if (c->win_tmp) cudaFree(c->win_tmp);

@@ -145,9 +145,10 @@ struct Ctx {
     uint16_t* pc_bre[3] = {};    // N x 2Np    [rho_ref | Re(rho - rho_ref)]
     uint16_t* pc_bim[3] = {};    // N x Np     -Im rho
     float* xp[tc::kMaxParts] = {};   // partial products of X (tensor-core forms)
-    // FP64_SLICED form: slices of S^-1, H or D, M or Y, Re rho, Im rho
+    // slice products: slices of S^-1, H or D, M or Y, Re rho, Im rho
     oz::Sliced oz[5];
     char* oz_raw[5] = {};
+    void* oz_mem = nullptr;      // FP64 form: memory of these slices, owned by the context
 
     // moving nuclei, FP32 form: FP32 copies of S^-1, H or D, rho_n; M or Y; X or Z
     float *md_sinv = nullptr, *md_b = nullptr, *md_rre = nullptr, *md_rim = nullptr;
