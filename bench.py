@@ -44,7 +44,7 @@ KERNEL_FLOPS = {
     # tensor-core split GEMMs: algorithmic flops (the split products execute 3x or 6x this)
     "tc_gemm_dM": lambda N: 2 * N ** 3,
     "tc_gemm_X": lambda N: 4 * N ** 3,
-    # integer-slice products (21 slice products each)
+    # integer-slice products (21 slice products each in the FP64-sliced form, 34 in FP64)
     "oz_gemm_M": lambda N: 2 * N ** 3,
     "oz_gemm_X": lambda N: 4 * N ** 3,
 }
@@ -810,7 +810,7 @@ def kernel_roofline(name: str, t_ms: float, form: str, N: int, peaks: dict, src:
     if name.startswith(("tc_gemm", "oz_gemm")):
         ach = KERNEL_FLOPS[name](N) / (t_ms * 1e-3) / 1e12
         peak = peaks["bf16_tflops"]
-        products = {"bf16x3": 3, "fp16x3": 3, "fp16x6": 6, "fp64s": 21}.get(form, 3)
+        products = {"bf16x3": 3, "fp16x3": 3, "fp16x6": 6, "fp64s": 21, "fp64": 34}.get(form, 3)
         executed = {"tc_gemm_X": 6 * N ** 3}.get(name, KERNEL_FLOPS[name](N)) * products
         out = {"kernel": name, "bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
                "frac": ach / peak, "traffic": _traffic(name, form),

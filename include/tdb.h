@@ -394,7 +394,8 @@ tdb_status tdb_split_gemm_noalloc(int M, int N, int K, const double* A, const do
  * frequencies, Ha); re, im: nsig x nw host doubles (written).  t_damp > 0, or 0 / +inf for
  * no damping; dt > 0.  FP64 on the GPU (the library allocates and frees its device
  * buffers; synchronises).  TDB_ERR_ARG for bad sizes, pointers or values, TDB_ERR_NOMEM if
- * the device buffers do not fit, TDB_ERR_CUDA for other CUDA failures. */
+ * the device buffers do not fit, TDB_ERR_TIMEOUT if a bounded device wait ran out,
+ * TDB_ERR_CUDA for other CUDA failures. */
 tdb_status tdb_damped_transform(int nsig, long K, const double* x, double dt, double t_damp,
                                 int nw, const double* omega, double* re, double* im);
 

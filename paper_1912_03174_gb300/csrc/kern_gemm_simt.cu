@@ -47,7 +47,7 @@ struct Ham {
 // product is bound by that pipe whatever the tile, and the tile only has to spread the work:
 // 64 x 64 tiles left all but N^2 / 4096 of the 152 SMs idle below N = 800.  Each output sums
 // its K terms in order.  A frozen FP64 step at N = 40: 173 us with 64 x 64 tiles and three
-// product launches, 26 us with these and two.
+// product launches, 18.7 us with these and two (whole steps in one launch: 11.2, k_small_steps).
 constexpr int kT8 = 8, kK8 = 64;
 
 template <class LB>
@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(kT8* kT8)
 // loaded into registers while this one is multiplied (32 rather than 16: a block's multiplications
 // then outlast a load).  64 x 64 rather than 128 x 128, so that
 // the three X products of a middle-sized system fill the chip (N = 532: 243 tiles; 128 x 128
-// tiles gave 25 blocks a product; the step there went from 425 to 100 us).  Each output sums its
+// tiles gave 25 blocks a product; the step there went from 427 to 92 us).  Each output sums its
 // K terms in order.
 constexpr int kF32Tile = 64, kF32K = 32, kF32Threads = 128, kF32Loads = 4;
 

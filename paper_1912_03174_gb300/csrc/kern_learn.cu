@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(256)
 // stores the new values into all NC networks.  The arithmetic per sample is that of k_net_grad.
 // A mini-batch is a few MFLOP, so what bounds it is latency: two launches, an atomic sum and
 // layers with one output per thread cost 121 us a batch of 512 at 16 x 64 (4 blocks of 128
-// samples), this 21; here a thread takes 2 samples x 4 hidden units, and nothing leaves the
+// samples), this 17.8; here a thread takes 2 samples x 4 hidden units, and nothing leaves the
 // cluster between batches.  Hidden units are padded to 64 with zero weights, which add nothing.
 constexpr int kES = 32, kEH = 64, kEF = 32, kEStride = kEH + 4, kEThreads = 256;
 constexpr int kEMaxOwn = 4;            // parameters per thread and CTA: 6337 / 8 / 256

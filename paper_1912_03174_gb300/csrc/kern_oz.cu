@@ -544,10 +544,9 @@ __global__ void k_colmax(const double* __restrict__ B, int ldb, int K, int cols,
 }
 
 // Slices of B^T through a 64 x 32 shared-memory transpose (coalesced on both sides).
-template <int SCH>
 __global__ void k_slice_cols(const double* __restrict__ B, int ldb, int K, int cols,
                              const uint32_t* __restrict__ colmax, SlicePtrs out) {
-    constexpr int NS = Cfg<SCH>::NS, BITS = Cfg<SCH>::BITS;
+    constexpr int NS = Cfg<kSix>::NS, BITS = Cfg<kSix>::BITS;
     __shared__ double t[64][33];
     const int k0 = blockIdx.y * 64, c0 = blockIdx.x * 32;
 #pragma unroll
@@ -657,10 +656,7 @@ void slice_cols(const double* B, int ldb, Sliced& out, double* colmax, cudaStrea
     cudaMemsetAsync(cm, 0, sizeof(uint32_t) * cols, st);
     k_colmax<<<dim3((cols + 31) / 32, 16), dim3(32, 8), 0, st>>>(B, ldb, K, cols, cm);
     const dim3 g((cols + 31) / 32, (K + 63) / 64), b(32, 8);
-    if (out.scheme == kSeven)
-        k_slice_cols<kSeven><<<g, b, 0, st>>>(B, ldb, K, cols, cm, ptrs(out));
-    else
-        k_slice_cols<kSix><<<g, b, 0, st>>>(B, ldb, K, cols, cm, ptrs(out));
+    k_slice_cols<<<g, b, 0, st>>>(B, ldb, K, cols, cm, ptrs(out));
 }
 
 cudaError_t prepare() {

@@ -181,26 +181,11 @@ void run_direct(dim3 grid, int nsig, long long K, long long span, const double* 
 
 size_t up(size_t b) { return (b + 255) & ~(size_t)255; }
 
-}  // namespace
-
-extern "C" tdb_status tdb_damped_transform(int nsig, long K, const double* x, double dt,
-                                           double t_damp, int nw, const double* omega, double* re,
-                                           double* im) {
-    if (nsig < 1 || K < 1 || nw < 1 || !x || !omega || !re || !im || !std::isfinite(dt) ||
-        !(dt > 0) || std::isnan(t_damp) || t_damp < 0 || nsig > 65535 * 8)
-        return fail(TDB_ERR_ARG, "tdb_damped_transform: invalid sizes, pointers, dt or t_damp");
-    for (int k = 0; k < nw; ++k)
-        if (!std::isfinite(omega[k]))
-            return fail(TDB_ERR_ARG, "tdb_damped_transform: non-finite frequency");
-    const double inv_td = (t_damp == 0.0 || std::isinf(t_damp)) ? 0.0 : 1.0 / t_damp;
-    // blocked path: rows (signal, block) of 512 samples, the frequencies in chunks whose
-    // products stay within kChunkBytes.  The slices are exact relative to a row's largest
-    // value, so the damping must not spread a block's twiddles over many binades (e^-8 at most).
+// The transform by the blocked or the direct path (checked arguments).
+tdb_status transform(bool blocked, int nsig, long K, const double* x, double dt, double inv_td, int nw,
+                     const double* omega, double* re, double* im) {
     const long long nb = ((long long)K + kBlk - 1) / kBlk;
     const long long rows = nb * nsig;
-    const bool blocked = (double)nsig * (double)K * nw >= kTensorWork && nb <= 65535 &&
-                         kBlk * dt * inv_td <= 8.0 &&
-                         nsig <= 65535 && rows * 2048 <= (long long)kChunkBytes;
     int cw = nw;   // frequencies per chunk
     if (blocked) {
         const long long fit = (long long)(kChunkBytes / 16) / rows;
@@ -309,5 +294,30 @@ extern "C" tdb_status tdb_damped_transform(int nsig, long K, const double* x, do
     cudaFree(base);
     if (st) cudaStreamDestroy(st);
     if (rc != TDB_OK) tdb::set_last_error("tdb_damped_transform: a CUDA call failed");
+    return rc;
+}
+
+}  // namespace
+
+extern "C" tdb_status tdb_damped_transform(int nsig, long K, const double* x, double dt,
+                                           double t_damp, int nw, const double* omega, double* re,
+                                           double* im) {
+    if (nsig < 1 || K < 1 || nw < 1 || !x || !omega || !re || !im || !std::isfinite(dt) ||
+        !(dt > 0) || std::isnan(t_damp) || t_damp < 0 || nsig > 65535 * 8)
+        return fail(TDB_ERR_ARG, "tdb_damped_transform: invalid sizes, pointers, dt or t_damp");
+    for (int k = 0; k < nw; ++k)
+        if (!std::isfinite(omega[k]))
+            return fail(TDB_ERR_ARG, "tdb_damped_transform: non-finite frequency");
+    const double inv_td = (t_damp == 0.0 || std::isinf(t_damp)) ? 0.0 : 1.0 / t_damp;
+    // blocked path: rows (signal, block) of 512 samples, the frequencies in chunks whose
+    // products stay within kChunkBytes.  The slices are exact relative to a row's largest
+    // value, so the damping must not spread a block's twiddles over many binades (e^-8 at most).
+    // Where its buffers do not fit, the direct path's do with less.
+    const long long nb = ((long long)K + kBlk - 1) / kBlk;
+    const bool blocked = (double)nsig * (double)K * nw >= kTensorWork && nb <= 65535 &&
+                         kBlk * dt * inv_td <= 8.0 &&
+                         nsig <= 65535 && nb * nsig * 2048 <= (long long)kChunkBytes;
+    tdb_status rc = transform(blocked, nsig, K, x, dt, inv_td, nw, omega, re, im);
+    if (blocked && rc == TDB_ERR_NOMEM) rc = transform(false, nsig, K, x, dt, inv_td, nw, omega, re, im);
     return rc;
 }

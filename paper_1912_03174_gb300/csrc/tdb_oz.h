@@ -72,8 +72,8 @@ struct Gate {
 // njobs <= 3 matrices of the same rows, K and scheme in one launch.
 void slice_rows(const SliceJob* jobs, int njobs, cudaStream_t st, Gate gate = {});
 void slice_rows(const double* A, int lda, double sign, Sliced& out, cudaStream_t st);
-// Slices of B^T for a general B (K x cols, row-major FP64, row stride ldb); colmax is
-// a device scratch of cols doubles.
+// Slices of B^T (scheme kSix) for a general B (K x cols, row-major FP64, row stride ldb);
+// colmax is a device scratch of cols doubles.
 void slice_cols(const double* B, int ldb, Sliced& out, double* colmax, cudaStream_t st);
 
 // One product sharing the A operand: C (M x N, row-major FP64, row stride ldc) = A B.

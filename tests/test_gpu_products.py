@@ -229,3 +229,32 @@ def test_cluster_steps_give_the_bits_of_the_separate_kernels(B, n_atoms, n_speci
                         p.observables()["E_total"]))
     for o in out[1:]:
         assert o[0] == out[0][0] and np.array_equal(o[1], out[0][1]) and o[2] == out[0][2]
+
+
+# one orbital per atom gives N that is no multiple of 4 or 2: rows without 16-byte alignment in
+# every form (N = 13, 70 and 193, the last with the FP64 form's sliced products)
+@pytest.mark.parametrize("form,n_atoms,tol", [
+    ("fp64", 193, 1e-10), ("fp64s", 13, 2e-8), ("fp64s", 70, 2e-8), ("fp32", 13, 1e-6),
+    ("fp32", 70, 1e-6), ("fp16x6", 13, 1e-6), ("fp16x6", 70, 1e-6), ("bf16x3", 13, 2e-5),
+    ("bf16x3", 70, 2e-5)])
+def test_rows_without_alignment_match_the_oracle(B, form, n_atoms, tol):
+    # the bounds of each form's parity tests; a clone half way steps to the same bits
+    import dataclasses
+    sysm = dataclasses.replace(I.small_flake(n_atoms, seed=8), orbs_per_atom=1,
+                               n_electrons=1.0 * n_atoms)
+    run = I.Run(dt=0.2, n_steps=0, scc=True, kick=1e-3, kT=I.SCC_KT)
+    n = 60
+    with B.Propagator(sysm, run, form) as p:
+        p.setup()
+        p.step(n // 2)
+        c = B.tdb_clone(p.ctx)
+        p.step(n - n // 2)
+        B.tdb_step(c, n - n // 2)
+        hist = B.tdb_dipole_history(p.ctx, n)
+        rho = B.tdb_get_rho(p.ctx)
+        same = B.tdb_get_state(p.ctx) == B.tdb_get_state(c)
+        B.tdb_destroy(c)
+    tr = O.propagate(sysm, run, O.setup(sysm, run)[0], n)
+    assert np.max(np.abs(hist - tr.dipole[:n])) < tol
+    assert np.max(np.abs(rho - tr.rho)) < tol
+    assert same
