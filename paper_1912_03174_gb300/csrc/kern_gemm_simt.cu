@@ -91,15 +91,14 @@ __global__ void __launch_bounds__(kT8* kT8)
     if (gm < M && gn < Ncol) (blockIdx.z ? C1 : C0)[(size_t)gm * ldc + gn] = acc;
 }
 
-// FP32: a 64 x 64 tile of C per block of 128 threads, 8 x 4 consecutive outputs each, for one
-// of up to three products of the same shape (blockIdx.z).  Bound by FFMA issue: a warp's step
-// of K reads 2 + 2 shared-memory wavefronts for its 32 FFMA, and the next 32-deep block is
-// loaded into registers while this one is multiplied (32 rather than 16: a block's multiplications
-// then outlast a load).  64 x 64 rather than 128 x 128, so that
-// the three X products of a middle-sized system fill the chip (N = 532: 243 tiles; 128 x 128
-// tiles gave 25 blocks a product; the step there went from 427 to 92 us).  Each output sums its
-// K terms in order.
-constexpr int kF32Tile = 64, kF32K = 32, kF32Threads = 128, kF32Loads = 4;
+// FP32, large systems: a 64 x 64 tile of C per block of 128 threads, 8 x 4 consecutive outputs
+// each, for one of up to three products of the same shape (blockIdx.z).  Bound by FFMA issue: a
+// warp's step of K reads 2 + 2 shared-memory wavefronts for its 32 FFMA, and the next 32-deep
+// block is loaded into registers while this one is multiplied (32 rather than 16: a block's
+// multiplications then outlast a load).  Nothing may use a loaded value before the
+// multiplications: delta H is formed where B goes to shared memory (formed in the load, it made
+// delta M at N = 1024 take 113 us, now 75; X 178, now 173).  Each output sums its K terms in order.
+constexpr int kF32Tile = 64, kF32K = 32, kF32Threads = 128, kF32Loads = 4, kF32Sms = 152;
 
 struct F32Parts {
     F32Part p[3];
@@ -110,7 +109,8 @@ template <bool DHAM>
 __global__ void __launch_bounds__(kF32Threads, 3)
     k_gemm_f32(int M, int Ncol, int K, const __grid_constant__ F32Parts parts,
                const float* dv, const float* add, float* C2) {
-    __shared__ __align__(16) float As[2][kF32K][kF32Tile + 4];
+    // A transposed; row r of k lies at r ^ 4 (k / 4 mod 8): the transposing stores hit all 32 banks
+    __shared__ __align__(16) float As[2][kF32K][kF32Tile];
     __shared__ __align__(16) float Bs[2][kF32K][kF32Tile];
     const F32Part& P = parts.p[blockIdx.z];
     const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(kF32Threads, 3)
     const int ar = tid / 8, ak = 4 * (tid % 8), bk = tid / 16, bn = 4 * (tid % 16);
     const bool va = (P.lda % 4 == 0) && (reinterpret_cast<uintptr_t>(P.A) & 15) == 0;
     const bool vb = (P.ldb % 4 == 0) && (reinterpret_cast<uintptr_t>(P.B) & 15) == 0;
-    float ra[kF32Loads][4], rb[kF32Loads][4];
+    float ra[kF32Loads][4], rb[kF32Loads][4], dk[kF32Loads];
     float dvn[4] = {0.f, 0.f, 0.f, 0.f};
     pdl_wait();
     if (DHAM)
@@ -147,18 +147,17 @@ __global__ void __launch_bounds__(kF32Threads, 3)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) rb[h][j] = gk < K && gn + j < Ncol ? pb[j] : 0.f;
             }
-            if (DHAM) {
-                const float dk = gk < K ? dv[gk] : 0.f;
-#pragma unroll
-                for (int j = 0; j < 4; ++j) rb[h][j] = 0.5f * rb[h][j] * (dk + dvn[j]);
-            }
+            if (DHAM) dk[h] = gk < K ? dv[gk] : 0.f;
         }
     };
     auto store = [&](int s) {
 #pragma unroll
         for (int h = 0; h < kF32Loads; ++h) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) As[s][ak + j][ar + 16 * h] = ra[h][j];
+            for (int j = 0; j < 4; ++j) As[s][ak + j][(ar + 16 * h) ^ ak] = ra[h][j];
+            if (DHAM)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) rb[h][j] = 0.5f * rb[h][j] * (dk[h] + dvn[j]);
             *reinterpret_cast<float4*>(&Bs[s][bk + 8 * h][bn]) =
                 make_float4(rb[h][0], rb[h][1], rb[h][2], rb[h][3]);
         }
@@ -177,8 +176,8 @@ __global__ void __launch_bounds__(kF32Threads, 3)
         if (more) load(k0 + kF32K);
 #pragma unroll
         for (int kk = 0; kk < kF32K; ++kk) {
-            const float4 a0 = *reinterpret_cast<const float4*>(&As[s][kk][8 * ty]);
-            const float4 a1 = *reinterpret_cast<const float4*>(&As[s][kk][8 * ty + 4]);
+            const float4 a0 = *reinterpret_cast<const float4*>(&As[s][kk][(8 * ty) ^ (kk & ~3)]);
+            const float4 a1 = *reinterpret_cast<const float4*>(&As[s][kk][(8 * ty + 4) ^ (kk & ~3)]);
             const float4 b0 = *reinterpret_cast<const float4*>(&Bs[s][kk][4 * tx]);
             const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
             const float b[4] = {b0.x, b0.y, b0.z, b0.w};
@@ -205,6 +204,184 @@ __global__ void __launch_bounds__(kF32Threads, 3)
                 // M = M_gs + delta M beside delta M
                 if (DHAM && C2) C2[(size_t)gm * P.ldc + gn + j] = add[(size_t)gm * Ncol + gn + j] + acc[i][j];
             }
+    }
+}
+
+// FP32, up to one 64 x 64 tile per SM and product: smaller tiles, TM x TN of C per block, RM x RN
+// outputs per thread (rows CY apart, columns in groups of four consecutive ones), for one of up to
+// three products of the same shape (blockIdx.z).  With so little work per SM what bounds it is
+// the latency of each K block: operands go to shared memory by asynchronous copies two blocks
+// ahead, A as it lies in memory (a thread reads four K of its rows at a time), so that a block
+// costs one barrier and few instructions beside its FFMA.  Each output sums its K terms in order.
+// Microseconds, delta M / the three X products, 64 x 64 tiles of k_gemm_f32 and this: N = 40 7.6 / 5.8
+// and 3.8 / 2.7, N = 260 16.8 / 17.3 and 11.1 / 8.2, N = 532 28.7 / 45.8 and 25.6 / 30.6.
+template <int TM, int TN, int RM, int RN, int KB, int ST>
+struct F32Tile {
+    static constexpr int M = TM, N = TN, R = RM, C = RN, K = KB, S = ST, CX = TN / RN, CY = TM / RM,
+                         T = CX * CY;
+    static constexpr int KA = KB / 4, NB = TN / 4, LA = TM * KA / T, LB = KB * NB / T;
+    static_assert(T % KA == 0 && T % NB == 0 && RN % 4 == 0 && LA * T == TM * KA && LB * T == KB * NB, "");
+};
+
+// 16 bytes (or 4) to shared memory, of which the first `bytes` are read and the rest are zero
+__device__ __forceinline__ void copy16(float* dst, const float* src, int bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                     static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+                 "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void copy4(float* dst, const float* src, int bytes) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                     static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+                 "l"(src), "r"(bytes) : "memory");
+}
+// Four elements p[0 .. 3] of which the first n (any integer) exist; base is any valid address.
+__device__ __forceinline__ void copy_row4(float* dst, const float* p, const float* base, int n, bool vec) {
+    n = max(0, min(n, 4));
+    if (vec) {
+        copy16(dst, n ? p : base, 4 * n);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) copy4(dst + j, j < n ? p + j : base, j < n ? 4 : 0);
+    }
+}
+
+template <bool DHAM, class X>
+__global__ void __launch_bounds__(X::T)
+    k_gemm_f32_small(int M, int Ncol, int K, const __grid_constant__ F32Parts parts,
+               const float* dv, const float* add, float* C2) {
+    __shared__ __align__(16) float As[X::S][X::M][X::K + 4];
+    __shared__ __align__(16) float Bs[X::S][X::K][X::N];
+    __shared__ float dks[DHAM ? X::S : 1][X::LB][X::T];
+    const F32Part& P = parts.p[blockIdx.z];
+    const int tid = threadIdx.x, tx = tid % X::CX, ty = tid / X::CX;
+    const int m0 = blockIdx.y * X::M, n0 = blockIdx.x * X::N;
+    const int ar = tid / X::KA, ak = 4 * (tid % X::KA), bk = tid / X::NB, bn = 4 * (tid % X::NB);
+    const bool va = (P.lda % 4 == 0) && (reinterpret_cast<uintptr_t>(P.A) & 15) == 0;
+    const bool vb = (P.ldb % 4 == 0) && (reinterpret_cast<uintptr_t>(P.B) & 15) == 0;
+    const bool vc = (P.ldc % 4 == 0) && (reinterpret_cast<uintptr_t>(P.C) & 15) == 0;
+    float dvn[4] = {0.f, 0.f, 0.f, 0.f};
+    pdl_wait();
+    if (DHAM)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) dvn[j] = n0 + bn + j < Ncol ? dv[n0 + bn + j] : 0.f;
+    auto load = [&](int k0, int s) {
+        if (k0 < K) {
+#pragma unroll
+            for (int h = 0; h < X::LA; ++h) {
+                const int r = ar + X::T / X::KA * h, gm = m0 + r;
+                copy_row4(&As[s][r][ak], P.A + (size_t)gm * P.lda + k0 + ak, P.A,
+                          gm < M ? K - k0 - ak : 0, va);
+            }
+#pragma unroll
+            for (int h = 0; h < X::LB; ++h) {
+                const int r = bk + X::T / X::NB * h, gk = k0 + r;
+                copy_row4(&Bs[s][r][bn], P.B + (size_t)gk * P.ldb + n0 + bn, P.B,
+                          gk < K ? Ncol - n0 - bn : 0, vb);
+                if (DHAM) copy4(&dks[s][h][tid], gk < K ? dv + gk : dv, gk < K ? 4 : 0);
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float acc[X::R][X::C];
+#pragma unroll
+    for (int i = 0; i < X::R; ++i)
+#pragma unroll
+        for (int j = 0; j < X::C; ++j) acc[i][j] = 0.f;
+#pragma unroll
+    for (int s = 0; s < X::S - 1; ++s) load(s * X::K, s);
+    int s = 0;
+    for (int k0 = 0; k0 < K; k0 += X::K, s = s + 1 == X::S ? 0 : s + 1) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(X::S - 2) : "memory");
+        if (DHAM)   // each thread turns the elements of S that it has copied into delta H
+#pragma unroll
+            for (int h = 0; h < X::LB; ++h) {
+                float4* b = reinterpret_cast<float4*>(&Bs[s][bk + X::T / X::NB * h][bn]);
+                const float dk = dks[s][h][tid];
+                float4 v = *b;
+                v.x = 0.5f * v.x * (dk + dvn[0]);
+                v.y = 0.5f * v.y * (dk + dvn[1]);
+                v.z = 0.5f * v.z * (dk + dvn[2]);
+                v.w = 0.5f * v.w * (dk + dvn[3]);
+                *b = v;
+            }
+        __syncthreads();
+        load(k0 + (X::S - 1) * X::K, s == 0 ? X::S - 1 : s - 1);
+#pragma unroll
+        for (int k4 = 0; k4 < X::K; k4 += 4) {
+            float4 a4[X::R];
+#pragma unroll
+            for (int i = 0; i < X::R; ++i) a4[i] = *reinterpret_cast<const float4*>(&As[s][ty + X::CY * i][k4]);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+                float b[X::C];
+#pragma unroll
+                for (int q = 0; q < X::C; q += 4) {
+                    const float4 v = *reinterpret_cast<const float4*>(&Bs[s][k4 + kk][4 * tx + X::CX * q]);
+                    b[q] = v.x, b[q + 1] = v.y, b[q + 2] = v.z, b[q + 3] = v.w;
+                }
+#pragma unroll
+                for (int i = 0; i < X::R; ++i) {
+                    const float a = kk == 0 ? a4[i].x : kk == 1 ? a4[i].y : kk == 2 ? a4[i].z : a4[i].w;
+#pragma unroll
+                    for (int j = 0; j < X::C; ++j) acc[i][j] = fmaf(a, b[j], acc[i][j]);
+                }
+            }
+        }
+    }
+    pdl_launch_dependents();
+#pragma unroll
+    for (int i = 0; i < X::R; ++i) {
+        const int gm = m0 + ty + X::CY * i;
+        if (gm >= M) break;
+#pragma unroll
+        for (int q = 0; q < X::C; q += 4) {
+            const int gn = n0 + 4 * tx + X::CX * q;
+            float* c = P.C + (size_t)gm * P.ldc + gn;
+            if (vc && gn + 4 <= Ncol) {
+                *reinterpret_cast<float4*>(c) = make_float4(acc[i][q], acc[i][q + 1], acc[i][q + 2], acc[i][q + 3]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (gn + j < Ncol) c[j] = acc[i][q + j];
+            }
+            // M = M_gs + delta M beside delta M
+            if (DHAM && C2)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (gn + j < Ncol)
+                        C2[(size_t)gm * P.ldc + gn + j] = add[(size_t)gm * Ncol + gn + j] + acc[i][q + j];
+        }
+    }
+}
+
+// 64 x 32 tiles, or 32 x 32 where they leave fewer outputs on the fullest SM (N = 532: 36 and 31 us
+// for X; where both leave as many the larger tile reads less, N = 700: 57 and 71).
+using F32Wide = F32Tile<64, 32, 4, 4, 32, 3>;
+using F32Narrow = F32Tile<32, 32, 4, 4, 32, 3>;
+
+template <bool DHAM>
+void run_f32(int M, int Ncol, int K, const F32Parts& p, int nparts, const float* dv, const float* add,
+             float* C2, cudaStream_t st) {
+    auto tiles = [&](int tm, int tn) { return ((M + tm - 1) / tm) * ((Ncol + tn - 1) / tn); };
+    bool aligned = true;
+    for (int z = 0; z < nparts; ++z)
+        aligned = aligned && p.p[z].lda % 4 == 0 && p.p[z].ldb % 4 == 0 &&
+                  ((reinterpret_cast<uintptr_t>(p.p[z].A) | reinterpret_cast<uintptr_t>(p.p[z].B)) & 15) == 0;
+    // rows without 16-byte alignment go element by element: at N = 70 delta M / X 6.2 / 3.8 us against
+    // 9.5 / 7.4 in 64 x 64 tiles, at N = 801 80 / 142 against 70 / 98
+    auto go = [&](auto kernel, int tm, int tn, int threads) {
+        launch_pdl(kernel, dim3((Ncol + tn - 1) / tn, (M + tm - 1) / tm, nparts), dim3(threads), 0, st, M,
+                   Ncol, K, p, dv, add, C2);
+    };
+    if (tiles(64, 64) > (aligned ? kF32Sms : 9)) {
+        go(k_gemm_f32<DHAM>, kF32Tile, kF32Tile, kF32Threads);
+    } else {
+        auto fullest = [&](int tm, int tn) { return (tiles(tm, tn) * nparts + kF32Sms - 1) / kF32Sms * tm * tn; };
+        const bool narrow = tiles(64, 32) * nparts > kF32Sms && fullest(32, 32) < fullest(64, 32);
+        if (narrow)
+            go(k_gemm_f32_small<DHAM, F32Narrow>, F32Narrow::M, F32Narrow::N, F32Narrow::T);
+        else
+            go(k_gemm_f32_small<DHAM, F32Wide>, F32Wide::M, F32Wide::N, F32Wide::T);
     }
 }
 
@@ -237,18 +414,14 @@ void gemm_f64_ham(int N, const double* A, const double* H0, const double* S, con
 void gemm_f32(int M, int Ncol, int K, const F32Part* parts, int nparts, cudaStream_t st) {
     F32Parts p{};
     for (int z = 0; z < nparts; ++z) p.p[z] = parts[z];
-    const dim3 g((Ncol + kF32Tile - 1) / kF32Tile, (M + kF32Tile - 1) / kF32Tile, nparts);
-    launch_pdl(k_gemm_f32<false>, g, dim3(kF32Threads), 0, st, M, Ncol, K, p,
-               static_cast<const float*>(nullptr), static_cast<const float*>(nullptr),
-               static_cast<float*>(nullptr));
+    run_f32<false>(M, Ncol, K, p, nparts, nullptr, nullptr, nullptr, st);
 }
 
 void gemm_f32_dham(int N, const float* A, const float* S, const float* dv, float* dM, float* Msum,
                    int ldc, const float* Mgs, cudaStream_t st) {
     F32Parts p{};
     p.p[0] = {A, N, S, N, dM, ldc};
-    const dim3 g((N + kF32Tile - 1) / kF32Tile, (N + kF32Tile - 1) / kF32Tile);
-    launch_pdl(k_gemm_f32<true>, g, dim3(kF32Threads), 0, st, N, N, N, p, dv, Mgs, Msum);
+    run_f32<true>(N, N, N, p, 1, dv, Mgs, Msum, st);
 }
 
 }  // namespace tdb

@@ -91,6 +91,24 @@ def test_fp32_form_matches_the_oracle_at_tile_edges(B, n_atoms):
     assert np.max(np.abs(rho - tr.rho)) < 1e-6
 
 
+# N = 532 (32 x 32 tiles for X: 64 x 32 ones would leave a nearly empty round), 772 (the smallest
+# aligned size past one 64 x 64 tile per SM); the bounds of the test above
+@pytest.mark.parametrize("n_atoms", [133, 193])
+def test_fp32_form_matches_the_oracle_past_its_tile_rules(B, n_atoms):
+    sysm = I.small_flake(n_atoms, seed=8)
+    run = I.Run(dt=0.2, n_steps=0, scc=True, kick=1e-3, kT=I.SCC_KT)
+    n = 10
+    with B.Propagator(sysm, run, "fp32") as p:
+        p.setup()
+        p.step(n)
+        hist = B.tdb_dipole_history(p.ctx, n)
+        rho = B.tdb_get_rho(p.ctx)
+    ref, _, _, _ = O.setup(sysm, run)
+    tr = O.propagate(sysm, run, ref, n)
+    assert np.max(np.abs(hist - tr.dipole[:n])) < 1e-6
+    assert np.max(np.abs(rho - tr.rho)) < 1e-6
+
+
 @pytest.mark.parametrize("dt_over_damp", [0.0, 0.004, 0.5])
 @pytest.mark.parametrize("nsig,K,nw", [(1, 513, 24000), (3, 4608, 901), (10, 1023, 1300)])
 def test_damped_transform_of_large_problems_matches_the_oracle(B, nsig, K, nw, dt_over_damp):
@@ -235,7 +253,7 @@ def test_cluster_steps_give_the_bits_of_the_separate_kernels(B, n_atoms, n_speci
 # every form (N = 13, 70 and 193, the last with the FP64 form's sliced products)
 @pytest.mark.parametrize("form,n_atoms,tol", [
     ("fp64", 193, 1e-10), ("fp64s", 13, 2e-8), ("fp64s", 70, 2e-8), ("fp32", 13, 1e-6),
-    ("fp32", 70, 1e-6), ("fp16x6", 13, 1e-6), ("fp16x6", 70, 1e-6), ("bf16x3", 13, 2e-5),
+    ("fp32", 70, 1e-6), ("fp32", 193, 1e-6), ("fp16x6", 13, 1e-6), ("fp16x6", 70, 1e-6), ("bf16x3", 13, 2e-5),
     ("bf16x3", 70, 2e-5)])
 def test_rows_without_alignment_match_the_oracle(B, form, n_atoms, tol):
     # the bounds of each form's parity tests; a clone half way steps to the same bits
