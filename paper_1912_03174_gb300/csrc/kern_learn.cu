@@ -10,9 +10,11 @@
 #include <cuda_bf16.h>
 
 #include <cmath>
+#include <cstddef>
 #include <cstdint>
 
 #include "tdb_internal.h"
+#include "tdb_learn.h"
 
 namespace tdb {
 namespace learn {
@@ -195,46 +197,86 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// One epoch of Adam in one thread-block cluster: every CTA keeps the whole network in shared
-// memory (weights rounded to bfloat16) and owns 1/NC of the parameters' FP32 masters and Adam
-// moments.  Per mini-batch the CTAs take equal shares of the samples (chunks of 32), write their
-// gradient sums into their own shared memory, and after a cluster barrier each owner adds the NC
-// sums of its parameters in rank order through distributed shared memory, updates them and
-// stores the new values into all NC networks.  The arithmetic per sample is that of k_net_grad.
+// One parameter's Adam step with the bias corrections c1, c2 (k_adam and k_net_epoch; the
+// roundings are written out, so that both are the same).
+__device__ __forceinline__ void adam(float& p, float& m, float& v, float g, float lr, float b1, float b2,
+                                     float c1, float c2, float eps) {
+    m = fmaf(b1, m, __fmul_rn(1.f - b1, g));
+    v = fmaf(b2, v, __fmul_rn(__fmul_rn(1.f - b2, g), g));
+    p -= lr * (m / c1) / (sqrtf(v / c2) + eps);
+}
+
+// Mini-batches of Adam in one thread-block cluster: every CTA keeps the whole network in shared
+// memory (weights rounded to bfloat16).  The CTAs work in groups of four; a group takes a block
+// of 128 samples of the mini-batch, each of its CTAs (members) the activations of 32 of them.
+// They hand those on through distributed shared memory, all first-layer activations to every
+// member and the rest to the member whose 16 columns they belong to, and after a cluster barrier
+// each member forms its columns' gradient sums over the block's 128 samples.  After another
+// barrier each owner adds the groups' sums of its parameters in group order, updates them (FP32
+// masters and moments in registers) and stores the new values into every network.
+//
+// The sums round as those of k_net_grad do: a chain over the 128 samples of a block for each
+// parameter, blocks added one after another, and per sample the same chains.  Where a mini-batch has
+// one block or two (a sum of two does not depend on its order) the results are bit for bit those
+// of k_net_grad and k_adam; with more, k_net_grad's atomic order varies from run to run and this
+// is one of its orders up to one block a group.  (Sums in other chains are as accurate, but a master
+// near a tie of the bfloat16 rounding then rounds the other way now and then, and an epoch's
+// parameters moved by up to 2e-5 against 1e-5 between two runs of k_net_grad.)
+//
 // A mini-batch is a few MFLOP, so what bounds it is latency: two launches, an atomic sum and
 // layers with one output per thread cost 121 us a batch of 512 at 16 x 64 (4 blocks of 128
-// samples), this 17.8; here a thread takes 2 samples x 4 hidden units, and nothing leaves the
-// cluster between batches.  Hidden units are padded to 64 with zero weights, which add nothing.
-constexpr int kES = 32, kEH = 64, kEF = 32, kEStride = kEH + 4, kEThreads = 256;
-constexpr int kEMaxOwn = 4;            // parameters per thread and CTA: 6337 / 8 / 256
+// samples), this 14.2; with sums over 32 samples in every CTA and block barriers between the layers it was
+// 17.9.  A thread takes 2 samples x 4 hidden units; a warp's four samples need no other
+// warp, so the layers follow one another without a block barrier.  Hidden units are padded to
+// 64 with zero weights and zero activations.  Bias corrections 1 - beta^t come from the host.
+constexpr int kES = 32, kEMembers = 4, kEH = 64, kEF = 32, kEC = kEH / kEMembers, kEStride = kEH + 4,
+              kEThreads = 256;
+constexpr int kESlice = (kEF + kEH + 3) * kEC + 1;   // gradient sums of a member: W1, W2, b1, b2, w3, b3
+static_assert(kES * kEMembers == kBlockSamples, "sizes");
 struct EpochSmem {
     float W1[kEF][kEH], W2[kEH][kEH], W2T[kEH][kEH];
     float b1[kEH], b2[kEH], w3[kEH], b3;
-    alignas(16) float x[kES][kEF + 4], h1[kES][kEStride], h2[kES][kEStride], d1[kES][kEStride],
-        d2[kES][kEStride];
-    float y[kES], dy[kES];
-    double sse[kEThreads / 32];
-    float g[kEF * kEH + 2 * kEH + kEH * kEH + kEH + 1];
+    alignas(16) float h2[kES][kEStride], d2[kES][kEStride];   // own samples
+    // the block's samples: inputs (of this batch and the next), activations, columns of this member
+    alignas(16) float x[2][kBlockSamples][kEF + 4], h1[kBlockSamples][kEStride];
+    float h2c[kBlockSamples][kEC + 4], d1c[kBlockSamples][kEC + 4], d2c[kBlockSamples][kEC + 4];
+    float dy[kBlockSamples], r2[kBlockSamples];
+    float g[kESlice];
 };
 
-// network value of packed parameter i (used by the owner to fill every CTA's copy)
-__device__ void put_param(const Layout& L, EpochSmem& s, int i, float v) {
-    const int H = L.H;
+// Entry e of member's gradient slice: its packed parameter (-1: none).
+__device__ __forceinline__ int slice_param(const Layout& L, int member, int e) {
+    if (e == (L.F + L.H + 3) * kEC) return member == 0 ? L.ob3 : -1;
+    const int row = e / kEC, col = kEC * member + e % kEC;
+    if (col >= L.H) return -1;
+    if (row < L.F) return L.oW1 + row * L.H + col;
+    if (row < L.F + L.H) return L.oW2 + (row - L.F) * L.H + col;
+    return (row == L.F + L.H ? L.ob1 : row == L.F + L.H + 1 ? L.ob2 : L.ow3) + col;
+}
+// Where packed parameter i lies in a network, in floats from its start: `at` (and `at2`, W2
+// transposed, or -1); true for a weight, which is kept rounded to bfloat16.
+__device__ __forceinline__ bool param_place(const Layout& L, int i, int& at, int& at2) {
+    auto f = [](size_t bytes) { return static_cast<int>(bytes / sizeof(float)); };
+    at2 = -1;
     if (i < L.ob1) {
-        s.W1[i / H][i % H] = bf(v);
+        at = f(offsetof(EpochSmem, W1)) + i / L.H * kEH + i % L.H;
     } else if (i < L.oW2) {
-        s.b1[i - L.ob1] = v;
+        at = f(offsetof(EpochSmem, b1)) + i - L.ob1;
+        return false;
     } else if (i < L.ob2) {
-        const int k = i - L.oW2;
-        s.W2[k / H][k % H] = bf(v);
-        s.W2T[k % H][k / H] = bf(v);
+        const int r = (i - L.oW2) / L.H, c = (i - L.oW2) % L.H;
+        at = f(offsetof(EpochSmem, W2)) + r * kEH + c;
+        at2 = f(offsetof(EpochSmem, W2T)) + c * kEH + r;
     } else if (i < L.ow3) {
-        s.b2[i - L.ob2] = v;
+        at = f(offsetof(EpochSmem, b2)) + i - L.ob2;
+        return false;
     } else if (i < L.ob3) {
-        s.w3[i - L.ow3] = bf(v);
+        at = f(offsetof(EpochSmem, w3)) + i - L.ow3;
     } else {
-        s.b3 = v;
+        at = f(offsetof(EpochSmem, b3));
+        return false;
     }
+    return true;
 }
 
 // acc[q][j] += sum_k A[2 ty + q][k] W[k][4 tx + j], k < K (a multiple of 4)
@@ -258,124 +300,177 @@ __device__ __forceinline__ void layer(const float* A, int lda, const float* W, i
         }
     }
 }
-__device__ __forceinline__ void put2(float (*o)[kEStride], int tx, int ty, const float (&v)[2][4]) {
+__device__ __forceinline__ void put4(float* o, const float (&v)[4]) {
+    *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
+}
+// Column sums over the block of a tile of 2 rows x 4 columns: g[r][j] = sum_q A[q][r] D[q][j], q in order
+__device__ __forceinline__ void column_sums(const float* A, int lda, const float* D, float (&g)[2][4]) {
 #pragma unroll
-    for (int q = 0; q < 2; ++q)
-        *reinterpret_cast<float4*>(&o[2 * ty + q][4 * tx]) =
-            make_float4(v[q][0], v[q][1], v[q][2], v[q][3]);
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) g[r][j] = 0.f;
+#pragma unroll 8
+    for (int q = 0; q < kBlockSamples; ++q) {
+        const float2 a = *reinterpret_cast<const float2*>(A + q * lda);
+        const float4 d = *reinterpret_cast<const float4*>(D + q * (kEC + 4));
+        const float ar[2] = {a.x, a.y}, dj[4] = {d.x, d.y, d.z, d.w};
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) g[r][j] = fmaf(ar[r], dj[j], g[r][j]);
+    }
 }
 
+// NG: groups of the cluster
+template <int NG>
 __global__ void __launch_bounds__(kEThreads)
     k_net_epoch(int F, int H, float* __restrict__ params, float* __restrict__ am,
                 float* __restrict__ av, const float* __restrict__ X, const float* __restrict__ Y,
-                long n, long batch, float lr, float beta1, float beta2, float eps, long t0,
-                double* __restrict__ sse) {
+                long n, long batch, float lr, float beta1, float beta2, float eps,
+                const __grid_constant__ Corrections corr, double* __restrict__ sse) {
     extern __shared__ __align__(16) uint8_t epoch_raw[];
     EpochSmem& s = *reinterpret_cast<EpochSmem*>(epoch_raw);
+    float* const net = reinterpret_cast<float*>(epoch_raw);
     cg::cluster_group cluster = cg::this_cluster();
-    const int rank = static_cast<int>(cluster.block_rank()), NC = static_cast<int>(cluster.num_blocks());
+    constexpr int NC = NG * kEMembers, kOwn = (kESlice + NG * kEThreads - 1) / (NG * kEThreads);
+    const int rank = static_cast<int>(cluster.block_rank());
+    const int group = rank / kEMembers, member = rank % kEMembers;
     const Layout L = layout(F, H);
-    const int t = threadIdx.x, tx = t % 16, ty = t / 16;
+    const int t = threadIdx.x, lane = t % 32, warp = t / 32, tx = t % 16, ty = t / 16;
     // everything starts at zero (padded rows and columns stay there)
     for (int i = t; i < static_cast<int>(sizeof(EpochSmem) / 4); i += kEThreads)
         reinterpret_cast<uint32_t*>(epoch_raw)[i] = 0;
     __syncthreads();
-    for (int i = t; i < L.n; i += kEThreads) put_param(L, s, i, params[i]);
-    // this CTA's parameters
-    const int own = (L.n + NC - 1) / NC, o0 = rank * own;
-    float pp[kEMaxOwn], pm[kEMaxOwn], pv[kEMaxOwn];
-#pragma unroll
-    for (int u = 0; u < kEMaxOwn; ++u) {
-        const int k = t + u * kEThreads, i = o0 + k;
-        const bool mine = k < own && i < L.n;
-        pp[u] = mine ? params[i] : 0.f;
-        pm[u] = mine ? am[i] : 0.f;
-        pv[u] = mine ? av[i] : 0.f;
+    for (int i = t; i < L.n; i += kEThreads) {
+        int at, at2;
+        const float v = params[i], w = param_place(L, i, at, at2) ? bf(v) : v;
+        net[at] = w;
+        if (at2 >= 0) net[at2] = w;
     }
-    double sq = 0.0;
-    long step = t0;
-    // this thread's values of a chunk, loaded one chunk ahead (rows past the share: x = 0)
-    constexpr int kPre = kES * kEF / kEThreads;
-    float xn[kPre], yn = 0.f;
-    auto fetch = [&](long b0, long c0) {
-        const long nb = batch < n - b0 ? batch : n - b0;
-        const long per = (nb + NC - 1) / NC, lo = rank * per, hi = lo + per < nb ? lo + per : nb;
+    // this CTA's parameters: its share of the member's slice
+    const int slice = (F + H + 3) * kEC + 1, own = (slice + NG - 1) / NG;
+    float pp[kOwn], pm[kOwn], pv[kOwn];
+    int pe[kOwn], pi[kOwn], at[kOwn], at2[kOwn];
+    bool weight[kOwn];
 #pragma unroll
-        for (int u = 0; u < kPre; ++u) {
-            const int e = t + u * kEThreads, q = e / F;
-            const long r = lo + c0 + q;
-            xn[u] = q < kES && r < hi ? __ldg(X + (b0 + r) * F + (e - q * F)) : 0.f;
+    for (int u = 0; u < kOwn; ++u) {
+        const int k = t + u * kEThreads;
+        pe[u] = group * own + k;
+        pi[u] = k < own && pe[u] < slice ? slice_param(L, member, pe[u]) : -1;
+        pp[u] = pm[u] = pv[u] = 0.f;
+        at[u] = at2[u] = -1;
+        weight[u] = false;
+        if (pi[u] >= 0) {
+            pp[u] = params[pi[u]];
+            pm[u] = am[pi[u]];
+            pv[u] = av[pi[u]];
+            weight[u] = param_place(L, pi[u], at[u], at2[u]);
         }
-        yn = t < kES && lo + c0 + t < hi ? __ldg(Y + b0 + lo + c0 + t) : 0.f;
+    }
+    // block `round NG + group` of the mini-batch at b0: its inputs into x[buf] (rows past the batch:
+    // zero), asynchronously, and this lane's target
+    const bool vec = F % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+    const int row = kES * member + 4 * warp + (lane & 3);   // of the block: this lane's sample
+    float yn = 0.f;
+    auto fetch = [&](long b0, long round, int buf) {
+        const long nb = batch < n - b0 ? batch : n - b0, r0 = (round * NG + group) * kBlockSamples;
+        const int q = t >> 1;
+        const bool in = r0 + q < nb;
+        const float* src = X + (in ? b0 + r0 + q : b0) * F;
+        float* dst = s.x[buf][q];
+        if (vec)
+            for (int c = 4 * (t & 1); c < F; c += 8)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                                 static_cast<uint32_t>(__cvta_generic_to_shared(dst + c))),
+                             "l"(src + c), "r"(in ? 16 : 0) : "memory");
+        else
+            for (int c = t & 1; c < F; c += 2)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                                 static_cast<uint32_t>(__cvta_generic_to_shared(dst + c))),
+                             "l"(src + c), "r"(in ? 4 : 0) : "memory");
+        yn = r0 + row < nb ? __ldg(Y + b0 + r0 + row) : 0.f;
     };
-    fetch(0, 0);
-    for (long b0 = 0; b0 < n; b0 += batch) {
+    double sq = 0.0;
+    int buf = 0;
+    fetch(0, 0, 0);
+    cluster.sync();   // no CTA writes into another one's memory before that is cleared
+    for (long b0 = 0, step = 0; b0 < n; b0 += batch, ++step) {
         const long nb = batch < n - b0 ? batch : n - b0;
-        const long per = (nb + NC - 1) / NC, lo = rank * per, hi = lo + per < nb ? lo + per : nb;
+        const long blocks = (nb + kBlockSamples - 1) / kBlockSamples, rounds = (blocks + NG - 1) / NG;
         const float scale = 1.0f / static_cast<float>(nb);
-        for (long c0 = 0; c0 < per; c0 += kES) {
-            // samples lo + c0 .. of the batch (rows past the share carry x = 0 and dy = 0)
+        for (long round = 0; round < rounds; ++round, buf ^= 1) {
+            const bool real = (round * NG + group) * kBlockSamples + row < nb;   // this lane's sample
+            const float y_ref = yn;
+            asm volatile("cp.async.wait_all;" ::: "memory");
             __syncthreads();
-#pragma unroll
-            for (int u = 0; u < kPre; ++u) {
-                const int e = t + u * kEThreads, q = e / F;
-                if (q < kES) s.x[q][e - q * F] = xn[u];
-            }
-            if (t < kES) s.y[t] = yn;
-            __syncthreads();
-            if (c0 + kES < per)
-                fetch(b0, c0 + kES);
+            if (round + 1 < rounds)
+                fetch(b0, round + 1, buf ^ 1);
             else if (b0 + batch < n)
-                fetch(b0 + batch, 0);
-            float v[2][4], dv[2][4];
+                fetch(b0 + batch, 0, buf ^ 1);
+            const int r = kES * member + 2 * ty;   // of the block: this thread's first sample
+            float v[2][4], h1[2][4], h2[2][4];
             auto bias = [&](const float* b) {
 #pragma unroll
                 for (int q = 0; q < 2; ++q)
 #pragma unroll
                     for (int j = 0; j < 4; ++j) v[q][j] = b[4 * tx + j];
             };
-            // h1 = tanh(x W1 + b1); rows of W1 past F are zero
+            // h1 = tanh(x W1 + b1) to every member; rows of W1 past F are zero
             bias(s.b1);
-            layer(&s.x[0][0], kEF + 4, &s.W1[0][0], (F + 3) & ~3, tx, ty, v);
-            float h1[2][4];
-#pragma unroll
-            for (int q = 0; q < 2; ++q)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) h1[q][j] = tanhf(v[q][j]);
-            put2(s.h1, tx, ty, h1);
-            __syncthreads();
-            // h2 = tanh(h1 W2 + b2)
-            bias(s.b2);
-            layer(&s.h1[0][0], kEStride, &s.W2[0][0], kEH, tx, ty, v);
-            float h2[2][4];
-#pragma unroll
-            for (int q = 0; q < 2; ++q)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) h2[q][j] = tanhf(v[q][j]);
-            put2(s.h2, tx, ty, h2);
-            // y = h2 w3 + b3, dy = 2 (y - Y) / nb: the 16 threads of a sample pair
-            float z[2] = {0.f, 0.f};
+            layer(s.x[buf][kES * member], kEF + 4, &s.W1[0][0], (F + 3) & ~3, tx, ty, v);
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) z[q] = fmaf(h2[q][j], s.w3[4 * tx + j], z[q]);
-                for (int o = 8; o > 0; o >>= 1) z[q] += __shfl_xor_sync(0xffffffffu, z[q], o);
-                const long r = lo + c0 + 2 * ty + q;
-                const float res = r < hi ? z[q] + s.b3 - s.y[2 * ty + q] : 0.f;
-                z[q] = 2.f * res * scale;
-                if (tx == 0) {
-                    s.dy[2 * ty + q] = z[q];
-                    sq += static_cast<double>(res * res);
+                for (int j = 0; j < 4; ++j) h1[q][j] = tanhf(v[q][j]);
+#pragma unroll
+                for (int m = 0; m < kEMembers; ++m) {
+                    float* o = &s.h1[r + q][4 * tx];   // (this CTA reads its own rows in a moment)
+                    put4(m == member ? o : cluster.map_shared_rank(o, group * kEMembers + m), h1[q]);
                 }
             }
-            // dz2 = dy w3 (1 - h2^2)
+            __syncwarp();
+            // h2 = tanh(h1 W2 + b2)
+            bias(s.b2);
+            layer(s.h1[kES * member], kEStride, &s.W2[0][0], kEH, tx, ty, v);
 #pragma unroll
-            for (int q = 0; q < 2; ++q)
+            for (int q = 0; q < 2; ++q) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    dv[q][j] = z[q] * s.w3[4 * tx + j] * (1.f - h2[q][j] * h2[q][j]);
-            put2(s.d2, tx, ty, dv);
-            __syncthreads();
+                for (int j = 0; j < 4; ++j) h2[q][j] = tanhf(v[q][j]);
+                put4(&s.h2[2 * ty + q][4 * tx], h2[q]);
+            }
+            __syncwarp();
+            // y = h2 w3 + b3, dy = 2 (y - Y) / nb, every lane for one of the warp's four samples
+            float y = s.b3;
+#pragma unroll 4
+            for (int j = 0; j < kEH; j += 4) {
+                const float4 h = *reinterpret_cast<const float4*>(&s.h2[4 * warp + (lane & 3)][j]);
+                const float4 w = *reinterpret_cast<const float4*>(&s.w3[j]);
+                y = fmaf(h.x, w.x, y);
+                y = fmaf(h.y, w.y, y);
+                y = fmaf(h.z, w.z, y);
+                y = fmaf(h.w, w.w, y);
+            }
+            const float res = real ? y - y_ref : 0.f;
+            const float dy = 2.f * res * scale;
+            // lane l stores the sample l & 3 to member l >> 2
+            if (lane < 4 * kEMembers) {
+                EpochSmem* to = cluster.map_shared_rank(&s, group * kEMembers + (lane >> 2));
+                to->dy[row] = dy;
+                to->r2[row] = res * res;
+            }
+            // dz2 = dy w3 (1 - h2^2); this thread's four columns belong to member tx / 4
+            EpochSmem* to = cluster.map_shared_rank(&s, group * kEMembers + tx / 4);
+            const int col = 4 * (tx % 4);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const float z = __shfl_sync(0xffffffffu, dy, 2 * (ty & 1) + q);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) v[q][j] = z * s.w3[4 * tx + j] * (1.f - h2[q][j] * h2[q][j]);
+                put4(&s.d2[2 * ty + q][4 * tx], v[q]);
+                put4(&to->d2c[r + q][col], v[q]);
+                put4(&to->h2c[r + q][col], h2[q]);
+            }
+            __syncwarp();
             // dz1 = (dz2 W2^T) (1 - h1^2)
 #pragma unroll
             for (int q = 0; q < 2; ++q)
@@ -383,118 +478,83 @@ __global__ void __launch_bounds__(kEThreads)
                 for (int j = 0; j < 4; ++j) v[q][j] = 0.f;
             layer(&s.d2[0][0], kEStride, &s.W2T[0][0], kEH, tx, ty, v);
 #pragma unroll
-            for (int q = 0; q < 2; ++q)
+            for (int q = 0; q < 2; ++q) {
 #pragma unroll
                 for (int j = 0; j < 4; ++j) v[q][j] *= 1.f - h1[q][j] * h1[q][j];
-            put2(s.d1, tx, ty, v);
-            // gradient sums of W2 (rows 4 ty .., columns 4 tx ..): h1^T dz2
-            {
-                float g2[4][4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) g2[i][j] = 0.f;
-#pragma unroll 4
-                for (int q = 0; q < kES; ++q) {
-                    const float4 a = *reinterpret_cast<const float4*>(&s.h1[q][4 * ty]);
-                    const float4 d = *reinterpret_cast<const float4*>(&s.d2[q][4 * tx]);
-                    const float ai[4] = {a.x, a.y, a.z, a.w}, dj[4] = {d.x, d.y, d.z, d.w};
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) g2[i][j] = fmaf(ai[i], dj[j], g2[i][j]);
-                }
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        if (4 * ty + i < H && 4 * tx + j < H) {
-                            float& o = s.g[L.oW2 + (4 * ty + i) * H + 4 * tx + j];
-                            o = c0 ? o + g2[i][j] : g2[i][j];
-                        }
+                put4(&to->d1c[r + q][col], v[q]);
             }
-            __syncthreads();
-            // W1: x^T dz1 (rows ty, ty + 16); then the biases, w3 and b3
+            cluster.sync();
+            // gradient sums of the block: W2 by warps 0 - 3, W1 by 4 and 5, the rest by 6 and 7
+            auto add = [&](int e, float g) { s.g[e] = round ? s.g[e] + g : g; };
+            if (warp < 6) {
+                const bool first = warp >= 4;
+                const int k = first ? t - 128 : t, i = 2 * (k / 4), c = 4 * (k % 4);
+                if (i < (first ? F : H)) {
+                    float g[2][4];
+                    if (first)
+                        column_sums(&s.x[buf][0][i], kEF + 4, &s.d1c[0][c], g);
+                    else
+                        column_sums(&s.h1[0][i], kEStride, &s.d2c[0][c], g);
 #pragma unroll
-            for (int r = 0; r < kEF / 16; ++r) {
-                const int f = ty + 16 * r;
-                if (f >= F) break;
-                float g1[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-                for (int q = 0; q < kES; ++q) {
-                    const float4 d = *reinterpret_cast<const float4*>(&s.d1[q][4 * tx]);
-                    const float xf = s.x[q][f];
-                    g1[0] = fmaf(xf, d.x, g1[0]);
-                    g1[1] = fmaf(xf, d.y, g1[1]);
-                    g1[2] = fmaf(xf, d.z, g1[2]);
-                    g1[3] = fmaf(xf, d.w, g1[3]);
+                    for (int q = 0; q < 2; ++q)
+                        if (i + q < (first ? F : H))
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) add(((first ? 0 : F) + i + q) * kEC + c + j, g[q][j]);
                 }
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (4 * tx + j < H) {
-                        float& o = s.g[L.oW1 + f * H + 4 * tx + j];
-                        o = c0 ? o + g1[j] : g1[j];
-                    }
-            }
-            {
-                const int kind = t / kEH, j = t % kEH;
+            } else {
+                const int k = t - 192, kind = k / kEC, c = k % kEC;
                 float g = 0.f;
                 if (kind == 0)
 #pragma unroll 8
-                    for (int q = 0; q < kES; ++q) g += s.d1[q][j];
+                    for (int q = 0; q < kBlockSamples; ++q) g += s.d1c[q][c];
                 else if (kind == 1)
 #pragma unroll 8
-                    for (int q = 0; q < kES; ++q) g += s.d2[q][j];
+                    for (int q = 0; q < kBlockSamples; ++q) g += s.d2c[q][c];
                 else if (kind == 2)
 #pragma unroll 8
-                    for (int q = 0; q < kES; ++q) g = fmaf(s.h2[q][j], s.dy[q], g);
-                else if (j == 0)
-                    for (int q = 0; q < kES; ++q) g += s.dy[q];
-                if ((kind < 3 && j < H) || (kind == 3 && j == 0)) {
-                    float& o = s.g[kind == 0 ? L.ob1 + j : kind == 1 ? L.ob2 + j
-                                                       : kind == 2   ? L.ow3 + j
-                                                                     : L.ob3];
-                    o = c0 ? o + g : g;
+                    for (int q = 0; q < kBlockSamples; ++q) g = fmaf(s.h2c[q][c], s.dy[q], g);
+                else if (c == 0)
+#pragma unroll 8
+                    for (int q = 0; q < kBlockSamples; ++q) g += s.dy[q];
+                if (kind < 3 || c == 0) add((F + H + kind) * kEC + c, g);
+                if (warp == 6 && member == 0) {
+                    float r2 = 0.f;
+#pragma unroll
+                    for (int q = 0; q < kBlockSamples; q += 32) r2 += s.r2[q + lane];
+                    for (int o = 16; o > 0; o >>= 1) r2 += __shfl_xor_sync(0xffffffffu, r2, o);
+                    sq += static_cast<double>(r2);
                 }
             }
+            cluster.sync();   // the block's sums are complete, and its activations read
         }
-        cluster.sync();
-        // owners: sum over the CTAs in rank order, Adam, new values into every network
-        ++step;
-        const float c1 = 1.0f - powf(beta1, static_cast<float>(step));
-        const float c2 = 1.0f - powf(beta2, static_cast<float>(step));
+        // owners: sum over the groups in order, Adam, new values into every network
+        const float2 c = corr.c[step];
 #pragma unroll
-        for (int u = 0; u < kEMaxOwn; ++u) {
-            const int k = t + u * kEThreads, i = o0 + k;
-            if (k < own && i < L.n) {
+        for (int u = 0; u < kOwn; ++u)
+            if (pi[u] >= 0) {
                 float g = 0.f;
-#pragma unroll 8
-                for (int c = 0; c < NC; ++c) g += *cluster.map_shared_rank(&s.g[i], c);
-                pm[u] = beta1 * pm[u] + (1.f - beta1) * g;
-                pv[u] = beta2 * pv[u] + (1.f - beta2) * g * g;
-                pp[u] -= lr * (pm[u] / c1) / (sqrtf(pv[u] / c2) + eps);
-                for (int c = 0; c < NC; ++c) put_param(L, *cluster.map_shared_rank(&s, c), i, pp[u]);
+#pragma unroll
+                for (int k = 0; k < NG; ++k)
+                    g += *cluster.map_shared_rank(&s.g[pe[u]], k * kEMembers + member);
+                adam(pp[u], pm[u], pv[u], g, lr, beta1, beta2, c.x, c.y, eps);
+                const float w = weight[u] ? bf(pp[u]) : pp[u];
+#pragma unroll 4
+                for (int k = 0; k < NC; ++k) {
+                    float* o = cluster.map_shared_rank(net, k);
+                    o[at[u]] = w;
+                    if (at2[u] >= 0) o[at2[u]] = w;
+                }
             }
-        }
         cluster.sync();
     }
 #pragma unroll
-    for (int u = 0; u < kEMaxOwn; ++u) {
-        const int k = t + u * kEThreads, i = o0 + k;
-        if (k < own && i < L.n) {
-            params[i] = pp[u];
-            am[i] = pm[u];
-            av[i] = pv[u];
+    for (int u = 0; u < kOwn; ++u)
+        if (pi[u] >= 0) {
+            params[pi[u]] = pp[u];
+            am[pi[u]] = pm[u];
+            av[pi[u]] = pv[u];
         }
-    }
-    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-    if (t % 32 == 0) s.sse[t / 32] = sq;
-    __syncthreads();
-    if (t == 0) {
-        double x = 0.0;
-        for (int w = 0; w < kEThreads / 32; ++w) x += s.sse[w];
-        atomicAdd(sse, x);
-    }
+    if (warp == 6 && member == 0 && lane == 0) atomicAdd(sse, sq);
 }
 
 __global__ void k_adam(int n, float* __restrict__ p, const float* __restrict__ g,
@@ -502,9 +562,7 @@ __global__ void k_adam(int n, float* __restrict__ p, const float* __restrict__ g
                        float c1, float c2, float eps) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    m[i] = b1 * m[i] + (1.f - b1) * g[i];
-    v[i] = b2 * v[i] + (1.f - b2) * g[i] * g[i];
-    p[i] -= lr * (m[i] / c1) / (sqrtf(v[i] / c2) + eps);
+    adam(p[i], m[i], v[i], g[i], lr, b1, b2, c1, c2, eps);
 }
 
 // Closed-form leapfrog window in the eigenbasis: for element (a, b), theta = (e_a - e_b) dt,
@@ -560,10 +618,13 @@ cudaError_t prepare(int, int) {
     cudaError_t e = cudaFuncSetAttribute(k_net_grad, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(grad_smem(32, 64)));
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_net_epoch, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(k_net_epoch<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  static_cast<int>(sizeof(EpochSmem)));
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_net_epoch, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        e = cudaFuncSetAttribute(k_net_epoch<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 static_cast<int>(sizeof(EpochSmem)));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_net_epoch<4>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_net_forward, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  static_cast<int>(sizeof(float) * layout(32, 64).n));
@@ -610,16 +671,17 @@ struct EpochLaunch {
 int epoch_cluster() {
     int fits = 0;
     EpochLaunch l(16, nullptr);
-    if (cudaOccupancyMaxActiveClusters(&fits, k_net_epoch, &l.cfg) != cudaSuccess) cudaGetLastError();
+    if (cudaOccupancyMaxActiveClusters(&fits, k_net_epoch<4>, &l.cfg) != cudaSuccess) cudaGetLastError();
     return fits > 0 ? 16 : 8;
 }
 
 cudaError_t launch_epoch(int nc, int F, int H, float* params, float* m, float* v, const float* X,
                          const float* Y, long n, long batch, float lr, float b1, float b2, float eps,
-                         long t0, double* sse, cudaStream_t st) {
+                         const Corrections& corr, double* sse, cudaStream_t st) {
     EpochLaunch l(nc, st);
-    return cudaLaunchKernelEx(&l.cfg, k_net_epoch, F, H, params, m, v, X, Y, n, batch, lr, b1, b2,
-                              eps, t0, sse);
+    auto kernel = nc == 16 ? k_net_epoch<4> : k_net_epoch<2>;
+    return cudaLaunchKernelEx(&l.cfg, kernel, F, H, params, m, v, X, Y, n, batch, lr, b1, b2, eps, corr,
+                              sse);
 }
 
 void launch_window(int N, const double* eps, double dt, int k, double* x0re, double* x0im,

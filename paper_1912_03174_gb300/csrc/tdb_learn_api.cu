@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "tdb.h"
+#include "tdb_learn.h"
 
 namespace tdb {
 void set_last_error(const char* msg);
@@ -24,7 +25,7 @@ void launch_adam(int n, float* p, const float* g, float* m, float* v, float lr, 
 int epoch_cluster();
 cudaError_t launch_epoch(int nc, int F, int H, float* params, float* m, float* v, const float* X,
                          const float* Y, long n, long batch, float lr, float b1, float b2, float eps,
-                         long t0, double* sse, cudaStream_t st);
+                         const Corrections& corr, double* sse, cudaStream_t st);
 }  // namespace learn
 }  // namespace tdb
 
@@ -42,9 +43,16 @@ struct tdb_shiftnet {
 namespace {
 
 // Mini-batches up to this size train an epoch in one cluster launch; larger ones give every SM
-// 128-sample blocks of k_net_grad.  Microseconds a batch, cluster / grid, 16 x 64 network: 21 / 121
-// at 512 samples, 44 / 124 at 2048, 74 / 124 at 4096, 135 / 127 at 8192 (the cluster has 16 SMs).
+// 128-sample blocks of k_net_grad.  Microseconds a batch, cluster / grid, 16 x 64 network: 14 / 121
+// at 512 samples, 38 / 124 at 2048, 68 / 124 at 4096, 99 / 123 at 6144; the cluster (16 SMs) takes
+// another 8 us for every 512 samples, the grid 123 up to 152 blocks.
 constexpr long kEpochBatch = 6144;
+
+// Adam's bias corrections 1 - beta^t of step t.
+float2 bias_corrections(float b1, float b2, long t) {
+    return make_float2(1.0f - std::pow(b1, static_cast<float>(t)),
+                       1.0f - std::pow(b2, static_cast<float>(t)));
+}
 
 tdb_status fail(const char* msg, tdb_status s) {
     tdb::set_last_error(msg);
@@ -191,14 +199,18 @@ tdb_status tdb_shiftnet_train(tdb_shiftnet* net, const float* X, const float* Y,
     double last = 0.0;
     for (int ep = 0; ep < epochs; ++ep) {
         cudaMemsetAsync(net->sse, 0, sizeof(double), net->st);
-        if (batch <= kEpochBatch) {
-            if (tdb::learn::launch_epoch(net->cluster, net->F, net->H, net->p, net->m, net->v, net->X,
-                                         net->Y, n, batch, lr, b1, b2, eps, net->t, net->sse,
-                                         net->st) != cudaSuccess) {
+        for (long s = 0; batch <= kEpochBatch && s < n; s += tdb::learn::kEpochSteps * batch) {
+            const long nb = std::min(tdb::learn::kEpochSteps * batch, n - s);
+            const int steps = static_cast<int>((nb + batch - 1) / batch);
+            tdb::learn::Corrections corr;
+            for (int k = 0; k < steps; ++k) corr.c[k] = bias_corrections(b1, b2, net->t + k + 1);
+            if (tdb::learn::launch_epoch(net->cluster, net->F, net->H, net->p, net->m, net->v,
+                                         net->X + s * net->F, net->Y + s, nb, batch, lr, b1, b2, eps,
+                                         corr, net->sse, net->st) != cudaSuccess) {
                 cudaGetLastError();
                 return fail("tdb_shiftnet_train: CUDA error", TDB_ERR_CUDA);
             }
-            net->t += (n + batch - 1) / batch;
+            net->t += steps;
         }
         for (long s = 0; batch > kEpochBatch && s < n; s += batch) {
             const long nb = std::min(batch, n - s);
@@ -206,9 +218,8 @@ tdb_status tdb_shiftnet_train(tdb_shiftnet* net, const float* X, const float* Y,
             tdb::learn::launch_grad(net->F, net->H, net->p, net->X + s * net->F, net->Y + s, nb,
                                     1.0f / nb, net->g, net->sse, net->st);
             ++net->t;
-            const float c1 = 1.0f - std::pow(b1, static_cast<float>(net->t));
-            const float c2 = 1.0f - std::pow(b2, static_cast<float>(net->t));
-            tdb::learn::launch_adam(net->np, net->p, net->g, net->m, net->v, lr, b1, b2, c1, c2, eps,
+            const float2 c = bias_corrections(b1, b2, net->t);
+            tdb::learn::launch_adam(net->np, net->p, net->g, net->m, net->v, lr, b1, b2, c.x, c.y, eps,
                                     net->st);
         }
         if (ep == epochs - 1) {

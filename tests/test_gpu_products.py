@@ -276,3 +276,33 @@ def test_rows_without_alignment_match_the_oracle(B, form, n_atoms, tol):
     assert np.max(np.abs(hist - tr.dipole[:n])) < tol
     assert np.max(np.abs(rho - tr.rho)) < tol
     assert same
+
+
+# less than a block of 128 samples, one block and a ragged one, two whole ones (a sum of two does not
+# depend on its order); more batches than one launch takes; hidden and feature counts that are
+# no multiples of 4
+@pytest.mark.parametrize("F,H,n,batch", [(16, 64, 2048, 256), (5, 7, 400, 100), (32, 64, 1250, 250),
+                                         (3, 33, 390, 130), (1, 1, 300, 1)])
+def test_training_epochs_give_the_bits_of_the_gradient_kernel_and_adam(B, F, H, n, batch):
+    # the same steps from tdb_shiftnet_gradient (same block sums) and Adam in FP32: moments by one
+    # fused multiply-add each, bias corrections from powers rounded once
+    f, d = np.float32, np.float64
+    rng = np.random.default_rng(F * 100 + H)
+    p = (rng.normal(size=F * H + H + H * H + 2 * H + 1) * 0.3).astype(f)
+    X = rng.normal(size=(n, F)).astype(f)
+    Y = rng.normal(size=n).astype(f)
+    lr, b1, b2 = f(2e-3), f(0.9), f(0.999)
+    with B.ShiftNet(F, H) as net:
+        net.set_params(p)
+        net.train(X, Y, epochs=1, batch=batch, lr=lr)
+        got = net.params()
+        q, m, v = p, np.zeros_like(p), np.zeros_like(p)
+        for t, s in enumerate(range(0, n, batch), 1):
+            net.set_params(q)
+            g = net.gradient(X[s:s + batch], Y[s:s + batch])[1]
+            m = (d(b1) * m + ((f(1) - b1) * g).astype(d)).astype(f)
+            v = (d(b2) * v + ((f(1) - b2) * g * g).astype(d)).astype(f)
+            c1, c2 = (f(1) - f(float(b) ** t) for b in (b1, b2))
+            q = q - (lr * (m / c1)) / (np.sqrt(v / c2) + f(1e-8))
+            assert q.dtype == f
+    assert np.array_equal(got, q)
