@@ -415,13 +415,14 @@ __global__ void __launch_bounds__(kEThreads)
 #pragma unroll
                     for (int j = 0; j < 4; ++j) v[q][j] = b[4 * tx + j];
             };
-            // h1 = tanh(x W1 + b1) to every member; rows of W1 past F are zero
+            // h1 = tanh(x W1 + b1) to every member; rows of W1 past F are zero.  (Padded units are
+            // set to zero: an infinite input times their zero weights is not.)
             bias(s.b1);
             layer(s.x[buf][kES * member], kEF + 4, &s.W1[0][0], (F + 3) & ~3, tx, ty, v);
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) h1[q][j] = tanhf(v[q][j]);
+                for (int j = 0; j < 4; ++j) h1[q][j] = 4 * tx + j < H ? tanhf(v[q][j]) : 0.f;
 #pragma unroll
                 for (int m = 0; m < kEMembers; ++m) {
                     float* o = &s.h1[r + q][4 * tx];   // (this CTA reads its own rows in a moment)

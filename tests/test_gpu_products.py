@@ -306,3 +306,23 @@ def test_training_epochs_give_the_bits_of_the_gradient_kernel_and_adam(B, F, H, 
             q = q - (lr * (m / c1)) / (np.sqrt(v / c2) + f(1e-8))
             assert q.dtype == f
     assert np.array_equal(got, q)
+
+
+@pytest.mark.parametrize("H", [5, 64])
+def test_an_infinite_feature_saturates_its_units_and_no_others(B, H):
+    # tanh takes +-inf to +-1, so the loss stays finite and only the gradient of the infinite
+    # feature's weights (inf times a derivative of zero) is NaN, as in the gradient kernel
+    F, n = 3, 100
+    rng = np.random.default_rng(H)
+    p = (rng.normal(size=F * H + H + H * H + 2 * H + 1) * 0.3).astype(np.float32)
+    X = rng.normal(size=(n, F)).astype(np.float32)
+    X[17, 1] = np.inf
+    Y = rng.normal(size=n).astype(np.float32)
+    with B.ShiftNet(F, H) as net:
+        net.set_params(p)
+        loss, g = net.gradient(X, Y)
+        net.set_params(p)
+        assert net.train(X, Y, epochs=1, batch=n, lr=1e-3) == pytest.approx(loss, rel=1e-6)
+        q = net.params()
+    assert np.isfinite(loss) and np.isfinite(g).sum() == len(g) - H
+    assert np.array_equal(np.isfinite(q), np.isfinite(g))
