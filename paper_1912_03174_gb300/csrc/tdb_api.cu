@@ -33,7 +33,19 @@ struct tdb_ctx : public Ctx {};
 
 namespace {
 thread_local std::string g_err;
+
+// Failures that a test cannot bring about otherwise, one at a time and for the calling thread only:
+// after tdb_test_fail_once(site) the next call at that site fails on the host as if CUDA had.
+enum FailSite { kFailNone = 0, kFailGraph = 1 };
+thread_local int g_fail = kFailNone;
+bool injected(FailSite site) {
+    if (g_fail != site) return false;
+    g_fail = kFailNone;
+    return true;
 }
+}  // namespace
+
+extern "C" void tdb_test_fail_once(int site) { g_fail = site; }
 
 namespace tdb {
 // message returned by tdb_last_error() on this thread
@@ -1299,8 +1311,12 @@ tdb_status ensure_graph(Ctx& c, int cur) {
     cudaGraph_t g = nullptr;
     CK(cudaStreamBeginCapture(c.stream, cudaStreamCaptureModeThreadLocal));
     int nl = 0;
+    // nothing runs while it is captured: which step S, H0, gamma and S^-1 belong to stays as it is
+    const long long model_n = c.model_n, line_n = c.line_n;
     tdb_status st = c.prm.move_nuclei ? enqueue_step_md(c, cur, false, &nl)
                                       : enqueue_step(c, cur, false, &nl);
+    c.model_n = model_n;
+    c.line_n = line_n;
     cudaError_t e = cudaStreamEndCapture(c.stream, &g);
     if (st != TDB_OK) {
         if (g) cudaGraphDestroy(g);
@@ -1310,7 +1326,7 @@ tdb_status ensure_graph(Ctx& c, int cur) {
         set_err("graph capture failed: %s", cudaGetErrorString(e));
         return TDB_ERR_CUDA;
     }
-    e = cudaGraphInstantiate(&c.graph[cur], g, 0);
+    e = injected(kFailGraph) ? cudaErrorMemoryAllocation : cudaGraphInstantiate(&c.graph[cur], g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) {
         set_err("graph instantiate failed: %s", cudaGetErrorString(e));

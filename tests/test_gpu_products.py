@@ -326,3 +326,30 @@ def test_an_infinite_feature_saturates_its_units_and_no_others(B, H):
         q = net.params()
     assert np.isfinite(loss) and np.isfinite(g).sum() == len(g) - H
     assert np.array_equal(np.isfinite(q), np.isfinite(g))
+
+
+@pytest.mark.parametrize("form,n_atoms", [("fp64", 12), ("fp64s", 12), ("fp64s", 49)])
+@pytest.mark.parametrize("failures", [1, 2])
+def test_a_failed_graph_leaves_an_ehrenfest_run_as_it_was(B, form, n_atoms, failures):
+    # the calls that would capture a step fail on the host (out of memory, say); the same steps taken
+    # afterwards give the bits of an undisturbed run
+    sysm = I.small_cluster(n_atoms, seed=7, T=3000.0, rep_A=60.0)
+    run = I.Run(dt=0.2, n_steps=0, scc=True, move_nuclei=True, kick=1e-2, kT=I.SCC_KT)
+    out = []
+    for fail in (0, failures):
+        with B.Propagator(sysm, run, form) as p:
+            p.setup()
+            done = 0
+            while done < 12:
+                if fail:
+                    B.load().tdb_test_fail_once(1)
+                try:
+                    p.step(1)
+                    done += 1
+                except B.TdbError as e:
+                    assert e.status == 3 and "graph" in str(e)
+                    fail -= 1
+            B.load().tdb_test_fail_once(0)
+            assert fail == 0
+            out.append((B.tdb_get_state(p.ctx), B.tdb_dipole_history(p.ctx, 12)))
+    assert out[0][0] == out[1][0] and np.array_equal(out[0][1], out[1][1])
