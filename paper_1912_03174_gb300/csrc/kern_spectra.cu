@@ -152,9 +152,10 @@ __global__ void k_outer_twiddles(int nb, int nw, const double* __restrict__ omeg
     E[(size_t)b * nw + k] = e;
 }
 
-// F_s(w_k) = dt sum_b E[b][k] P[s nb + b][2 k .. 2 k + 1]
+// F_s(w_k) = dt sum_b E[b][k] P[s nb + b][2 k .. 2 k + 1]; *nonfinite set where a sum is not finite
 __global__ void k_outer_sum(int nb, int nw, const double2* __restrict__ E, const double2* __restrict__ P,
-                            double dt, int ldo, double* __restrict__ re, double* __restrict__ im) {
+                            double dt, int ldo, double* __restrict__ re, double* __restrict__ im,
+                            int* __restrict__ nonfinite) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x, s = blockIdx.y;
     if (k >= nw) return;
     double a = 0.0, c = 0.0;
@@ -166,6 +167,7 @@ __global__ void k_outer_sum(int nb, int nw, const double2* __restrict__ E, const
     }
     re[(size_t)s * ldo + k] = dt * a;
     im[(size_t)s * ldo + k] = dt * c;
+    if (!isfinite(a) || !isfinite(c)) *nonfinite = 1;
 }
 
 tdb_status fail(tdb_status st, const char* msg) {
@@ -181,9 +183,10 @@ void run_direct(dim3 grid, int nsig, long long K, long long span, const double* 
 
 size_t up(size_t b) { return (b + 255) & ~(size_t)255; }
 
-// The transform by the blocked or the direct path (checked arguments).
+// The transform by the blocked or the direct path (checked arguments).  The blocked path sets
+// nonfinite where a result is not finite: its slices make a block with an infinite sample NaN.
 tdb_status transform(bool blocked, int nsig, long K, const double* x, double dt, double inv_td, int nw,
-                     const double* omega, double* re, double* im) {
+                     const double* omega, double* re, double* im, bool& nonfinite) {
     const long long nb = ((long long)K + kBlk - 1) / kBlk;
     const long long rows = nb * nsig;
     int cw = nw;   // frequencies per chunk
@@ -230,7 +233,7 @@ tdb_status transform(bool blocked, int nsig, long K, const double* x, double dt,
         double* dim_ = reinterpret_cast<double*>(base + bx + bw + bo);
         char* q = base + bx + bw + 2 * bo;
         int* err = reinterpret_cast<int*>(q + bt + be + bp + bsa + bsb);
-        int h_err = 0;
+        int h_err[2] = {0, 0};
         if (blocked && xrow != (size_t)K) ok(cudaMemsetAsync(dx, 0, bx, st));
         ok(cudaMemcpy2DAsync(dx, sizeof(double) * xrow, x, sizeof(double) * K, sizeof(double) * K, nsig,
                              cudaMemcpyHostToDevice, st));
@@ -240,7 +243,7 @@ tdb_status transform(bool blocked, int nsig, long K, const double* x, double dt,
             double2* E = reinterpret_cast<double2*>(q + bt);
             double* P = reinterpret_cast<double*>(q + bt + be);
             oz::Sliced a, b;
-            ok(cudaMemsetAsync(err, 0, sizeof(int), st));
+            ok(cudaMemsetAsync(err, 0, 2 * sizeof(int), st));
             ok(oz::prepare());
             if (!oz::sliced_init(a, q + bt + be + bp, (int)rows, kBlk, 128, oz::kSeven)) rc = TDB_ERR_CUDA;
             oz::slice_rows(dx, kBlk, 1.0, a, st);
@@ -261,9 +264,10 @@ tdb_status transform(bool blocked, int nsig, long K, const double* x, double dt,
                 part.ldc = 2 * w;
                 ok(oz::gemm(a, &part, 1, err, st));
                 k_outer_sum<<<dim3((w + 63) / 64, nsig), 64, 0, st>>>(
-                    (int)nb, w, E, reinterpret_cast<const double2*>(P), dt, nw, dre + w0, dim_ + w0);
+                    (int)nb, w, E, reinterpret_cast<const double2*>(P), dt, nw, dre + w0, dim_ + w0,
+                    err + 1);
             }
-            ok(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, st));
+            ok(cudaMemcpyAsync(h_err, err, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
         } else {
             double2* part = reinterpret_cast<double2*>(q);
             const dim3 grid(gx, groups, (unsigned)nz);
@@ -285,7 +289,8 @@ tdb_status transform(bool blocked, int nsig, long K, const double* x, double dt,
         ok(cudaMemcpyAsync(re, dre, sizeof(double) * no, cudaMemcpyDeviceToHost, st));
         ok(cudaMemcpyAsync(im, dim_, sizeof(double) * no, cudaMemcpyDeviceToHost, st));
         ok(cudaStreamSynchronize(st));
-        if (rc == TDB_OK && h_err != 0) {
+        nonfinite = h_err[1] != 0;
+        if (rc == TDB_OK && h_err[0] != 0) {
             cudaFree(base);
             cudaStreamDestroy(st);
             return fail(TDB_ERR_TIMEOUT, "tdb_damped_transform: a bounded device wait timed out");
@@ -312,12 +317,15 @@ extern "C" tdb_status tdb_damped_transform(int nsig, long K, const double* x, do
     // blocked path: rows (signal, block) of 512 samples, the frequencies in chunks whose
     // products stay within kChunkBytes.  The slices are exact relative to a row's largest
     // value, so the damping must not spread a block's twiddles over many binades (e^-8 at most).
-    // Where its buffers do not fit, the direct path's do with less.
+    // Where its buffers do not fit, the direct path's do with less; where a result is not finite, the
+    // direct path takes infinite samples as FP64 arithmetic does.
     const long long nb = ((long long)K + kBlk - 1) / kBlk;
     const bool blocked = (double)nsig * (double)K * nw >= kTensorWork && nb <= 65535 &&
                          kBlk * dt * inv_td <= 8.0 &&
                          nsig <= 65535 && nb * nsig * 2048 <= (long long)kChunkBytes;
-    tdb_status rc = transform(blocked, nsig, K, x, dt, inv_td, nw, omega, re, im);
-    if (blocked && rc == TDB_ERR_NOMEM) rc = transform(false, nsig, K, x, dt, inv_td, nw, omega, re, im);
+    bool nonfinite = false;
+    tdb_status rc = transform(blocked, nsig, K, x, dt, inv_td, nw, omega, re, im, nonfinite);
+    if (blocked && (rc == TDB_ERR_NOMEM || (rc == TDB_OK && nonfinite)))
+        rc = transform(false, nsig, K, x, dt, inv_td, nw, omega, re, im, nonfinite);
     return rc;
 }

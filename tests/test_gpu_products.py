@@ -353,3 +353,26 @@ def test_a_failed_graph_leaves_an_ehrenfest_run_as_it_was(B, form, n_atoms, fail
             assert fail == 0
             out.append((B.tdb_get_state(p.ctx), B.tdb_dipole_history(p.ctx, 12)))
     assert out[0][0] == out[1][0] and np.array_equal(out[0][1], out[1][1])
+
+
+def test_damped_transform_of_large_problems_takes_infinite_samples_as_fp64_does(B):
+    # an infinite sample times the cosine and sine of its phase: infinities of their signs (those
+    # above 1e-9 keep them: the twiddles are good to tens of ulps); a NaN makes its own signal NaN,
+    # other signals are as without them
+    from oracle import tdb_spectra as SP
+    rng = np.random.default_rng(3)
+    x = rng.normal(size=(4, 4608))
+    om = rng.uniform(0.1, 5.0, size=901)
+    dt, t_damp = 0.2, 200.0
+    x[1, 700], x[2, 3000], x[3, 4607] = np.inf, -np.inf, np.nan
+    re, im = np.empty((4, 901)), np.empty((4, 901))   # (a complex array has no infinite parts of its own)
+    assert B.load().tdb_damped_transform(4, 4608, B._ptr(x), dt, t_damp, 901, B._ptr(om), B._ptr(re),
+                                         B._ptr(im)) == 0
+    ref = SP.damped_transform(x[:1], dt, t_damp, om)
+    assert np.max(np.abs(re[0] + 1j * im[0] - ref[0])) < 1e-13 * dt * np.sum(np.abs(x[0]))
+    for s, n, sign in ((1, 700, 1.0), (2, 3000, -1.0)):
+        c, d = np.cos(om * n * dt), np.sin(om * n * dt)
+        assert np.min(np.abs(c)) > 1e-9 and np.min(np.abs(d)) > 1e-9
+        assert np.array_equal(re[s], sign * np.sign(c) * np.inf)
+        assert np.array_equal(im[s], sign * np.sign(d) * np.inf)
+    assert np.all(np.isnan(re[3])) and np.all(np.isnan(im[3]))
