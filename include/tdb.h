@@ -152,7 +152,8 @@ size_t tdb_workspace_bytes(const tdb_system* sys, const tdb_params* prm);
  * Beside the workspace, and also when that is the caller's, a TDB_FP64 context of
  * 192 <= N <= 4096 orbitals allocates the integer slices of its products (70 N^2
  * bytes, rows padded to 64; freed by tdb_destroy).  If they cannot be had, its products
- * run in FP64 arithmetic instead: slower, within the same accuracy. */
+ * run in FP64 arithmetic instead: slower, within the same accuracy but not to the bit (a
+ * state loaded into such a context does not continue bit for bit). */
 tdb_status tdb_create(const tdb_system* sys, const tdb_params* prm, void* workspace,
                       size_t workspace_bytes, tdb_ctx** out);
 
@@ -178,7 +179,8 @@ tdb_status tdb_step(tdb_ctx* ctx, long n);
  * parameters and precision form, its own device workspace (workspace as in
  * tdb_create, or NULL) and stream (cuda_stream, or NULL for a new one); the
  * device state is copied device to device, so a branch costs no ground state and
- * no host round trip.  Stepping the clone reproduces stepping src bit for bit.
+ * no host round trip.  Stepping the clone reproduces stepping src bit for bit (unless its
+ * product slices could not be had and those of src could, see tdb_create).
  * This is how a probe run branches from a pump run at delay tau (Sec. 3.2):
  * step the pump to tau, clone, kick the clone. */
 tdb_status tdb_clone(tdb_ctx* src, void* cuda_stream, void* workspace, size_t workspace_bytes,

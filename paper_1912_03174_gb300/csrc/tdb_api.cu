@@ -36,7 +36,7 @@ thread_local std::string g_err;
 
 // Failures that a test cannot bring about otherwise, one at a time and for the calling thread only:
 // after tdb_test_fail_once(site) the next call at that site fails on the host as if CUDA had.
-enum FailSite { kFailNone = 0, kFailGraph = 1 };
+enum FailSite { kFailNone = 0, kFailGraph = 1, kFailSlices = 2 };
 thread_local int g_fail = kFailNone;
 bool injected(FailSite site) {
     if (g_fail != site) return false;
@@ -161,7 +161,7 @@ void take_slices(Ctx& c, Carver& k) {
 void alloc_slices(Ctx& c) {
     Carver size{nullptr};
     take_slices(c, size);
-    if (cudaMalloc(&c.oz_mem, size.off) != cudaSuccess) {
+    if (injected(kFailSlices) || cudaMalloc(&c.oz_mem, size.off) != cudaSuccess) {
         cudaGetLastError();
         c.oz_mem = nullptr;
         return;
@@ -1927,15 +1927,11 @@ tdb_status tdb_clone(tdb_ctx* src, void* cuda_stream, void* workspace, size_t wo
     prm.cuda_stream = cuda_stream;
     TRY(tdb_create(&sys, &prm, workspace, workspace_bytes, out));
     tdb_ctx* c = *out;
-    // the source's kind of products, so that both step alike
+    // the source's kind of products, so that both step alike; a clone whose slices cannot be had
+    // keeps its DFMA products
     if (!src->oz_mem && c->oz_mem) {
         cudaFree(c->oz_mem);
         c->oz_mem = nullptr;
-    } else if (src->oz_mem && !c->oz_mem) {
-        tdb_destroy(c);
-        *out = nullptr;
-        set_err("tdb_clone: cudaMalloc of the product slices failed");
-        return TDB_ERR_NOMEM;
     }
     // the device state is the workspace (same layout: no device pointers inside it)
     tdb_status rc = TDB_OK;

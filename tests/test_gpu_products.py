@@ -376,3 +376,30 @@ def test_damped_transform_of_large_problems_takes_infinite_samples_as_fp64_does(
         assert np.array_equal(re[s], sign * np.sign(c) * np.inf)
         assert np.array_equal(im[s], sign * np.sign(d) * np.inf)
     assert np.all(np.isnan(re[3])) and np.all(np.isnan(im[3]))
+
+
+def test_contexts_and_clones_without_product_slices_step_with_fp64_products(B):
+    # the slices' memory cannot be had, for the source, the clone or both: every call is served, a pair
+    # of the same kind steps to the same bits and any two of them within the form's bound; the clone of
+    # a source without slices has none either
+    sysm = I.small_flake(49, seed=8)
+    run = I.Run(dt=0.2, n_steps=0, scc=True, kick=1e-2, kT=I.SCC_KT)
+    n = 40
+    ends = []
+    for no_src, no_clone in ((0, 0), (0, 1), (1, 0), (1, 1)):
+        B.load().tdb_test_fail_once(2 * no_src)
+        with B.Propagator(sysm, run, "fp64") as p:
+            p.setup()
+            p.step(n // 2)
+            B.load().tdb_test_fail_once(2 * no_clone)
+            c = B.tdb_clone(p.ctx)
+            B.load().tdb_test_fail_once(0)
+            p.step(n // 2)
+            B.tdb_step(c, n // 2)
+            same = B.tdb_get_state(p.ctx) == B.tdb_get_state(c)
+            assert same == (no_src or not no_clone)
+            ends += [B.tdb_get_rho(p.ctx), B.tdb_get_rho(c)]
+            B.tdb_destroy(c)
+    assert not np.array_equal(ends[0], ends[4])     # (slices and DFMA products differ in the last bits)
+    for e in ends[1:]:
+        assert np.max(np.abs(e - ends[0])) < 1e-10
