@@ -54,14 +54,16 @@ __device__ void twiddle(double w, double dt, double inv_td, double n, double& re
     im = d * fma(cs, pe, sn);
 }
 
-// Partial sums of the samples [n0, n1) of blockIdx.z for the signals of blockIdx.y.  The
+// Partial sums of the samples [n0, n1) of blockIdx.z for the signals of blockIdx.y, or without
+// `part` the results themselves (one block takes all samples).  The
 // twiddle is exact every 32 samples and advanced by the one-step factor in between, which keeps
 // its error at a few tens of ulps.
 template <int SIGS>
 __global__ void __launch_bounds__(kFreqs)
     k_damped_transform(int nsig, long long K, long long span, const double* __restrict__ x, double dt,
                        double inv_td, int nw, const double* __restrict__ omega,
-                       double2* __restrict__ part) {
+                       double2* __restrict__ part, double* __restrict__ re,
+                       double* __restrict__ im) {
     __shared__ double xs[SIGS][kSamp];
     const int k = blockIdx.x * kFreqs + threadIdx.x;
     const int s0 = blockIdx.y * SIGS;
@@ -102,8 +104,15 @@ __global__ void __launch_bounds__(kFreqs)
     if (k >= nw) return;
 #pragma unroll
     for (int s = 0; s < SIGS; ++s)
-        if (s0 + s < nsig)
-            part[((size_t)blockIdx.z * nsig + s0 + s) * nw + k] = make_double2(ar[s], ai[s]);
+        if (s0 + s < nsig) {
+            const size_t i = ((size_t)blockIdx.z * nsig + s0 + s) * nw + k;
+            if (part) {
+                part[i] = make_double2(ar[s], ai[s]);
+            } else {
+                re[i] = dt * ar[s];
+                im[i] = dt * ai[s];
+            }
+        }
 }
 
 // dt times the sum of nz partial sums, in order
@@ -177,8 +186,10 @@ tdb_status fail(tdb_status st, const char* msg) {
 
 template <int SIGS>
 void run_direct(dim3 grid, int nsig, long long K, long long span, const double* x, double dt,
-                double inv_td, int nw, const double* omega, double2* part, cudaStream_t st) {
-    k_damped_transform<SIGS><<<grid, kFreqs, 0, st>>>(nsig, K, span, x, dt, inv_td, nw, omega, part);
+                double inv_td, int nw, const double* omega, double2* part, double* re, double* im,
+                cudaStream_t st) {
+    k_damped_transform<SIGS><<<grid, kFreqs, 0, st>>>(nsig, K, span, x, dt, inv_td, nw, omega, part, re,
+                                                      im);
 }
 
 size_t up(size_t b) { return (b + 255) & ~(size_t)255; }
@@ -214,8 +225,8 @@ tdb_status transform(bool blocked, int nsig, long K, const double* x, double dt,
         bp = up(sizeof(double2) * rows * cw);
         bsa = up(oz::sliced_bytes((int)rows, kBlk, oz::kSeven));
         bsb = up(oz::sliced_bytes(2 * cw, kBlk, oz::kSeven));
-    } else {
-        bp = up(sizeof(double2) * nz * no);
+    } else if (nz > 1) {
+        bp = up(sizeof(double2) * nz * no);   // 608 x 128 x 9 partial sums at most
     }
     tdb_status rc = TDB_OK;
     cudaStream_t st = nullptr;
@@ -269,9 +280,11 @@ tdb_status transform(bool blocked, int nsig, long K, const double* x, double dt,
             }
             ok(cudaMemcpyAsync(h_err, err, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
         } else {
-            double2* part = reinterpret_cast<double2*>(q);
+            double2* part = nz > 1 ? reinterpret_cast<double2*>(q) : nullptr;
             const dim3 grid(gx, groups, (unsigned)nz);
-            auto go = [&](auto fn) { fn(grid, nsig, (long long)K, span, dx, dt, inv_td, nw, dw, part, st); };
+            auto go = [&](auto fn) {
+                fn(grid, nsig, (long long)K, span, dx, dt, inv_td, nw, dw, part, dre, dim_, st);
+            };
             switch (sigs) {
                 case 1: go(run_direct<1>); break;
                 case 2: go(run_direct<2>); break;
@@ -283,7 +296,8 @@ tdb_status transform(bool blocked, int nsig, long K, const double* x, double dt,
                 case 8: go(run_direct<8>); break;
                 default: go(run_direct<9>); break;
             }
-            k_sum_parts<<<(unsigned)((no + 127) / 128), 128, 0, st>>>((int)nz, no, part, dt, dre, dim_);
+            if (part)
+                k_sum_parts<<<(unsigned)((no + 127) / 128), 128, 0, st>>>((int)nz, no, part, dt, dre, dim_);
         }
         ok(cudaGetLastError());
         ok(cudaMemcpyAsync(re, dre, sizeof(double) * no, cudaMemcpyDeviceToHost, st));

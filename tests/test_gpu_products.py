@@ -403,3 +403,22 @@ def test_contexts_and_clones_without_product_slices_step_with_fp64_products(B):
     assert not np.array_equal(ends[0], ends[4])     # (slices and DFMA products differ in the last bits)
     for e in ends[1:]:
         assert np.max(np.abs(e - ends[0])) < 1e-10
+
+
+def test_damped_transform_needs_no_more_memory_than_its_samples_and_results(B):
+    # 320 MB of results where 420 MB are free; damped too strongly within a block for the blocked
+    # path; two samples, so that the reference is a closed form
+    import torch
+    rng = np.random.default_rng(9)
+    x, om = rng.normal(size=(100, 2)), rng.uniform(0.0, 5.0, size=200000)
+    dt, t_damp = 0.2, 0.5
+    B.tdb_damped_transform(x, dt, t_damp, om[:1])
+    torch.cuda.empty_cache()
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - (420 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        got = B.tdb_damped_transform(x, dt, t_damp, om)
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+    ref = dt * (x[:, :1] + x[:, 1:] * np.exp((1j * om - 1 / t_damp) * dt)[None])
+    assert np.max(np.abs(got - ref) / (dt * np.sum(np.abs(x), axis=1, keepdims=True))) < 1e-13
