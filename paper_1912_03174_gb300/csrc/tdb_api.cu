@@ -1966,6 +1966,16 @@ tdb_status tdb_clone(tdb_ctx* src, void* cuda_stream, void* workspace, size_t wo
     c->field_on = src->field_on;
     c->model_n = src->model_n;
     c->line_n = src->line_n;
+    // the tuned tile width, which changes the time of a step and not its result
+    if (tensor(*c) && src->x_bn) {
+        if (!make_x_maps(*c, src->x_bn, c->maps_x)) {
+            tdb_destroy(c);
+            *out = nullptr;
+            set_err("cuTensorMapEncodeTiled failed");
+            return TDB_ERR_CUDA;
+        }
+        c->x_bn = src->x_bn;
+    }
     return TDB_OK;
 }
 

@@ -422,3 +422,24 @@ def test_damped_transform_needs_no_more_memory_than_its_samples_and_results(B):
         torch.cuda.empty_cache()
     ref = dt * (x[:, :1] + x[:, 1:] * np.exp((1j * om - 1 / t_damp) * dt)[None])
     assert np.max(np.abs(got - ref) / (dt * np.sum(np.abs(x), axis=1, keepdims=True))) < 1e-13
+
+
+def test_clones_step_with_the_tuned_tile_width_of_their_source(B):
+    # a width is tuned once (tens of launches); the clone of a context that has none tunes its own
+    sysm = I.small_flake(40, seed=8)
+    run = I.Run(dt=0.2, n_steps=0, scc=True, kick=1e-3, kT=I.SCC_KT)
+    with B.Propagator(sysm, run, "bf16x3") as p:
+        p.setup()
+        early = B.tdb_clone(p.ctx)
+        B.tdb_set_x_tile(p.ctx, 176)
+        p.step(3)
+        c = B.tdb_clone(p.ctx)
+        assert B.tdb_x_tile(early) == 0 and B.tdb_x_tile(c) == 176
+        for x in (p.ctx, c):
+            B.tdb_step(x, 10)
+        B.tdb_step(early, 13)
+        assert B.tdb_x_tile(c) == 176 and B.tdb_x_tile(early) in (128, 176, 256)
+        state = B.tdb_get_state(p.ctx)
+        assert B.tdb_get_state(c) == state and B.tdb_get_state(early) == state
+        for x in (c, early):
+            B.tdb_destroy(x)
