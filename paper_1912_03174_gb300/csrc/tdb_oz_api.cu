@@ -11,8 +11,11 @@ namespace tdb {
 void set_last_error(const char* msg);
 }
 
-extern "C" tdb_status tdb_slice_gemm(int M, int N, int K, const double* A, const double* B,
-                                     double* C, double* ms) {
+namespace {
+
+// scheme kSix: B is K x N; kSeven: B is the transpose, N x K, sliced by rows as the propagator does
+tdb_status slice_gemm(int scheme, int M, int N, int K, const double* A, const double* B, double* C,
+                      double* ms) {
     namespace oz = tdb::oz;
     if (M < 1 || N < 1 || K < 1 || !A || !B || !C || M > 32768 || N > 32768 || K > oz::kMaxK) {
         tdb::set_last_error("tdb_slice_gemm: invalid sizes or pointers (K <= 4096)");
@@ -33,14 +36,14 @@ extern "C" tdb_status tdb_slice_gemm(int M, int N, int K, const double* A, const
     ok(cudaMalloc(&dB, sizeof(double) * K * N));
     ok(cudaMalloc(&dC, sizeof(double) * M * N));
     ok(cudaMalloc(&colmax, sizeof(double) * N));
-    ok(cudaMalloc(&bufA, oz::sliced_bytes(M, K)));
-    ok(cudaMalloc(&bufB, oz::sliced_bytes(N, K)));
+    ok(cudaMalloc(&bufA, oz::sliced_bytes(M, K, scheme)));
+    ok(cudaMalloc(&bufB, oz::sliced_bytes(N, K, scheme)));
     ok(cudaMalloc(&err, sizeof(int)));
     ok(cudaEventCreate(&e0));
     ok(cudaEventCreate(&e1));
     oz::Sliced sa, sb;
     if (rc == TDB_OK &&
-        (!oz::sliced_init(sa, bufA, M, K, 128) || !oz::sliced_init(sb, bufB, N, K, 64)))
+        (!oz::sliced_init(sa, bufA, M, K, 128, scheme) || !oz::sliced_init(sb, bufB, N, K, 64, scheme)))
         rc = TDB_ERR_CUDA;
     if (rc == TDB_OK) {
         ok(oz::prepare());
@@ -48,7 +51,10 @@ extern "C" tdb_status tdb_slice_gemm(int M, int N, int K, const double* A, const
         ok(cudaMemcpyAsync(dA, A, sizeof(double) * M * K, cudaMemcpyHostToDevice, st));
         ok(cudaMemcpyAsync(dB, B, sizeof(double) * K * N, cudaMemcpyHostToDevice, st));
         oz::slice_rows(dA, K, 1.0, sa, st);
-        oz::slice_cols(dB, N, sb, colmax, st);
+        if (scheme == oz::kSeven)
+            oz::slice_rows(dB, K, 1.0, sb, st);
+        else
+            oz::slice_cols(dB, N, sb, colmax, st);
         ok(cudaGetLastError());
         oz::Part part;
         part.b = &sb;
@@ -80,4 +86,18 @@ extern "C" tdb_status tdb_slice_gemm(int M, int N, int K, const double* A, const
     if (e1) cudaEventDestroy(e1);
     if (st) cudaStreamDestroy(st);
     return rc;
+}
+
+}  // namespace
+
+extern "C" tdb_status tdb_slice_gemm(int M, int N, int K, const double* A, const double* B,
+                                     double* C, double* ms) {
+    return slice_gemm(tdb::oz::kSix, M, N, K, A, B, C, ms);
+}
+
+// The seven-digit product of the FP64 form and the damped transforms on its own, for its test:
+// C = A Bt^T.
+extern "C" tdb_status tdb_test_slice_gemm7(int M, int N, int K, const double* A, const double* Bt,
+                                           double* C) {
+    return slice_gemm(tdb::oz::kSeven, M, N, K, A, Bt, C, nullptr);
 }

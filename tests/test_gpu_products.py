@@ -443,3 +443,79 @@ def test_clones_step_with_the_tuned_tile_width_of_their_source(B):
         assert B.tdb_get_state(c) == state and B.tdb_get_state(early) == state
         for x in (c, early):
             B.tdb_destroy(x)
+
+
+# N = 48, 188 and 192 (the largest size of that inverse)
+@pytest.mark.parametrize("n_atoms,s0", [(12, 7.1373463), (47, 6.7347821), (48, 6.8602551)])
+def test_the_fp64_repair_of_an_ill_conditioned_inverse_is_needed_and_taken(B, n_atoms, s0):
+    # cond(S) = 1.09e6.  A stable FP64 inverse and ground state leave a small multiple of N cond 2^-52
+    # of the forces (three eigensolvers differ by 2e-9); two Newton-Schulz steps from an FP32 inverse
+    # without the repair leave 1e-6 to 4e-5, at least 19 times the bound
+    import dataclasses
+    sysm = dataclasses.replace(I.small_cluster(n_atoms, seed=5), s0=s0)
+    S, H0 = O.model_matrices(sysm, sysm.R)
+    ev = np.linalg.eigvalsh(S)
+    run = I.Run(dt=1e-6, n_steps=0, scc=False, move_nuclei=True, kT=I.SCC_KT)
+    with B.Propagator(sysm, run, "fp64") as p:
+        p.setup()
+        f = p.observables(forces=True)["forces"]
+    rho, gs, S, Sinv = O.setup(sysm, run)
+    G = O.gamma_matrix(sysm, sysm.R)
+    q = O.mulliken(sysm, rho, S) - O.reference_populations(sysm)
+    E = np.zeros(3)
+    v = O.atom_potential(G, q, sysm.R, E, False)
+    ref = O.forces(sysm, rho, S, Sinv, O.scc_hamiltonian(sysm, H0, S, v), G, q, v, sysm.R, E, False)
+    assert np.max(np.abs(f - ref)) < 10 * sysm.n_orb * ev[-1] / ev[0] * 2.0 ** -52 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("n_atoms", [47, 48, 65])
+def test_windows_of_the_fp64_form_match_the_oracle_on_both_sides_of_the_slice_rule(B, n_atoms):
+    # N = 188 (DFMA products), 192 and 260 (slices); the FP64 form's bound of the window tests
+    sysm = I.small_flake(n_atoms, seed=8)
+    run = I.Run(dt=0.2, n_steps=0, scc=True, kick=0.02, kT=I.SCC_KT)
+    with B.Propagator(sysm, run, "fp64") as p:
+        p.setup()
+        p.step(5)
+        rho, prev = B.tdb_get_rho(p.ctx, prev=True)
+        v = B.tdb_scc_shift(p.ctx)
+        B.tdb_step_window(p.ctx, v, 9)
+        got, got_prev = B.tdb_get_rho(p.ctx, prev=True)
+    S, H0 = O.model_matrices(sysm, np.asarray(sysm.R))
+    a, b = O.window_propagate(prev, rho, S, O.scc_hamiltonian(sysm, H0, S, v), run.dt, 9)
+    assert np.max(np.abs(got_prev - a)) < 1e-10
+    assert np.max(np.abs(got - b)) < 1e-10
+
+
+# one element; one K element short of, at and past the exact chunk of 128; ragged tiles; the largest K;
+# "spread" gives a row's elements 60 binades, "extreme" makes every digit product as large as it gets
+# (x0: digits -127, -128, ..., -128) with one sign, which fills the FP32 accumulators and 64-bit sums,
+# "cancel" leaves 2^-40 of the terms' size
+@pytest.mark.parametrize("M,N,K,kind", [(1, 1, 1, "normal"), (5, 7, 127, "normal"), (130, 66, 128, "normal"),
+                                        (129, 65, 129, "spread"), (129, 65, 1025, "normal"),
+                                        (3, 5, 4096, "spread"), (3, 5, 4096, "extreme"),
+                                        (130, 66, 128, "extreme"), (33, 40, 1000, "cancel")])
+def test_seven_digit_slice_products_keep_their_error_bound(B, M, N, K, kind):
+    # operands to 2^-55 of their row's largest value (twice, over K terms), digit pairs from 2^-64 of the
+    # row scales on dropped (20.1 2^-64 of the largest values a term), the sum rounded once
+    import ctypes
+    rng = np.random.default_rng(M + N + K)
+    A, Bt = rng.normal(size=(M, K)), rng.normal(size=(N, K))
+    if kind == "spread":
+        A *= 2.0 ** rng.integers(-60, 1, A.shape)
+        Bt *= 2.0 ** rng.integers(-60, 1, Bt.shape)
+    if kind == "extreme":
+        x0 = (127 + sum(128 * 2.0 ** (-8 * s) for s in range(1, 7))) / 128
+        A[:], Bt[:] = -x0, -x0
+    if kind == "cancel":
+        A[:, K // 2:], Bt[:, K // 2:] = -A[:, :K // 2], Bt[:, :K // 2]
+        A[:, 0] *= 1 + 2.0 ** -40
+    C = np.zeros((M, N))
+    dp = ctypes.POINTER(ctypes.c_double)
+    fn = B.load().tdb_test_slice_gemm7
+    fn.restype, fn.argtypes = ctypes.c_int, [ctypes.c_int] * 3 + [dp] * 3
+    assert fn(M, N, K, B._ptr(A), B._ptr(Bt), B._ptr(C)) == 0
+    ref = A.astype(np.longdouble) @ Bt.T.astype(np.longdouble)
+    eps = float(np.finfo(np.longdouble).eps)   # of the reference's own sums
+    big = K * np.abs(A).max(1)[:, None] * np.abs(Bt).max(1)[None]
+    bound = big * (2.0 ** -54 + 20.1 * 2.0 ** -64 + K * eps) + 2.0 ** -53 * np.abs(ref)
+    assert np.all(np.abs(C - ref) <= bound)
