@@ -877,6 +877,31 @@ def roofline(prof: dict, form: str, N: int, peaks: dict, src: str, ms_step_dev: 
     return out
 
 
+def short_line(line: dict) -> dict:
+    """The line on standard output: the contract's keys, rates per form and the dominant kernel and
+    the step of the roofline, numbers to six digits: well below the 3000 characters that a log's tail may
+    be cut to.  The full line, with every section, goes to standard error."""
+    def six(x):
+        if isinstance(x, dict):
+            return {k: six(v) for k, v in x.items()}
+        if isinstance(x, list):
+            return [six(v) for v in x]
+        return float(f"{x:.6g}") if isinstance(x, float) else x
+
+    def rates(forms):
+        return {f: v["steps_per_s"] for f, v in forms.items()}
+
+    c = line["config"]
+    cfg = {k: c[k] for k in ("workload", "N", "precision", "parallelism", "l2", "fp64_steps_per_s",
+                             "speedup_vs_fp64", "max_dipole_err_vs_fp64_au", "x_tile")}
+    cfg["steps_per_s"] = rates(c["forms"])
+    if c.get("n2048"):
+        cfg["n2048_steps_per_s"] = {k: rates(c["n2048"][k]["forms"]) for k in ("frozen", "ehrenfest_c3")}
+    out = dict(line, config=cfg)
+    out["roofline"] = {k: v for k, v in line["roofline"].items() if k not in ("kernels", "note")}
+    return {k: v if k in ("value", "ms_per_step") else six(v) for k, v in out.items()}
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -1025,7 +1050,8 @@ def main():
     if rank == 0:
         if not args.no_e2e:
             line["e2e"] = e2e_run(B, sysm, run, head, min(args.steps, 100), args.warmup)
-        print(json.dumps(line), flush=True)
+        print(json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(short_line(line)), flush=True)
     if dist:
         dist.barrier()
         dist.destroy_process_group()

@@ -65,3 +65,45 @@ def test_profiled_traffic_is_dropped_when_a_source_changes(tmp_path, monkeypatch
     assert bench._traffic("update", "fp16x6") is None
     src.write_text("kernel v2")
     assert bench._traffic("tc_gemm_X", "fp16x6") is None
+
+
+def test_the_printed_line_keeps_the_contract_and_fits_a_cut_log():
+    # every section as long as a full run makes it; a log keeps the last 3000 characters of a run
+    import json
+    forms = ["fp64", "fp64s", "fp32", "bf16x3", "fp16x3", "fp16x6"]
+    x = 1.0 / 3.0
+    form = {f: {"steps_per_s": x, "max_dipole_err_vs_fp64_au": x, "phase_ms": {str(k): x for k in range(9)}}
+            for f in forms}
+    kernels = {f: {"kernel": f, "note": "n" * 300, "achieved": x} for f in forms}
+    line = {"metric": bench.METRIC, "value": 14085.123456789012, "unit": "steps/s", "n_gpus": 1, "steps": 200,
+            "warmup": 20, "ms_per_step": 0.070997, "higher_is_better": True, "scaling": "weak",
+            "vs_baseline": None, "dtype": "fp16x6", "data": "synthetic",
+            "config": {"workload": bench.WORKLOAD, "N": 1024, "precision": "fp16x6", "parallelism": "replicas",
+                       "l2": "flushed between timed steps (256 MB write)", "fp64_steps_per_s": x,
+                       "speedup_vs_fp64": x, "max_dipole_err_vs_fp64_au": x, "forms": form,
+                       "x_tile": {f: 176 for f in forms[3:]}, "kernel_ms": {f: form for f in forms},
+                       "n2048": {"frozen": {"workload": "w" * 99, "forms": form},
+                                 "ehrenfest_c3": {"workload": "w" * 99, "forms": form, "note": "n" * 99}},
+                       "pump_probe_c4": {str(k): x for k in range(99)}, "learned_c5": kernels,
+                       "accuracy": kernels, "section_seconds": {f: x for f in forms}},
+            "roofline": {"kernel": "tc_gemm_X", "bound": "tensor", "achieved": x, "peak": 1945.7,
+                         "unit": "TFLOP/s", "frac": x, "traffic": None, "peak_source": "m" * 60,
+                         "executed_tflops": x, "executed_frac": x, "note": "n" * 200, "operand_gbs": x,
+                         "operand_hbm_frac": x, "kernels": kernels,
+                         "step": {k: x for k in ("time_us", "tensor_floor_us", "hbm_floor_us", "bound",
+                                                 "algorithmic_bytes", "method_flops", "frac")}},
+            "gpu_launches": 1200,
+            "clocks": {"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "reasons": [], "samples": 956},
+            "cpu_baseline": {"value": x, "unit": "steps/s", "cores": 16, "kind": "oracle", "sample": "s" * 120},
+            "e2e": {"value": x, "unit": "steps/s", "h2d_bytes_per_step": 88, "d2h_bytes_per_step": 24}}
+    short = bench.short_line(line)
+    assert len(json.dumps(short)) < 2900
+    assert short.keys() == line.keys()
+    for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "vs_baseline", "dtype",
+              "data", "gpu_launches", "clocks"):
+        assert short[k] == line[k]
+    assert short["config"]["N"] == 1024 and set(short["config"]["steps_per_s"]) == set(forms)
+    assert set(short["config"]["n2048_steps_per_s"]["frozen"]) == set(forms)
+    assert short["e2e"]["value"] == pytest.approx(x, rel=1e-5)
+    line["config"]["n2048"] = None
+    assert "n2048_steps_per_s" not in bench.short_line(line)["config"]
