@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(kT8* kT8)
 // multiplications then outlast a load).  Nothing may use a loaded value before the
 // multiplications: delta H is formed where B goes to shared memory (formed in the load, it made
 // delta M at N = 1024 take 113 us, now 75; X 178, now 173).  Each output sums its K terms in order.
-constexpr int kF32Tile = 64, kF32K = 32, kF32Threads = 128, kF32Loads = 4, kF32Sms = 152;
+constexpr int kF32Tile = 64, kF32K = 32, kF32Threads = 128, kF32Loads = 4;
 
 struct F32Parts {
     F32Part p[3];
@@ -367,17 +367,19 @@ void run_f32(int M, int Ncol, int K, const F32Parts& p, int nparts, const float*
     for (int z = 0; z < nparts; ++z)
         aligned = aligned && p.p[z].lda % 4 == 0 && p.p[z].ldb % 4 == 0 &&
                   ((reinterpret_cast<uintptr_t>(p.p[z].A) | reinterpret_cast<uintptr_t>(p.p[z].B)) & 15) == 0;
-    // rows without 16-byte alignment go element by element: at N = 70 delta M / X 6.2 / 3.8 us against
-    // 9.5 / 7.4 in 64 x 64 tiles, at N = 801 80 / 142 against 70 / 98
+    // rows without 16-byte alignment are copied element by element, four times the copies of a block:
+    // a step with these tiles / 64 x 64 ones, us: N = 70 23.5 / 30.7, 161 30.9 / 40.0, 193 32.8 / 43.3, 321
+    // 47.1 / 57.3, 385 62.6 / 71.7, 513 95.0 / 90.8, 641 144 / 126.  (The line at 9 tiles, N = 192, is on
+    // the safe side of that crossover.)
     auto go = [&](auto kernel, int tm, int tn, int threads) {
         launch_pdl(kernel, dim3((Ncol + tn - 1) / tn, (M + tm - 1) / tm, nparts), dim3(threads), 0, st, M,
                    Ncol, K, p, dv, add, C2);
     };
-    if (tiles(64, 64) > (aligned ? kF32Sms : 9)) {
+    if (tiles(64, 64) > (aligned ? kSmCount : 9)) {
         go(k_gemm_f32<DHAM>, kF32Tile, kF32Tile, kF32Threads);
     } else {
-        auto fullest = [&](int tm, int tn) { return (tiles(tm, tn) * nparts + kF32Sms - 1) / kF32Sms * tm * tn; };
-        const bool narrow = tiles(64, 32) * nparts > kF32Sms && fullest(32, 32) < fullest(64, 32);
+        auto fullest = [&](int tm, int tn) { return (tiles(tm, tn) * nparts + kSmCount - 1) / kSmCount * tm * tn; };
+        const bool narrow = tiles(64, 32) * nparts > kSmCount && fullest(32, 32) < fullest(64, 32);
         if (narrow)
             go(k_gemm_f32_small<DHAM, F32Narrow>, F32Narrow::M, F32Narrow::N, F32Narrow::T);
         else

@@ -210,7 +210,7 @@ tdb_status transform(bool blocked, int nsig, long K, const double* x, double dt,
     const int groups = (nsig + kMaxSigs - 1) / kMaxSigs, sigs = (nsig + groups - 1) / groups;
     const int gx = (nw + kFreqs - 1) / kFreqs;
     long long nz = std::max<long long>(1, std::min<long long>((K + kSamp - 1) / kSamp,
-                                                              608 / std::max(1, gx * groups)));
+                                                              4 * kSmCount / std::max(1, gx * groups)));
     const long long span = ((K + nz - 1) / nz + kExact - 1) / kExact * kExact;
     nz = (K + span - 1) / span;
 
@@ -226,7 +226,7 @@ tdb_status transform(bool blocked, int nsig, long K, const double* x, double dt,
         bsa = up(oz::sliced_bytes((int)rows, kBlk, oz::kSeven));
         bsb = up(oz::sliced_bytes(2 * cw, kBlk, oz::kSeven));
     } else if (nz > 1) {
-        bp = up(sizeof(double2) * nz * no);   // 608 x 128 x 9 partial sums at most
+        bp = up(sizeof(double2) * nz * no);   // 4 kSmCount x 128 x 9 partial sums at most
     }
     tdb_status rc = TDB_OK;
     cudaStream_t st = nullptr;

@@ -96,7 +96,6 @@ void set_err(const char* fmt, ...) {
         if (s_ != TDB_OK) return s_;   \
     } while (0)
 
-constexpr int kSmCount = 152;
 constexpr int kObsBlocks = 2 * kSmCount;
 
 // Carves named sub-buffers out of one workspace, 256-byte aligned.

@@ -15,6 +15,7 @@
 namespace tdb {
 
 constexpr int kTile = 32;          // tile edge of the O(N^2) kernels (update, Mulliken partials)
+constexpr int kSmCount = 152;
 
 // Laser field parameters as the kernels read them (eq:pumpf).
 struct FieldDev {
@@ -316,7 +317,6 @@ void launch_charges_df(const Ctx& c, const float2* partial, double* q, double* d
 void launch_master_absmax(const Ctx& c, const MasterPtrs& m, double* out, cudaStream_t st);
 void launch_master_pieces(const Ctx& c, const MasterPtrs& m, const UpdateOperands& ops,
                           const double* mx_exact, const float* dev_scale, cudaStream_t st);
-// FP16X6: head pieces of rho - rho_ref (scale from c.dyn->max_drho[slot]) into the B operands
 // FP64 form, frozen nuclei, N <= kSmallStepN: leapfrog steps in one cluster launch (kern_small.cu)
 constexpr int kSmallStepN = 64;
 struct SmallStepArgs {
@@ -330,11 +330,15 @@ struct SmallStepArgs {
 };
 bool small_steps_prepare();   // whether the device can place the cluster
 cudaError_t launch_small_steps(const SmallStepArgs& a, cudaStream_t st);
-// GEMM: C[M x Ncol] = A[M x K] * B[K x Ncol], row-major, FP64 SIMT.
-enum class BKind { Dense = 0, Hamiltonian = 1 };
+// FP64 product C[M x Ncol] = A[M x K] B[K x Ncol], row-major
 void gemm_f64(int M, int Ncol, int K, const double* A, int lda, const double* B, int ldb,
               double* C, int ldc, cudaStream_t st);
-// C = A * H with H_kj = H0_kj + 1/2 S_kj (v_k + v_j) formed while loading B (eq:hscc).
+// C0 = A B0 and C1 = A B1 (N x N) in one launch
+void gemm_f64_pair(int N, const double* A, const double* B0, const double* B1, double* C0,
+                   double* C1, cudaStream_t st);
+// C = A H with H_kj = H0_kj + 1/2 S_kj (v_k + v_j) formed while loading B (eq:hscc)
+void gemm_f64_ham(int N, const double* A, const double* H0, const double* S, const double* v_orb,
+                  double* C, cudaStream_t st);
 // FP32 products C = A B (row-major), up to three of the same shape in one launch
 struct F32Part {
     const float* A;
@@ -348,13 +352,5 @@ void gemm_f32(int M, int Ncol, int K, const F32Part* parts, int nparts, cudaStre
 // dM = A dH with dH_kj = 1/2 S_kj (dv_k + dv_j), and Msum = Mgs + dM (row strides ldc; Mgs: N)
 void gemm_f32_dham(int N, const float* A, const float* S, const float* dv, float* dM, float* Msum,
                    int ldc, const float* Mgs, cudaStream_t st);
-// C0 = A B0 and C1 = A B1 (N x N) in one launch
-void gemm_f64_pair(int N, const double* A, const double* B0, const double* B1, double* C0,
-                   double* C1, cudaStream_t st);
-void gemm_f64_ham(int N, const double* A, const double* H0, const double* S, const double* v_orb,
-                  double* C, cudaStream_t st);
-// FP32 SIMT: C = A * B (+ Cadd if non-null).
-void gemm_f32(int M, int Ncol, int K, const float* A, int lda, const float* B, int ldb, float* C,
-              int ldc, cudaStream_t st);
 
 }  // namespace tdb

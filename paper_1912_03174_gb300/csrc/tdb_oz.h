@@ -14,9 +14,13 @@
 //           K max_k|A_ik| max_k|B_kj| -- the TDB_FP64_SLICED form.
 //   kSeven  7 digits of 8 bits, W = 8 (34 pairs), chunks of 128: 55-bit operands, the
 //           first dropped weight is 2^-64.  On the products of the propagation (S^-1 H,
-//           M rho, N = 132 .. 520) its error is 0.3 to 0.65 of the DFMA product's in the
-//           2-norm and below a tenth of it in the largest element: it replaces the DFMA
-//           product of the TDB_FP64 form where N is large enough (see use_slices).
+//           M Re rho, M Im rho; N = 132 .. 520) its error is 0.29 to 0.61 of the DFMA
+//           product's in the 2-norm and 0.03 to 0.14 in the largest element: it replaces
+//           the DFMA product of the TDB_FP64 form where N is large enough (see use_slices).
+//
+// The bounds are relative to the largest entry of a row of A times that of a column of B: an element
+// of C far below those (rows of S^-1 and rho decay with distance) has their absolute error, not,
+// as from DFMA, a relative one of its own.
 #pragma once
 
 #include <cuda.h>
