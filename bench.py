@@ -8,7 +8,8 @@ dipole, M = S^-1 H, X = M rho, leapfrog update (eq:leapfrog, eq:eomrho).
 The headline value is the reduced-precision form (the fastest form built);
 the FP64 form runs on the same trajectory as the accuracy reference (it is
 itself pinned to the CPU oracle by the parity tests) and as the speed
-baseline.  One JSON line is printed by rank 0.
+baseline.  Rank 0 prints one JSON line, and the same with every section on
+standard error.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 """
